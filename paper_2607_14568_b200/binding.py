@@ -92,6 +92,21 @@ def lib():
     return _lib
 
 
+_call = None
+
+
+def _native():
+    """The native side of this binding (csrc/py_call.cpp): one function per entry point that checks the tensors,
+    calls the library and returns its status, or -1 for arguments it does not take.  The Python code behind it words
+    the error for those, and serves the few forms only it converts (a stream or chunk that is not a plain int)."""
+    global _call
+    if _call is None:
+        lib()                       # raises if the library has not been built
+        from . import _call as module
+        _call = module
+    return _call
+
+
 def gdn_status_string(status: int) -> str:
     return lib().gdn_status_string(int(status)).decode()
 
@@ -170,6 +185,12 @@ def _stream(stream):
 
 def _prefill(fn_name, io_dtype, q, k, v, log_alpha, beta, initial_state, out, final_state,
              cu_seqlens, chunk, stream):
+    rc = getattr(_call or _native(), fn_name)(q, k, v, log_alpha, beta, initial_state, out, final_state, cu_seqlens, chunk,
+                                              stream)
+    if rc == 0:
+        return out, final_state
+    if rc > 0:
+        raise GdnError(rc, fn_name)
     f32 = torch.float32
     _check([("q", q, io_dtype), ("k", k, io_dtype), ("v", v, io_dtype), ("out", out, io_dtype),
             ("log_alpha", log_alpha, f32), ("beta", beta, f32), ("initial_state", initial_state, f32),
@@ -246,6 +267,12 @@ def gdn_chunk_prefill_raw(q_raw, k_raw, v, a_raw, b_raw, gate_scale, norm_eps, i
                           cu_seqlens=None, chunk: int = 64, stream=None):
     """gdn_chunk_prefill on raw projections: the L2 norms of q, k and the gates sigmoid(b_raw),
     -softplus(a_raw) * gate_scale are computed inside the kernels.  Needs gdn_set_workspace.  See include/gdn.h."""
+    rc = (_call or _native()).gdn_chunk_prefill_raw(q_raw, k_raw, v, a_raw, b_raw, gate_scale, norm_eps, initial_state, out,
+                                                    final_state, cu_seqlens, chunk, stream)
+    if rc == 0:
+        return out, final_state
+    if rc > 0:
+        raise GdnError(rc, "gdn_chunk_prefill_raw")
     f32, bf = torch.float32, torch.bfloat16
     _check([("q_raw", q_raw, bf), ("k_raw", k_raw, bf), ("v", v, bf), ("out", out, bf), ("a_raw", a_raw, f32),
             ("b_raw", b_raw, f32), ("initial_state", initial_state, f32), ("final_state", final_state, f32),
@@ -270,6 +297,12 @@ def gdn_chunk_prefill_gated(q, k, v, log_alpha, beta, initial_state, gate_z, nor
                             cu_seqlens=None, chunk: int = 64, stream=None):
     """gdn_chunk_prefill with the output stage fused in: out = o / sqrt(mean o^2 + norm_eps) * norm_weight * silu(gate_z)
     per (token, head); gate_z bf16 like out, norm_weight fp32 [d_v].  Needs gdn_set_workspace.  See include/gdn.h."""
+    rc = (_call or _native()).gdn_chunk_prefill_gated(q, k, v, log_alpha, beta, initial_state, gate_z, norm_weight, norm_eps,
+                                                      out, final_state, cu_seqlens, chunk, stream)
+    if rc == 0:
+        return out, final_state
+    if rc > 0:
+        raise GdnError(rc, "gdn_chunk_prefill_gated")
     f32, bf = torch.float32, torch.bfloat16
     _check([("q", q, bf), ("k", k, bf), ("v", v, bf), ("out", out, bf), ("gate_z", gate_z, bf), ("log_alpha", log_alpha, f32),
             ("beta", beta, f32), ("initial_state", initial_state, f32), ("final_state", final_state, f32),
@@ -290,6 +323,12 @@ def gdn_chunk_prefill_gated(q, k, v, log_alpha, beta, initial_state, gate_z, nor
 def gdn_attn_causal_prefill(q, k, v, out, scale=None, cu_seqlens=None, stream=None):
     """Causal softmax attention with grouped queries: q, out [B,T,Hq,d], k, v [B,T,Hkv,d] bf16 on the device
     (packed [T,H,d] with int32 cu_seqlens [B+1]); scale defaults to 1/sqrt(d).  See include/gdn_attn.h."""
+    rc = (_call or _native()).gdn_attn_causal_prefill(q, k, v, out, cu_seqlens, float(q.shape[-1]) ** -0.5 if scale is None else scale,
+                                                      stream)
+    if rc == 0:
+        return out
+    if rc > 0:
+        raise GdnError(rc, "gdn_attn_causal_prefill")
     bf = torch.bfloat16
     _check([("q", q, bf), ("k", k, bf), ("v", v, bf), ("out", out, bf), ("cu_seqlens", cu_seqlens, torch.int32)],
            bf, "cuda")
@@ -314,6 +353,11 @@ def gdn_attn_causal_prefill(q, k, v, out, scale=None, cu_seqlens=None, stream=No
 def gdn_decode_step(q, k, v, log_alpha, beta, state, out, stream=None):
     """One token per sequence: q, k [B,H,d_k], v, out [B,H,d_v] bf16; log_alpha, beta [B,H] fp32;
     state [B,H,d_k,d_v] fp32, updated in place.  See include/gdn.h."""
+    rc = (_call or _native()).gdn_decode_step(q, k, v, log_alpha, beta, state, out, stream)
+    if rc == 0:
+        return out, state
+    if rc > 0:
+        raise GdnError(rc, "gdn_decode_step")
     f32, bf = torch.float32, torch.bfloat16
     _check([("q", q, bf), ("k", k, bf), ("v", v, bf), ("out", out, bf), ("log_alpha", log_alpha, f32),
             ("beta", beta, f32), ("state", state, f32)], bf, "cuda")
