@@ -98,7 +98,7 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     volatile uint32_t* sMisc = reinterpret_cast<volatile uint32_t*>(sm + AS_MISC);
     AWaiter w{base + AS_BARS, reinterpret_cast<volatile int*>(sm + AS_MISC + 4)};
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     // which sequence and which pair of query tiles: batched input takes them from the grid; packed input
     // walks the sequence boundaries (grid.y covers an upper bound of the pair count, the surplus CTAs leave)
     int tok0, len, t;
@@ -255,8 +255,10 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
         }
     } else if (warp == 8) {
-        // =========================== MMA issue (one thread) ===========================
-        if (lane == 0) {
+        // =========================== MMA issue (one elected thread) ===========================
+        {
+            const uint32_t tmem = warp_uniform(sMisc[0]);
+            const bool lead = elect_one();
             // operand descriptors are built once: issuing costs tens of nanoseconds per instruction and
             // sits on each tile's softmax -> P V -> Q K^T chain
             const uint64_t dq0 = make_smem_desc(base + AS_Q, 16, 1024), dk0 = make_smem_desc(base + AS_K, 16, 1024);
@@ -266,15 +268,15 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (uint32_t ks = 0; ks < 8; ++ks) {
                     const uint64_t off = ((ks >> 2) * 16384 + (ks & 3) * 32) >> 4;   // the address field counts 16 bytes
-                    mma_ss(tmem + TM_S + X * 128, dq + off, dk + off, ID_QK, ks > 0);
+                    if (lead) mma_ss(tmem + TM_S + X * 128, dq + off, dk + off, ID_QK, ks > 0);
                 }
-                mma_commit(w.bar(AB_SFULL0 + X));
+                if (lead) mma_commit(w.bar(AB_SFULL0 + X));
             };
             auto issue_pv = [&](uint32_t X, int j) {       // O_X += P_X V_j, 16 keys per step
                 const uint64_t dv = dv0 + ((uint64_t)((j & 1) * TILE_BYTES) >> 4);
 #pragma unroll
                 for (uint32_t ks = 0; ks < 8; ++ks)
-                    mma_ts(tmem + TM_O + X * 128, tmem + TM_S + X * 128 + ks * 8, dv + ((ks * 2048) >> 4), ID_PV,
+                    if (lead) mma_ts(tmem + TM_O + X * 128, tmem + TM_S + X * 128 + ks * 8, dv + ((ks * 2048) >> 4), ID_PV,
                            (j > 0 || ks > 0) ? 1u : 0u);
             };
             w.wait(AB_Q, 0);
@@ -282,7 +284,7 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             tc_fence_after_sync();
             issue_qk(0, 0);
             if (hasB) issue_qk(1, 0);
-            mma_commit(w.bar(AB_KFREE0));
+            if (lead) mma_commit(w.bar(AB_KFREE0));
             for (int j = 0; j < ntiles; ++j) {
                 const uint32_t s = j & 1, s1 = (j + 1) & 1;
                 const bool more = (j + 1 < ntiles);
@@ -297,7 +299,7 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (j + 1 < nA) {
                         issue_qk(0, j + 1);
                     } else {
-                        mma_commit(w.bar(AB_PVDONE0 + 0));
+                        if (lead) mma_commit(w.bar(AB_PVDONE0 + 0));
                     }
                 }
                 if (hasB) {
@@ -307,11 +309,11 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (more) {
                         issue_qk(1, j + 1);
                     } else {
-                        mma_commit(w.bar(AB_PVDONE0 + 1));
+                        if (lead) mma_commit(w.bar(AB_PVDONE0 + 1));
                     }
                 }
-                mma_commit(w.bar(AB_VFREE0 + s));
-                if (more) mma_commit(w.bar(AB_KFREE0 + s1));
+                if (lead) mma_commit(w.bar(AB_VFREE0 + s));
+                if (more && lead) mma_commit(w.bar(AB_KFREE0 + s1));
             }
         }
     } else {

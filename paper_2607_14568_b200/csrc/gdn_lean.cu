@@ -250,7 +250,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     volatile uint32_t* sMisc = reinterpret_cast<volatile uint32_t*>(sm + PS_MISC);
     Waiter w{base + PS_BARS, reinterpret_cast<volatile int*>(sm + PS_MISC + 4)};
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int H = p.H;
     pdl_trigger();                      // the next kernel of the call may set itself up while this one runs
     if (tid == 0) {
@@ -267,7 +267,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = sMisc[0];
+    const uint32_t tmem = warp_uniform(sMisc[0]);
 
     // Items are handed out through a global ticket: the time per item differs between SMs by a
     // quarter, so a fixed assignment would leave the fast ones idle at the end.  The issuing thread
@@ -275,16 +275,21 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const long nitems = p.nslots * H;
     int nh = 0, nR = 0;      // issuing thread: head, first token of the item it drew last
     long ntok = 0;
-    auto draw = [&]() -> int {           // next ticket that names a used slot, or -1
+    auto draw = [&]() -> int {           // (whole warp 4) next ticket that names a used slot, or -1
         while (true) {
-            const int t = atomicAdd(p.ticket, 1);
+            int t = 0;
+            if (lane == 0) t = atomicAdd(p.ticket, 1);
+            t = (int)warp_uniform((uint32_t)t);
             if (t >= nitems) return -1;
             if (decode_item(p, t, &nh, &ntok, &nR)) return t;
         }
     };
-    if (warp == 4 && lane == 0) {
-        sMisc[2] = (uint32_t)draw();
-        mbar_arrive(w.bar(PB_ITEM));
+    if (warp == 4) {
+        const int first = draw();
+        if (lane == 0) {
+            sMisc[2] = (uint32_t)first;
+            mbar_arrive(w.bar(PB_ITEM));
+        }
     }
     int it = 0;     // items this CTA has processed (barrier phases)
     while (true) {
@@ -581,11 +586,13 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             tc_fence_before_sync();
             mbar_arrive(w.bar(PB_DONE));
         } else if (warp == 4) {
-            // ================= TMA + MMA issue (one thread) =================
-            if (lane == 0) {
+            // ================= TMA + MMA issue (one elected thread) =================
+            {
+                const bool lead = elect_one();
                 const uint32_t kq = base + PS_KQ, full = w.bar(PB_FULL);
                 const uint64_t pol_k = (p.l2 & 1) ? l2_policy_evict_last() : l2_policy_evict_normal();
                 auto load_tiles = [&](int hh, long tk) {
+                    if (!lead) return;
                     mbar_arrive_expect_tx(full, 32768);
                     tma_load_3d_hint(kq, &map_k, 0, hh, (int)tk, full, pol_k);
                     tma_load_3d_hint(kq + 16384, &map_k, 64, hh, (int)tk, full, pol_k);
@@ -599,24 +606,26 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
                 for (uint32_t ks = 0; ks < 8; ++ks) {
                     const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-                    mma_ss(tmem, make_smem_desc(kq + off, 16, 1024), make_smem_desc(kq + off, 16, 1024), ID_G, ks > 0);
+                    if (lead) mma_ss(tmem, make_smem_desc(kq + off, 16, 1024), make_smem_desc(kq + off, 16, 1024), ID_G, ks > 0);
                 }
-                mma_commit(w.bar(PB_G));
+                if (lead) mma_commit(w.bar(PB_G));
                 const int nxt = draw();                             // the atomic's latency hides behind the solve
                 w.wait(PB_TREADY, par);
                 tc_fence_after_sync();
 #pragma unroll
                 for (uint32_t ks = 0; ks < 4; ++ks)
-                    mma_ss(tmem, make_smem_desc(kq + ks * 2048, 16384, 1024),
+                    if (lead) mma_ss(tmem, make_smem_desc(kq + ks * 2048, 16384, 1024),
                            make_smem_desc(base + PS_T1 + ks * 2048, 1024, 1024), ID_WU, ks > 0);
-                mma_commit(w.bar(PB_W));
+                if (lead) mma_commit(w.bar(PB_W));
                 // request the tiles of the next item as soon as the K/Q space is free, then publish it
                 if (nxt >= 0) {
                     w.wait(PB_KQFREE, par);
                     load_tiles(nh, ntok);
                 }
-                sMisc[2 + ((it + 1) & 1)] = (uint32_t)nxt;
-                mbar_arrive(w.bar(PB_ITEM));
+                if (lead) {
+                    sMisc[2 + ((it + 1) & 1)] = (uint32_t)nxt;
+                    mbar_arrive(w.bar(PB_ITEM));
+                }
             }
         } else {
             // ================= step a: chunk-local cumulative log gate (one warp) =================
@@ -770,7 +779,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                                            const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
     const int n = cta.z / p.nseg, seg = cta.z % p.nseg;
     const int H = p.H, dv = p.dv;
@@ -1031,7 +1040,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     } else {
         // =============================== control warpgroup ===============================
         if (!SCAN) setmaxnreg_dec<56>();
-        if (warp == 8 && lane == 0) {
+        if (warp == 8) {
+            const bool lead = elect_one();
             // ---- MMA issuer of the sequential chain: v_new and the state update, nothing else ----
             // (issuing costs tens of nanoseconds per instruction; everything off the chain is
             //  issued by a second thread so that it does not sit between two dependent steps)
@@ -1049,23 +1059,24 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 if (c == tail_c) w.wait_hot(CB_CLEAN, 0);      // padded K rows have been cleared
                 w.wait_hot(CB_SREADY, c & 1);
                 tc_fence_after_sync();
-                stamp(1, c, 0);
+                if (lead) stamp(1, c, 0);
 #pragma unroll
                 for (uint32_t ks = 0; ks < 8; ++ks)            // v^T = U^T - S^T W^T
-                    mma_ts(tmem + TM_DV, tmem + TM_SBF + ks * 8, dW + ks * 128, ID_1, 1);
-                mma_commit(w.bar(CB_V));
-                stamp(1, c, 1);
+                    if (lead) mma_ts(tmem + TM_DV, tmem + TM_SBF + ks * 8, dW + ks * 128, ID_1, 1);
+                if (lead) mma_commit(w.bar(CB_V));
+                if (lead) stamp(1, c, 1);
                 w.wait_hot(CB_VREADY, c & 1);
                 tc_fence_after_sync();
-                stamp(1, c, 3);
+                if (lead) stamp(1, c, 3);
 #pragma unroll
                 for (uint32_t ks = 0; ks < 4; ++ks)            // dS^T = (v e^{gC-g})^T K
-                    mma_ts(tmem + TM_DS, tmem + TM_VT + ks * 8, dK + ks * 128, ID_2, ks > 0);
-                mma_commit(w.bar(CB_S));
-                mma_commit(w.bar(CB_FREEA0 + s));
-                stamp(1, c, 4);
+                    if (lead) mma_ts(tmem + TM_DS, tmem + TM_VT + ks * 8, dK + ks * 128, ID_2, ks > 0);
+                if (lead) mma_commit(w.bar(CB_S));
+                if (lead) mma_commit(w.bar(CB_FREEA0 + s));
+                if (lead) stamp(1, c, 4);
             }
-        } else if (warp == 10 && lane == 0) {
+        } else if (warp == 10) {
+            const bool lead = elect_one();
             // ---- MMA issuer of everything off the chain: U^T, O1^T, O2^T ----
             // (descriptors are built once; a stage or a k-step is an add on the 16-byte address field.  Every warp
             //  role runs its loop at the same time, so the size of these loops shows in the instruction cache.)
@@ -1082,9 +1093,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 8; ++ks)        // O1^T = S^T Q^T
-                        mma_ts(tmem + TM_O1, tmem + TM_SBF + ks * 8, dQ0 + soff + (uint64_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4),
+                        if (lead) mma_ts(tmem + TM_O1, tmem + TM_SBF + ks * 8, dQ0 + soff + (uint64_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4),
                                ID_O, ks > 0);
-                    mma_commit(w.bar(CB_O1));
+                    if (lead) mma_commit(w.bar(CB_O1));
                     w.wait(CB_VREADY, c & 1);
                     tc_fence_after_sync();
                 }
@@ -1095,16 +1106,16 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     if (c + 1 == tail_c) w.wait(CB_CLEAN, 0);  // padded V rows have been cleared
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)
-                        mma_ss(tmem + TM_DV, dV0 + boff + ks * 128, dT0 + boff + ks * 128, ID_WU, ks > 0);
-                    mma_commit(w.bar(CB_FREEB0 + sB));
-                    mma_commit(w.bar(CB_U));
+                        if (lead) mma_ss(tmem + TM_DV, dV0 + boff + ks * 128, dT0 + boff + ks * 128, ID_WU, ks > 0);
+                    if (lead) mma_commit(w.bar(CB_FREEB0 + sB));
+                    if (lead) mma_commit(w.bar(CB_U));
                 }
                 if (c >= 0) {
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)        // O2^T = v^T P^T
-                        mma_ts(tmem + TM_O2, tmem + TM_V + ks * 8, dP0 + soff + ks * 2, ID_O, ks > 0);
-                    mma_commit(w.bar(CB_O));
-                    mma_commit(w.bar(CB_FREEA0 + s));
+                        if (lead) mma_ts(tmem + TM_O2, tmem + TM_V + ks * 8, dP0 + soff + ks * 2, ID_O, ks > 0);
+                    if (lead) mma_commit(w.bar(CB_O));
+                    if (lead) mma_commit(w.bar(CB_FREEA0 + s));
                 }
             }
         } else if (warp == 9 && lane == 0) {
@@ -1174,7 +1185,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = sMisc[0];
+    const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_wait();                         // scratch items and incoming states come from the kernels before this one
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
     chain_body<DBG, false, GATED>(&map_q, &map_k, &map_v, p, cta, w, Handover{nullptr, 0});
@@ -1245,7 +1256,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                                              const Cta& cta, const Waiter& w) {
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
     const int nsum = p.nseg - 1;                      // the last segment needs no summary
     const int n = cta.z / nsum, seg = cta.z % nsum;
@@ -1353,7 +1364,8 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     } else {
         // =============================== control warpgroup ===============================
         if (!SCAN) setmaxnreg_dec<56>();
-        if ((warp == 8 || warp == 10) && lane == 0) {
+        if (warp == 8 || warp == 10) {
+            const bool lead = elect_one();
             // ---- one MMA issue thread per chain instance (they are independent) ----
             const int inst = (warp == 8) ? 0 : 1;
             if (inst < ninst) {
@@ -1366,24 +1378,24 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                         tc_fence_after_sync();
 #pragma unroll
                         for (uint32_t ks = 0; ks < 4; ++ks)        // U^T = V^T (T diag(b))^T
-                            mma_ss(tmem + sum_dv(0), make_smem_desc(sb + SS_V + ks * 2048, 8192, 1024),
+                            if (lead) mma_ss(tmem + sum_dv(0), make_smem_desc(sb + SS_V + ks * 2048, 8192, 1024),
                                    make_smem_desc(sb + SS_T2 + ks * 2048, 1024, 1024), ID_WU, ks > 0);
                     }
                     w.wait_hot(SB_SREADY0 + inst, c & 1);
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 8; ++ks)            // v^T = U^T - S^T W^T   (U = 0 for the identity chain)
-                        mma_ts(tmem + sum_dv(inst), tmem + sum_ds(inst) + ks * 8,
+                        if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_ds(inst) + ks * 8,
                                dW + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
-                    mma_commit(w.bar(SB_V0 + inst));
+                    if (lead) mma_commit(w.bar(SB_V0 + inst));
                     w.wait_hot(SB_VREADY0 + inst, c & 1);
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)            // dS^T = (v e^{gC-g})^T K
-                        mma_ts(tmem + sum_ds(inst), tmem + sum_vt(inst) + ks * 8,
+                        if (lead) mma_ts(tmem + sum_ds(inst), tmem + sum_vt(inst) + ks * 8,
                                dK + ks * 128, ID_2, ks > 0);
-                    mma_commit(w.bar(SB_S0 + inst));
-                    mma_commit(w.bar(SB_FREE0 + s));
+                    if (lead) mma_commit(w.bar(SB_S0 + inst));
+                    if (lead) mma_commit(w.bar(SB_FREE0 + s));
                 }
             }
         } else if (warp == 9 && lane == 0) {
@@ -1438,7 +1450,7 @@ gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = sMisc[0];
+    const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
     pdl_wait();                         // the scratch items come from the prepare kernel
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
@@ -1493,7 +1505,7 @@ __device__ __forceinline__ void combine_init_bars(const Waiter& w) {
 template <bool SCAN>
 __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& cta, const Waiter& w, int issue_warp) {
     const uint32_t base = cta.base, tmem = cta.tmem;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int j0 = cta.dvb * CMB_COLS, h = cta.h, n = cta.z;
     const int H = p.H, dv = p.dv, nhops = p.nseg - 1;
     auto seg_off = [&](int seg) { return ((size_t)(n * p.nseg + seg) * H + h) * DK * dv; };
@@ -1558,7 +1570,8 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
             }
         }
         store_sin(nhops);
-    } else if (warp >= issue_warp && warp < issue_warp + 3 && lane == 0) {
+    } else if (warp >= issue_warp && warp < issue_warp + 3) {
+        const bool lead = elect_one();
         // ---- MMA issue, one thread per partial product (issuing costs tens of nanoseconds per instruction and the
         //      three products are independent); the first of them also copies the M images ----
         const uint32_t prod = (uint32_t)(warp - issue_warp);            // hi*hi, lo*hi, hi*lo
@@ -1567,6 +1580,7 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
         auto load_m = [&](int seg) {
             const uint32_t st = seg % CMB_STAGES, full = w.bar(MB_FULL0 + st);
             const uint8_t* src = reinterpret_cast<const uint8_t*>(p.seg_mt) + ((size_t)(n * p.nseg + seg) * H + h) * CMB_IMG;
+            if (!lead) return;
             mbar_arrive_expect_tx(full, CMB_IMG);
 #pragma unroll
             for (uint32_t q = 0; q < 4; ++q) bulk_load(base + st * CMB_IMG + q * 16384, src + q * 16384, 16384, full);
@@ -1581,10 +1595,10 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
             tc_fence_after_sync();
 #pragma unroll
             for (uint32_t ks = 0; ks < 8; ++ks)
-                mma_ss(tmem + prod * CMB_COLS, make_smem_desc(ma + (ks >> 2) * 16384 + (ks & 3) * 2048, 8192, 1024),
+                if (lead) mma_ss(tmem + prod * CMB_COLS, make_smem_desc(ma + (ks >> 2) * 16384 + (ks & 3) * 2048, 8192, 1024),
                        dB0 + (uint64_t)(((ks >> 2) * (CMB_COLS * 128) + (ks & 3) * 32) >> 4), ID_CMB, ks ? 1u : 0u);
-            mma_commit(w.bar(MB_D));
-            mma_commit(w.bar(MB_FREE0 + st));
+            if (lead) mma_commit(w.bar(MB_D));
+            if (lead) mma_commit(w.bar(MB_FREE0 + st));
             if (prod == 0 && seg + (int)CMB_STAGES < nhops) {
                 w.wait(MB_FREE0 + st, (seg / CMB_STAGES) & 1);   // the tensor core has read this stage for all three products
                 load_m(seg + CMB_STAGES);
@@ -1618,7 +1632,7 @@ __global__ void __launch_bounds__(CMB_THREADS, 1) gdn_combine_kernel(CombinePara
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = sMisc[0];
+    const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
     combine_body<false>(p, cta, w, 4);
@@ -1701,7 +1715,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = sMisc[0];
+    const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_wait();                         // the scratch items come from the prepare kernel
     auto stamp = [&](int ev) {
         if (DBG && p.cp.dbg && tid == 0 && h == 0 && n == 0 && seg < 16)

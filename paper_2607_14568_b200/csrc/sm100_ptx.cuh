@@ -211,6 +211,17 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                  : "memory");
 }
 
+// Issuing from one thread of a converged warp: the warp runs the loop, the waits and the address arithmetic together and
+// only the instruction itself is predicated, so the compiler sees warp-uniform values and keeps descriptors
+// and tensor-memory addresses in uniform registers.  Inside `if (lane == 0)` each operand of each MMA is first moved
+// there from a vector register.  Measured: attention at 10240 tokens 396 -> 363 us.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-serialization attribute may start while its predecessor in the
 // stream is still running; pdl_wait() blocks until that predecessor has completed and its writes are
