@@ -154,14 +154,20 @@ __device__ __forceinline__ void bulk_store_hint(void* gdst, uint32_t smem_src, u
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;"
                  ::"l"(reinterpret_cast<uint64_t>(gdst)), "r"(smem_src), "r"(bytes), "l"(pol) : "memory");
 }
-// 16 bytes global -> shared by one thread, waited for by the same thread
-__device__ __forceinline__ void cp_async16(uint32_t smem_dst, const void* gsrc) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(gsrc)) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// z / (1 + e^-z); the reciprocal is refined by one Newton step (about one unit in the last place, as a division, without
+// the branches of one: 64 of them per thread and chunk took longer than the chain step they must hide behind)
+__device__ __forceinline__ float silu(float z) {
+    const float d = 1.0f + __expf(-z);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    r = r * fmaf(-d, r, 2.0f);
+    return d > 8e37f ? 0.0f : z * r;
+}
 
 // slot of chunk 0 of sequence n: disjoint ranges for any lengths, total <= tokens/64 + B
 __device__ __forceinline__ long slot_base(long tok0, int n) { return (tok0 >> 6) + n; }
@@ -680,29 +686,37 @@ constexpr int CHAIN_THREADS = 384;
 // tensor memory columns
 constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384;
 constexpr uint32_t CT_COLS = 512;
-// shared memory: two stages of {K/Q tiles, V tile, -W^T, T2, P, gates}
-// shared memory: operands are staged in two rings with different lifetimes.
-//   ring A (2 deep): K/Q tiles, -W^T, P   -- used from the v_new MMA of a chunk to its last output MMA
-//   ring B (3 deep): V tile, (T diag b)^T -- used only by the U^T MMA, which is issued one chunk early
-//   gate vectors (4 deep): read by threads, not by MMAs; a slot is reused four chunks later, when
-//   every reader of its previous contents has provably finished (no barrier needed)
-// A slot is released by the completion of the last MMA that reads it, so its refill starts early.
-constexpr uint32_t ST_KQ = 0, ST_W = 32768, ST_P = 49152;
-constexpr uint32_t STAGE_A = 57344, STAGE_A_TX = 32768 + 16384 + 8192 + 1280;   // + the gate vectors
+// shared memory: every operand has a ring of its own, released by the completion of the MMAs that read it, so that a
+// slot is refilled as soon as its one use is over and a load has well over a chunk step to arrive.  (With
+// K, Q, -W and P in one two-deep ring, released together by the last of them, a load could only start when its
+// chunk's predecessor but one was completely done: a CTA by itself then ran at half the sum of load latency and
+// step, 1.55 us a chunk, its issuing thread waiting for tiles two thirds of the time.)
+//   -W^T    2 deep   v_new MMA
+//   Q       2 deep   O1 MMA
+//   K       2 deep   state-update MMA
+//   P       2 deep   O2 MMA
+//   V, T2   2 deep   U^T MMA, which is issued one chunk early
+//   gate vectors: 6 deep, read by threads, not by MMAs; they arrive with -W^T and a slot is reused six chunks later,
+//   when every reader of its previous contents has provably finished (no barrier needed)
 constexpr uint32_t ST_V = 0, ST_T2 = 16384;
 constexpr uint32_t STAGE_B = 24576, STAGE_B_TX = 16384 + 8192;
-constexpr uint32_t CS_A = 0, CS_B = 2 * STAGE_A, CS_GATES = CS_B + 3 * STAGE_B;
-constexpr uint32_t CS_OST = CS_GATES + 4 * 1280;       // bf16 output staging [64][128]
-constexpr uint32_t CS_BARS = CS_OST + 16384;
-constexpr uint32_t CS_MISC = CS_BARS + 24 * 8;
+constexpr uint32_t CS_W = 0, CS_Q = CS_W + 2 * 16384, CS_K = CS_Q + 2 * 16384, CS_P = CS_K + 2 * 16384;
+constexpr uint32_t CS_B = CS_P + 2 * 8192;
+constexpr uint32_t GATE_SLOTS = 6;
+constexpr uint32_t CS_OST = CS_B + 2 * STAGE_B;        // two output tiles [2 halves of the columns][64 tokens][64], 128-byte swizzle
+constexpr uint32_t CS_GATES = CS_OST + 2 * 16384;
+constexpr uint32_t CS_BARS = (CS_GATES + GATE_SLOTS * 1280 + 1023) / 1024 * 1024;
+constexpr uint32_t CS_MISC = CS_BARS + 32 * 8;
 constexpr uint32_t CS_TOTAL = CS_MISC + 64;
 constexpr uint32_t CHAIN_SMEM = CS_TOTAL + 1024;
-constexpr uint32_t CS_Z = CS_TOTAL;                    // fused output stage only: gate_z of one chunk, 16 KiB
-constexpr uint32_t CHAIN_SMEM_GATED = CHAIN_SMEM + 16384;
-static_assert(CS_Z % 16 == 0 && CHAIN_SMEM_GATED <= 232448, "shared memory per CTA");
+// fused output stage only: the gate_z tile of a chunk, the partial row sums of two chunks, the inverse norms of each warp
+constexpr uint32_t CS_Z = (CS_TOTAL + 1023) / 1024 * 1024, CS_RED = CS_Z + 16384, CS_INV = CS_RED + 2 * 4 * 64 * 4;
+constexpr uint32_t CHAIN_SMEM_GATED = CS_INV + 4 * 64 * 4 + 1024;
+static_assert(CS_OST % 1024 == 0 && CHAIN_SMEM_GATED <= 232448, "shared memory per CTA");
 
-enum CBar : uint32_t { CB_FULLA0 = 0, CB_FREEA0 = 2, CB_FULLB0 = 4, CB_FREEB0 = 7, CB_V = 10, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE,
-                       CB_U, CB_O1, CB_CLEAN };
+enum CBar : uint32_t { CB_FULLW0 = 0, CB_FREEW0 = 2, CB_FULLQ0 = 4, CB_FREEQ0 = 6, CB_FULLK0 = 8, CB_FREEK0 = 10, CB_FULLP0 = 12, CB_FREEP0 = 14,
+                       CB_FULLB0 = 16, CB_FREEB0 = 18, CB_ZFULL = 20, CB_ZFREE, CB_V, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE, CB_U, CB_O1, CB_CLEAN };
+static_assert(CB_CLEAN < 32, "barrier area");
 
 struct ChainParams {
     const float* s0;          // [N,H,d_k,d_v] or nullptr
@@ -764,9 +778,8 @@ __device__ __forceinline__ bool handover_wait(const Handover& hv, volatile int* 
 }
 
 __device__ __forceinline__ void chain_init_bars(const Waiter& w) {
-    for (uint32_t i = 0; i < 2; ++i) { mbar_init(w.bar(CB_FULLA0 + i), 1); mbar_init(w.bar(CB_FREEA0 + i), 2); }   // both issuers
+    for (uint32_t i = CB_FULLW0; i < CB_V; ++i) mbar_init(w.bar(i), i == CB_ZFREE ? 128 : 1);
     mbar_init(w.bar(CB_U), 1); mbar_init(w.bar(CB_O1), 1);
-    for (uint32_t i = 0; i < 3; ++i) { mbar_init(w.bar(CB_FULLB0 + i), 1); mbar_init(w.bar(CB_FREEB0 + i), 1); }
     mbar_init(w.bar(CB_V), 1); mbar_init(w.bar(CB_S), 1); mbar_init(w.bar(CB_O), 1);
     mbar_init(w.bar(CB_SREADY), 128); mbar_init(w.bar(CB_VREADY), 128); mbar_init(w.bar(CB_OFREE), 128);
     mbar_init(w.bar(CB_CLEAN), 128);
@@ -776,7 +789,7 @@ __device__ __forceinline__ void chain_init_bars(const Waiter& w) {
 // incoming state is awaited through `hv` and read past the L1 cache, since another SM wrote it in this launch).
 template <bool DBG, bool SCAN, bool GATED>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
-                                           const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
+                                           const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
@@ -837,7 +850,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             mbar_arrive(w.bar(CB_SREADY));
         }
         for (int c = 0; c < nchunks; ++c) {
-            const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c & 3) * 1280);
+            const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
             if (c > 0) w.wait_hot(CB_O, (c - 1) & 1);     // O2 of the previous chunk no longer reads bf16 v_new
             w.wait_hot(CB_V, c & 1);
             tc_fence_after_sync();
@@ -919,35 +932,33 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         // =============================== epilogue warpgroup ===============================
         const int j = tid - 128, we = j >> 5;
         const uint32_t lane_base = (uint32_t)(we * 32) << 16;
-        __nv_bfloat16* ost = reinterpret_cast<__nv_bfloat16*>(sm + CS_OST);
-        // Fused output stage: every thread fetches the eight 16-byte pieces of gate_z it will use itself, one chunk
-        // ahead (each thread waits for and reads only its own copies).  Loaded where they are used, they cost eight
-        // memory latencies per chunk on the warpgroup that must keep up with the chain: 154 -> 106 us for the
-        // kernel on 4 x 1500 tokens, 16 heads.
-        auto fetch_z = [&](int c) {
-            if (!GATED || c >= nchunks) return;
-            const int Rz = min(C, len - c * C);
-            const __nv_bfloat16* src = p.gate_z + ((size_t)(tok0 + c * C) * H + h) * dv + (j & 15) * 8;
+        // The accumulators are read as matrix fragments (thread: 4 value columns x 16 tokens, tokens in pairs), so that a
+        // pair of tokens packs into one register and stmatrix transposes 8x8 blocks into rows of the output tile,
+        // which leaves as two TMA stores (a last, partial chunk by plain stores: the rows behind it belong to others).
+        // This role must stay shorter than a chain step: with one 2-byte store per value and row copies by
+        // the threads it took 1.6 us a chunk and set the pace of the whole kernel.
+        const int l4 = lane & 3, l8 = lane >> 2;                 // fragment: columns 8q + 2 l4 (+1) are tokens, rows l8 (+8) values
+        // lane's part in stmatrix / ldmatrix: value columns 8 piece .. +7 of token 8q + (lane & 7)
+        const uint32_t piece = 4u * (uint32_t)we + (uint32_t)(lane >> 3);
+        const uint32_t frag_off = (piece >> 3) * 8192 + (uint32_t)(lane & 7) * 128 + (((piece & 7) ^ (uint32_t)(lane & 7)) << 4);
+        float wv[4] = {0.f, 0.f, 0.f, 0.f};
+        if (GATED) {
 #pragma unroll
-            for (int it = 0; it < 8; ++it) {
-                const int r = it * 8 + (j >> 4);
-                if (r < Rz) cp_async16(base + CS_Z + (it * 128 + j) * 16, src + (size_t)r * H * dv);
-            }
-        };
-        fetch_z(0);
+            for (int m = 0; m < 4; ++m) wv[m] = __ldg(p.norm_w + 32 * we + 8 * m + l8);
+        }
         for (int c = 0; c < nchunks; ++c) {
             const int R = min(C, len - c * C);
-            const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c & 3) * 1280);
+            const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
             if (tail_c >= 0 && c == max(tail_c - 1, 0)) {
                 const int Rt = len - tail_c * C;
-                const uint32_t sa = base + CS_A + (uint32_t)(tail_c & 1) * STAGE_A + ST_KQ;
-                const uint32_t sv = base + CS_B + (uint32_t)(tail_c % 3) * STAGE_B + ST_V;
-                w.wait(CB_FULLA0 + (tail_c & 1), (tail_c >> 1) & 1);
-                w.wait(CB_FULLB0 + tail_c % 3, (tail_c / 3) & 1);
+                const uint32_t sk = base + CS_K + (uint32_t)(tail_c & 1) * 16384;
+                const uint32_t sv = base + CS_B + (uint32_t)(tail_c & 1) * STAGE_B + ST_V;
+                w.wait(CB_FULLK0 + (tail_c & 1), (tail_c >> 1) & 1);
+                w.wait(CB_FULLB0 + (tail_c & 1), (tail_c >> 1) & 1);
                 const uint32_t pieces = (uint32_t)(C - Rt) * 8u;
                 for (uint32_t x = j; x < 4 * pieces; x += 128) {             // K_lo, K_hi, V_lo, V_hi
                     const uint32_t t4 = x / pieces, y = x - t4 * pieces;
-                    const uint32_t tile = t4 == 0 ? sa : t4 == 1 ? sa + 16384 : t4 == 2 ? sv : sv + 8192;
+                    const uint32_t tile = t4 == 0 ? sk : t4 == 1 ? sk + 8192 : t4 == 2 ? sv : sv + 8192;
                     st_shared_v4(tile + ((uint32_t)Rt + (y >> 3)) * 128 + ((y & 7) << 4), 0u, 0u, 0u, 0u);
                 }
                 fence_proxy_async_smem();
@@ -957,86 +968,104 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             tc_fence_after_sync();
             // take both accumulators out of tensor memory first and hand them back at once: the next
             // chunk's output MMAs wait for this
-            uint32_t o1a[32], o1b[32], o2a[32], o2b[32];
-            tmem_ld32(tmem + lane_base + TM_O1, o1a);
-            tmem_ld32(tmem + lane_base + TM_O1 + 32, o1b);
-            tmem_ld32(tmem + lane_base + TM_O2, o2a);
-            tmem_ld32(tmem + lane_base + TM_O2 + 32, o2b);
+            uint32_t o1[2][32], o2[2][32];
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O1, o1[hh]);
+                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O2, o2[hh]);
+            }
             tmem_wait_ld();
             tc_fence_before_sync();
             mbar_arrive(w.bar(CB_OFREE));
+            const uint32_t ost = base + CS_OST + (uint32_t)(c & 1) * 16384;
+            float o[2][32];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + 8 * q + 2 * l4);
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh)
+                        o[hh][4 * q + x] = fmaf((x & 1) ? eg.y : eg.x, __uint_as_float(o1[hh][4 * q + x]), __uint_as_float(o2[hh][4 * q + x]));
+            }
             if (GATED) {
                 // Fused output stage (the per-position kernels behind the scan, Section "Prefill projections:
                 // dequantize, then call the vendor"): root-mean-square norm of each output row over the value
-                // axis, weight vector, SiLU gate.  The rows go through shared memory in fp32, 32 tokens at a
-                // time; sixteen neighbouring lanes hold one row and add up its squares by shuffles.
-                float* fst = reinterpret_cast<float*>(sm + CS_OST);           // [32][128] fp32, the same 16 KiB
-                const size_t row0 = (size_t)(tok0 + c * C) * H + h;
-                const int col = (j & 15) * 8;
-                const float4 w0 = __ldg(reinterpret_cast<const float4*>(p.norm_w + col));
-                const float4 w1 = __ldg(reinterpret_cast<const float4*>(p.norm_w + col + 4));
-                const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-                cp_async_wait_all();
+                // axis, weight vector, SiLU gate.  A token's squares lie in the eight lanes of equal l4 of every warp:
+                // a butterfly that halves the tokens at each step leaves two tokens' sums per lane, the four warps' sums meet
+                // in shared memory.  gate_z comes by TMA a chunk ahead and is read in the same fragments.
+                float ss[16];
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
+                for (int q = 0; q < 8; ++q)
 #pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        fst[i * DVB + j] = half ? fmaf(gates[160 + i], __uint_as_float(o1b[i]), __uint_as_float(o2b[i]))
-                                                : fmaf(gates[128 + i], __uint_as_float(o1a[i]), __uint_as_float(o2a[i]));
-                    named_bar_sync(2, 128);
-#pragma unroll 1
-                    for (int it = 0; it < 4; ++it) {          // one copy: the divisions are the bulk of this role's code
-                        const int rr = (it * 128 + j) >> 4, r = 32 * half + rr;
-                        const float4 x0 = *reinterpret_cast<const float4*>(fst + rr * DVB + col);
-                        const float4 x1 = *reinterpret_cast<const float4*>(fst + rr * DVB + col + 4);
-                        const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-                        float ss = 0.f;
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) ss = fmaf(xv[e], xv[e], ss);
-#pragma unroll
-                        for (int d = 1; d < 16; d <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
-                        const float inv = rsqrtf(ss * (1.0f / DVB) + p.norm_eps);
-                        if (r < R) {
-                            const size_t off = (row0 + (size_t)r * H) * dv + col;
-                            const uint4 zz = *reinterpret_cast<const uint4*>(sm + CS_Z + ((half * 4 + it) * 128 + j) * 16);
-                            const uint32_t zu[4] = {zz.x, zz.y, zz.z, zz.w};
-                            uint32_t pk[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float z0 = __uint_as_float(zu[e] << 16), z1 = __uint_as_float(zu[e] & 0xffff0000u);
-                                const float y0 = xv[2 * e] * inv * wv[2 * e] * (z0 / (1.0f + __expf(-z0)));
-                                const float y1 = xv[2 * e + 1] * inv * wv[2 * e + 1] * (z1 / (1.0f + __expf(-z1)));
-                                pk[e] = pack_bf16(y0, y1);
-                            }
-                            *reinterpret_cast<uint4*>(p.out + off) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        }
+                    for (int x = 0; x < 2; ++x) {
+                        const float a0 = o[0][4 * q + x], a1 = o[0][4 * q + 2 + x], a2 = o[1][4 * q + x], a3 = o[1][4 * q + 2 + x];
+                        ss[2 * q + x] = fmaf(a0, a0, a1 * a1) + fmaf(a2, a2, a3 * a3);
                     }
-                    named_bar_sync(2, 128);
+#pragma unroll
+                for (int st = 0; st < 3; ++st) {
+                    const int half = 8 >> st;                    // values kept: the upper half of the tokens where the lane bit is set
+                    const bool up = (lane & (16 >> st)) != 0;
+#pragma unroll
+                    for (int i = 0; i < half; ++i) {
+                        const float give = up ? ss[i] : ss[half + i], keep = up ? ss[half + i] : ss[i];
+                        ss[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16 >> st);
+                    }
                 }
-                fetch_z(c + 1);
-                continue;
+                float* red = reinterpret_cast<float*>(sm + CS_RED) + (c & 1) * 256;
+                // tokens 8q + 2 l4 (+1) with q = (lane bits 4, 3, 2)
+                const int qk = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+                *reinterpret_cast<float2*>(red + we * 64 + 8 * qk + 2 * l4) = make_float2(ss[0], ss[1]);
+                named_bar_sync(2, 128);
+                float* inv = reinterpret_cast<float*>(sm + CS_INV) + we * 64;
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    const int tk = lane + 32 * x;
+                    const float sum = (red[tk] + red[64 + tk]) + (red[128 + tk] + red[192 + tk]);
+                    inv[tk] = rsqrtf(sum * (1.0f / DVB) + p.norm_eps);
+                }
+                __syncwarp();
+                w.wait(CB_ZFULL, c & 1);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    uint32_t z[4];
+                    ldmatrix_x4_trans(base + CS_Z + frag_off + (uint32_t)q * 1024, z[0], z[1], z[2], z[3]);
+                    const float2 iv = *reinterpret_cast<const float2*>(inv + 8 * q + 2 * l4);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {                // matrix m: value rows 8m + l8 of the warp's 32
+                        float* y = &o[m >> 1][4 * q + 2 * (m & 1)];
+                        y[0] *= iv.x * wv[m] * silu(__uint_as_float(z[m] << 16));
+                        y[1] *= iv.y * wv[m] * silu(__uint_as_float(z[m] & 0xffff0000u));
+                    }
+                }
+                mbar_arrive(w.bar(CB_ZFREE));
             }
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const float oa = fmaf(gates[128 + i], __uint_as_float(o1a[i]), __uint_as_float(o2a[i]));
-                const float ob = fmaf(gates[160 + i], __uint_as_float(o1b[i]), __uint_as_float(o2b[i]));
-                ost[i * DVB + j] = __float2bfloat16_rn(oa);           // transpose through shared memory
-                ost[(32 + i) * DVB + j] = __float2bfloat16_rn(ob);
-            }
-            named_bar_sync(2, 128);
-            {
+            for (int q = 0; q < 8; ++q)
+                stmatrix_x4_trans(ost + frag_off + (uint32_t)q * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
+                                  pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
+            if (R == C) {
+                fence_proxy_async_smem();
+                if (j == 0) bulk_wait_read_all();              // the tile the next chunk writes has left (stored a chunk ago)
+                named_bar_sync(2, 128);
+                if (j == 0) {
+                    const int tok = (int)(tok0 + (long)c * C);
+                    tma_store_3d(map_o, dvb * DVB, h, tok, ost);
+                    tma_store_3d(map_o, dvb * DVB + 64, h, tok, ost + 8192);
+                    bulk_commit();
+                }
+            } else {
+                named_bar_sync(2, 128);
                 __nv_bfloat16* obase = p.out + ((size_t)(tok0 + c * C) * H + h) * dv + (size_t)dvb * DVB;
-#pragma unroll
-                for (int it = 0; it < 8; ++it) {
-                    const int qd = it * 128 + j, r = qd >> 4, col = (qd & 15) * 8;
-                    if (r < R) {
-                        const uint4 val = *reinterpret_cast<const uint4*>(ost + r * DVB + col);
-                        *reinterpret_cast<uint4*>(obase + (size_t)r * H * dv + col) = val;
-                    }
+#pragma unroll 1
+                for (int qd = j; qd < R * 16; qd += 128) {
+                    const uint32_t r = (uint32_t)qd >> 4, pc = (uint32_t)qd & 15u;
+                    const uint4 val = *reinterpret_cast<const uint4*>(sm + CS_OST + (c & 1) * 16384 + (pc >> 3) * 8192 + swz(r, pc & 7));
+                    *reinterpret_cast<uint4*>(obase + (size_t)r * H * dv + pc * 8) = val;
                 }
             }
-            named_bar_sync(2, 128);
         }
+        if (j == 0) bulk_wait_all();
     } else {
         // =============================== control warpgroup ===============================
         if (!SCAN) setmaxnreg_dec<56>();
@@ -1047,14 +1076,14 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             //  issued by a second thread so that it does not sit between two dependent steps)
             // operand descriptors are built once per stage, outside the dependent chain: the address field
             // counts 16-byte units, so a k-step is a plain add
-            const uint64_t dW0 = make_smem_desc(base + CS_A + ST_W, 1024, 1024);
-            const uint64_t dK0 = make_smem_desc(base + CS_A + ST_KQ, 16384, 1024);
+            const uint64_t dW0 = make_smem_desc(base + CS_W, 1024, 1024), dK0 = make_smem_desc(base + CS_K, 8192, 1024);
             for (int c = 0; c < nchunks; ++c) {
-                const uint32_t s = c & 1;
-                const uint64_t dW = dW0 + (uint64_t)((s * STAGE_A) >> 4), dK = dK0 + (uint64_t)((s * STAGE_A) >> 4);
+                const uint32_t s = c & 1, par = (c >> 1) & 1;
+                const uint64_t dW = dW0 + (uint64_t)((s * 16384) >> 4), dK = dK0 + (uint64_t)((s * 16384) >> 4);
                 // the waits that are normally long satisfied come first: whatever follows the wait on the
                 // state sits on the dependent chain
-                w.wait_hot(CB_FULLA0 + s, (c >> 1) & 1);
+                w.wait_hot(CB_FULLW0 + s, par);
+                w.wait_hot(CB_FULLK0 + s, par);
                 w.wait_hot(CB_U, c & 1);                       // U^T of this chunk is in the accumulator
                 if (c == tail_c) w.wait_hot(CB_CLEAN, 0);      // padded K rows have been cleared
                 w.wait_hot(CB_SREADY, c & 1);
@@ -1064,6 +1093,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 for (uint32_t ks = 0; ks < 8; ++ks)            // v^T = U^T - S^T W^T
                     if (lead) mma_ts(tmem + TM_DV, tmem + TM_SBF + ks * 8, dW + ks * 128, ID_1, 1);
                 if (lead) mma_commit(w.bar(CB_V));
+                if (lead) mma_commit(w.bar(CB_FREEW0 + s));
                 if (lead) stamp(1, c, 1);
                 w.wait_hot(CB_VREADY, c & 1);
                 tc_fence_after_sync();
@@ -1072,7 +1102,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 for (uint32_t ks = 0; ks < 4; ++ks)            // dS^T = (v e^{gC-g})^T K
                     if (lead) mma_ts(tmem + TM_DS, tmem + TM_VT + ks * 8, dK + ks * 128, ID_2, ks > 0);
                 if (lead) mma_commit(w.bar(CB_S));
-                if (lead) mma_commit(w.bar(CB_FREEA0 + s));
+                if (lead) mma_commit(w.bar(CB_FREEK0 + s));
                 if (lead) stamp(1, c, 4);
             }
         } else if (warp == 10) {
@@ -1081,28 +1111,28 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             // (descriptors are built once; a stage or a k-step is an add on the 16-byte address field.  Every warp
             //  role runs its loop at the same time, so the size of these loops shows in the instruction cache.)
             const uint64_t dV0 = make_smem_desc(base + CS_B + ST_V, 8192, 1024), dT0 = make_smem_desc(base + CS_B + ST_T2, 1024, 1024);
-            const uint64_t dQ0 = make_smem_desc(base + CS_A + ST_KQ + 8192, 16, 1024), dP0 = make_smem_desc(base + CS_A + ST_P, 16, 1024);
+            const uint64_t dQ0 = make_smem_desc(base + CS_Q, 16, 1024), dP0 = make_smem_desc(base + CS_P, 16, 1024);
             for (int c = -1; c < nchunks; ++c) {
-                const uint32_t s = c & 1;
-                const uint64_t soff = (uint64_t)((s * STAGE_A) >> 4);
+                const uint32_t s = c & 1, par = (c >> 1) & 1;
                 if (c >= 0) {
                     w.wait(CB_SREADY, c & 1);
-                    w.wait(CB_FULLA0 + s, (c >> 1) & 1);
+                    w.wait(CB_FULLQ0 + s, par);
                     if (c > 0) w.wait(CB_OFREE, (c - 1) & 1);  // the epilogue has read the previous O1, O2
                     w.wait_hot(CB_V, c & 1);                   // stay out of the tensor pipe until v_new is done
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 8; ++ks)        // O1^T = S^T Q^T
-                        if (lead) mma_ts(tmem + TM_O1, tmem + TM_SBF + ks * 8, dQ0 + soff + (uint64_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4),
+                        if (lead) mma_ts(tmem + TM_O1, tmem + TM_SBF + ks * 8, dQ0 + (uint64_t)((s * 16384 + (ks >> 2) * 8192 + (ks & 3) * 32) >> 4),
                                ID_O, ks > 0);
                     if (lead) mma_commit(w.bar(CB_O1));
+                    if (lead) mma_commit(w.bar(CB_FREEQ0 + s));
                     w.wait(CB_VREADY, c & 1);
                     tc_fence_after_sync();
                 }
                 if (c + 1 < nchunks) {                         // U^T = V^T (T diag(b))^T of chunk c + 1: D_v is free,
-                    const uint32_t sB = (c + 1) % 3;           // v_new of chunk c has been read
+                    const uint32_t sB = (c + 1) & 1;           // v_new of chunk c has been read
                     const uint64_t boff = (uint64_t)((sB * STAGE_B) >> 4);
-                    w.wait(CB_FULLB0 + sB, ((c + 1) / 3) & 1);
+                    w.wait(CB_FULLB0 + sB, ((c + 1) >> 1) & 1);
                     if (c + 1 == tail_c) w.wait(CB_CLEAN, 0);  // padded V rows have been cleared
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)
@@ -1111,11 +1141,12 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     if (lead) mma_commit(w.bar(CB_U));
                 }
                 if (c >= 0) {
+                    w.wait(CB_FULLP0 + s, par);
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)        // O2^T = v^T P^T
-                        if (lead) mma_ts(tmem + TM_O2, tmem + TM_V + ks * 8, dP0 + soff + ks * 2, ID_O, ks > 0);
+                        if (lead) mma_ts(tmem + TM_O2, tmem + TM_V + ks * 8, dP0 + (uint64_t)((s * 8192) >> 4) + ks * 2, ID_O, ks > 0);
                     if (lead) mma_commit(w.bar(CB_O));
-                    if (lead) mma_commit(w.bar(CB_FREEA0 + s));
+                    if (lead) mma_commit(w.bar(CB_FREEP0 + s));
                 }
             }
         } else if (warp == 9 && lane == 0) {
@@ -1123,41 +1154,72 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             prefetch_tensormap(map_q);
             prefetch_tensormap(map_k);
             prefetch_tensormap(map_v);
+            prefetch_tensormap(map_o);
             const uint64_t pol_done = (p.l2 & 1) ? l2_policy_evict_first() : l2_policy_evict_normal();
             const uint64_t pol_item = (p.l2 & 2) ? l2_policy_evict_first() : l2_policy_evict_normal();
             for (int c = 0; c < nchunks; ++c) {
                 if (c == p.drop_chunk && dvb == 0 && h == 0 && cta.z == 0) continue;
                 const int tok = (int)(tok0 + (long)c * C);
                 const uint8_t* item = p.items + (size_t)((slot0 + c) * H + h) * ITEM_BYTES;
-                {   // ring B: V tile and (T diag(b))^T
-                    const uint32_t sB = c % 3, bb = base + CS_B + sB * STAGE_B, full = w.bar(CB_FULLB0 + sB);
-                    if (c >= 3) w.wait(CB_FREEB0 + sB, ((c / 3) - 1) & 1);
+                // in the order in which the slots come free
+                const uint32_t s = c & 1, par = ((c >> 1) - 1) & 1;
+                {   // V tile and (T diag b)^T
+                    const uint32_t bb = base + CS_B + s * STAGE_B, full = w.bar(CB_FULLB0 + s);
+                    if (c >= 2) w.wait(CB_FREEB0 + s, par);
                     mbar_arrive_expect_tx(full, STAGE_B_TX);
                     tma_load_3d_hint(bb + ST_V, map_v, dvb * DVB, h, tok, full, pol_done);
                     tma_load_3d_hint(bb + ST_V + 8192, map_v, dvb * DVB + 64, h, tok, full, pol_done);
                     bulk_load_hint(bb + ST_T2, item + IT_T2, 8192, full, pol_item);
                 }
-                {   // ring A: K/Q tiles, -W^T, P, and the gate vectors (own 4-deep ring, same barrier)
-                    const uint32_t s = c & 1, sb = base + CS_A + s * STAGE_A, full = w.bar(CB_FULLA0 + s);
-                    if (c >= 2) w.wait(CB_FREEA0 + s, ((c >> 1) - 1) & 1);
-                    mbar_arrive_expect_tx(full, STAGE_A_TX);
-                    bulk_load_hint(sb + ST_W, item + IT_W, 16384, full, pol_item);
-                    tma_load_3d_hint(sb + ST_KQ, map_k, 0, h, tok, full, pol_done);
-                    tma_load_3d_hint(sb + ST_KQ + 8192, map_q, 0, h, tok, full, pol_done);
-                    tma_load_3d_hint(sb + ST_KQ + 16384, map_k, 64, h, tok, full, pol_done);
-                    tma_load_3d_hint(sb + ST_KQ + 24576, map_q, 64, h, tok, full, pol_done);
-                    bulk_load(sb + ST_P, item + IT_P, 8192, full);
-                    bulk_load(base + CS_GATES + (c & 3) * 1280, item + IT_GATES, 1280, full);
+                {
+                    const uint32_t full = w.bar(CB_FULLW0 + s);
+                    if (c >= 2) w.wait(CB_FREEW0 + s, par);
+                    mbar_arrive_expect_tx(full, 16384 + 1280);
+                    bulk_load_hint(base + CS_W + s * 16384, item + IT_W, 16384, full, pol_item);
+                    bulk_load(base + CS_GATES + (c % (int)GATE_SLOTS) * 1280, item + IT_GATES, 1280, full);
+                }
+                {
+                    const uint32_t full = w.bar(CB_FULLQ0 + s), dst = base + CS_Q + s * 16384;
+                    if (c >= 2) w.wait(CB_FREEQ0 + s, par);
+                    mbar_arrive_expect_tx(full, 16384);
+                    tma_load_3d_hint(dst, map_q, 0, h, tok, full, pol_done);
+                    tma_load_3d_hint(dst + 8192, map_q, 64, h, tok, full, pol_done);
+                }
+                {
+                    const uint32_t full = w.bar(CB_FULLK0 + s), dst = base + CS_K + s * 16384;
+                    if (c >= 2) w.wait(CB_FREEK0 + s, par);
+                    mbar_arrive_expect_tx(full, 16384);
+                    tma_load_3d_hint(dst, map_k, 0, h, tok, full, pol_done);
+                    tma_load_3d_hint(dst + 8192, map_k, 64, h, tok, full, pol_done);
+                }
+                {
+                    const uint32_t full = w.bar(CB_FULLP0 + s);
+                    if (c >= 2) w.wait(CB_FREEP0 + s, par);
+                    mbar_arrive_expect_tx(full, 8192);
+                    bulk_load(base + CS_P + s * 8192, item + IT_P, 8192, full);
                 }
             }
             if (*w.abort_flag) {
                 // let copies in flight land before shared memory is released (bounded)
                 const unsigned long long t0 = globaltimer_ns();
-                for (int c = max(0, nchunks - 3); c < nchunks; ++c) {
-                    while (!mbar_try_wait(w.bar(CB_FULLB0 + c % 3), (c / 3) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
-                    if (c >= nchunks - 2)
-                        while (!mbar_try_wait(w.bar(CB_FULLA0 + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
-                }
+                for (int c = max(0, nchunks - 2); c < nchunks; ++c)
+                    for (uint32_t b = CB_FULLW0; b <= CB_FULLB0; b += 4)
+                        while (!mbar_try_wait(w.bar(b + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+            }
+        } else if (GATED && warp == 11 && lane == 0) {
+            // ---- TMA producer of the gate tile ----
+            prefetch_tensormap(map_z);
+            const uint32_t full = w.bar(CB_ZFULL);
+            for (int c = 0; c < nchunks; ++c) {
+                if (c > 0) w.wait(CB_ZFREE, (c - 1) & 1);
+                const int tok = (int)(tok0 + (long)c * C);
+                mbar_arrive_expect_tx(full, 16384);
+                tma_load_3d(base + CS_Z, map_z, 0, h, tok, full);
+                tma_load_3d(base + CS_Z + 8192, map_z, 64, h, tok, full);
+            }
+            if (*w.abort_flag) {
+                const unsigned long long t0 = globaltimer_ns();
+                while (!mbar_try_wait(full, (nchunks - 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
             }
         }
     }
@@ -1166,7 +1228,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
 template <bool DBG, bool GATED>
 __global__ void __launch_bounds__(CHAIN_THREADS, 1)
 gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                 const __grid_constant__ CUtensorMap map_v, ChainParams p) {
+                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
+                 const __grid_constant__ CUtensorMap map_z, ChainParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
@@ -1188,7 +1251,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_wait();                         // scratch items and incoming states come from the kernels before this one
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
-    chain_body<DBG, false, GATED>(&map_q, &map_k, &map_v, p, cta, w, Handover{nullptr, 0});
+    chain_body<DBG, false, GATED>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1666,7 +1729,7 @@ constexpr int SCAN_THREADS = 384;
 constexpr uint32_t SC_BARS1 = CS_BARS;                 // behind the largest data layout (the chain phase's)
 constexpr uint32_t SC_BARS2 = SC_BARS1 + 24 * 8;
 constexpr uint32_t SC_BARS3 = SC_BARS2 + 16 * 8;
-constexpr uint32_t SC_MISC = SC_BARS3 + 24 * 8;
+constexpr uint32_t SC_MISC = SC_BARS3 + 32 * 8;
 constexpr uint32_t SCAN_SMEM = SC_MISC + 64 + 1024;
 static_assert(SUS_BARS <= CS_BARS && CM_BARS <= CS_BARS, "phase layouts must end before the barrier area");
 static_assert(SCAN_SMEM <= 232448, "shared memory per CTA");
@@ -1686,7 +1749,7 @@ __device__ __forceinline__ void mbar_inval(uint32_t bar) {
 template <bool DBG>
 __global__ void __launch_bounds__(SCAN_THREADS, 1)
 gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                const __grid_constant__ CUtensorMap map_v, ScanParams p) {
+                const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, ScanParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
@@ -1767,7 +1830,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         stamp(3);
         // ---------------- phase 3: chain over this segment's chunks ----------------
         const Cta c3{base, sm, tmem, 0, h, (int)blockIdx.z};
-        chain_body<DBG, true, false>(&map_q, &map_k, &map_v, p.cp, c3, w3, Handover{fl + 1, nowners});
+        chain_body<DBG, true, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
         stamp(4);
         tc_fence_before_sync();
         cta_sync();
@@ -1923,10 +1986,12 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
         nseg = 1;
         seg_chunks = (a.T + C - 1) / C > 0 ? (a.T + C - 1) / C : 1;
     }
-    CUtensorMap mq, mk, mv;
+    CUtensorMap mq, mk, mv, mo, mz;
     if (!tc_make_map(&mq, a.q, tokens, a.H, a.d_k) || !tc_make_map(&mk, a.k, tokens, a.H, a.d_k) ||
-        !tc_make_map(&mv, a.v, tokens, a.H, a.d_v))
+        !tc_make_map(&mv, a.v, tokens, a.H, a.d_v) || !tc_make_map(&mo, a.out, tokens, a.H, a.d_v) ||
+        (opt.gate_z && !tc_make_map(&mz, opt.gate_z, tokens, a.H, a.d_v)))
         return GDN_ERR_CUDA;
+    if (!opt.gate_z) mz = mo;
     int* ticket = static_cast<int*>(workspace);                      // header, zeroed by lean_init_workspace
     uint8_t* ws = static_cast<uint8_t*>(workspace) + kWorkspaceHeader;
     const long nslots = (long)(tokens >> 6) + a.B;
@@ -1963,8 +2028,8 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                            snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps};
             ScanParams scp{sp, cb, cp, static_cast<int*>(workspace) + kScanFlagOffset};
             dim3 grid(1, a.H, a.B * nseg);
-            if (g_lean_dbg) launch_after(gdn_scan_kernel<true>, grid, SCAN_THREADS, SCAN_SMEM, stream, mq, mk, mv, scp);
-            else launch_after(gdn_scan_kernel<false>, grid, SCAN_THREADS, SCAN_SMEM, stream, mq, mk, mv, scp);
+            if (g_lean_dbg) launch_after(gdn_scan_kernel<true>, grid, SCAN_THREADS, SCAN_SMEM, stream, mq, mk, mv, mo, scp);
+            else launch_after(gdn_scan_kernel<false>, grid, SCAN_THREADS, SCAN_SMEM, stream, mq, mk, mv, mo, scp);
             count_launch();
             g_lean_scan_last = true;
             mark(4);
@@ -1986,9 +2051,9 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                    ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, nseg, seg_chunks,
                    snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps};
     dim3 grid(a.d_v / DVB, a.H, a.B * nseg);
-    if (opt.gate_z) launch_after(gdn_chain_kernel<false, true>, grid, CHAIN_THREADS, CHAIN_SMEM_GATED, stream, mq, mk, mv, cp);
-    else if (g_lean_dbg) launch_after(gdn_chain_kernel<true, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, cp);
-    else launch_after(gdn_chain_kernel<false, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, cp);
+    if (opt.gate_z) launch_after(gdn_chain_kernel<false, true>, grid, CHAIN_THREADS, CHAIN_SMEM_GATED, stream, mq, mk, mv, mo, mz, cp);
+    else if (g_lean_dbg) launch_after(gdn_chain_kernel<true, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
+    else launch_after(gdn_chain_kernel<false, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
     count_launch();
     mark(4);
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
@@ -2082,9 +2147,9 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
         scratch_of_device[dev] = ptr;
     }
     uint8_t* ws = static_cast<uint8_t*>(scratch_of_device[dev]);
-    CUtensorMap mq, mk, mv;
+    CUtensorMap mq, mk, mv, mo;
     if (!tc_make_map(&mq, a.q, tokens, a.H, a.d_k) || !tc_make_map(&mk, a.k, tokens, a.H, a.d_k) ||
-        !tc_make_map(&mv, a.v, tokens, a.H, a.d_v))
+        !tc_make_map(&mv, a.v, tokens, a.H, a.d_v) || !tc_make_map(&mo, a.out, tokens, a.H, a.d_v))
         return GDN_ERR_CUDA;
     const long nitems = (long)nslots * a.H;
     const long cap = 4L * sms_of_device[dev];
@@ -2097,7 +2162,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
                    ws, nullptr, nullptr, -1, a.B, a.T, a.H, a.d_v, 1, packed ? (1 << 24) : (nch > 0 ? nch : 1),
                    nullptr, 1, 0};
     dim3 grid(a.d_v / DVB, a.H, a.B);
-    gdn_chain_kernel<false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, cp);
+    gdn_chain_kernel<false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }

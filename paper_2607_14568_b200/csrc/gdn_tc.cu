@@ -766,7 +766,7 @@ EncodeTiledFn encode_fn() {
 // again, so the last few encodings are kept per host thread and the driver call is skipped on a repeat.
 bool make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d) {
     struct Entry { const void* ptr; uint64_t tokens, H, d; CUtensorMap map; bool used; };
-    constexpr int kEntries = 8;
+    constexpr int kEntries = 32;          // four to five tensors a call, a handful of buffer sets in rotation
     static thread_local Entry cache[kEntries] = {};
     static thread_local int next = 0;
     for (int i = 0; i < kEntries; ++i)
