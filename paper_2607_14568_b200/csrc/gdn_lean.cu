@@ -160,9 +160,9 @@ __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bu
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // z / (1 + e^-z); the reciprocal is refined by one Newton step (about one unit in the last place, as a division, without
-// the branches of one: 64 of them per thread and chunk took longer than the chain step they must hide behind)
+// the branches of one)
 __device__ __forceinline__ float silu(float z) {
-    const float d = 1.0f + __expf(-z);
+    const float d = 1.0f + ex2(z * -LOG2E);
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
     r = r * fmaf(-d, r, 2.0f);
@@ -682,9 +682,10 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // =====================================================================================
 // chain kernel (steps c and d)
 // =====================================================================================
-constexpr int CHAIN_THREADS = 384;
+constexpr int CHAIN_THREADS = 512;          // two chain warpgroups, output warpgroup, control warpgroup
 // tensor memory columns
-constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384;
+constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384,
+                   TM_OG = 448;   // fused output stage: the combined fp32 output rows
 constexpr uint32_t CT_COLS = 512;
 // shared memory: every operand has a ring of its own, released by the completion of the MMAs that read it, so that a
 // slot is refilled as soon as its one use is over and a load has well over a chunk step to arrive.  (With
@@ -715,8 +716,8 @@ constexpr uint32_t CHAIN_SMEM_GATED = CS_INV + 4 * 64 * 4 + 1024;
 static_assert(CS_OST % 1024 == 0 && CHAIN_SMEM_GATED <= 232448, "shared memory per CTA");
 
 enum CBar : uint32_t { CB_FULLW0 = 0, CB_FREEW0 = 2, CB_FULLQ0 = 4, CB_FREEQ0 = 6, CB_FULLK0 = 8, CB_FREEK0 = 10, CB_FULLP0 = 12, CB_FREEP0 = 14,
-                       CB_FULLB0 = 16, CB_FREEB0 = 18, CB_ZFULL = 20, CB_ZFREE, CB_V, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE, CB_U, CB_O1, CB_CLEAN };
-static_assert(CB_CLEAN < 32, "barrier area");
+                       CB_FULLB0 = 16, CB_FREEB0 = 18, CB_ZFULL = 20, CB_ZFREE, CB_V, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE, CB_U, CB_O1, CB_CLEAN, CB_VPLAIN };
+static_assert(CB_VPLAIN < 32, "barrier area");
 
 struct ChainParams {
     const float* s0;          // [N,H,d_k,d_v] or nullptr
@@ -781,7 +782,7 @@ __device__ __forceinline__ void chain_init_bars(const Waiter& w) {
     for (uint32_t i = CB_FULLW0; i < CB_V; ++i) mbar_init(w.bar(i), i == CB_ZFREE ? 128 : 1);
     mbar_init(w.bar(CB_U), 1); mbar_init(w.bar(CB_O1), 1);
     mbar_init(w.bar(CB_V), 1); mbar_init(w.bar(CB_S), 1); mbar_init(w.bar(CB_O), 1);
-    mbar_init(w.bar(CB_SREADY), 128); mbar_init(w.bar(CB_VREADY), 128); mbar_init(w.bar(CB_OFREE), 128);
+    mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256); mbar_init(w.bar(CB_OFREE), 128);
     mbar_init(w.bar(CB_CLEAN), 128);
 }
 
@@ -820,30 +821,34 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     const float* s_in = p.seg_sin ? p.seg_sin + ((size_t)(n * p.nseg + seg) * H + h) * DK * dv + (size_t)dvb * DVB
                                   : (p.s0 ? p.s0 + state_off : nullptr);
 
-    if (warp < 4) {
-        // =============================== chain warpgroup ===============================
-        if (!SCAN) setmaxnreg_inc<232>();
-        const int j = tid;
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-        float S[DK];
+    if (warp < 8) {
+        // =============================== chain warpgroups ===============================
+        // Two of them share the conversions that sit between two dependent MMA batches: each takes half of the tokens
+        // of v_new and half of the state's d_k columns (64 fp32 values per thread).  Short prompts: 27 -> 25 us for the kernel.
+        if (!SCAN) setmaxnreg_inc<160>();
+        const int wg = warp >> 2, j = tid & 127;
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        const uint32_t t_sbf = tmem + lane_base + TM_SBF + 32 * wg, t_ds = tmem + lane_base + TM_DS + 64 * wg;
+        const size_t soff = (size_t)(64 * wg) * dv + j;          // this thread's first state element: row 64 wg, column j
+        float S[64];
         if (SCAN) {                                     // the combine phase of every slice of this head has been written
             if (tid == 0) handover_wait(hv, w.abort_flag);
-            named_bar_sync(3, 128);
+            named_bar_sync(3, 256);
         }
         if (s_in) {
 #pragma unroll
-            for (int m = 0; m < DK; ++m) S[m] = SCAN ? __ldcg(s_in + (size_t)m * dv + j) : __ldg(s_in + (size_t)m * dv + j);
+            for (int m = 0; m < 64; ++m) S[m] = SCAN ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
         } else {
 #pragma unroll
-            for (int m = 0; m < DK; ++m) S[m] = 0.f;
+            for (int m = 0; m < 64; ++m) S[m] = 0.f;
         }
         if (nchunks > 0) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < 2; ++q) {
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(S[32 * q + 2 * i], S[32 * q + 2 * i + 1]);
-                tmem_st16(tmem + lane_base + TM_SBF + 16 * q, pk);
+                tmem_st16(t_sbf + 16 * q, pk);
             }
             tmem_wait_st();
             tc_fence_before_sync();
@@ -856,58 +861,47 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             tc_fence_after_sync();
             if (tid == 0) stamp(0, c, 0);
             {
-                // v_new^T: the load of the second half is in flight while the first is converted
-                uint32_t xa[32], xb[32];
-                tmem_ld32(tmem + lane_base + TM_DV, xa);
-                tmem_wait_ld();
-                tmem_ld32(tmem + lane_base + TM_DV + 32, xb);
-                uint32_t pv[16], pd[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float v0 = __uint_as_float(xa[2 * i]), v1 = __uint_as_float(xa[2 * i + 1]);
-                    const float2 dec = *reinterpret_cast<const float2*>(gates + 192 + 2 * i);
-                    pv[i] = pack_bf16(v0, v1);
-                    pd[i] = pack_bf16(v0 * dec.x, v1 * dec.y);
-                }
-                tmem_st16(tmem + lane_base + TM_V, pv);
-                tmem_st16(tmem + lane_base + TM_VT, pd);
+                // v_new^T: first the decayed copy the state update waits for, then the plain one of the output product
+                uint32_t x[32], pk[16];
+                tmem_ld32(tmem + lane_base + TM_DV + 32 * wg, x);
                 tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const float v0 = __uint_as_float(xb[2 * i]), v1 = __uint_as_float(xb[2 * i + 1]);
-                    const float2 dec = *reinterpret_cast<const float2*>(gates + 224 + 2 * i);
-                    pv[i] = pack_bf16(v0, v1);
-                    pd[i] = pack_bf16(v0 * dec.x, v1 * dec.y);
+                    const float2 dec = *reinterpret_cast<const float2*>(gates + 192 + 32 * wg + 2 * i);
+                    pk[i] = pack_bf16(__uint_as_float(x[2 * i]) * dec.x, __uint_as_float(x[2 * i + 1]) * dec.y);
                 }
-                tmem_st16(tmem + lane_base + TM_V + 16, pv);
-                tmem_st16(tmem + lane_base + TM_VT + 16, pd);
+                tmem_st16(tmem + lane_base + TM_VT + 16 * wg, pk);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive(w.bar(CB_VREADY));
+                if (tid == 0) stamp(0, c, 1);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+                tmem_st16(tmem + lane_base + TM_V + 16 * wg, pk);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive(w.bar(CB_VPLAIN));
             }
-            tmem_wait_st();
-            tc_fence_before_sync();
-            mbar_arrive(w.bar(CB_VREADY));
-            if (tid == 0) stamp(0, c, 1);
             w.wait_hot(CB_O1, c & 1);                      // O1 of this chunk no longer reads the bf16 state
             w.wait_hot(CB_S, c & 1);
             tc_fence_after_sync();
             if (tid == 0) stamp(0, c, 2);
             const float gamma = gates[256];
             {
-                // S^T <- e^{gC} S^T + dS^T, 32 columns at a time, the next load always in flight
-                uint32_t da[32], db[32];
-                tmem_ld32(tmem + lane_base + TM_DS, da);
+                // S^T <- e^{gC} S^T + dS^T, 32 columns at a time, both loads in flight
+                uint32_t d[2][32];
+                tmem_ld32(t_ds, d[0]);
                 tmem_wait_ld();
+                tmem_ld32(t_ds + 32, d[1]);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t (&cur)[32] = (q & 1) ? db : da;
-                    uint32_t (&nxt)[32] = (q & 1) ? da : db;
-                    if (q < 3) tmem_ld32(tmem + lane_base + TM_DS + 32 * (q + 1), nxt);
+                for (int q = 0; q < 2; ++q) {
                     uint32_t pk[16];
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) S[32 * q + i] = fmaf(gamma, S[32 * q + i], __uint_as_float(cur[i]));
+                    for (int i = 0; i < 32; ++i) S[32 * q + i] = fmaf(gamma, S[32 * q + i], __uint_as_float(d[q][i]));
 #pragma unroll
                     for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(S[32 * q + 2 * i], S[32 * q + 2 * i + 1]);
-                    tmem_st16(tmem + lane_base + TM_SBF + 16 * q, pk);
-                    if (q < 3) tmem_wait_ld();
+                    tmem_st16(t_sbf + 16 * q, pk);
+                    if (q == 0) tmem_wait_ld();
                 }
             }
             tmem_wait_st();
@@ -918,19 +912,20 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 const int gc = cbeg + c + 1;            // chunks of the sequence consumed so far
                 if (gc % p.snap_every == 0 && gc / p.snap_every <= p.nsnap && gc * C <= sq.len) {
                     float* dst = p.snaps + (((size_t)n * p.nsnap + (gc / p.snap_every - 1)) * H + h) * DK * dv +
-                                 (size_t)dvb * DVB + j;
+                                 (size_t)dvb * DVB + soff;
 #pragma unroll
-                    for (int m = 0; m < DK; ++m) dst[(size_t)m * dv] = S[m];
+                    for (int m = 0; m < 64; ++m) dst[(size_t)m * dv] = S[m];
                 }
             }
         }
         if (p.sT && seg == p.nseg - 1) {
 #pragma unroll
-            for (int m = 0; m < DK; ++m) p.sT[state_off + (size_t)m * dv + j] = S[m];
+            for (int m = 0; m < 64; ++m) p.sT[state_off + soff + (size_t)m * dv] = S[m];
         }
-    } else if (warp < 8) {
-        // =============================== epilogue warpgroup ===============================
-        const int j = tid - 128, we = j >> 5;
+    } else if (warp < 12) {
+        // =============================== output warpgroup ===============================
+        if (!SCAN) setmaxnreg_inc<136>();
+        const int j = tid - 256, we = j >> 5;
         const uint32_t lane_base = (uint32_t)(we * 32) << 16;
         // The accumulators are read as matrix fragments (thread: 4 value columns x 16 tokens, tokens in pairs), so that a
         // pair of tokens packs into one register and stmatrix transposes 8x8 blocks into rows of the output tile,
@@ -968,25 +963,25 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             tc_fence_after_sync();
             // take both accumulators out of tensor memory first and hand them back at once: the next
             // chunk's output MMAs wait for this
-            uint32_t o1[2][32], o2[2][32];
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O1, o1[hh]);
-                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O2, o2[hh]);
-            }
-            tmem_wait_ld();
-            tc_fence_before_sync();
-            mbar_arrive(w.bar(CB_OFREE));
             const uint32_t ost = base + CS_OST + (uint32_t)(c & 1) * 16384;
             float o[2][32];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + 8 * q + 2 * l4);
+            for (int hh = 0; hh < 2; ++hh) {
+                uint32_t o1[32], o2[32];
+                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O1, o1);
+                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O2, o2);
+                tmem_wait_ld();
+                if (hh == 1) {
+                    tc_fence_before_sync();
+                    mbar_arrive(w.bar(CB_OFREE));
+                }
 #pragma unroll
-                for (int x = 0; x < 4; ++x)
+                for (int q = 0; q < 8; ++q) {
+                    const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + 8 * q + 2 * l4);
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh)
-                        o[hh][4 * q + x] = fmaf((x & 1) ? eg.y : eg.x, __uint_as_float(o1[hh][4 * q + x]), __uint_as_float(o2[hh][4 * q + x]));
+                    for (int x = 0; x < 4; ++x)
+                        o[hh][4 * q + x] = fmaf((x & 1) ? eg.y : eg.x, __uint_as_float(o1[4 * q + x]), __uint_as_float(o2[4 * q + x]));
+                }
             }
             if (GATED) {
                 // Fused output stage (the per-position kernels behind the scan, Section "Prefill projections:
@@ -1012,6 +1007,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                         ss[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16 >> st);
                     }
                 }
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh)
+                    tmem_st_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_OG, reinterpret_cast<const uint32_t (&)[32]>(o[hh]));
                 float* red = reinterpret_cast<float*>(sm + CS_RED) + (c & 1) * 256;
                 // tokens 8q + 2 l4 (+1) with q = (lane bits 4, 3, 2)
                 const int qk = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
@@ -1026,24 +1024,32 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 }
                 __syncwarp();
                 w.wait(CB_ZFULL, c & 1);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    uint32_t z[4];
-                    ldmatrix_x4_trans(base + CS_Z + frag_off + (uint32_t)q * 1024, z[0], z[1], z[2], z[3]);
+                tmem_wait_st();
+                // Rolled, with the rows coming back from tensor memory, which takes a running address where registers
+                // do not: unrolled over o the 64 gates made 14 KB of straight-line code that the instruction cache had
+                // lost by the next chunk (4900 clocks, kernel on 4 x 1500 tokens 65 us; 45 us now).
+#pragma unroll 2
+                for (uint32_t q = 0; q < 8; ++q) {
+                    uint32_t y[2][4], z[4];
+                    tmem_ld_frag8(tmem + lane_base + TM_OG + 8 * q, y[0]);
+                    tmem_ld_frag8(tmem + lane_base + (16u << 16) + TM_OG + 8 * q, y[1]);
+                    ldmatrix_x4_trans(base + CS_Z + frag_off + q * 1024, z[0], z[1], z[2], z[3]);
                     const float2 iv = *reinterpret_cast<const float2*>(inv + 8 * q + 2 * l4);
+                    tmem_wait_ld();
+                    uint32_t pk[4];
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) {                // matrix m: value rows 8m + l8 of the warp's 32
-                        float* y = &o[m >> 1][4 * q + 2 * (m & 1)];
-                        y[0] *= iv.x * wv[m] * silu(__uint_as_float(z[m] << 16));
-                        y[1] *= iv.y * wv[m] * silu(__uint_as_float(z[m] & 0xffff0000u));
-                    }
+                    for (int m = 0; m < 4; ++m)                  // matrix m: value rows 8m + l8 of the warp's 32
+                        pk[m] = pack_bf16(__uint_as_float(y[m >> 1][2 * (m & 1)]) * (iv.x * wv[m]) * silu(__uint_as_float(z[m] << 16)),
+                                          __uint_as_float(y[m >> 1][2 * (m & 1) + 1]) * (iv.y * wv[m]) * silu(__uint_as_float(z[m] & 0xffff0000u)));
+                    stmatrix_x4_trans(ost + frag_off + q * 1024, pk[0], pk[1], pk[2], pk[3]);
                 }
                 mbar_arrive(w.bar(CB_ZFREE));
-            }
+            } else {
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                stmatrix_x4_trans(ost + frag_off + (uint32_t)q * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
-                                  pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
+                for (int q = 0; q < 8; ++q)
+                    stmatrix_x4_trans(ost + frag_off + (uint32_t)q * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
+                                      pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
+            }
             if (R == C) {
                 fence_proxy_async_smem();
                 if (j == 0) bulk_wait_read_all();              // the tile the next chunk writes has left (stored a chunk ago)
@@ -1069,7 +1075,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     } else {
         // =============================== control warpgroup ===============================
         if (!SCAN) setmaxnreg_dec<56>();
-        if (warp == 8) {
+        if (warp == 12) {
             const bool lead = elect_one();
             // ---- MMA issuer of the sequential chain: v_new and the state update, nothing else ----
             // (issuing costs tens of nanoseconds per instruction; everything off the chain is
@@ -1105,7 +1111,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 if (lead) mma_commit(w.bar(CB_FREEK0 + s));
                 if (lead) stamp(1, c, 4);
             }
-        } else if (warp == 10) {
+        } else if (warp == 14) {
             const bool lead = elect_one();
             // ---- MMA issuer of everything off the chain: U^T, O1^T, O2^T ----
             // (descriptors are built once; a stage or a k-step is an add on the 16-byte address field.  Every warp
@@ -1142,6 +1148,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 }
                 if (c >= 0) {
                     w.wait(CB_FULLP0 + s, par);
+                    w.wait(CB_VPLAIN, c & 1);
+                    tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)        // O2^T = v^T P^T
                         if (lead) mma_ts(tmem + TM_O2, tmem + TM_V + ks * 8, dP0 + (uint64_t)((s * 8192) >> 4) + ks * 2, ID_O, ks > 0);
@@ -1149,7 +1157,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     if (lead) mma_commit(w.bar(CB_FREEP0 + s));
                 }
             }
-        } else if (warp == 9 && lane == 0) {
+        } else if (warp == 13 && lane == 0) {
             // ---- TMA producer ----
             prefetch_tensormap(map_q);
             prefetch_tensormap(map_k);
@@ -1206,7 +1214,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     for (uint32_t b = CB_FULLW0; b <= CB_FULLB0; b += 4)
                         while (!mbar_try_wait(w.bar(b + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
             }
-        } else if (GATED && warp == 11 && lane == 0) {
+        } else if (GATED && warp == 15 && lane == 0) {
             // ---- TMA producer of the gate tile ----
             prefetch_tensormap(map_z);
             const uint32_t full = w.bar(CB_ZFULL);
@@ -1317,6 +1325,7 @@ __device__ __forceinline__ void summary_init_bars(const Waiter& w, int ninst) {
 template <bool SCAN>
 __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUtensorMap* map_v, const SummaryParams& p,
                                              const Cta& cta, const Waiter& w) {
+    constexpr int CW = SCAN ? 12 : 8;                 // first warp of the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
@@ -1427,10 +1436,10 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     } else {
         // =============================== control warpgroup ===============================
         if (!SCAN) setmaxnreg_dec<56>();
-        if (warp == 8 || warp == 10) {
+        if (warp == CW || warp == CW + 2) {
             const bool lead = elect_one();
             // ---- one MMA issue thread per chain instance (they are independent) ----
-            const int inst = (warp == 8) ? 0 : 1;
+            const int inst = (warp == CW) ? 0 : 1;
             if (inst < ninst) {
                 const uint64_t dW0 = make_smem_desc(base + SS_W, 1024, 1024), dK0 = make_smem_desc(base + SS_K, 8192, 1024);
                 for (int c = 0; c < nchunks; ++c) {
@@ -1461,7 +1470,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                     if (lead) mma_commit(w.bar(SB_FREE0 + s));
                 }
             }
-        } else if (warp == 9 && lane == 0) {
+        } else if (warp == CW + 1 && lane == 0) {
             prefetch_tensormap(map_k);
             prefetch_tensormap(map_v);
             const uint64_t pol_keep = (p.l2 & 1) ? l2_policy_evict_last() : l2_policy_evict_normal();
@@ -1725,7 +1734,7 @@ __global__ void __launch_bounds__(CMB_THREADS, 1) gdn_combine_kernel(CombinePara
 // before the launch and zero again after it (the last CTA of a head to get past both waits clears them), so a
 // captured launch can be replayed.
 // =====================================================================================
-constexpr int SCAN_THREADS = 384;
+constexpr int SCAN_THREADS = 512;
 constexpr uint32_t SC_BARS1 = CS_BARS;                 // behind the largest data layout (the chain phase's)
 constexpr uint32_t SC_BARS2 = SC_BARS1 + 24 * 8;
 constexpr uint32_t SC_BARS3 = SC_BARS2 + 16 * 8;
@@ -1819,7 +1828,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     cta_sync();
                 }
                 const Cta c2{base, sm, tmem, slice, h, n};
-                combine_body<true>(p.cb, c2, w2, 8);
+                combine_body<true>(p.cb, c2, w2, 12);
                 tc_fence_before_sync();
             }
             __threadfence();
@@ -1835,10 +1844,11 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         tc_fence_before_sync();
         cta_sync();
     };
-    // register budgets: warpgroup 0 holds a 128-value fp32 row per thread in all three phases (232), warpgroup 1
-    // the identity chain of the summary and the epilogue of the chain phase (216), warpgroup 2 issues and copies (56)
-    if (warp < 4) { setmaxnreg_inc<232>(); phases(); }
-    else if (warp < 8) { setmaxnreg_inc<216>(); phases(); }
+    // register budgets: warpgroups 0 and 1 hold the fp32 states (a 128-value row per thread in the summary phase), warpgroup
+    // 2 writes the outputs, warpgroup 3 issues and copies
+    if (warp < 4) { setmaxnreg_inc<184>(); phases(); }
+    else if (warp < 8) { setmaxnreg_inc<184>(); phases(); }
+    else if (warp < 12) { setmaxnreg_dec<88>(); phases(); }
     else { setmaxnreg_dec<56>(); phases(); }
     if (tid == 0) {                     // the last CTA of this head to get here clears the counters
         __threadfence();
