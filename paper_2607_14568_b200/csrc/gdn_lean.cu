@@ -72,7 +72,7 @@ constexpr uint32_t IT_GATES = 32768;  //  1280: g log2e | beta | e^g | e^{gC-g} 
 constexpr uint32_t GATE_FLOATS = 320;
 constexpr uint32_t ITEM_BYTES = 34048;
 
-constexpr uint32_t LDA = 68, LDY = 32;
+constexpr uint32_t LDA = 68;
 
 // Bounded waits.  Their slow path is inlined at some thirty sites of kernels whose warp roles all run their
 // loops at once, and the instruction footprint decides the chain kernel's speed (measured: with 82 KiB of code
@@ -188,12 +188,11 @@ constexpr uint32_t PS_A = 32768;                      // fp32 A [64][68], turned
                                                       // later the staging space of the -W^T image
 constexpr uint32_t PS_T1 = PS_KQ + 24576;             // (T diag(b e^g))^T image over the Q_hi tile (dead after G)
 constexpr uint32_t PS_T2 = PS_KQ + 8192;              // (T diag(b))^T image over the Q_lo tile, after the P image
-constexpr uint32_t PS_Y = PS_A + 64 * LDA * 4;
-constexpr uint32_t PS_GATES = PS_Y + 32 * LDY * 4;
+constexpr uint32_t PS_GATES = PS_A + 64 * LDA * 4;
 constexpr uint32_t PS_RN = PS_GATES + GATE_FLOATS * 4;     // raw inputs: 1/|k_i| (64), 1/|q_r| (64)
 constexpr uint32_t PS_BARS = PS_RN + 128 * 4;
 constexpr uint32_t PS_MISC = PS_BARS + 16 * 8;
-constexpr uint32_t PS_TOTAL = PS_MISC + 64;
+constexpr uint32_t PS_TOTAL = PS_MISC + 64;          // tensor-memory address, abort flag, two item slots of four words
 constexpr uint32_t PREP_SMEM = PS_TOTAL + 1024;
 constexpr int PREP_THREADS = 192;
 constexpr uint32_t PT_COLS = 64;
@@ -208,7 +207,7 @@ struct PrepParams {
     long nslots;
     int B, T, H;
     float gate_scale, eps;     // raw inputs only
-    int* ticket;               // {next item, CTAs done}: both zero before the launch, both zero again after it
+    int* ticket;               // next item beyond the first one of every CTA: zero before the launch; the chain kernel zeroes it again
     int l2;                    // bit 0: the K tiles are read again by later kernels of this call and fit in L2: keep them there;
                                // bit 1: the same for the W and T2 images this kernel writes
 };
@@ -259,6 +258,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int H = p.H;
     pdl_trigger();                      // the next kernel of the call may set itself up while this one runs
+    if (warp == 4) { prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); }
     if (tid == 0) {
         mbar_init(w.bar(PB_FULL), 1); mbar_init(w.bar(PB_G), 1); mbar_init(w.bar(PB_W), 1);
         mbar_init(w.bar(PB_TREADY), 128); mbar_init(w.bar(PB_GREADY), 32); mbar_init(w.bar(PB_DONE), 128);
@@ -275,36 +275,42 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
 
-    // Items are handed out through a global ticket: the time per item differs between SMs by a
-    // quarter, so a fixed assignment would leave the fast ones idle at the end.  The issuing thread
-    // draws the ticket one item ahead and publishes it in shared memory (slot it & 1, barrier PB_ITEM).
+    pdl_wait();                         // the scratch may still be read, and the inputs written, by what ran before
+
+    // Every CTA starts with the item of its own index; further ones are handed out through a global ticket: the time per
+    // item differs between SMs by a quarter, so a fixed assignment would leave the fast ones idle at the end.  The
+    // issuing warp draws the ticket one item ahead and publishes the item (number, head, first token, rows) in shared
+    // memory (slot it & 1, barrier PB_ITEM), so that nobody else looks the sequence up.
     const long nitems = p.nslots * H;
-    int nh = 0, nR = 0;      // issuing thread: head, first token of the item it drew last
+    int nh = 0, nR = 0;      // issuing warp: head, first token of the item it drew last
     long ntok = 0;
-    auto draw = [&]() -> int {           // (whole warp 4) next ticket that names a used slot, or -1
+    auto draw = [&](int t) -> int {      // (whole warp 4) t, or the next ticket, that names a used slot; -1 = no more
         while (true) {
-            int t = 0;
-            if (lane == 0) t = atomicAdd(p.ticket, 1);
-            t = (int)warp_uniform((uint32_t)t);
+            if (t < 0) {
+                if (lane == 0) t = (int)gridDim.x + atomicAdd(p.ticket, 1);
+                t = (int)warp_uniform((uint32_t)t);
+            }
             if (t >= nitems) return -1;
             if (decode_item(p, t, &nh, &ntok, &nR)) return t;
+            t = -1;
         }
     };
-    if (warp == 4) {
-        const int first = draw();
+    auto publish = [&](int slot, int item) {
         if (lane == 0) {
-            sMisc[2] = (uint32_t)first;
+            volatile uint32_t* m = sMisc + 4 + 4 * slot;
+            m[0] = (uint32_t)item; m[1] = (uint32_t)nh; m[2] = (uint32_t)ntok; m[3] = (uint32_t)nR;
             mbar_arrive(w.bar(PB_ITEM));
         }
-    }
+    };
+    if (warp == 4) publish(0, draw((int)blockIdx.x));
     int it = 0;     // items this CTA has processed (barrier phases)
     while (true) {
         w.wait(PB_ITEM, it & 1);
-        const long item = (int)sMisc[2 + (it & 1)];
+        volatile uint32_t* m_item = sMisc + 4 + 4 * (it & 1);
+        const long item = (int)m_item[0];
+        const int h = (int)m_item[1], R = (int)m_item[3];
+        const long tok = (int)m_item[2];
         if (item < 0 || *w.abort_flag) break;
-        int h, R;
-        long tok;
-        decode_item(p, item, &h, &tok, &R);
         uint8_t* out_item = p.items + (size_t)item * ITEM_BYTES;
         const uint32_t par = it & 1;
 
@@ -336,6 +342,9 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 sRN[tp] = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
                 named_bar_sync(1, 128);
             }
+            // the -W^T image of the previous item has left the space of A by now; everybody is about to write there
+            if (tp == 0) bulk_wait_read_all();
+            named_bar_sync(1, 128);
             w.wait(PB_G, par);
             tc_fence_after_sync();
             // ---- step b1: decay masks on G = [K;Q] K^T ----
@@ -575,6 +584,10 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 tmem_wait_ld();
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
+                    if (hh == 1 && ch == 0) {                  // accumulator and gate vectors have been read: the next item's G may come
+                        tc_fence_before_sync();
+                        mbar_arrive(w.bar(PB_DONE));
+                    }
                     uint32_t pk[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
@@ -587,10 +600,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (tp == 0) {                                     // staged over the fp32 T, which is dead by now
                 bulk_store_hint(out_item + IT_W, base + PS_A, 16384, (p.l2 & 2) ? l2_policy_evict_last() : l2_policy_evict_normal());
                 bulk_commit();
-                bulk_wait_read_all();                          // the staging space may now be overwritten
             }
-            tc_fence_before_sync();
-            mbar_arrive(w.bar(PB_DONE));
         } else if (warp == 4) {
             // ================= TMA + MMA issue (one elected thread) =================
             {
@@ -615,7 +625,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     if (lead) mma_ss(tmem, make_smem_desc(kq + off, 16, 1024), make_smem_desc(kq + off, 16, 1024), ID_G, ks > 0);
                 }
                 if (lead) mma_commit(w.bar(PB_G));
-                const int nxt = draw();                             // the atomic's latency hides behind the solve
+                const int nxt = draw(-1);                           // the atomic's latency hides behind the solve
                 w.wait(PB_TREADY, par);
                 tc_fence_after_sync();
 #pragma unroll
@@ -628,10 +638,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     w.wait(PB_KQFREE, par);
                     load_tiles(nh, ntok);
                 }
-                if (lead) {
-                    sMisc[2 + ((it + 1) & 1)] = (uint32_t)nxt;
-                    mbar_arrive(w.bar(PB_ITEM));
-                }
+                publish((it + 1) & 1, nxt);
             }
         } else {
             // ================= step a: chunk-local cumulative log gate (one warp) =================
@@ -668,14 +675,6 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (warp == 0) {
         tc_fence_after_sync();
         tmem_dealloc(tmem, PT_COLS);
-    }
-    if (tid == 0) {      // the last CTA to leave re-arms the ticket for the next launch
-        __threadfence();
-        if (atomicAdd(p.ticket + 1, 1) == (int)gridDim.x - 1) {
-            p.ticket[0] = 0;
-            p.ticket[1] = 0;
-            __threadfence();
-        }
     }
 }
 
@@ -738,6 +737,7 @@ struct ChainParams {
     const __nv_bfloat16* gate_z;   // [.., H, d_v] like out, or nullptr
     const float* norm_w;           // [d_v]
     float norm_eps;
+    int* ticket;                   // the prepare kernel's item ticket: zeroed here for the next call (that kernel has completed)
 };
 
 // One CTA's identity inside a kernel: aligned shared-memory base (address and pointer), tensor-memory base,
@@ -795,6 +795,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
+    if (tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
     const int n = cta.z / p.nseg, seg = cta.z % p.nseg;
     const int H = p.H, dv = p.dv;
     const SeqInfo sq = seq_info(p.cu, n, p.T);
@@ -1257,6 +1258,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
+    pdl_trigger();                      // the next call's prepare kernel may set itself up as SMs come free
     pdl_wait();                         // scratch items and incoming states come from the kernels before this one
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
     chain_body<DBG, false, GATED>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
@@ -1868,24 +1870,32 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
-// Sequence split: only for batched (equal-length) input with few chains.  Returns the number
-// of segments per sequence (1 = no split) and the chunks per segment.
+// Sequence split: only for batched (equal-length) input.  Returns the number of segments per sequence (1 = no split) and
+// the chunks per segment: the cheapest by the model below, whose constants are fits of the kernels' times on a B200 in units
+// of 0.1 us (d_v = 128; n chunks per segment).  A step of a chain takes 1.04 us by itself and longer when the CTAs
+// together ask for more than the memory delivers (98 KB per chain step, 57 KB per summary step); summaries and chains cost
+// about 12 and 9 us besides their steps, the combination 5 us and 1.5 us a hop for every round of its CTAs (one per
+// SM), and programmatic launches hide about 8 us of a split's start-ups.  So a split pays from about 28 chunks on for 16
+// chains (2048 tokens: 52 us in one piece, 49.5 us in eight), and not at all when fewer than three segments per chain
+// fit the GPU (4 x 1500 tokens, 16 heads: 64 us in one piece, 86 us in two).
+constexpr int kMaxSeg = 16;
 static void plan_split(int B, int T, int H, int d_v, bool packed, int num_sms, int* nseg, int* seg_chunks) {
     const int nch = (T + C - 1) / C;
     *nseg = 1;
     *seg_chunks = nch > 0 ? nch : 1;
-    if (packed || nch < 16) return;
     const long chains = (long)B * H * (d_v / DVB);
-    if (chains * 2 > num_sms) return;
-    int want = (int)(num_sms / chains);
-    if (want > 16) want = 16;
-    if (want > nch / 4) want = nch / 4;                 // at least four chunks per segment
-    if (want < 2) return;
-    const int sc = (nch + want - 1) / want;
-    *seg_chunks = sc;
-    *nseg = (nch + sc - 1) / sc;
+    if (packed || nch < 2 || chains * 2 > num_sms) return;
+    auto steps = [](long ctas, int n, double per_cta) { return n * (ctas * per_cta > 10.4 ? ctas * per_cta : 10.4); };
+    double best = 90 + steps(chains, nch, 0.137);
+    const int most = (int)(num_sms / chains) < kMaxSeg ? (int)(num_sms / chains) : kMaxSeg;
+    for (int want = 2; want <= most; ++want) {
+        const int sc = (nch + want - 1) / want, ns = (nch + sc - 1) / sc;
+        if (ns < 2) break;
+        const long rounds = (chains * (DVB / CMB_COLS) + num_sms - 1) / num_sms;
+        const double cost = 125 + steps(chains * (ns - 1), sc, 0.092) + rounds * (50 + 15 * (ns - 1)) + 90 + steps(chains * ns, sc, 0.137) - 80;
+        if (cost < best) { best = cost; *nseg = ns; *seg_chunks = sc; }
+    }
 }
-constexpr int kMaxSeg = 16;
 
 // In front of the items: the prepare kernel's item ticket (two ints) and, from int 16 on, the scan kernel's
 // counters (four ints per (sequence, head)).  All of it reads zero before a call and zero again after it.
@@ -2014,8 +2024,8 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     const int pgrid = (int)(nitems < 4L * num_sms ? nitems : 4L * num_sms);
     auto mark = [&](int i) { if (g_lean_timing && g_lean_events[i]) cudaEventRecord(g_lean_events[i], stream); };
     mark(0);
-    if (opt.raw) gdn_prep_kernel<true><<<pgrid, PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
-    else gdn_prep_kernel<false><<<pgrid, PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
+    if (opt.raw) launch_after(gdn_prep_kernel<true>, dim3(pgrid), PREP_THREADS, PREP_SMEM, stream, mq, mk, pp);
+    else launch_after(gdn_prep_kernel<false>, dim3(pgrid), PREP_THREADS, PREP_SMEM, stream, mq, mk, pp);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
     mark(1);
@@ -2035,7 +2045,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
         if (g_lean_use_scan && !opt.gate_z && a.d_v == DVB && (long)a.B * a.H * nseg <= num_sms && (long)a.B * a.H <= kMaxScanChains) {
             ChainParams cp{a.initial_state, static_cast<__nv_bfloat16*>(a.out), a.final_state, a.cu_seqlens,
                            ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, nseg, seg_chunks,
-                           snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps};
+                           snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket};
             ScanParams scp{sp, cb, cp, static_cast<int*>(workspace) + kScanFlagOffset};
             dim3 grid(1, a.H, a.B * nseg);
             if (g_lean_dbg) launch_after(gdn_scan_kernel<true>, grid, SCAN_THREADS, SCAN_SMEM, stream, mq, mk, mv, mo, scp);
@@ -2059,7 +2069,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // ---- steps c, d ----
     ChainParams cp{a.initial_state, static_cast<__nv_bfloat16*>(a.out), a.final_state, a.cu_seqlens,
                    ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, nseg, seg_chunks,
-                   snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps};
+                   snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket};
     dim3 grid(a.d_v / DVB, a.H, a.B * nseg);
     if (opt.gate_z) launch_after(gdn_chain_kernel<false, true>, grid, CHAIN_THREADS, CHAIN_SMEM_GATED, stream, mq, mk, mv, mo, mz, cp);
     else if (g_lean_dbg) launch_after(gdn_chain_kernel<true, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
@@ -2170,7 +2180,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
     const int nch = packed ? 1 : (a.T + C - 1) / C;            // one segment: the whole sequence
     ChainParams cp{a.initial_state, static_cast<__nv_bfloat16*>(a.out), a.final_state, a.cu_seqlens,
                    ws, nullptr, nullptr, -1, a.B, a.T, a.H, a.d_v, 1, packed ? (1 << 24) : (nch > 0 ? nch : 1),
-                   nullptr, 1, 0};
+                   nullptr, 1, 0, 0, nullptr, nullptr, 0.f, static_cast<int*>(ticket_of_device[dev])};
     dim3 grid(a.d_v / DVB, a.H, a.B);
     gdn_chain_kernel<false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
     count_launch();
