@@ -159,14 +159,11 @@ __device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// z / (1 + e^-z); the reciprocal is refined by one Newton step (about one unit in the last place, as a division, without
-// the branches of one)
+// z / (1 + e^-z) with the hardware reciprocal (one unit in the last place; 0 for e^-z = inf)
 __device__ __forceinline__ float silu(float z) {
-    const float d = 1.0f + ex2(z * -LOG2E);
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    r = r * fmaf(-d, r, 2.0f);
-    return d > 8e37f ? 0.0f : z * r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + ex2(z * -LOG2E)));
+    return z * r;
 }
 
 // slot of chunk 0 of sequence n: disjoint ranges for any lengths, total <= tokens/64 + B
@@ -682,6 +679,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // chain kernel (steps c and d)
 // =====================================================================================
 constexpr int CHAIN_THREADS = 512;          // two chain warpgroups, output warpgroup, control warpgroup
+constexpr int CHAIN_THREADS_GATED = 640;    // two output warpgroups, 32 tokens each
 // tensor memory columns
 constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384,
                    TM_OG = 448;   // fused output stage: the combined fp32 output rows
@@ -778,19 +776,27 @@ __device__ __forceinline__ bool handover_wait(const Handover& hv, volatile int* 
     return true;
 }
 
-__device__ __forceinline__ void chain_init_bars(const Waiter& w) {
-    for (uint32_t i = CB_FULLW0; i < CB_V; ++i) mbar_init(w.bar(i), i == CB_ZFREE ? 128 : 1);
+__device__ __forceinline__ void chain_init_bars(const Waiter& w, int out_threads) {
+    for (uint32_t i = CB_FULLW0; i < CB_V; ++i) mbar_init(w.bar(i), i == CB_ZFREE ? out_threads : 1);
     mbar_init(w.bar(CB_U), 1); mbar_init(w.bar(CB_O1), 1);
     mbar_init(w.bar(CB_V), 1); mbar_init(w.bar(CB_S), 1); mbar_init(w.bar(CB_O), 1);
-    mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256); mbar_init(w.bar(CB_OFREE), 128);
+    mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256); mbar_init(w.bar(CB_OFREE), out_threads);
     mbar_init(w.bar(CB_CLEAN), 128);
 }
+
+// fragment loads and stores by the number of registers
+__device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[32]) { tmem_ld_frag64(a, r); }
+__device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { tmem_ld_frag32(a, r); }
+__device__ __forceinline__ void put_frags(uint32_t a, const float (&o)[16]) { tmem_st_frag32(a, reinterpret_cast<const uint32_t (&)[16]>(o)); }
+__device__ __forceinline__ void put_frags(uint32_t, const float (&)[32]) {}                  // (plain output: never called)
 
 // Steps c and d for one CTA.  SCAN: called from the merged scan kernel (register budgets are set there, the
 // incoming state is awaited through `hv` and read past the L1 cache, since another SM wrote it in this launch).
 template <bool DBG, bool SCAN, bool GATED>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
+    constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments of each
+    constexpr int CW = 8 + 4 * NOUT;                         // first warp of the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
@@ -826,7 +832,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         // =============================== chain warpgroups ===============================
         // Two of them share the conversions that sit between two dependent MMA batches: each takes half of the tokens
         // of v_new and half of the state's d_k columns (64 fp32 values per thread).  Short prompts: 27 -> 25 us for the kernel.
-        if (!SCAN) setmaxnreg_inc<160>();
+        if (!SCAN) setmaxnreg_inc<GATED ? 136 : 160>();
         const int wg = warp >> 2, j = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t t_sbf = tmem + lane_base + TM_SBF + 32 * wg, t_ds = tmem + lane_base + TM_DS + 64 * wg;
@@ -923,16 +929,18 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
 #pragma unroll
             for (int m = 0; m < 64; ++m) p.sT[state_off + soff + (size_t)m * dv] = S[m];
         }
-    } else if (warp < 12) {
-        // =============================== output warpgroup ===============================
-        if (!SCAN) setmaxnreg_inc<136>();
-        const int j = tid - 256, we = j >> 5;
+    } else if (warp < CW) {
+        // =============================== output warpgroup(s) ===============================
+        if (!SCAN) { if (GATED) setmaxnreg_dec<80>(); else setmaxnreg_inc<136>(); }
+        const int og = (warp - 8) >> 2, q0 = og * QN;            // this warpgroup's tokens: 8 q0 .. 8 (q0 + QN) - 1
+        const int j = (tid - 256) & 127, we = j >> 5;
         const uint32_t lane_base = (uint32_t)(we * 32) << 16;
         // The accumulators are read as matrix fragments (thread: 4 value columns x 16 tokens, tokens in pairs), so that a
         // pair of tokens packs into one register and stmatrix transposes 8x8 blocks into rows of the output tile,
         // which leaves as two TMA stores (a last, partial chunk by plain stores: the rows behind it belong to others).
         // This role must stay shorter than a chain step: with one 2-byte store per value and row copies by
-        // the threads it took 1.6 us a chunk and set the pace of the whole kernel.
+        // the threads it took 1.6 us a chunk and set the pace of the whole kernel.  (With the fused output stage a single
+        // warpgroup is limited by how fast one warp per scheduler can issue, so two of them take 32 tokens each.)
         const int l4 = lane & 3, l8 = lane >> 2;                 // fragment: columns 8q + 2 l4 (+1) are tokens, rows l8 (+8) values
         // lane's part in stmatrix / ldmatrix: value columns 8 piece .. +7 of token 8q + (lane & 7)
         const uint32_t piece = 4u * (uint32_t)we + (uint32_t)(lane >> 3);
@@ -945,7 +953,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         for (int c = 0; c < nchunks; ++c) {
             const int R = min(C, len - c * C);
             const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
-            if (tail_c >= 0 && c == max(tail_c - 1, 0)) {
+            if (og == 0 && tail_c >= 0 && c == max(tail_c - 1, 0)) {
                 const int Rt = len - tail_c * C;
                 const uint32_t sk = base + CS_K + (uint32_t)(tail_c & 1) * 16384;
                 const uint32_t sv = base + CS_B + (uint32_t)(tail_c & 1) * STAGE_B + ST_V;
@@ -965,20 +973,20 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             // take both accumulators out of tensor memory first and hand them back at once: the next
             // chunk's output MMAs wait for this
             const uint32_t ost = base + CS_OST + (uint32_t)(c & 1) * 16384;
-            float o[2][32];
+            float o[2][4 * QN];
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-                uint32_t o1[32], o2[32];
-                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O1, o1);
-                tmem_ld_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O2, o2);
+                uint32_t o1[4 * QN], o2[4 * QN];
+                tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O1 + 8 * q0, o1);
+                tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O2 + 8 * q0, o2);
                 tmem_wait_ld();
                 if (hh == 1) {
                     tc_fence_before_sync();
                     mbar_arrive(w.bar(CB_OFREE));
                 }
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + 8 * q + 2 * l4);
+                for (int q = 0; q < QN; ++q) {
+                    const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + 8 * (q0 + q) + 2 * l4);
 #pragma unroll
                     for (int x = 0; x < 4; ++x)
                         o[hh][4 * q + x] = fmaf((x & 1) ? eg.y : eg.x, __uint_as_float(o1[4 * q + x]), __uint_as_float(o2[4 * q + x]));
@@ -990,17 +998,18 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 // axis, weight vector, SiLU gate.  A token's squares lie in the eight lanes of equal l4 of every warp:
                 // a butterfly that halves the tokens at each step leaves two tokens' sums per lane, the four warps' sums meet
                 // in shared memory.  gate_z comes by TMA a chunk ahead and is read in the same fragments.
-                float ss[16];
+                float ss[2 * QN];
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
+                for (int q = 0; q < QN; ++q)
 #pragma unroll
                     for (int x = 0; x < 2; ++x) {
                         const float a0 = o[0][4 * q + x], a1 = o[0][4 * q + 2 + x], a2 = o[1][4 * q + x], a3 = o[1][4 * q + 2 + x];
                         ss[2 * q + x] = fmaf(a0, a0, a1 * a1) + fmaf(a2, a2, a3 * a3);
                     }
+                // eight values over eight lanes: after the three steps a lane holds one token's sum over its warp
 #pragma unroll
                 for (int st = 0; st < 3; ++st) {
-                    const int half = 8 >> st;                    // values kept: the upper half of the tokens where the lane bit is set
+                    const int half = QN >> st;                   // values kept: the upper half where the lane bit is set
                     const bool up = (lane & (16 >> st)) != 0;
 #pragma unroll
                     for (int i = 0; i < half; ++i) {
@@ -1008,18 +1017,15 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                         ss[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16 >> st);
                     }
                 }
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh)
-                    tmem_st_frag64(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_OG, reinterpret_cast<const uint32_t (&)[32]>(o[hh]));
+                put_frags(tmem + lane_base + TM_OG + 8 * q0, o[0]);
+                put_frags(tmem + lane_base + (16u << 16) + TM_OG + 8 * q0, o[1]);
+                // value index = lane bits 4, 3, 2 = 2 q + x: token 8 (q0 + q) + 2 l4 + x
                 float* red = reinterpret_cast<float*>(sm + CS_RED) + (c & 1) * 256;
-                // tokens 8q + 2 l4 (+1) with q = (lane bits 4, 3, 2)
-                const int qk = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-                *reinterpret_cast<float2*>(red + we * 64 + 8 * qk + 2 * l4) = make_float2(ss[0], ss[1]);
-                named_bar_sync(2, 128);
+                red[we * 64 + 8 * (q0 + (lane >> 4) * 2 + ((lane >> 3) & 1)) + 2 * l4 + ((lane >> 2) & 1)] = ss[0];
+                named_bar_sync(5 + og, 128);
                 float* inv = reinterpret_cast<float*>(sm + CS_INV) + we * 64;
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    const int tk = lane + 32 * x;
+                {
+                    const int tk = 8 * q0 + lane;                // 32 tokens, one per lane
                     const float sum = (red[tk] + red[64 + tk]) + (red[128 + tk] + red[192 + tk]);
                     inv[tk] = rsqrtf(sum * (1.0f / DVB) + p.norm_eps);
                 }
@@ -1027,10 +1033,10 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 w.wait(CB_ZFULL, c & 1);
                 tmem_wait_st();
                 // Rolled, with the rows coming back from tensor memory, which takes a running address where registers
-                // do not: unrolled over o the 64 gates made 14 KB of straight-line code that the instruction cache had
-                // lost by the next chunk (4900 clocks, kernel on 4 x 1500 tokens 65 us; 45 us now).
+                // do not: unrolled over o the gates made 14 KB of straight-line code that the instruction cache had
+                // lost by the next chunk.
 #pragma unroll 2
-                for (uint32_t q = 0; q < 8; ++q) {
+                for (uint32_t q = q0; q < (uint32_t)(q0 + QN); ++q) {
                     uint32_t y[2][4], z[4];
                     tmem_ld_frag8(tmem + lane_base + TM_OG + 8 * q, y[0]);
                     tmem_ld_frag8(tmem + lane_base + (16u << 16) + TM_OG + 8 * q, y[1]);
@@ -1047,36 +1053,36 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 mbar_arrive(w.bar(CB_ZFREE));
             } else {
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    stmatrix_x4_trans(ost + frag_off + (uint32_t)q * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
+                for (int q = 0; q < QN; ++q)
+                    stmatrix_x4_trans(ost + frag_off + (uint32_t)(q0 + q) * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
                                       pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
             }
             if (R == C) {
                 fence_proxy_async_smem();
-                if (j == 0) bulk_wait_read_all();              // the tile the next chunk writes has left (stored a chunk ago)
-                named_bar_sync(2, 128);
-                if (j == 0) {
+                if (j == 0 && og == 0) bulk_wait_read_all();              // the tile the next chunk writes has left (stored a chunk ago)
+                named_bar_sync(2, 128 * NOUT);
+                if (j == 0 && og == 0) {
                     const int tok = (int)(tok0 + (long)c * C);
                     tma_store_3d(map_o, dvb * DVB, h, tok, ost);
                     tma_store_3d(map_o, dvb * DVB + 64, h, tok, ost + 8192);
                     bulk_commit();
                 }
             } else {
-                named_bar_sync(2, 128);
+                named_bar_sync(2, 128 * NOUT);
                 __nv_bfloat16* obase = p.out + ((size_t)(tok0 + c * C) * H + h) * dv + (size_t)dvb * DVB;
 #pragma unroll 1
-                for (int qd = j; qd < R * 16; qd += 128) {
+                for (int qd = j + 128 * og; qd < R * 16; qd += 128 * NOUT) {
                     const uint32_t r = (uint32_t)qd >> 4, pc = (uint32_t)qd & 15u;
                     const uint4 val = *reinterpret_cast<const uint4*>(sm + CS_OST + (c & 1) * 16384 + (pc >> 3) * 8192 + swz(r, pc & 7));
                     *reinterpret_cast<uint4*>(obase + (size_t)r * H * dv + pc * 8) = val;
                 }
             }
         }
-        if (j == 0) bulk_wait_all();
+        if (j == 0 && og == 0) bulk_wait_all();
     } else {
         // =============================== control warpgroup ===============================
-        if (!SCAN) setmaxnreg_dec<56>();
-        if (warp == 12) {
+        if (!SCAN) setmaxnreg_dec<GATED ? 48 : 56>();
+        if (warp == CW) {
             const bool lead = elect_one();
             // ---- MMA issuer of the sequential chain: v_new and the state update, nothing else ----
             // (issuing costs tens of nanoseconds per instruction; everything off the chain is
@@ -1112,7 +1118,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 if (lead) mma_commit(w.bar(CB_FREEK0 + s));
                 if (lead) stamp(1, c, 4);
             }
-        } else if (warp == 14) {
+        } else if (warp == CW + 2) {
             const bool lead = elect_one();
             // ---- MMA issuer of everything off the chain: U^T, O1^T, O2^T ----
             // (descriptors are built once; a stage or a k-step is an add on the 16-byte address field.  Every warp
@@ -1158,7 +1164,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     if (lead) mma_commit(w.bar(CB_FREEP0 + s));
                 }
             }
-        } else if (warp == 13 && lane == 0) {
+        } else if (warp == CW + 1 && lane == 0) {
             // ---- TMA producer ----
             prefetch_tensormap(map_q);
             prefetch_tensormap(map_k);
@@ -1215,7 +1221,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     for (uint32_t b = CB_FULLW0; b <= CB_FULLB0; b += 4)
                         while (!mbar_try_wait(w.bar(b + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
             }
-        } else if (GATED && warp == 15 && lane == 0) {
+        } else if (GATED && warp == CW + 3 && lane == 0) {
             // ---- TMA producer of the gate tile ----
             prefetch_tensormap(map_z);
             const uint32_t full = w.bar(CB_ZFULL);
@@ -1235,7 +1241,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
 }
 
 template <bool DBG, bool GATED>
-__global__ void __launch_bounds__(CHAIN_THREADS, 1)
+__global__ void __launch_bounds__(GATED ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
 gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                  const __grid_constant__ CUtensorMap map_z, ChainParams p) {
@@ -1246,7 +1252,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     Waiter w{base + CS_BARS, reinterpret_cast<volatile int*>(sm + CS_MISC + 4)};
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        chain_init_bars(w);
+        chain_init_bars(w, GATED ? 256 : 128);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -1778,7 +1784,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (tid == 0) {
         summary_init_bars(w1, 2);
         combine_init_bars(w2);
-        chain_init_bars(w3);
+        chain_init_bars(w3, 128);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -2071,7 +2077,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                    ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, nseg, seg_chunks,
                    snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket};
     dim3 grid(a.d_v / DVB, a.H, a.B * nseg);
-    if (opt.gate_z) launch_after(gdn_chain_kernel<false, true>, grid, CHAIN_THREADS, CHAIN_SMEM_GATED, stream, mq, mk, mv, mo, mz, cp);
+    if (opt.gate_z) launch_after(gdn_chain_kernel<false, true>, grid, CHAIN_THREADS_GATED, CHAIN_SMEM_GATED, stream, mq, mk, mv, mo, mz, cp);
     else if (g_lean_dbg) launch_after(gdn_chain_kernel<true, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
     else launch_after(gdn_chain_kernel<false, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
     count_launch();
