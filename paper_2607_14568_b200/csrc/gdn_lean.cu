@@ -682,7 +682,7 @@ constexpr int CHAIN_THREADS = 512;          // two chain warpgroups, output warp
 constexpr int CHAIN_THREADS_GATED = 640;    // two output warpgroups, 32 tokens each
 // tensor memory columns
 constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384,
-                   TM_OG = 448;   // fused output stage: the combined fp32 output rows
+                   TM_OG = 448;   // fused output stage: norm_w * silu(gate_z) of the chunk, fp32
 constexpr uint32_t CT_COLS = 512;
 // shared memory: every operand has a ring of its own, released by the completion of the MMAs that read it, so that a
 // slot is refilled as soon as its one use is over and a load has well over a chunk step to arrive.  (With
@@ -787,8 +787,6 @@ __device__ __forceinline__ void chain_init_bars(const Waiter& w, int out_threads
 // fragment loads and stores by the number of registers
 __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[32]) { tmem_ld_frag64(a, r); }
 __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { tmem_ld_frag32(a, r); }
-__device__ __forceinline__ void put_frags(uint32_t a, const float (&o)[16]) { tmem_st_frag32(a, reinterpret_cast<const uint32_t (&)[16]>(o)); }
-__device__ __forceinline__ void put_frags(uint32_t, const float (&)[32]) {}                  // (plain output: never called)
 
 // Steps c and d for one CTA.  SCAN: called from the merged scan kernel (register budgets are set there, the
 // incoming state is awaited through `hv` and read past the L1 cache, since another SM wrote it in this launch).
@@ -968,6 +966,26 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 fence_proxy_async_smem();
                 mbar_arrive(w.bar(CB_CLEAN));
             }
+            if (GATED) {
+                // The gates do not depend on the chain: they are formed while this chunk's outputs are still on their way, and
+                // wait in tensor memory, which takes a running address where registers do not (unrolled, the
+                // gates made 14 KB of straight-line code that the instruction cache had lost by the next chunk).
+                w.wait(CB_ZFULL, c & 1);
+#pragma unroll 2
+                for (uint32_t q = q0; q < (uint32_t)(q0 + QN); ++q) {
+                    uint32_t z[4], y[2][4];
+                    ldmatrix_x4_trans(base + CS_Z + frag_off + q * 1024, z[0], z[1], z[2], z[3]);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {                // matrix m: value rows 8m + l8 of the warp's 32
+                        y[m >> 1][2 * (m & 1)] = __float_as_uint(wv[m] * silu(__uint_as_float(z[m] << 16)));
+                        y[m >> 1][2 * (m & 1) + 1] = __float_as_uint(wv[m] * silu(__uint_as_float(z[m] & 0xffff0000u)));
+                    }
+                    tmem_st_frag8(tmem + lane_base + TM_OG + 8 * q, y[0]);
+                    tmem_st_frag8(tmem + lane_base + (16u << 16) + TM_OG + 8 * q, y[1]);
+                }
+                tmem_wait_st();
+                mbar_arrive(w.bar(CB_ZFREE));
+            }
             w.wait_hot(CB_O, c & 1);
             tc_fence_after_sync();
             // take both accumulators out of tensor memory first and hand them back at once: the next
@@ -1017,8 +1035,6 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                         ss[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16 >> st);
                     }
                 }
-                put_frags(tmem + lane_base + TM_OG + 8 * q0, o[0]);
-                put_frags(tmem + lane_base + (16u << 16) + TM_OG + 8 * q0, o[1]);
                 // value index = lane bits 4, 3, 2 = 2 q + x: token 8 (q0 + q) + 2 l4 + x
                 float* red = reinterpret_cast<float*>(sm + CS_RED) + (c & 1) * 256;
                 red[we * 64 + 8 * (q0 + (lane >> 4) * 2 + ((lane >> 3) & 1)) + 2 * l4 + ((lane >> 2) & 1)] = ss[0];
@@ -1030,33 +1046,23 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     inv[tk] = rsqrtf(sum * (1.0f / DVB) + p.norm_eps);
                 }
                 __syncwarp();
-                w.wait(CB_ZFULL, c & 1);
-                tmem_wait_st();
-                // Rolled, with the rows coming back from tensor memory, which takes a running address where registers
-                // do not: unrolled over o the gates made 14 KB of straight-line code that the instruction cache had
-                // lost by the next chunk.
-#pragma unroll 2
-                for (uint32_t q = q0; q < (uint32_t)(q0 + QN); ++q) {
-                    uint32_t y[2][4], z[4];
-                    tmem_ld_frag8(tmem + lane_base + TM_OG + 8 * q, y[0]);
-                    tmem_ld_frag8(tmem + lane_base + (16u << 16) + TM_OG + 8 * q, y[1]);
-                    ldmatrix_x4_trans(base + CS_Z + frag_off + q * 1024, z[0], z[1], z[2], z[3]);
-                    const float2 iv = *reinterpret_cast<const float2*>(inv + 8 * q + 2 * l4);
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    uint32_t g[4 * QN];
+                    tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_OG + 8 * q0, g);
                     tmem_wait_ld();
-                    uint32_t pk[4];
 #pragma unroll
-                    for (int m = 0; m < 4; ++m)                  // matrix m: value rows 8m + l8 of the warp's 32
-                        pk[m] = pack_bf16(__uint_as_float(y[m >> 1][2 * (m & 1)]) * (iv.x * wv[m]) * silu(__uint_as_float(z[m] << 16)),
-                                          __uint_as_float(y[m >> 1][2 * (m & 1) + 1]) * (iv.y * wv[m]) * silu(__uint_as_float(z[m] & 0xffff0000u)));
-                    stmatrix_x4_trans(ost + frag_off + q * 1024, pk[0], pk[1], pk[2], pk[3]);
+                    for (int q = 0; q < QN; ++q) {
+                        const float2 iv = *reinterpret_cast<const float2*>(inv + 8 * (q0 + q) + 2 * l4);
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) o[hh][4 * q + x] *= ((x & 1) ? iv.y : iv.x) * __uint_as_float(g[4 * q + x]);
+                    }
                 }
-                mbar_arrive(w.bar(CB_ZFREE));
-            } else {
-#pragma unroll
-                for (int q = 0; q < QN; ++q)
-                    stmatrix_x4_trans(ost + frag_off + (uint32_t)(q0 + q) * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
-                                      pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
             }
+#pragma unroll
+            for (int q = 0; q < QN; ++q)
+                stmatrix_x4_trans(ost + frag_off + (uint32_t)(q0 + q) * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
+                                  pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
             if (R == C) {
                 fence_proxy_async_smem();
                 if (j == 0 && og == 0) bulk_wait_read_all();              // the tile the next chunk writes has left (stored a chunk ago)
