@@ -53,6 +53,7 @@ static bool g_lean_use_scan = false;       // true = summary, combination and ch
                                            // slower than the three kernels under programmatic dependent launch: 0.162 vs 0.152 ms on
                                            // the 10240-token workload, 0.074 vs 0.060 ms at 2048 tokens, so it is off by default)
 static bool g_lean_scan_last = false;
+static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size (-1 = by the rule)
 
 namespace {
 
@@ -239,7 +240,10 @@ __device__ __forceinline__ bool decode_item(const PrepParams& p, long item, int*
 // inverse row norms scale A, P and the columns of T diag(b e^g), and they ride to the chain kernels
 // inside the gate vectors (e^g / |q| for the output rows, e^{gC-g} / |k| for the state update), so
 // the K and Q tiles themselves are used as they are.
-template <bool RAW>
+// COMPACT: the item is (T diag(b))^T, P and the gate vectors only, 17 KB instead of 33: the chain kernels then form
+// S^T K^T where they used S^T W^T and multiply by T diag(b) afterwards (see chain_body).  The first row of the gate vectors is
+// e^g / |k| there instead of g.
+template <bool RAW, bool COMPACT>
 __global__ void __launch_bounds__(PREP_THREADS, 4)
 gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, PrepParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -529,16 +533,21 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     *reinterpret_cast<float2*>(sTf + (32 + 16 * mb + g + 8) * LDA + 16 * nb + 8 * q + 2 * t) = make_float2(-r[q][2], -r[q][3]);
                 }
             }
-            if (tp == 0) bulk_wait_read_all();                 // the P image has left the Q_lo tile
+            if (tp == 0) {
+                bulk_wait_read_all();                          // the P image has left the Q_lo tile
+                if (COMPACT) mbar_arrive(w.bar(PB_KQFREE));    // and nothing else will use the tiles: the next item's may land
+            }
             named_bar_sync(1, 128);
             // ---- step b3 operands: row i = cc of (T diag(b e^g))^T (shared) and (T diag(b))^T (scratch) ----
             {
                 const int cc = tp & 63, half = tp >> 6;
                 const float b = gates[64 + cc], bg = b * gates[128 + cc] * (RAW ? sRN[cc] : 1.f);
+                const uint32_t t2img = base + (COMPACT ? PS_A : PS_T2);      // COMPACT: over the fp32 T, once everybody has read it
                 float t[32];
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
                     t[i] = (half == 0 && cc >= 32) ? 0.f : sTf[(32 * half + i) * LDA + cc];
+                if (COMPACT) named_bar_sync(1, 128);
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
                     uint32_t p1[4], p2[4];
@@ -548,23 +557,37 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                         p1[e] = pack_bf16(t0 * bg, t1 * bg);
                         p2[e] = pack_bf16(t0 * b, t1 * b);
                     }
-                    st_shared_v4(base + PS_T1 + swz(cc, 4 * half + ch), p1[0], p1[1], p1[2], p1[3]);
-                    st_shared_v4(base + PS_T2 + swz(cc, 4 * half + ch), p2[0], p2[1], p2[2], p2[3]);
+                    if (!COMPACT) st_shared_v4(base + PS_T1 + swz(cc, 4 * half + ch), p1[0], p1[1], p1[2], p1[3]);
+                    st_shared_v4(t2img + swz(cc, 4 * half + ch), p2[0], p2[1], p2[2], p2[3]);
                 }
             }
             fence_proxy_async_smem();
-            tc_fence_before_sync();
-            mbar_arrive(w.bar(PB_TREADY));
+            if (!COMPACT) {
+                tc_fence_before_sync();
+                mbar_arrive(w.bar(PB_TREADY));
+            }
             named_bar_sync(1, 128);
-            if (tp == 0) { bulk_store_hint(out_item + IT_T2, base + PS_T2, 8192, (p.l2 & 2) ? l2_policy_evict_last() : l2_policy_evict_normal()); bulk_commit(); }
+            if (tp == 0) {
+                bulk_store_hint(out_item + IT_T2, base + (COMPACT ? PS_A : PS_T2), 8192, (p.l2 & 2) ? l2_policy_evict_last() : l2_policy_evict_normal());
+                bulk_commit();
+            }
             // ---- step b3 result: -W^T image to scratch; gate vectors to scratch ----
             if (tp < GATE_FLOATS / 4) {
-                float4 gv = *reinterpret_cast<const float4*>(gates + 4 * tp);
+                float4 gv = *reinterpret_cast<const float4*>(gates + 4 * (COMPACT && tp < 16 ? tp + 32 : tp));   // COMPACT: row 0 is e^g
                 if (RAW && tp >= 32 && tp < 64) {      // e^g -> e^g / |q|   and   e^{gC-g} -> e^{gC-g} / |k|
                     const float4 rn = *reinterpret_cast<const float4*>(sRN + (tp < 48 ? 64 + 4 * (tp - 32) : 4 * (tp - 48)));
                     gv.x *= rn.x; gv.y *= rn.y; gv.z *= rn.z; gv.w *= rn.w;
                 }
+                if (RAW && COMPACT && tp < 16) {       // e^g / |k|
+                    const float4 rn = *reinterpret_cast<const float4*>(sRN + 4 * tp);
+                    gv.x *= rn.x; gv.y *= rn.y; gv.z *= rn.z; gv.w *= rn.w;
+                }
                 *reinterpret_cast<float4*>(out_item + IT_GATES + tp * 16) = gv;
+            }
+            if (COMPACT) {
+                mbar_arrive(w.bar(PB_DONE));           // the gate vectors have been read
+                ++it;
+                continue;
             }
             w.wait(PB_W, par);
             tc_fence_after_sync();
@@ -613,7 +636,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     tma_load_3d(kq + 24576, &map_q, 64, hh, (int)tk, full);
                 };
                 if (it == 0) load_tiles(h, tok);                    // later items were requested one item ahead
-                else w.wait(PB_DONE, (it - 1) & 1);                 // the accumulator columns of the last item are free
+                else if (!COMPACT) w.wait(PB_DONE, (it - 1) & 1);   // the accumulator columns of the last item are free (COMPACT: since PB_KQFREE)
                 tc_fence_after_sync();
                 w.wait(PB_FULL, par);
 #pragma unroll
@@ -623,6 +646,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 }
                 if (lead) mma_commit(w.bar(PB_G));
                 const int nxt = draw(-1);                           // the atomic's latency hides behind the solve
+                if (!COMPACT) {
                 w.wait(PB_TREADY, par);
                 tc_fence_after_sync();
 #pragma unroll
@@ -630,11 +654,12 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     if (lead) mma_ss(tmem, make_smem_desc(kq + ks * 2048, 16384, 1024),
                            make_smem_desc(base + PS_T1 + ks * 2048, 1024, 1024), ID_WU, ks > 0);
                 if (lead) mma_commit(w.bar(PB_W));
-                // request the tiles of the next item as soon as the K/Q space is free, then publish it
-                if (nxt >= 0) {
-                    w.wait(PB_KQFREE, par);
-                    load_tiles(nh, ntok);
                 }
+                // request the tiles of the next item as soon as the K/Q space is free, then publish it
+                // (the end is published no earlier: everybody must have taken this item before the next phase of PB_ITEM
+                //  completes, or a wait for this one would see the parity of the one after)
+                w.wait(PB_KQFREE, par);
+                if (nxt >= 0) load_tiles(nh, ntok);
                 publish((it + 1) & 1, nxt);
             }
         } else {
@@ -715,6 +740,18 @@ static_assert(CS_OST % 1024 == 0 && CHAIN_SMEM_GATED <= 232448, "shared memory p
 enum CBar : uint32_t { CB_FULLW0 = 0, CB_FREEW0 = 2, CB_FULLQ0 = 4, CB_FREEQ0 = 6, CB_FULLK0 = 8, CB_FREEK0 = 10, CB_FULLP0 = 12, CB_FREEP0 = 14,
                        CB_FULLB0 = 16, CB_FREEB0 = 18, CB_ZFULL = 20, CB_ZFREE, CB_V, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE, CB_U, CB_O1, CB_CLEAN, CB_VPLAIN };
 static_assert(CB_VPLAIN < 32, "barrier area");
+// COMPACT chains read no -W^T: K has a third slot in its place (it is used from the first to the last MMA of a step), and
+// the barriers of the -W^T ring serve that slot and the extra hand-over.
+enum CBarCompact : uint32_t { CB_FULLK2 = CB_FULLW0, CB_X = CB_FULLW0 + 1, CB_FREEK2 = CB_FREEW0, CB_YREADY = CB_FREEW0 + 1 };
+constexpr uint32_t CS_K2 = CS_W;
+// slot of K tile c and its barriers
+template <bool COMPACT> struct KRing {
+    static __device__ __forceinline__ uint32_t slot(int c) { return COMPACT ? (uint32_t)(c % 3) : (uint32_t)(c & 1); }
+    static __device__ __forceinline__ uint32_t parity(int c) { return COMPACT ? (uint32_t)((c / 3) & 1) : (uint32_t)((c >> 1) & 1); }
+    static __device__ __forceinline__ uint32_t offset(uint32_t s) { return s == 2 ? CS_K2 : CS_K + s * 16384; }
+    static __device__ __forceinline__ uint32_t full(uint32_t s) { return s == 2 ? (uint32_t)CB_FULLK2 : CB_FULLK0 + s; }
+    static __device__ __forceinline__ uint32_t free(uint32_t s) { return s == 2 ? (uint32_t)CB_FREEK2 : CB_FREEK0 + s; }
+};
 
 struct ChainParams {
     const float* s0;          // [N,H,d_k,d_v] or nullptr
@@ -776,8 +813,9 @@ __device__ __forceinline__ bool handover_wait(const Handover& hv, volatile int* 
     return true;
 }
 
-__device__ __forceinline__ void chain_init_bars(const Waiter& w, int out_threads) {
-    for (uint32_t i = CB_FULLW0; i < CB_V; ++i) mbar_init(w.bar(i), i == CB_ZFREE ? out_threads : 1);
+__device__ __forceinline__ void chain_init_bars(const Waiter& w, int out_threads, bool compact) {
+    for (uint32_t i = CB_FULLW0; i < CB_V; ++i)
+        mbar_init(w.bar(i), i == CB_ZFREE ? out_threads : (compact && i == CB_YREADY) ? 256 : 1);
     mbar_init(w.bar(CB_U), 1); mbar_init(w.bar(CB_O1), 1);
     mbar_init(w.bar(CB_V), 1); mbar_init(w.bar(CB_S), 1); mbar_init(w.bar(CB_O), 1);
     mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256); mbar_init(w.bar(CB_OFREE), out_threads);
@@ -790,7 +828,12 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 
 // Steps c and d for one CTA.  SCAN: called from the merged scan kernel (register budgets are set there, the
 // incoming state is awaited through `hv` and read past the L1 cache, since another SM wrote it in this launch).
-template <bool DBG, bool SCAN, bool GATED>
+//
+// COMPACT: v_new = T diag(b) (V - diag(e^g) K S) instead of U - W S: S^T K^T, a conversion that applies -e^g, and a product
+// with (T diag(b))^T onto U^T.  One hop more per step (about 0.25 us), but 16 KB less to write and to read
+// per chunk and head, so it is the form for grids that are bound by memory (see launch_lean).  As many roundings: Y
+// here, W there.
+template <bool DBG, bool SCAN, bool GATED, bool COMPACT>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
     constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments of each
@@ -861,6 +904,23 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
         for (int c = 0; c < nchunks; ++c) {
             const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
+            if (COMPACT) {
+                // Y^T = -e^g (S^T K^T) as bf16; the accumulator borrows columns of dS^T, which is idle now
+                w.wait_hot(CB_X, c & 1);
+                tc_fence_after_sync();
+                uint32_t x[32], pk[16];
+                tmem_ld32(tmem + lane_base + TM_DS + 32 * wg, x);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float2 eg = *reinterpret_cast<const float2*>(gates + 32 * wg + 2 * i);
+                    pk[i] = pack_bf16(-eg.x * __uint_as_float(x[2 * i]), -eg.y * __uint_as_float(x[2 * i + 1]));
+                }
+                tmem_st16(tmem + lane_base + TM_DS + 64 + 16 * wg, pk);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive(w.bar(CB_YREADY));
+            }
             if (c > 0) w.wait_hot(CB_O, (c - 1) & 1);     // O2 of the previous chunk no longer reads bf16 v_new
             w.wait_hot(CB_V, c & 1);
             tc_fence_after_sync();
@@ -953,9 +1013,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
             if (og == 0 && tail_c >= 0 && c == max(tail_c - 1, 0)) {
                 const int Rt = len - tail_c * C;
-                const uint32_t sk = base + CS_K + (uint32_t)(tail_c & 1) * 16384;
+                const uint32_t ks = KRing<COMPACT>::slot(tail_c), sk = base + KRing<COMPACT>::offset(ks);
                 const uint32_t sv = base + CS_B + (uint32_t)(tail_c & 1) * STAGE_B + ST_V;
-                w.wait(CB_FULLK0 + (tail_c & 1), (tail_c >> 1) & 1);
+                w.wait(KRing<COMPACT>::full(ks), KRing<COMPACT>::parity(tail_c));
                 w.wait(CB_FULLB0 + (tail_c & 1), (tail_c >> 1) & 1);
                 const uint32_t pieces = (uint32_t)(C - Rt) * 8u;
                 for (uint32_t x = j; x < 4 * pieces; x += 128) {             // K_lo, K_hi, V_lo, V_hi
@@ -1095,24 +1155,41 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             //  issued by a second thread so that it does not sit between two dependent steps)
             // operand descriptors are built once per stage, outside the dependent chain: the address field
             // counts 16-byte units, so a k-step is a plain add
-            const uint64_t dW0 = make_smem_desc(base + CS_W, 1024, 1024), dK0 = make_smem_desc(base + CS_K, 8192, 1024);
+            const uint64_t dW0 = make_smem_desc(base + CS_W, 1024, 1024), dT0 = make_smem_desc(base + CS_B + ST_T2, 1024, 1024);
             for (int c = 0; c < nchunks; ++c) {
                 const uint32_t s = c & 1, par = (c >> 1) & 1;
-                const uint64_t dW = dW0 + (uint64_t)((s * 16384) >> 4), dK = dK0 + (uint64_t)((s * 16384) >> 4);
+                const uint32_t sk = KRing<COMPACT>::slot(c), ka = base + KRing<COMPACT>::offset(sk);
+                const uint64_t dW = dW0 + (uint64_t)((s * 16384) >> 4), dT = dT0 + (uint64_t)((s * STAGE_B) >> 4);
+                const uint64_t dK = make_smem_desc(ka, 8192, 1024), dKk = make_smem_desc(ka, 16, 1024);   // MN-major, K-major
                 // the waits that are normally long satisfied come first: whatever follows the wait on the
                 // state sits on the dependent chain
-                w.wait_hot(CB_FULLW0 + s, par);
-                w.wait_hot(CB_FULLK0 + s, par);
-                w.wait_hot(CB_U, c & 1);                       // U^T of this chunk is in the accumulator
+                if (!COMPACT) w.wait_hot(CB_FULLW0 + s, par);
+                w.wait_hot(KRing<COMPACT>::full(sk), KRing<COMPACT>::parity(c));
+                if (!COMPACT) w.wait_hot(CB_U, c & 1);         // U^T of this chunk is in the accumulator
                 if (c == tail_c) w.wait_hot(CB_CLEAN, 0);      // padded K rows have been cleared
                 w.wait_hot(CB_SREADY, c & 1);
                 tc_fence_after_sync();
                 if (lead) stamp(1, c, 0);
+                if (COMPACT) {
 #pragma unroll
-                for (uint32_t ks = 0; ks < 8; ++ks)            // v^T = U^T - S^T W^T
-                    if (lead) mma_ts(tmem + TM_DV, tmem + TM_SBF + ks * 8, dW + ks * 128, ID_1, 1);
-                if (lead) mma_commit(w.bar(CB_V));
-                if (lead) mma_commit(w.bar(CB_FREEW0 + s));
+                    for (uint32_t ks = 0; ks < 8; ++ks)        // X^T = S^T K^T
+                        if (lead) mma_ts(tmem + TM_DS, tmem + TM_SBF + ks * 8, dKk + (uint64_t)(((ks >> 2) * 8192 + (ks & 3) * 32) >> 4), ID_O, ks > 0);
+                    if (lead) mma_commit(w.bar(CB_X));
+                    w.wait_hot(CB_U, c & 1);
+                    w.wait_hot(CB_YREADY, c & 1);
+                    tc_fence_after_sync();
+#pragma unroll
+                    for (uint32_t ks = 0; ks < 4; ++ks)        // v^T = U^T + Y^T (T diag(b))^T
+                        if (lead) mma_ts(tmem + TM_DV, tmem + TM_DS + 64 + ks * 8, dT + ks * 128, ID_1, 1);
+                    if (lead) mma_commit(w.bar(CB_V));
+                    if (lead) mma_commit(w.bar(CB_FREEB0 + s));
+                } else {
+#pragma unroll
+                    for (uint32_t ks = 0; ks < 8; ++ks)        // v^T = U^T - S^T W^T
+                        if (lead) mma_ts(tmem + TM_DV, tmem + TM_SBF + ks * 8, dW + ks * 128, ID_1, 1);
+                    if (lead) mma_commit(w.bar(CB_V));
+                    if (lead) mma_commit(w.bar(CB_FREEW0 + s));
+                }
                 if (lead) stamp(1, c, 1);
                 w.wait_hot(CB_VREADY, c & 1);
                 tc_fence_after_sync();
@@ -1121,7 +1198,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 for (uint32_t ks = 0; ks < 4; ++ks)            // dS^T = (v e^{gC-g})^T K
                     if (lead) mma_ts(tmem + TM_DS, tmem + TM_VT + ks * 8, dK + ks * 128, ID_2, ks > 0);
                 if (lead) mma_commit(w.bar(CB_S));
-                if (lead) mma_commit(w.bar(CB_FREEK0 + s));
+                if (lead) mma_commit(w.bar(KRing<COMPACT>::free(sk)));
                 if (lead) stamp(1, c, 4);
             }
         } else if (warp == CW + 2) {
@@ -1137,7 +1214,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     w.wait(CB_SREADY, c & 1);
                     w.wait(CB_FULLQ0 + s, par);
                     if (c > 0) w.wait(CB_OFREE, (c - 1) & 1);  // the epilogue has read the previous O1, O2
-                    w.wait_hot(CB_V, c & 1);                   // stay out of the tensor pipe until v_new is done
+                    w.wait_hot(COMPACT ? (uint32_t)CB_X : (uint32_t)CB_V, c & 1);   // stay out of the tensor pipe until v_new (COMPACT: X) is done
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 8; ++ks)        // O1^T = S^T Q^T
@@ -1156,7 +1233,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)
                         if (lead) mma_ss(tmem + TM_DV, dV0 + boff + ks * 128, dT0 + boff + ks * 128, ID_WU, ks > 0);
-                    if (lead) mma_commit(w.bar(CB_FREEB0 + sB));
+                    if (!COMPACT && lead) mma_commit(w.bar(CB_FREEB0 + sB));
                     if (lead) mma_commit(w.bar(CB_U));
                 }
                 if (c >= 0) {
@@ -1192,7 +1269,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     tma_load_3d_hint(bb + ST_V + 8192, map_v, dvb * DVB + 64, h, tok, full, pol_done);
                     bulk_load_hint(bb + ST_T2, item + IT_T2, 8192, full, pol_item);
                 }
-                {
+                if (!COMPACT) {
                     const uint32_t full = w.bar(CB_FULLW0 + s);
                     if (c >= 2) w.wait(CB_FREEW0 + s, par);
                     mbar_arrive_expect_tx(full, 16384 + 1280);
@@ -1207,11 +1284,13 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     tma_load_3d_hint(dst + 8192, map_q, 64, h, tok, full, pol_done);
                 }
                 {
-                    const uint32_t full = w.bar(CB_FULLK0 + s), dst = base + CS_K + s * 16384;
-                    if (c >= 2) w.wait(CB_FREEK0 + s, par);
-                    mbar_arrive_expect_tx(full, 16384);
+                    const uint32_t sk = KRing<COMPACT>::slot(c), full = w.bar(KRing<COMPACT>::full(sk)), dst = base + KRing<COMPACT>::offset(sk);
+                    constexpr int KD = COMPACT ? 3 : 2;
+                    if (c >= KD) w.wait(KRing<COMPACT>::free(sk), KRing<COMPACT>::parity(c - KD));
+                    mbar_arrive_expect_tx(full, 16384 + (COMPACT ? 1280 : 0));
                     tma_load_3d_hint(dst, map_k, 0, h, tok, full, pol_done);
                     tma_load_3d_hint(dst + 8192, map_k, 64, h, tok, full, pol_done);
+                    if (COMPACT) bulk_load(base + CS_GATES + (c % (int)GATE_SLOTS) * 1280, item + IT_GATES, 1280, full);
                 }
                 {
                     const uint32_t full = w.bar(CB_FULLP0 + s);
@@ -1224,8 +1303,12 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 // let copies in flight land before shared memory is released (bounded)
                 const unsigned long long t0 = globaltimer_ns();
                 for (int c = max(0, nchunks - 2); c < nchunks; ++c)
-                    for (uint32_t b = CB_FULLW0; b <= CB_FULLB0; b += 4)
-                        while (!mbar_try_wait(w.bar(b + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+                    for (uint32_t b = COMPACT ? CB_FULLQ0 : CB_FULLW0; b <= CB_FULLB0; b += 4)
+                        while (!(COMPACT && b == CB_FULLK0) && !mbar_try_wait(w.bar(b + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+                if (COMPACT)
+                    for (int c = max(0, nchunks - 3); c < nchunks; ++c)
+                        while (!mbar_try_wait(w.bar(KRing<COMPACT>::full(KRing<COMPACT>::slot(c))), KRing<COMPACT>::parity(c)) &&
+                               globaltimer_ns() - t0 < TIMEOUT_NS) {}
             }
         } else if (GATED && warp == CW + 3 && lane == 0) {
             // ---- TMA producer of the gate tile ----
@@ -1246,7 +1329,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     }
 }
 
-template <bool DBG, bool GATED>
+template <bool DBG, bool GATED, bool COMPACT>
 __global__ void __launch_bounds__(GATED ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
 gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
@@ -1258,7 +1341,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     Waiter w{base + CS_BARS, reinterpret_cast<volatile int*>(sm + CS_MISC + 4)};
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        chain_init_bars(w, GATED ? 256 : 128);
+        chain_init_bars(w, GATED ? 256 : 128, COMPACT);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -1273,7 +1356,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     pdl_trigger();                      // the next call's prepare kernel may set itself up as SMs come free
     pdl_wait();                         // scratch items and incoming states come from the kernels before this one
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
-    chain_body<DBG, false, GATED>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
+    chain_body<DBG, false, GATED, COMPACT>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1312,7 +1395,8 @@ __device__ __forceinline__ uint32_t sum_ds(int inst) { return inst ? 288u : 64u;
 __device__ __forceinline__ uint32_t sum_vt(int inst) { return inst ? 416u : 192u; }   // bf16 decayed v_new^T
 constexpr uint32_t SUM_COLS = 512;
 
-enum SBar : uint32_t { SB_FULL0 = 0, SB_FREE0 = 3, SB_V0 = 6, SB_S0 = 8, SB_SREADY0 = 10, SB_VREADY0 = 12 };
+enum SBar : uint32_t { SB_FULL0 = 0, SB_FREE0 = 3, SB_V0 = 6, SB_S0 = 8, SB_SREADY0 = 10, SB_VREADY0 = 12,
+                       SB_X0 = 14, SB_YREADY0 = 16 };
 
 struct SummaryParams {
     const int32_t* cu;
@@ -1332,11 +1416,12 @@ __device__ __forceinline__ void summary_init_bars(const Waiter& w, int ninst) {
     for (uint32_t i = 0; i < 2; ++i) {
         mbar_init(w.bar(SB_V0 + i), 1); mbar_init(w.bar(SB_S0 + i), 1);
         mbar_init(w.bar(SB_SREADY0 + i), 128); mbar_init(w.bar(SB_VREADY0 + i), 128);
+        mbar_init(w.bar(SB_X0 + i), 1); mbar_init(w.bar(SB_YREADY0 + i), 128);
     }
 }
 
-// Segment summary (M_seg, N_seg) of one CTA; cta.z = sequence * (nseg - 1) + segment.
-template <bool SCAN>
+// Segment summary (M_seg, N_seg) of one CTA; cta.z = sequence * (nseg - 1) + segment.  COMPACT: as in chain_body.
+template <bool SCAN, bool COMPACT>
 __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUtensorMap* map_v, const SummaryParams& p,
                                              const Cta& cta, const Waiter& w) {
     constexpr int CW = SCAN ? 12 : 8;                 // first warp of the control warpgroup
@@ -1381,6 +1466,29 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
             for (int c = 0; c < nchunks; ++c) {
                 const uint32_t s = c % SUM_STAGES;
                 const float* gates = reinterpret_cast<const float*>(sm + s * SUM_STAGE + SS_GATES);
+                if (COMPACT) {
+                    // Y^T = -e^g (S^T K^T): accumulator in the upper columns of dS^T, bf16 in the place of the decayed v_new
+                    w.wait_hot(SB_X0 + inst, c & 1);
+                    tc_fence_after_sync();
+                    uint32_t x[2][32];
+                    tmem_ld32(tmem + lane_base + sum_ds(inst) + 64, x[0]);
+                    tmem_wait_ld();
+                    tmem_ld32(tmem + lane_base + sum_ds(inst) + 96, x[1]);
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {
+                        uint32_t pk[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const float2 eg = *reinterpret_cast<const float2*>(gates + 32 * hh + 2 * i);
+                            pk[i] = pack_bf16(-eg.x * __uint_as_float(x[hh][2 * i]), -eg.y * __uint_as_float(x[hh][2 * i + 1]));
+                        }
+                        tmem_st16(tmem + lane_base + sum_vt(inst) + 16 * hh, pk);
+                        if (hh == 0) tmem_wait_ld();
+                    }
+                    tmem_wait_st();
+                    tc_fence_before_sync();
+                    mbar_arrive(w.bar(SB_YREADY0 + inst));
+                }
                 w.wait_hot(SB_V0 + inst, c & 1);
                 tc_fence_after_sync();
 #pragma unroll
@@ -1469,10 +1577,24 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                     }
                     w.wait_hot(SB_SREADY0 + inst, c & 1);
                     tc_fence_after_sync();
+                    if (COMPACT) {
+                        const uint64_t dKk = make_smem_desc(sb + SS_K, 16, 1024), dT = make_smem_desc(sb + SS_T2, 1024, 1024);
 #pragma unroll
-                    for (uint32_t ks = 0; ks < 8; ++ks)            // v^T = U^T - S^T W^T   (U = 0 for the identity chain)
-                        if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_ds(inst) + ks * 8,
-                               dW + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
+                        for (uint32_t ks = 0; ks < 8; ++ks)        // X^T = S^T K^T
+                            if (lead) mma_ts(tmem + sum_ds(inst) + 64, tmem + sum_ds(inst) + ks * 8,
+                                   dKk + (uint64_t)(((ks >> 2) * 8192 + (ks & 3) * 32) >> 4), ID_O, ks > 0);
+                        if (lead) mma_commit(w.bar(SB_X0 + inst));
+                        w.wait_hot(SB_YREADY0 + inst, c & 1);
+                        tc_fence_after_sync();
+#pragma unroll
+                        for (uint32_t ks = 0; ks < 4; ++ks)        // v^T = U^T + Y^T (T diag(b))^T
+                            if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_vt(inst) + ks * 8, dT + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
+                    } else {
+#pragma unroll
+                        for (uint32_t ks = 0; ks < 8; ++ks)        // v^T = U^T - S^T W^T   (U = 0 for the identity chain)
+                            if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_ds(inst) + ks * 8,
+                                   dW + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
+                    }
                     if (lead) mma_commit(w.bar(SB_V0 + inst));
                     w.wait_hot(SB_VREADY0 + inst, c & 1);
                     tc_fence_after_sync();
@@ -1495,12 +1617,12 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                 const uint32_t full = w.bar(SB_FULL0 + s);
                 const int tok = (int)(tok0 + (long)c * C);
                 const uint8_t* item = p.items + (size_t)((slot0 + c) * H + h) * ITEM_BYTES;
-                mbar_arrive_expect_tx(full, SUM_STAGE_TX);
+                mbar_arrive_expect_tx(full, COMPACT ? SUM_STAGE_TX - 16384 : SUM_STAGE_TX);
                 tma_load_3d_hint(sb + SS_K, map_k, 0, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_K + 8192, map_k, 64, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_V, map_v, dvb * DVB, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_V + 8192, map_v, dvb * DVB + 64, h, tok, full, pol_keep);
-                bulk_load_hint(sb + SS_W, item + IT_W, 16384, full, pol_item);
+                if (!COMPACT) bulk_load_hint(sb + SS_W, item + IT_W, 16384, full, pol_item);
                 bulk_load_hint(sb + SS_T2, item + IT_T2, 8192, full, pol_item);
                 bulk_load(sb + SS_GATES, item + IT_GATES, 1280, full);
             }
@@ -1515,6 +1637,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     }
 }
 
+template <bool COMPACT>
 __global__ void __launch_bounds__(SUM_THREADS, 1)
 gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    SummaryParams p) {
@@ -1540,7 +1663,7 @@ gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     pdl_trigger();
     pdl_wait();                         // the scratch items come from the prepare kernel
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
-    summary_body<false>(&map_k, &map_v, p, cta, w);
+    summary_body<false, COMPACT>(&map_k, &map_v, p, cta, w);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1790,7 +1913,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (tid == 0) {
         summary_init_bars(w1, 2);
         combine_init_bars(w2);
-        chain_init_bars(w3, 128);
+        chain_init_bars(w3, 128, false);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -1816,7 +1939,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // ---------------- phase 1: summary of this segment (the last segment needs none) ----------------
         if (seg < nseg - 1) {
             const Cta c1{base, sm, tmem, 0, h, n * (nseg - 1) + seg};
-            summary_body<true>(&map_k, &map_v, p.sp, c1, w1);
+            summary_body<true, false>(&map_k, &map_v, p.sp, c1, w1);
             __threadfence();
             tc_fence_before_sync();
             cta_sync();
@@ -1853,7 +1976,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         stamp(3);
         // ---------------- phase 3: chain over this segment's chunks ----------------
         const Cta c3{base, sm, tmem, 0, h, (int)blockIdx.z};
-        chain_body<DBG, true, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
+        chain_body<DBG, true, false, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
         stamp(4);
         tc_fence_before_sync();
         cta_sync();
@@ -1971,16 +2094,20 @@ static int device_setup(int* sms_out) {
     if (sms_of_device[dev] == 0) {
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return GDN_ERR_CUDA;
-        if (cudaFuncSetAttribute(gdn_prep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_prep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_chain_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_chain_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_chain_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM_GATED) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_summary_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SUM_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CMB_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_scan_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCAN_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_scan_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCAN_SMEM) != cudaSuccess)
+        auto smem_limit = [](const void* kernel, uint32_t bytes) {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+        };
+#define GDN_K(...) reinterpret_cast<const void*>(__VA_ARGS__)
+        if (!smem_limit(GDN_K(gdn_prep_kernel<false, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, false>), PREP_SMEM) ||
+            !smem_limit(GDN_K(gdn_prep_kernel<false, true>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, true>), PREP_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<false, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<true, false, false>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<false, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<false, false, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<false, true, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_summary_kernel<false>), SUM_SMEM) || !smem_limit(GDN_K(gdn_summary_kernel<true>), SUM_SMEM) ||
+            !smem_limit(GDN_K(gdn_combine_kernel), CMB_SMEM) ||
+            !smem_limit(GDN_K(gdn_scan_kernel<false>), SCAN_SMEM) || !smem_limit(GDN_K(gdn_scan_kernel<true>), SCAN_SMEM))
             return GDN_ERR_CUDA;
+#undef GDN_K
         sms_of_device[dev] = sms;
     }
     *sms_out = sms_of_device[dev];
@@ -2033,11 +2160,21 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // earlier readers ask L2 to keep them and the last reader releases them.
     const int l2 = (nseg > 1 && tokens * a.H * (uint64_t)(a.d_k + a.d_v) * 2 <= (96ull << 20)) ? (g_lean_l2_hints & 3) : 0;
     PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, nslots, a.B, a.T, a.H, opt.gate_scale, opt.eps, ticket, l2};
+    // Items without -W^T (24 % less memory traffic over both kernels, one hop more per chain step) pay when the chains of a call
+    // together are bound by memory: one segment each, at least three fifths of the SMs busy to the end (equal
+    // lengths), every chain reading its own K and Q (with d_v = 256 two chains share them through L2).  One B200, calls
+    // with / without: 4 x 8192 tokens x 32 heads 380 / 452 us, 4 x 4096 x 24 157 / 174 us, but 1 x 4096 x 64 heads 149 / 144 us
+    // and 4 x 4096 x 16 heads with d_v = 256 148 / 148 us.  With the fused output stage a step is longer anyway
+    // and the line lies lower (4 x 1500 x 16: 74 / 78 us).
+    const bool compact = !g_lean_dbg && !g_lean_use_scan &&
+                         (g_lean_compact >= 0 ? g_lean_compact == 1
+                                              : !packed && nseg == 1 && a.d_v == DVB && (long)a.B * a.H * 5 >= (opt.gate_z ? 2L : 3L) * num_sms);
     const int pgrid = (int)(nitems < 4L * num_sms ? nitems : 4L * num_sms);
     auto mark = [&](int i) { if (g_lean_timing && g_lean_events[i]) cudaEventRecord(g_lean_events[i], stream); };
     mark(0);
-    if (opt.raw) launch_after(gdn_prep_kernel<true>, dim3(pgrid), PREP_THREADS, PREP_SMEM, stream, mq, mk, pp);
-    else launch_after(gdn_prep_kernel<false>, dim3(pgrid), PREP_THREADS, PREP_SMEM, stream, mq, mk, pp);
+    auto prep = compact ? (opt.raw ? gdn_prep_kernel<true, true> : gdn_prep_kernel<false, true>)
+                        : (opt.raw ? gdn_prep_kernel<true, false> : gdn_prep_kernel<false, false>);
+    launch_after(prep, dim3(pgrid), PREP_THREADS, PREP_SMEM, stream, mq, mk, pp);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
     mark(1);
@@ -2068,7 +2205,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
             return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
         }
         dim3 sgrid(a.d_v / DVB, a.H, a.B * (nseg - 1));
-        launch_after(gdn_summary_kernel, sgrid, SUM_THREADS, SUM_SMEM, stream, mk, mv, sp);
+        launch_after(compact ? gdn_summary_kernel<true> : gdn_summary_kernel<false>, sgrid, SUM_THREADS, SUM_SMEM, stream, mk, mv, sp);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
         mark(2);
@@ -2083,14 +2220,17 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                    ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, nseg, seg_chunks,
                    snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket};
     dim3 grid(a.d_v / DVB, a.H, a.B * nseg);
-    if (opt.gate_z) launch_after(gdn_chain_kernel<false, true>, grid, CHAIN_THREADS_GATED, CHAIN_SMEM_GATED, stream, mq, mk, mv, mo, mz, cp);
-    else if (g_lean_dbg) launch_after(gdn_chain_kernel<true, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
-    else launch_after(gdn_chain_kernel<false, false>, grid, CHAIN_THREADS, CHAIN_SMEM, stream, mq, mk, mv, mo, mz, cp);
+    auto chain = opt.gate_z ? (compact ? gdn_chain_kernel<false, true, true> : gdn_chain_kernel<false, true, false>)
+                 : g_lean_dbg ? gdn_chain_kernel<true, false, false>
+                              : (compact ? gdn_chain_kernel<false, false, true> : gdn_chain_kernel<false, false, false>);
+    launch_after(chain, grid, opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
+                 mq, mk, mv, mo, mz, cp);
     count_launch();
     mark(4);
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
+void lean_set_compact(int mode) { g_lean_compact = mode; }
 void lean_set_scan(int enable) { g_lean_use_scan = enable != 0; }
 void lean_set_l2_hints(int enable) { g_lean_l2_hints = enable; }
 void lean_force_segments(int nseg) { g_lean_force_nseg = nseg; }
@@ -2171,9 +2311,9 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             return GDN_ERR_CUDA;
-        if (cudaFuncSetAttribute(gdn_prep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-        cudaFuncSetAttribute(gdn_prep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_chain_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
+        if (cudaFuncSetAttribute(gdn_prep_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(gdn_prep_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(gdn_chain_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
             return GDN_ERR_CUDA;
         sms_of_device[dev] = sms;
         scratch_of_device[dev] = ptr;
@@ -2186,7 +2326,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
     const long nitems = (long)nslots * a.H;
     const long cap = 4L * sms_of_device[dev];
     PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, (long)nslots, a.B, a.T, a.H, 1.f, 0.f, static_cast<int*>(ticket_of_device[dev])};
-    gdn_prep_kernel<false><<<(int)(nitems < cap ? nitems : cap), PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
+    gdn_prep_kernel<false, false><<<(int)(nitems < cap ? nitems : cap), PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
     const int nch = packed ? 1 : (a.T + C - 1) / C;            // one segment: the whole sequence
@@ -2194,7 +2334,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
                    ws, nullptr, nullptr, -1, a.B, a.T, a.H, a.d_v, 1, packed ? (1 << 24) : (nch > 0 ? nch : 1),
                    nullptr, 1, 0, 0, nullptr, nullptr, 0.f, static_cast<int*>(ticket_of_device[dev])};
     dim3 grid(a.d_v / DVB, a.H, a.B);
-    gdn_chain_kernel<false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
+    gdn_chain_kernel<false, false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
