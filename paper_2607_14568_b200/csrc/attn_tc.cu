@@ -52,7 +52,7 @@ constexpr uint32_t AS_TOTAL = AS_MISC + 64;
 constexpr uint32_t ATTN_SMEM = AS_TOTAL + 1024;
 
 enum ABar : uint32_t { AB_Q = 0, AB_KFULL0 = 1, AB_KFREE0 = 3, AB_VFULL0 = 5, AB_VFREE0 = 7, AB_SFULL0 = 9 /* A, B */,
-                       AB_PFULL0 = 11 /* A, B */, AB_PVDONE0 = 13 /* A, B */ };
+                       AB_PFULL0 = 11 /* A, B: first 64 keys */, AB_PVDONE0 = 13 /* A, B */, AB_PFULL1 = 15 /* A, B: other 64 */ };
 
 struct AWaiter {
     uint32_t bars;
@@ -101,24 +101,33 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     // which sequence and which pair of query tiles: batched input takes them from the grid; packed input
     // walks the sequence boundaries (grid.y covers an upper bound of the pair count, the surplus CTAs leave)
+    // CTAs start in x-major order.  Everywhere the longest pairs of tiles come first and the short ones fill the tail: y
+    // counts pairs from the last of the longest sequence down, over all heads and sequences.
     int tok0, len, t;
     if (p.cu) {
-        int y = (int)blockIdx.y, n = 0;
-        tok0 = 0; len = 0; t = -1;
-        for (; n < p.B; ++n) {
-            const int a = p.cu[n], l = p.cu[n + 1] - a;
-            const int np = ((l + BM - 1) / BM + 1) / 2;
-            if (y < np) { tok0 = a; len = l; t = np - 1 - y; break; }
-            y -= np;
+        // pairs with an index of at least i, over all sequences: sum max(0, pairs - i); the largest i with more than y of
+        // them is this CTA's pair index, and the sequence follows from y's rank among the pairs of that index
+        const int y = (int)blockIdx.y;
+        auto pairs_of = [&](int n) { return ((p.cu[n + 1] - p.cu[n] + BM - 1) / BM + 1) / 2; };
+        auto at_least = [&](int i) { int s = 0; for (int n = 0; n < p.B; ++n) s += max(0, pairs_of(n) - i); return s; };
+        if (y >= at_least(0)) return;                      // uniform for the CTA; nothing has been set up yet
+        int lo = 0, hi = (p.T + 2 * BM - 1) / (2 * BM);    // at_least(lo) > y >= at_least(hi)
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (at_least(mid) > y) lo = mid; else hi = mid;
         }
-        if (t < 0) return;                                 // uniform for the CTA; nothing has been set up yet
+        t = lo;
+        int rank = y - at_least(t + 1);
+        tok0 = 0; len = 0;
+        for (int n = 0; n < p.B; ++n)
+            if (pairs_of(n) > t && rank-- == 0) { tok0 = p.cu[n]; len = p.cu[n + 1] - tok0; break; }
     } else {
-        tok0 = (int)blockIdx.z * p.T;
+        tok0 = (int)(blockIdx.x / p.Hq) * p.T;
         len = p.T;
-        t = (((len + BM - 1) / BM + 1) / 2) - 1 - (int)blockIdx.y;   // CTAs start in x-major order: every head's
-    }                                                      // longest pair of tiles first, the short ones fill the tail
+        t = (((len + BM - 1) / BM + 1) / 2) - 1 - (int)blockIdx.y;
+    }
     const int nqt = (len + BM - 1) / BM;
-    const int h = blockIdx.x;
+    const int h = (int)blockIdx.x % p.Hq;
     const int hk = h / (p.Hq / p.Hkv);                     // the key/value head this query head reads
     const bool hasB = (2 * t + 1 < nqt);
     const int nA = 2 * t + 1;                              // key tiles of A: 0..2t (the last is its diagonal)
@@ -130,7 +139,7 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (uint32_t s = 0; s < 2; ++s) {
             mbar_init(w.bar(AB_KFULL0 + s), 1); mbar_init(w.bar(AB_KFREE0 + s), 1);
             mbar_init(w.bar(AB_VFULL0 + s), 1); mbar_init(w.bar(AB_VFREE0 + s), 1);
-            mbar_init(w.bar(AB_SFULL0 + s), 1); mbar_init(w.bar(AB_PFULL0 + s), 128);
+            mbar_init(w.bar(AB_SFULL0 + s), 1); mbar_init(w.bar(AB_PFULL0 + s), 128); mbar_init(w.bar(AB_PFULL1 + s), 128);
             mbar_init(w.bar(AB_PVDONE0 + s), 1);
         }
         sMisc[1] = 0;
@@ -159,27 +168,25 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             // S_X of tile j is complete; so is every earlier MMA of the issuing thread (P V of tile j - 1)
             w.wait(AB_SFULL0 + X, j & 1);
             tc_fence_after_sync();
-            // pass 1: row maximum of the raw scores (c >= 0, so max(c s) = c max(s)); the scores are read
-            // again in pass 2 instead of being kept, so that both passes have registers to overlap their
-            // loads, special-function operations and conversions
+            // row maximum of the raw scores (c >= 0, so max(c s) = c max(s)); the scores stay in registers
             float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            {
-                uint32_t x[4][32];
+            uint32_t x[4][32];
+            tmem_ld32(ts, x[0]);
+            tmem_ld32(ts + 32, x[1]);
+            tmem_wait_ld();
+            tmem_ld32(ts + 64, x[2]);
+            tmem_ld32(ts + 96, x[3]);
 #pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) tmem_ld32(ts + 32 * q4, x[q4]);
-                tmem_wait_ld();
+            for (int q4 = 0; q4 < 4; ++q4) {
+                if (q4 == 2) tmem_wait_ld();
                 if (j == qt) {                             // diagonal tile: keys after the query do not count
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4)
-#pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (32 * q4 + i > r) x[q4][i] = 0xff800000u;       // -inf
+                    for (int i = 0; i < 32; ++i)
+                        if (32 * q4 + i > r) x[q4][i] = 0xff800000u;           // -inf
                 }
 #pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4)
-#pragma unroll
-                    for (int i = 0; i < 32; i += 2)
-                        mx4[(i >> 1) & 3] = max3(mx4[(i >> 1) & 3], __uint_as_float(x[q4][i]), __uint_as_float(x[q4][i + 1]));
+                for (int i = 0; i < 32; i += 2)
+                    mx4[(i >> 1) & 3] = max3(mx4[(i >> 1) & 3], __uint_as_float(x[q4][i]), __uint_as_float(x[q4][i + 1]));
             }
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * c;
             // raise the reference maximum only when it is first set or has grown by more than 2^8
@@ -187,47 +194,40 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const float m_new = grow ? mx : m_ref;
             const float alpha = grow ? ex2(m_ref - m_new) : 1.f;           // 0 on the first tile (m_ref = -inf)
             m_ref = m_new;
-            // pass 2: P = 2^(c s - m) as bf16 over the first 64 columns of the scores it came from; the
-            // next 32 columns are requested before the current 32 are worked on
+            if (j > 0 && __any_sync(0xffffffffu, grow)) {   // rescale the accumulator rows of this warp (P V of tile j - 1 is complete)
+#pragma unroll 1
+                for (int q4 = 0; q4 < 8; ++q4) {
+                    uint32_t o[16];
+                    tmem_ld16(to + 16 * q4, o);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                    tmem_st16(to + 16 * q4, o);
+                }
+            }
+            // P = 2^(c s - m) as bf16 over the first 64 columns of the scores it came from.  The first 64 keys are handed
+            // over while the others are worked on, so that half of P V runs under the second half of the softmax.
+            // (masked scores are -inf: exact zeros after the query's own position)
             float sum[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t xs[2][32];
-            tmem_ld32(ts, xs[0]);
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4) {
-                tmem_wait_ld();
-                if (q4 < 3) tmem_ld32(ts + 32 * (q4 + 1), xs[(q4 + 1) & 1]);
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const int e = 32 * q4 + 2 * i;
-                    float p0 = ex2(fmaf(__uint_as_float(xs[q4 & 1][2 * i]), c, -m_new));
-                    float p1 = ex2(fmaf(__uint_as_float(xs[q4 & 1][2 * i + 1]), c, -m_new));
-                    if (j == qt) {                         // exact zeros after the query's own position
-                        if (e > r) p0 = 0.f;
-                        if (e + 1 > r) p1 = 0.f;
-                    }
+                    const float p0 = ex2(fmaf(__uint_as_float(x[q4][2 * i]), c, -m_new));
+                    const float p1 = ex2(fmaf(__uint_as_float(x[q4][2 * i + 1]), c, -m_new));
                     sum[i & 1] += p0;
                     sum[2 + (i & 1)] += p1;
                     pk[i] = pack_bf16(p0, p1);
                 }
                 tmem_st16(ts + 16 * q4, pk);
-            }
-            const float sum0 = sum[0] + sum[1], sum1 = sum[2] + sum[3];
-            l = l * alpha + (sum0 + sum1);
-            if (j > 0 && __any_sync(0xffffffffu, grow)) {   // rescale the accumulator rows of this warp
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    uint32_t o[32];
-                    tmem_ld32(to + 32 * q4, o);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                    tmem_st32(to + 32 * q4, o);
+                if (q4 & 1) {
+                    tmem_wait_st();
+                    tc_fence_before_sync();
+                    mbar_arrive(w.bar((q4 == 1 ? AB_PFULL0 : AB_PFULL1) + X));
                 }
             }
-            tmem_wait_st();
-            tc_fence_before_sync();
-            mbar_arrive(w.bar(AB_PFULL0 + X));
+            l = l * alpha + ((sum[0] + sum[1]) + (sum[2] + sum[3]));
         }
         // ---- epilogue: O / l -> bf16 -> global (one 256-byte row per thread) ----
         if (nX > 0) {
@@ -272,12 +272,19 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
                 if (lead) mma_commit(w.bar(AB_SFULL0 + X));
             };
-            auto issue_pv = [&](uint32_t X, int j) {       // O_X += P_X V_j, 16 keys per step
+            auto issue_pv = [&](uint32_t X, int j) {       // O_X += P_X V_j, 16 keys per step, each half when its P is there
                 const uint64_t dv = dv0 + ((uint64_t)((j & 1) * TILE_BYTES) >> 4);
+                w.wait(AB_PFULL0 + X, j & 1);
+                tc_fence_after_sync();
 #pragma unroll
-                for (uint32_t ks = 0; ks < 8; ++ks)
+                for (uint32_t ks = 0; ks < 8; ++ks) {
+                    if (ks == 4) {
+                        w.wait(AB_PFULL1 + X, j & 1);
+                        tc_fence_after_sync();
+                    }
                     if (lead) mma_ts(tmem + TM_O + X * 128, tmem + TM_S + X * 128 + ks * 8, dv + ((ks * 2048) >> 4), ID_PV,
                            (j > 0 || ks > 0) ? 1u : 0u);
+                }
             };
             w.wait(AB_Q, 0);
             w.wait(AB_KFULL0, 0);
@@ -293,8 +300,6 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 w.wait(AB_VFULL0 + s, (j >> 1) & 1);
                 if (more) w.wait(AB_KFULL0 + s1, ((j + 1) >> 1) & 1);
                 if (j < nA) {
-                    w.wait(AB_PFULL0 + 0, j & 1);
-                    tc_fence_after_sync();
                     issue_pv(0, j);
                     if (j + 1 < nA) {
                         issue_qk(0, j + 1);
@@ -303,8 +308,6 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                 }
                 if (hasB) {
-                    w.wait(AB_PFULL0 + 1, j & 1);
-                    tc_fence_after_sync();
                     issue_pv(1, j);
                     if (more) {
                         issue_qk(1, j + 1);
@@ -390,7 +393,7 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, const in
         return GDN_ERR_CUDA;
     AttnParams p{static_cast<__nv_bfloat16*>(out), cu_seqlens, B, T, Hq, Hkv, scale * 1.4426950408889634f};
     // packed: sum over sequences of ceil(ceil(len / 128) / 2) <= T / 256 + B
-    dim3 grid(Hq, cu_seqlens ? T / (2 * BM) + B : ((T + BM - 1) / BM + 1) / 2, cu_seqlens ? 1 : B);
+    dim3 grid(cu_seqlens ? Hq : Hq * B, cu_seqlens ? T / (2 * BM) + B : ((T + BM - 1) / BM + 1) / 2);
     if (cudaFuncSetAttribute(attn_causal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ATTN_SMEM) !=
         cudaSuccess)
         return GDN_ERR_CUDA;
