@@ -99,6 +99,8 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     AWaiter w{base + AS_BARS, reinterpret_cast<volatile int*>(sm + AS_MISC + 4)};
 
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
+    pdl_trigger();                      // a following kernel of this library may set itself up as SMs come free
+    pdl_wait();                         // the inputs, and the buffer of the outputs, belong to what ran before
     // which sequence and which pair of query tiles: batched input takes them from the grid; packed input
     // walks the sequence boundaries (grid.y covers an upper bound of the pair count, the surplus CTAs leave)
     // CTAs start in x-major order.  Everywhere the longest pairs of tiles come first and the short ones fill the tail: y
@@ -391,13 +393,26 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, const in
     if (!tc_make_map(&mq, q, tokens, Hq, d) || !tc_make_map(&mk, k, tokens, Hkv, d) ||
         !tc_make_map(&mv, v, tokens, Hkv, d))
         return GDN_ERR_CUDA;
-    AttnParams p{static_cast<__nv_bfloat16*>(out), cu_seqlens, B, T, Hq, Hkv, scale * 1.4426950408889634f};
+    // masked scores are -inf, which a factor of zero would turn into NaN: the smallest normal number stands for zero (every
+    // 2^(c s - m) is 1 with it)
+    const float c = scale * 1.4426950408889634f;
+    AttnParams p{static_cast<__nv_bfloat16*>(out), cu_seqlens, B, T, Hq, Hkv, c > 1.17549435e-38f ? c : 1.17549435e-38f};
     // packed: sum over sequences of ceil(ceil(len / 128) / 2) <= T / 256 + B
     dim3 grid(cu_seqlens ? Hq : Hq * B, cu_seqlens ? T / (2 * BM) + B : ((T + BM - 1) / BM + 1) / 2);
     if (cudaFuncSetAttribute(attn_causal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ATTN_SMEM) !=
         cudaSuccess)
         return GDN_ERR_CUDA;
-    attn_causal_kernel<<<grid, ATTN_THREADS, ATTN_SMEM, stream>>>(mq, mk, mv, p);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(ATTN_THREADS);
+    cfg.dynamicSmemBytes = ATTN_SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, attn_causal_kernel, mq, mk, mv, p);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }

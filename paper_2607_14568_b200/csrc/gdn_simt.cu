@@ -30,6 +30,7 @@
 #include <mutex>
 
 #include "gdn_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace gdn {
 namespace {
@@ -296,6 +297,8 @@ __global__ void __launch_bounds__(NT, 1) gdn_simt_kernel(SimtParams p) {
     TIO* const sV = reinterpret_cast<TIO*>(sW + NC * LDT);               // two slices [C][NC]
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    ptx::pdl_trigger();
+    ptx::pdl_wait();                           // launched ahead of the previous kernel's end: nothing is read or written before it
     const uint32_t rank = cluster_rank();
     const int CS = (int)cluster_size();        // chunks prepared at a time, one per CTA
     const int h = blockIdx.y, n = blockIdx.z;
@@ -536,7 +539,9 @@ int launch_typed(const SimtParams& p, cudaStream_t stream) {
     if (cudaGetDevice(&dev) != cudaSuccess) return GDN_ERR_CUDA;
     if (dev < 0 || dev >= kMaxDevices) return GDN_ERR_UNSUPPORTED;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
@@ -570,6 +575,7 @@ int launch_typed(const SimtParams& p, cudaStream_t stream) {
     cfg.gridDim = dim3(p.dv / NC, p.H, p.B);
     cfg.dynamicSmemBytes = simt_smem<TIO, NC>(p.dk);
     cfg.stream = stream;
+    cfg.numAttrs = 2;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, gdn_simt_kernel<TIO, NC>, p);
     count_launch();
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
