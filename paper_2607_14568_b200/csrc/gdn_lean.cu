@@ -1724,7 +1724,10 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
         const int m = tid;
         const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
         float s[CMB_COLS];
-        if (p.s0) {   // the initial state is an input of the call: it may be read before the predecessor has finished
+        // M_seg, N_seg come from the summary kernel.  The initial state waits as well: with every kernel launched ahead of
+        // its predecessor's end, only this wait says that what ran before the call, which may have produced it, is done.
+        if (!SCAN) pdl_wait();
+        if (p.s0) {
             const float4* src = reinterpret_cast<const float4*>(p.s0 + (((size_t)n * H + h) * DK + m) * dv + j0);
 #pragma unroll
             for (int q = 0; q < CMB_COLS / 4; ++q) { const float4 x = __ldg(src + q); s[4 * q] = x.x; s[4 * q + 1] = x.y; s[4 * q + 2] = x.z; s[4 * q + 3] = x.w; }
@@ -1732,7 +1735,6 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
 #pragma unroll
             for (int j = 0; j < CMB_COLS; ++j) s[j] = 0.f;
         }
-        if (!SCAN) pdl_wait();          // M_seg, N_seg come from the summary kernel
         auto store_sin = [&](int seg) {
             float4* dst = reinterpret_cast<float4*>(p.seg_sin + seg_off(seg) + (size_t)m * dv + j0);
 #pragma unroll
