@@ -391,6 +391,7 @@ int gdn_debug_get_timing(float* ms5) { return ms5 ? lean_get_timing(ms5) : GDN_E
 // Not part of the public header: forces the number of sequence segments (0 = automatic); chooses between the
 // merged scan kernel (1: used whenever its grid fits the GPU at once) and the three stand-alone kernels (0, default).
 void gdn_debug_force_segments(int nseg) { lean_force_segments(nseg); }
+void gdn_debug_set_relay(int pieces) { lean_set_relay(pieces); }
 void gdn_debug_set_compact(int mode) { lean_set_compact(mode); }
 void gdn_debug_set_scan(int enable) { lean_set_scan(enable); }
 void gdn_debug_set_l2_hints(int enable) { lean_set_l2_hints(enable); }

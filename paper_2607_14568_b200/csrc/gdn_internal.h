@@ -69,6 +69,7 @@ void lean_set_debug(float* p);        // tests only: time stamps of the chain ke
 int lean_set_timing(int enable);      // benchmark only: record events around each kernel
 int lean_get_timing(float* ms5);      // {prepare, summary, combine, chain, scan} of the last call
 void lean_set_l2_hints(int enable);   // tests only: 0 = no L2 eviction-priority hints
+void lean_set_relay(int pieces);      // tests only: pieces per chain (0 = never, -1 = by the rule)
 void lean_set_compact(int mode);      // tests only: 0 / 1 = scratch items with / without W, -1 = by the rule
 void lean_set_scan(int enable);       // tests only: 0 = never merge summary, combine and chain into one launch
 

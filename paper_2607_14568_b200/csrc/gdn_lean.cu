@@ -53,6 +53,7 @@ static bool g_lean_use_scan = false;       // true = summary, combination and ch
                                            // slower than the three kernels under programmatic dependent launch: 0.162 vs 0.152 ms on
                                            // the 10240-token workload, 0.074 vs 0.060 ms at 2048 tokens, so it is off by default)
 static bool g_lean_scan_last = false;
+static int g_lean_relay = -1;              // tests: pieces per chain (0 = never, -1 = by the rule)
 static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size (-1 = by the rule)
 
 namespace {
@@ -277,6 +278,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t tmem = warp_uniform(sMisc[0]);
 
     pdl_wait();                         // the scratch may still be read, and the inputs written, by what ran before
+    if (blockIdx.x == 0 && tid == 0) p.ticket[1] = 0;                 // (the chain kernel's, see ChainParams::relay)
 
     // Every CTA starts with the item of its own index; further ones are handed out through a global ticket: the time per
     // item differs between SMs by a quarter, so a fixed assignment would leave the fast ones idle at the end.  The
@@ -772,7 +774,12 @@ struct ChainParams {
     const __nv_bfloat16* gate_z;   // [.., H, d_v] like out, or nullptr
     const float* norm_w;           // [d_v]
     float norm_eps;
-    int* ticket;                   // the prepare kernel's item ticket: zeroed here for the next call (that kernel has completed)
+    int* ticket;                   // the prepare kernel's item ticket: zeroed here for the next call (that kernel has completed);
+                                   // ticket[1]: the next piece of a relay
+    // Relay (more chains than SMs, see plan_relay): every chain is cut into nseg pieces that run one after the other, each
+    // possibly on another SM.  Pieces are taken in order through ticket[1], all first pieces before all second ones, so
+    // whoever waits for a piece knows that it is running or done; the state travels through sT.
+    int* relay;                    // [chains] pieces of the chain that are done (zero before and after every call), or nullptr
 };
 
 // One CTA's identity inside a kernel: aligned shared-memory base (address and pointer), tensor-memory base,
@@ -833,9 +840,13 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 // with (T diag(b))^T onto U^T.  One hop more per step (about 0.25 us), but 16 KB less to write and to read
 // per chunk and head, so it is the form for grids that are bound by memory (see launch_lean).  As many roundings: Y
 // here, W there.
-template <bool DBG, bool SCAN, bool GATED, bool COMPACT>
+// MODE: what only a debug build (time stamps) or a relay needs stays out of the plain kernel: as run-time branches the relay cost
+// the other calls 1 to 2 %.
+enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2 };
+template <int MODE, bool SCAN, bool GATED, bool COMPACT>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
+    constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay;
     constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments of each
     constexpr int CW = 8 + 4 * NOUT;                         // first warp of the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
@@ -866,7 +877,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     // With a split every segment, the first included, takes its incoming state from seg_sin (the combine
     // kernel copied the caller's initial state there): nothing reads initial_state once this kernel runs,
     // so final_state may alias it.
-    const float* s_in = p.seg_sin ? p.seg_sin + ((size_t)(n * p.nseg + seg) * H + h) * DK * dv + (size_t)dvb * DVB
+    auto done = [&]() { return p.relay + (n * H + h) * (dv / DVB) + dvb; };      // (few chains: see kMaxRelayChains)
+    const float* s_in = RELAY && seg > 0 ? p.sT + state_off
+                      : p.seg_sin ? p.seg_sin + ((size_t)(n * p.nseg + seg) * H + h) * DK * dv + (size_t)dvb * DVB
                                   : (p.s0 ? p.s0 + state_off : nullptr);
 
     if (warp < 8) {
@@ -879,13 +892,13 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         const uint32_t t_sbf = tmem + lane_base + TM_SBF + 32 * wg, t_ds = tmem + lane_base + TM_DS + 64 * wg;
         const size_t soff = (size_t)(64 * wg) * dv + j;          // this thread's first state element: row 64 wg, column j
         float S[64];
-        if (SCAN) {                                     // the combine phase of every slice of this head has been written
-            if (tid == 0) handover_wait(hv, w.abort_flag);
+        if (SCAN || (RELAY && seg > 0)) {               // the combine phase of every slice of this head, or the previous piece, has been written
+            if (tid == 0) handover_wait(SCAN ? hv : Handover{done(), seg}, w.abort_flag);
             named_bar_sync(3, 256);
         }
-        if (s_in) {
+        if (s_in) {                                     // (SCAN, RELAY: past the L1 cache, another SM may have written it during this launch)
 #pragma unroll
-            for (int m = 0; m < 64; ++m) S[m] = SCAN ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
+            for (int m = 0; m < 64; ++m) S[m] = (SCAN || RELAY) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
         } else {
 #pragma unroll
             for (int m = 0; m < 64; ++m) S[m] = 0.f;
@@ -983,9 +996,17 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 }
             }
         }
-        if (p.sT && seg == p.nseg - 1) {
+        if (p.sT && (RELAY || seg == p.nseg - 1)) {
 #pragma unroll
             for (int m = 0; m < 64; ++m) p.sT[state_off + soff + (size_t)m * dv] = S[m];
+        }
+        if (RELAY) {                                    // publish the piece; the last one leaves the counter at zero
+            __threadfence();
+            named_bar_sync(3, 256);
+            if (tid == 0) {
+                __threadfence();
+                atomicExch(done(), seg == p.nseg - 1 ? 0 : seg + 1);
+            }
         }
     } else if (warp < CW) {
         // =============================== output warpgroup(s) ===============================
@@ -1329,7 +1350,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     }
 }
 
-template <bool DBG, bool GATED, bool COMPACT>
+template <int MODE, bool GATED, bool COMPACT>
 __global__ void __launch_bounds__(GATED ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
 gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
@@ -1355,8 +1376,18 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();                      // the next call's prepare kernel may set itself up as SMs come free
     pdl_wait();                         // scratch items and incoming states come from the kernels before this one
-    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
-    chain_body<DBG, false, GATED, COMPACT>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
+    int dvb = (int)blockIdx.x, h = (int)blockIdx.y, z = (int)blockIdx.z;
+    if (MODE == kRelay) {
+        if (threadIdx.x == 0) sMisc[2] = (uint32_t)atomicAdd(p.ticket + 1, 1);
+        __syncthreads();
+        const int D = p.dv / DVB, chains = p.B * p.H * D, t = (int)warp_uniform(sMisc[2]);
+        const int seg = t / chains, c = t - seg * chains;       // the value columns of a head are neighbours: they share K and Q through L2
+        dvb = c % D;
+        h = (c / D) % p.H;
+        z = (c / (D * p.H)) * p.nseg + seg;
+    }
+    const Cta cta{base, sm, tmem, dvb, h, z};
+    chain_body<MODE, false, GATED, COMPACT>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1978,7 +2009,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         stamp(3);
         // ---------------- phase 3: chain over this segment's chunks ----------------
         const Cta c3{base, sm, tmem, 0, h, (int)blockIdx.z};
-        chain_body<DBG, true, false, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
+        chain_body<DBG ? kStamps : kPlain, true, false, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
         stamp(4);
         tc_fence_before_sync();
         cta_sync();
@@ -2034,10 +2065,28 @@ static void plan_split(int B, int T, int H, int d_v, bool packed, int num_sms, i
     }
 }
 
+// More chains than SMs: in one piece each, the last round of CTAs leaves SMs idle (256 chains on 148 SMs: the second round
+// fills 108).  Cut into pieces that relay the state, ceil(chains * pieces / SMs) rounds of shorter pieces follow
+// each other; a piece costs about six chunk steps of start and drain.  Returns the pieces (1 = whole chains), only for
+// a gain of more than a twentieth.
+// (One B200, d_v = 256: 192 chains of 128 steps 335 -> 285 us for the kernel, 476 -> 435 us a call; 192 of 64 steps
+// 190 -> 165 and 261 -> 240 us; 256 of 512 steps, which memory bounds when all SMs are busy, 1410 -> 1363 us.)
+static int plan_relay(long chains, int nch, int num_sms) {
+    auto cost = [&](int pieces) {
+        const long len = (nch + pieces - 1) / pieces, rounds = (chains * pieces + num_sms - 1) / num_sms;
+        return rounds * (len + 6);
+    };
+    int best = 1;
+    for (int q = 2; q <= 12 && nch / q >= 24; ++q)
+        if (cost(q) < cost(best)) best = q;
+    return cost(best) * 20 < cost(1) * 19 ? best : 1;
+}
+
 // In front of the items: the prepare kernel's item ticket (two ints) and, from int 16 on, the scan kernel's
 // counters (four ints per (sequence, head)).  All of it reads zero before a call and zero again after it.
 constexpr size_t kWorkspaceHeader = 4096;
 constexpr int kScanFlagOffset = 16;
+constexpr long kMaxRelayChains = (long)(kWorkspaceHeader / sizeof(int) - kScanFlagOffset);
 constexpr long kMaxScanChains = (long)(kWorkspaceHeader / sizeof(int) - kScanFlagOffset) / SCAN_FLAG_INTS;
 
 // The ticket must read zero before the first launch; every launch leaves it zero again.
@@ -2102,9 +2151,11 @@ static int device_setup(int* sms_out) {
 #define GDN_K(...) reinterpret_cast<const void*>(__VA_ARGS__)
         if (!smem_limit(GDN_K(gdn_prep_kernel<false, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, false>), PREP_SMEM) ||
             !smem_limit(GDN_K(gdn_prep_kernel<false, true>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, true>), PREP_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<false, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<true, false, false>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<false, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<false, false, true>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<false, true, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kStamps, false, false>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, false, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, true, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kRelay, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, false, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kRelay, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, true, true>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_summary_kernel<false>), SUM_SMEM) || !smem_limit(GDN_K(gdn_summary_kernel<true>), SUM_SMEM) ||
             !smem_limit(GDN_K(gdn_combine_kernel), CMB_SMEM) ||
             !smem_limit(GDN_K(gdn_scan_kernel<false>), SCAN_SMEM) || !smem_limit(GDN_K(gdn_scan_kernel<true>), SCAN_SMEM))
@@ -2147,6 +2198,15 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
         nseg = 1;
         seg_chunks = (a.T + C - 1) / C > 0 ? (a.T + C - 1) / C : 1;
     }
+    // ---- relay of chains that do not fill a whole number of rounds (the states travel through final_state) ----
+    const long chain_ctas = (long)a.B * a.H * (a.d_v / DVB);
+    const int nch_all = packed ? 0 : (a.T + C - 1) / C;
+    int pieces = 1;
+    if (nseg == 1 && !packed && !forced && a.final_state && !g_lean_dbg && chain_ctas <= kMaxRelayChains)
+        pieces = g_lean_relay > 0 ? (g_lean_relay < nch_all ? g_lean_relay : 1)
+                 : g_lean_relay < 0 && chain_ctas > num_sms ? plan_relay(chain_ctas, nch_all, num_sms) : 1;
+    const int piece_chunks = pieces > 1 ? (nch_all + pieces - 1) / pieces : seg_chunks;
+    if (pieces > 1) pieces = (nch_all + piece_chunks - 1) / piece_chunks;
     CUtensorMap mq, mk, mv, mo, mz;
     if (!tc_make_map(&mq, a.q, tokens, a.H, a.d_k) || !tc_make_map(&mk, a.k, tokens, a.H, a.d_k) ||
         !tc_make_map(&mv, a.v, tokens, a.H, a.d_v) || !tc_make_map(&mo, a.out, tokens, a.H, a.d_v) ||
@@ -2219,12 +2279,15 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     }
     // ---- steps c, d ----
     ChainParams cp{a.initial_state, static_cast<__nv_bfloat16*>(a.out), a.final_state, a.cu_seqlens,
-                   ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, nseg, seg_chunks,
-                   snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket};
-    dim3 grid(a.d_v / DVB, a.H, a.B * nseg);
-    auto chain = opt.gate_z ? (compact ? gdn_chain_kernel<false, true, true> : gdn_chain_kernel<false, true, false>)
-                 : g_lean_dbg ? gdn_chain_kernel<true, false, false>
-                              : (compact ? gdn_chain_kernel<false, false, true> : gdn_chain_kernel<false, false, false>);
+                   ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, pieces > 1 ? pieces : nseg, piece_chunks,
+                   snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket,
+                   pieces > 1 ? static_cast<int*>(workspace) + kScanFlagOffset : nullptr};
+    dim3 grid(a.d_v / DVB, a.H, a.B * (pieces > 1 ? pieces : nseg));
+    auto chain = pieces > 1 ? (opt.gate_z ? (compact ? gdn_chain_kernel<kRelay, true, true> : gdn_chain_kernel<kRelay, true, false>)
+                                          : (compact ? gdn_chain_kernel<kRelay, false, true> : gdn_chain_kernel<kRelay, false, false>))
+                 : opt.gate_z ? (compact ? gdn_chain_kernel<kPlain, true, true> : gdn_chain_kernel<kPlain, true, false>)
+                 : g_lean_dbg ? gdn_chain_kernel<kStamps, false, false>
+                              : (compact ? gdn_chain_kernel<kPlain, false, true> : gdn_chain_kernel<kPlain, false, false>);
     launch_after(chain, grid, opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
                  mq, mk, mv, mo, mz, cp);
     count_launch();
@@ -2232,6 +2295,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
+void lean_set_relay(int pieces) { g_lean_relay = pieces; }
 void lean_set_compact(int mode) { g_lean_compact = mode; }
 void lean_set_scan(int enable) { g_lean_use_scan = enable != 0; }
 void lean_set_l2_hints(int enable) { g_lean_l2_hints = enable; }
@@ -2315,7 +2379,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
             return GDN_ERR_CUDA;
         if (cudaFuncSetAttribute(gdn_prep_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(gdn_prep_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_chain_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
+            cudaFuncSetAttribute(gdn_chain_kernel<kPlain, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
             return GDN_ERR_CUDA;
         sms_of_device[dev] = sms;
         scratch_of_device[dev] = ptr;
@@ -2336,7 +2400,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
                    ws, nullptr, nullptr, -1, a.B, a.T, a.H, a.d_v, 1, packed ? (1 << 24) : (nch > 0 ? nch : 1),
                    nullptr, 1, 0, 0, nullptr, nullptr, 0.f, static_cast<int*>(ticket_of_device[dev])};
     dim3 grid(a.d_v / DVB, a.H, a.B);
-    gdn_chain_kernel<false, false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
+    gdn_chain_kernel<kPlain, false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
