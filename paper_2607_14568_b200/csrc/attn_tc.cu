@@ -50,12 +50,13 @@ constexpr uint32_t TILE_BYTES = 32768;
 constexpr uint32_t AS_Q = 0, AS_K = 2 * TILE_BYTES, AS_V = 4 * TILE_BYTES;      // Q: A, B; K, V: two stages each
 constexpr uint32_t AS_BARS = 6 * TILE_BYTES;
 constexpr uint32_t AS_MISC = AS_BARS + 24 * 8;
+constexpr uint32_t AS_TAKEN = AS_MISC + 48;
 constexpr uint32_t AS_TOTAL = AS_MISC + 64;
 constexpr uint32_t ATTN_SMEM = AS_TOTAL + 1024;
 
 enum ABar : uint32_t { AB_Q = 0, AB_KFULL0 = 1, AB_KFREE0 = 3, AB_VFULL0 = 5, AB_VFREE0 = 7, AB_SFULL0 = 9 /* A, B */,
                        AB_PFULL0 = 11 /* A, B: first 64 keys */, AB_PVDONE0 = 13 /* A, B */, AB_PFULL1 = 15 /* A, B: other 64 */,
-                       AB_QFREE = 17 /* Q tiles and item slot read */ };
+                       AB_QFREE = 17 /* Q tiles and item slot read */, AB_TAKEN = 18 };
 
 struct AWaiter {
     uint32_t bars;
@@ -95,13 +96,15 @@ constexpr uint32_t ID_PV = make_idesc(128, 128, kFmtBF16, kFmtBF16, kMajorK, kMa
 // probabilities, the tensor core runs P V and the next Q K^T of the other.  (Items of a single tile when
 // there are few: the rule is at the launch.)
 //
-// One CTA per SM walks its share of the items, sorted by length, the longest first, dealt out back and
-// forth.  The copies of the next item start when the last Q K^T of the current one has been issued, and its first
-// Q K^T and softmax run under the last softmax and the output of the current one; with a CTA per item the 5 us of
-// its start and end stood open between any two (16 heads: 6000 tokens 136 -> 126 us, 10240 tokens 400 -> 383 us at the
-// power limit, packed 1711 + 402 + 2048 + 65 + 977 tokens 54 -> 46.8 us).  The copy warp looks the items up and publishes them in shared
-// memory (item k in slot k & 1, barrier AB_Q; t < 0 is the end); a slot and the Q tiles are free again
-// when the softmax warps have read the one and the tensor core the others (AB_QFREE).
+// The grid has one CTA per item, the longest items first.  A CTA that has issued its item's last copies takes the item of a
+// CTA that has not started (which then never does), so every SM goes on to the longest item that is left, and the copies,
+// first Q K^T and softmax of the next item run under the last softmax and the output of the current one; started as a
+// CTA, each item left 5 us open.  16 heads: 6000 tokens 136 -> 124 us, 10240 tokens 400 -> 383 us at the power limit,
+// packed 1711 + 402 + 2048 + 65 + 977 tokens 54 -> 43 us, eight packed prompts of 33 to 3000 tokens 84 -> 66 us.  (One CTA per SM and
+// the items dealt out back and forth in advance: 126, 383, 47, 75 us.)
+// The copy warp looks the items up and publishes them in shared memory (item k in slot k & 1, barrier AB_Q; t < 0 is the
+// end); a slot and the Q tiles are free again when the softmax warps have read the one and the tensor core the others
+// (AB_QFREE).
 __global__ void __launch_bounds__(ATTN_THREADS, 1)
 attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, AttnParams p) {
@@ -136,23 +139,24 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // Items are numbered (y, x): x over heads (and sequences of one length), y from the last index of the longest sequence
     // down, over all sequences.  Packed: items with an index of at least i are sum max(0, count - i); the largest i with more
     // than y of them is the index of y, and its sequence follows from y's rank among the sequences that have it.  One warp does
-    // this together (a thread alone took 4.6 ms for 400 sequences of 64 tokens that now take 0.35 ms).
+    // this together (400 sequences of 64 tokens: 4.6 ms with a thread alone, 0.21 ms).
     const int span = p.per * BM;
     int first = 0;                                         // items of sequence `lane`: the first 32 are read once
+    int most = 0, ny = (p.T + span - 1) / span;            // items of the longest sequence, items of one head
     auto count_of = [&](int n) { return n < 32 ? first : (p.cu[n + 1] - p.cu[n] + span - 1) / span; };
     auto at_least = [&](int i) {
         int sum = max(0, first - i);
         for (int n = lane + 32; n < p.B; n += 32) sum += max(0, count_of(n) - i);
         return (int)__reduce_add_sync(0xffffffffu, sum);
     };
-    auto find = [&](uint32_t k, Item& it) {                // item k of this CTA; t < 0 when there are no more
-        const uint32_t G = gridDim.x, i = k * G + ((k & 1) ? G - 1 - blockIdx.x : blockIdx.x), X = p.cu ? p.Hq : p.Hq * p.B;
-        const int ny = p.cu ? at_least(0) : (p.T + span - 1) / span, y = (int)(i / X), x = (int)(i - y * X);
-        it.t = -1;                                         // (only the last row is partial: a CTA that is not in it is through)
+    auto find = [&](uint32_t i, Item& it) {                // item i, t < 0 if there are not that many
+        const uint32_t X = p.cu ? p.Hq : p.Hq * p.B;
+        const int y = (int)(i / X), x = (int)(i - y * X);
+        it.t = -1;
         if (y >= ny) return;
         it.h = x % p.Hq;
         if (p.cu) {
-            int lo = 0, hi = (p.T + span - 1) / span;      // at_least(lo) > y >= at_least(hi)
+            int lo = 0, hi = most;                         // at_least(lo) > y >= at_least(hi)
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
                 if (at_least(mid) > y) lo = mid; else hi = mid;
@@ -180,10 +184,11 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         shape(it);
     };
     Item it{};
-    if (warp == 9 && !p.cu) find(0, it);                   // the first one under the setup
+    if (warp == 9 && !p.cu) find(blockIdx.x, it);                   // the first one under the setup
 
     if (tid == 0) {
-        mbar_init(w.bar(AB_Q), 1); mbar_init(w.bar(AB_QFREE), 9);      // 8 softmax warps and the tensor core
+        mbar_init(w.bar(AB_Q), 1); mbar_init(w.bar(AB_TAKEN), 1);
+        mbar_init(w.bar(AB_QFREE), 9);                     // 8 softmax warps and the tensor core
         for (uint32_t s = 0; s < 2; ++s) {
             mbar_init(w.bar(AB_KFULL0 + s), 1); mbar_init(w.bar(AB_KFREE0 + s), 1);
             mbar_init(w.bar(AB_VFULL0 + s), 1); mbar_init(w.bar(AB_VFREE0 + s), 1);
@@ -395,12 +400,33 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         };
         if (p.cu) {
             if (lane < p.B) first = (p.cu[lane + 1] - p.cu[lane] + span - 1) / span;
-            find(0, it);
+            most = first;
+            for (int n = lane + 32; n < p.B; n += 32) most = max(most, count_of(n));
+            most = (int)__reduce_max_sync(0xffffffffu, most);
+            ny = at_least(0);
+            find(blockIdx.x, it);
         }
         uint32_t kt = 0;
-        int q_loads = 0;
+        int q_loads = 0, asked = 0;
+        auto next = [&](Item& it) {
+            do {
+                uint32_t i = ~0u;
+                if (lane == 0) {
+                    fence_proxy_async_smem();              // (the previous answer has been read)
+                    mbar_arrive_expect_tx(w.bar(AB_TAKEN), 16);
+                    take_pending_cta(base + AS_TAKEN, w.bar(AB_TAKEN));
+                    w.wait(AB_TAKEN, asked & 1);
+                    if (*w.abort_flag == 0) i = taken_cta_x(base + AS_TAKEN);
+                }
+                ++asked;
+                i = warp_uniform(i);
+                it.t = -1;
+                if (i == ~0u) return;
+                find(i, it);
+            } while (it.t < 0);
+        };
         for (int k = 0;; ++k) {
-            if (k > 0) find(k, it);                        // under the copies and products of item k - 1
+            if (k > 0) next(it);                           // under the last two rounds of item k - 1
             if (lane == 0) {
                 if (k > 0) w.wait(AB_QFREE, (k - 1) & 1);
                 volatile uint32_t* m = sMisc + 4 + 4 * (k & 1);
@@ -431,6 +457,7 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             // let copies in flight land before shared memory is released (bounded)
             const unsigned long long t0 = globaltimer_ns();
             while (q_loads > 0 && !mbar_try_wait(w.bar(AB_Q), (q_loads - 1) & 1) && globaltimer_ns() - t0 < ATTN_TIMEOUT_NS) {}
+            while (asked > 0 && !mbar_try_wait(w.bar(AB_TAKEN), (asked - 1) & 1) && globaltimer_ns() - t0 < ATTN_TIMEOUT_NS) {}
             for (uint32_t x = kt >= 2 ? kt - 2 : 0; x < kt; ++x)
                 for (uint32_t which = 0; which < 2; ++which)
                     while (!mbar_try_wait(w.bar((which ? AB_VFULL0 : AB_KFULL0) + (x & 1)), (x >> 1) & 1) &&
@@ -492,7 +519,8 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, const in
     };
     p.per = items_of(1) < 2ll * sms ? 1 : 2;
     const long long items = items_of(p.per);
-    const dim3 grid((unsigned)(items < sms ? items : sms));
+    if (items > 0x7fffffffll) return GDN_ERR_TOO_LARGE;
+    const dim3 grid((unsigned)items);
     if (cudaFuncSetAttribute(attn_causal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ATTN_SMEM) !=
         cudaSuccess)
         return GDN_ERR_CUDA;

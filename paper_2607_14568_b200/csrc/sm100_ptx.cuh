@@ -273,6 +273,22 @@ __device__ __forceinline__ uint32_t warp_uniform(uint32_t x) { return __shfl_syn
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Work stealing (cluster launch control): asks for one CTA of this grid that has not started; it then never does, and its
+// work is the caller's.  The 16-byte answer completes 16 bytes on the barrier.  Not to be asked again after a "none".
+__device__ __forceinline__ void take_pending_cta(uint32_t answer, uint32_t bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t taken_cta_x(uint32_t answer) {         // its blockIdx.x, or ~0 for none
+    uint32_t x;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 h;\n\tld.shared.b128 h, [%1];\n\tmov.u32 %0, 0xffffffff;\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+        : "=r"(x) : "r"(answer) : "memory");
+    return x;
+}
+
 // ---------------------------------------------------------------- small helpers
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);   // .x = lo -> low 16 bits

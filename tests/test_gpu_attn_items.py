@@ -1,5 +1,5 @@
 """Attention: how the query tiles are dealt out to the SMs (single tiles or pairs, one or several
-items per SM, packed sequences of every kind), against the fp64 oracle."""
+items per CTA, packed sequences of every kind), against the fp64 oracle."""
 import numpy as np
 import pytest
 import torch
@@ -40,7 +40,7 @@ def _check(B, T, Hq, Hkv, lens=None):
             assert_close(f64(out[s]), want, 5e-3, 2e-2, f"out of {n} tokens at {s.start}")
 
 
-# 148 SMs: one tile per item below 296 of them, pairs from there on; the last row of items full, partial or absent
+# 148 SMs: one tile per item below 296 of them, pairs from there on; one item per SM, two, or several taken over
 @pytest.mark.parametrize("B,T,Hq", [(1, 129, 74), (1, 257, 98), (1, 257, 99), (37, 129, 4), (5, 385, 30), (1, 1281, 29)])
 def test_items(B, T, Hq):
     _check(B, T, Hq, Hq)
