@@ -87,6 +87,18 @@ struct Prefill {
 };
 
 PyObject* result(long rc) { return PyLong_FromLong(rc); }
+
+// Calls the entry point without the interpreter lock, as ctypes does: a launch blocks when the queue is full, and what it waits
+// for may be a host callback or another stream's work that a Python thread has yet to run.  (The arguments are plain values by
+// then; the caller's frame holds the tensors.)
+template <typename... P, typename... A>
+PyObject* call(int (*entry)(P...), A... args) {
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = entry(args...);
+    Py_END_ALLOW_THREADS
+    return result(rc);
+}
 #define NEED(n) if (nargs != (n)) return result(kNotTaken)
 #define REFUSE_UNLESS(c) if (!(c)) return result(kNotTaken)
 
@@ -107,8 +119,8 @@ PyObject* prefill(PyObject*, PyObject* const* x, Py_ssize_t nargs) {
     int chunk;
     gdn_stream_t s;
     REFUSE_UNLESS(p.ok && int_of(x[9], &chunk) && stream_of(x[10], &s));
-    return result(F(p.q.ptr<void>(), p.k.ptr<void>(), p.v.ptr<void>(), p.a.ptr<float>(), p.b.ptr<float>(), p.s0.ptr<float>(),
-                    p.out.ptr<void>(), p.fin.ptr<float>(), p.cu.ptr<int32_t>(), p.B, p.T, p.H, p.dk, p.dv, chunk, s));
+    return call(F, p.q.ptr<void>(), p.k.ptr<void>(), p.v.ptr<void>(), p.a.ptr<float>(), p.b.ptr<float>(), p.s0.ptr<float>(),
+                p.out.ptr<void>(), p.fin.ptr<float>(), p.cu.ptr<int32_t>(), p.B, p.T, p.H, p.dk, p.dv, chunk, s);
 }
 
 // q_raw, k_raw, v, a_raw, b_raw, gate_scale, norm_eps, initial_state, out, final_state, cu_seqlens, chunk, stream
@@ -119,9 +131,8 @@ PyObject* prefill_raw(PyObject*, PyObject* const* x, Py_ssize_t nargs) {
     float scale, eps;
     gdn_stream_t s;
     REFUSE_UNLESS(p.ok && float_of(x[5], &scale) && float_of(x[6], &eps) && int_of(x[11], &chunk) && stream_of(x[12], &s));
-    return result(gdn_chunk_prefill_raw(p.q.ptr<void>(), p.k.ptr<void>(), p.v.ptr<void>(), p.a.ptr<float>(), p.b.ptr<float>(), scale, eps,
-                                        p.s0.ptr<float>(), p.out.ptr<void>(), p.fin.ptr<float>(), p.cu.ptr<int32_t>(), p.B, p.T, p.H, p.dk,
-                                        p.dv, chunk, s));
+    return call(gdn_chunk_prefill_raw, p.q.ptr<void>(), p.k.ptr<void>(), p.v.ptr<void>(), p.a.ptr<float>(), p.b.ptr<float>(), scale, eps,
+                p.s0.ptr<float>(), p.out.ptr<void>(), p.fin.ptr<float>(), p.cu.ptr<int32_t>(), p.B, p.T, p.H, p.dk, p.dv, chunk, s);
 }
 
 // q, k, v, log_alpha, beta, initial_state, gate_z, norm_weight, norm_eps, out, final_state, cu_seqlens, chunk, stream
@@ -134,9 +145,9 @@ PyObject* prefill_gated(PyObject*, PyObject* const* x, Py_ssize_t nargs) {
     gdn_stream_t s;
     REFUSE_UNLESS(p.ok && z.ok && w.ok && z.sizes() == p.out.sizes() && w.is({p.dv}) && float_of(x[8], &eps) && int_of(x[12], &chunk) &&
                   stream_of(x[13], &s));
-    return result(gdn_chunk_prefill_gated(p.q.ptr<void>(), p.k.ptr<void>(), p.v.ptr<void>(), p.a.ptr<float>(), p.b.ptr<float>(),
-                                          p.s0.ptr<float>(), z.ptr<void>(), w.ptr<float>(), eps, p.out.ptr<void>(), p.fin.ptr<float>(),
-                                          p.cu.ptr<int32_t>(), p.B, p.T, p.H, p.dk, p.dv, chunk, s));
+    return call(gdn_chunk_prefill_gated, p.q.ptr<void>(), p.k.ptr<void>(), p.v.ptr<void>(), p.a.ptr<float>(), p.b.ptr<float>(),
+                p.s0.ptr<float>(), z.ptr<void>(), w.ptr<float>(), eps, p.out.ptr<void>(), p.fin.ptr<float>(), p.cu.ptr<int32_t>(), p.B, p.T,
+                p.H, p.dk, p.dv, chunk, s);
 }
 
 // q, k, v, log_alpha, beta, state, out, stream
@@ -150,8 +161,8 @@ PyObject* decode(PyObject*, PyObject* const* x, Py_ssize_t nargs) {
     const int64_t dv = v.sizes()[2];
     REFUSE_UNLESS(k.sizes() == qs && v.is({qs[0], qs[1], dv}) && out.sizes() == v.sizes() && a.is({qs[0], qs[1]}) && b.is({qs[0], qs[1]}) &&
                   st.is({qs[0], qs[1], qs[2], dv}) && qs[0] <= INT32_MAX && qs[1] <= INT32_MAX);
-    return result(gdn_decode_step(q.ptr<void>(), k.ptr<void>(), v.ptr<void>(), a.ptr<float>(), b.ptr<float>(), st.ptr<float>(), out.ptr<void>(),
-                                  (int)qs[0], (int)qs[1], (int)qs[2], (int)dv, s));
+    return call(gdn_decode_step, q.ptr<void>(), k.ptr<void>(), v.ptr<void>(), a.ptr<float>(), b.ptr<float>(), st.ptr<float>(),
+                out.ptr<void>(), (int)qs[0], (int)qs[1], (int)qs[2], (int)dv, s);
 }
 
 // q, k, v, out, cu_seqlens, scale, stream
@@ -166,8 +177,8 @@ PyObject* attention(PyObject*, PyObject* const* x, Py_ssize_t nargs) {
     REFUSE_UNLESS(v.sizes() == ks && out.sizes() == qs && qs.slice(0, nd - 2) == ks.slice(0, nd - 2) && qs[nd - 1] == ks[nd - 1]);
     const int64_t B = cu.t ? cu.t->numel() - 1 : qs[0];
     REFUSE_UNLESS(B <= INT32_MAX && qs[nd - 3] <= INT32_MAX && qs[nd - 2] <= INT32_MAX);
-    return result(gdn_attn_causal_prefill(q.ptr<void>(), k.ptr<void>(), v.ptr<void>(), out.ptr<void>(), cu.ptr<int32_t>(), (int)B,
-                                          (int)qs[nd - 3], (int)qs[nd - 2], (int)ks[nd - 2], (int)qs[nd - 1], scale, s));
+    return call(gdn_attn_causal_prefill, q.ptr<void>(), k.ptr<void>(), v.ptr<void>(), out.ptr<void>(), cu.ptr<int32_t>(), (int)B,
+                (int)qs[nd - 3], (int)qs[nd - 2], (int)ks[nd - 2], (int)qs[nd - 1], scale, s);
 }
 
 #define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(fn)), METH_FASTCALL, nullptr}
