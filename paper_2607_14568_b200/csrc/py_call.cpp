@@ -7,6 +7,8 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#include <exception>
+
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -181,12 +183,26 @@ PyObject* attention(PyObject*, PyObject* const* x, Py_ssize_t nargs) {
                 (int)qs[nd - 3], (int)qs[nd - 2], (int)ks[nd - 2], (int)qs[nd - 1], scale, s);
 }
 
-#define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(fn)), METH_FASTCALL, nullptr}
+// torch throws when a tensor has no address (inside vmap), no plain sizes (nested tensors) or no device to ask for its stream:
+// an exception must not leave a function that the interpreter called.
+template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* x, Py_ssize_t nargs) {
+    try {
+        return F(self, x, nargs);
+    } catch (const c10::Error& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    }
+    return nullptr;
+}
+
+#define FAST(name, ...) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<__VA_ARGS__>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
-    FAST("gdn_chunk_prefill", (prefill<gdn_chunk_prefill, at::kBFloat16>)),
-    FAST("gdn_chunk_prefill_f32", (prefill<f32_entry, at::kFloat>)),
-    FAST("gdn_chunk_prefill_bf16_simt", (prefill<gdn_chunk_prefill_bf16_simt, at::kBFloat16>)),
-    FAST("gdn_chunk_prefill_noalloc", (prefill<gdn_chunk_prefill_noalloc, at::kBFloat16>)),
+    FAST("gdn_chunk_prefill", prefill<gdn_chunk_prefill, at::kBFloat16>),
+    FAST("gdn_chunk_prefill_f32", prefill<f32_entry, at::kFloat>),
+    FAST("gdn_chunk_prefill_bf16_simt", prefill<gdn_chunk_prefill_bf16_simt, at::kBFloat16>),
+    FAST("gdn_chunk_prefill_noalloc", prefill<gdn_chunk_prefill_noalloc, at::kBFloat16>),
     FAST("gdn_chunk_prefill_raw", prefill_raw),
     FAST("gdn_chunk_prefill_gated", prefill_gated),
     FAST("gdn_decode_step", decode),

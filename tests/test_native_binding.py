@@ -99,3 +99,21 @@ def test_other_threads_run_during_a_call(stand_in):
             t.join()
             assert rc == 0, f"{name}: no other thread ran while the entry point was waiting (status {rc})"
     """)
+
+
+def test_a_tensor_that_cannot_give_its_address_raises(stand_in):
+    """Inside a vmap a tensor has no address of its own and torch throws a C++ exception when it is asked for one: that has to
+    come out as a Python exception (it ended the process when it left the C function)."""
+    _run(stand_in, """
+        go.value = 1
+        for name, args in calls():
+            def mapped(x):
+                return getattr(native, name)(x, *args[1:])
+            batch = Cuda(5, *args[0].shape, dtype=args[0].dtype)
+            try:
+                torch.func.vmap(mapped)(batch)
+            except RuntimeError as e:
+                assert "data pointer" in str(e), f"{name}: {e}"
+            else:
+                raise AssertionError(f"{name}: no exception")
+    """)
