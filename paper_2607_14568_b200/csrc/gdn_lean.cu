@@ -424,6 +424,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 }
             }
             fence_proxy_async_smem();
+            if (COMPACT) tc_fence_before_sync();       // G has been read: PB_KQFREE, below, lets the next item's G overwrite it
             named_bar_sync(1, 128);
             // The images leave the SM as bulk copies from shared memory (a thread-per-row store would
             // touch 32 different lines per instruction); thread 0 issues them and later waits for their

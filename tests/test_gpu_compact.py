@@ -61,3 +61,31 @@ def test_compact_chain_matches_oracle(entry, kw, nseg):
         bar *= max(1.0, float(np.abs(o).max() / np.abs(plain).max()))
     assert_close(f64(d["out"]), o, BF16_REL_L2, bar, "out")
     assert_close(f64(d["final_state"]), fin, BF16_REL_L2, BF16_MAX_ABS, "final_state")
+
+
+def test_many_items_per_cta_match_oracle_and_repeat_bit_for_bit():
+    """2 x 41 chunks of 32 heads over four prepare CTAs per SM: each prepares four items and more, the next item's token-token product
+    following straight on the reads of the previous one (the accumulator is handed back with the tiles)."""
+    cfg = get_config("short", B=2, T=64 * 40 + 7, H=32, init_std=0.3, seed=79)
+    x = make_inputs(cfg)
+    d = to_device(x)
+    ws = torch.empty(gdn.gdn_workspace_bytes(cfg.B, cfg.T, cfg.H, cfg.d_k, cfg.d_v, False), dtype=torch.uint8, device="cuda")
+    gdn.gdn_set_workspace(ws)
+    gdn.lib().gdn_debug_force_segments(1)
+    gdn.lib().gdn_debug_set_compact(1)
+    first = None
+    try:
+        for _ in range(6):
+            d["out"].zero_(); d["final_state"].zero_()
+            gdn.gdn_chunk_prefill(d["q"], d["k"], d["v"], d["log_alpha"], d["beta"], d["initial_state"], d["out"], d["final_state"])
+            got = d["out"].clone(), d["final_state"].clone()
+            first = first or got
+            assert torch.equal(got[0], first[0]) and torch.equal(got[1], first[1])
+        assert gdn.gdn_query_status_stream() == 0
+    finally:
+        gdn.lib().gdn_debug_set_compact(-1)
+        gdn.lib().gdn_debug_force_segments(0)
+        gdn.gdn_set_workspace(None)
+    o, fin = oracle.sequential(widen(x.q), widen(x.k), widen(x.v), x.log_alpha, x.beta, x.initial_state, None)
+    assert_close(f64(first[0]), o, BF16_REL_L2, BF16_MAX_ABS, "out")
+    assert_close(f64(first[1]), fin, BF16_REL_L2, BF16_MAX_ABS, "final_state")
