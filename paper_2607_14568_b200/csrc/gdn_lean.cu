@@ -2223,15 +2223,19 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // earlier readers ask L2 to keep them and the last reader releases them.
     const int l2 = (nseg > 1 && tokens * a.H * (uint64_t)(a.d_k + a.d_v) * 2 <= (96ull << 20)) ? (g_lean_l2_hints & 3) : 0;
     PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, nslots, a.B, a.T, a.H, opt.gate_scale, opt.eps, ticket, l2};
-    // Items without -W^T (24 % less memory traffic over both kernels, one hop more per chain step) pay when the chains of a call
-    // together are bound by memory: one segment each, at least three fifths of the SMs busy to the end (equal
-    // lengths), every chain reading its own K and Q (with d_v = 256 two chains share them through L2).  One B200, calls
-    // with / without: 4 x 8192 tokens x 32 heads 380 / 452 us, 4 x 4096 x 24 157 / 174 us, but 1 x 4096 x 64 heads 149 / 144 us
-    // and 4 x 4096 x 16 heads with d_v = 256 148 / 148 us.  With the fused output stage a step is longer anyway
-    // and the line lies lower (4 x 1500 x 16: 74 / 78 us).
+    // Items without -W^T (24 % less memory traffic over both kernels, one hop more per chain step) are for calls of one segment
+    // per chain and equal lengths.  A plain or raw call takes them when its chains together are bound by memory: at least three
+    // fifths of the SMs busy to the end, every chain reading its own K and Q (with d_v = 256 two chains share them through
+    // L2: 4 x 4096 x 16 heads 148 / 148 us).  One B200, calls without / with W: 1500 tokens 64 chains 58.1 / 57.8 us, 80 64.0 / 66.4,
+    // 96 71.9 / 76.1, 144 94 / 112; 4096 tokens 64 chains 148 / 140 us, 80 169 / 162, 96 188 / 188, 112 204 / 218, 144 238 / 284; 8192
+    // tokens 64 chains 293 / 268 us, 96 370 / 364, 112 404 / 419, 144 466 / 552.  (The line lies at 89 chains: the crossing moves from
+    // 70 at 1500 tokens to 100 at 8192, with at most 3 % to gain on either side of it.)  With the fused output stage that stage and not
+    // the chain sets the step, which hides the hop, so there is no line: 64 tokens 1 to 24 chains 4 to 5 % less, 1500
+    // tokens 1 chain 54.7 / 54.4 us, 16 58.9 / 59.4, 32 65.7 / 67.6, 56 72.0 / 73.7, 64 73.5 / 77.1, 96 87 / 94, 144 113 / 126; 4096 tokens
+    // 32 155 / 158 us, 64 178 / 184, 128 271 / 288; 8192 tokens 48 319 / 329 us, 96 445 / 462.
     const bool compact = !g_lean_dbg && !g_lean_use_scan &&
                          (g_lean_compact >= 0 ? g_lean_compact == 1
-                                              : !packed && nseg == 1 && a.d_v == DVB && (long)a.B * a.H * 5 >= (opt.gate_z ? 2L : 3L) * num_sms);
+                                              : !packed && nseg == 1 && a.d_v == DVB && (opt.gate_z || (long)a.B * a.H * 5 >= 3L * num_sms));
     const int pgrid = (int)(nitems < 4L * num_sms ? nitems : 4L * num_sms);
     auto mark = [&](int i) { if (g_lean_timing && g_lean_events[i]) cudaEventRecord(g_lean_events[i], stream); };
     mark(0);
