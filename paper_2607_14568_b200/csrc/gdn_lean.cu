@@ -2041,12 +2041,17 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // ------------------------------------------------------------------------------------------
 // Sequence split: only for batched (equal-length) input.  Returns the number of segments per sequence (1 = no split) and
 // the chunks per segment: the cheapest by the model below, whose constants are fits of the kernels' times on a B200 in units
-// of 0.1 us (d_v = 128; n chunks per segment).  A step of a chain takes 1.04 us by itself and longer when the CTAs
-// together ask for more than the memory delivers (98 KB per chain step, 57 KB per summary step); summaries and chains cost
-// about 12 and 9 us besides their steps, the combination 5 us and 1.5 us a hop for every round of its CTAs (one per
-// SM), and programmatic launches hide about 8 us of a split's start-ups.  So a split pays from about 28 chunks on for 16
-// chains (2048 tokens: 52 us in one piece, 49.5 us in eight), and not at all when fewer than three segments per chain
-// fit the GPU (4 x 1500 tokens, 16 heads: 64 us in one piece, 86 us in two).
+// of 0.1 us (n chunks per segment).  A step of a chain takes 1.04 us by itself and longer when the CTAs together ask for more than
+// the memory delivers: 98 KB per chain step, 57 KB per summary step.  With D = d_v / 128 blocks of value columns the D CTAs of a
+// chain share all of that but their values and outputs through L2, which leaves 33 + 65 / D and 16 + 41 / D KB of
+// a step for the memory.  Summaries and chains cost about 12 and 9 us besides their steps, the combination 5 us and 1.5 us a hop
+// for every round of its CTAs (one per SM), and programmatic launches hide about 8 us of a split's start-ups.  So a split
+// pays from about 28 chunks on for 16 chains (2048 tokens: 47 us in one piece, 45 us in five), and not at all when fewer than
+// three segments per chain fit the GPU (4 x 1500 tokens, 16 heads: 58 us in one piece, 86 us in two).
+// Against every number of segments, 8 to 32 heads of 1024 to 32768 tokens, the choice is at most 7 % slower than the best
+// one with d_v = 128 (8 heads, 10240 tokens: 89 us in ten segments, 83 us in fourteen) and 3 % with 256 to 512.  There, with the
+// traffic of d_v = 128 for every CTA, it was up to 22 % slower: 24 heads 10240 tokens 237 -> 214 us, 32768 tokens 760 -> 623 us, 16
+// heads 4096 tokens 88 -> 79 us.
 constexpr int kMaxSeg = 16;
 static void plan_split(int B, int T, int H, int d_v, bool packed, int num_sms, int* nseg, int* seg_chunks) {
     const int nch = (T + C - 1) / C;
@@ -2055,13 +2060,14 @@ static void plan_split(int B, int T, int H, int d_v, bool packed, int num_sms, i
     const long chains = (long)B * H * (d_v / DVB);
     if (packed || nch < 2 || chains * 2 > num_sms) return;
     auto steps = [](long ctas, int n, double per_cta) { return n * (ctas * per_cta > 10.4 ? ctas * per_cta : 10.4); };
-    double best = 90 + steps(chains, nch, 0.137);
+    const double D = d_v / DVB, chain_cta = 0.137 * (33 + 65 / D) / 98, summary_cta = 0.092 * (16 + 41 / D) / 57;
+    double best = 90 + steps(chains, nch, chain_cta);
     const int most = (int)(num_sms / chains) < kMaxSeg ? (int)(num_sms / chains) : kMaxSeg;
     for (int want = 2; want <= most; ++want) {
         const int sc = (nch + want - 1) / want, ns = (nch + sc - 1) / sc;
         if (ns < 2) break;
         const long rounds = (chains * (DVB / CMB_COLS) + num_sms - 1) / num_sms;
-        const double cost = 125 + steps(chains * (ns - 1), sc, 0.092) + rounds * (50 + 15 * (ns - 1)) + 90 + steps(chains * ns, sc, 0.137) - 80;
+        const double cost = 125 + steps(chains * (ns - 1), sc, summary_cta) + rounds * (50 + 15 * (ns - 1)) + 90 + steps(chains * ns, sc, chain_cta) - 80;
         if (cost < best) { best = cost; *nseg = ns; *seg_chunks = sc; }
     }
 }

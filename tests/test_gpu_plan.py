@@ -1,0 +1,31 @@
+"""The plans the library makes from the sizes of a call: which kernels run (counted launches), and that what they return is the
+oracle's result on both sides of a line."""
+import pytest
+import torch
+
+import paper_2607_14568_b200 as gdn
+from workloads import get_config, make_inputs
+from gdn_testlib import BF16_MAX_ABS, BF16_REL_L2, assert_close, f64, run_oracle, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+# Two CTAs of a chain share its keys, queries and prepared items (d_v = 256): a split costs them less memory than two chains
+@pytest.mark.parametrize("T,H,d_v,launches", [(4096, 16, 256, 4), (10240, 24, 256, 4), (4096, 24, 256, 2), (2048, 16, 256, 2),
+                                              (2048, 16, 128, 4), (1024, 16, 128, 2)])
+def test_sequence_split_by_the_rule(T, H, d_v, launches):
+    cfg = get_config("short", B=1, T=T, H=H, d_v=d_v, init_std=0.02, seed=81)
+    x = make_inputs(cfg)
+    d = to_device(x)
+    ws = torch.empty(gdn.gdn_workspace_bytes(1, T, H, cfg.d_k, d_v, False), dtype=torch.uint8, device="cuda")
+    gdn.gdn_set_workspace(ws)
+    try:
+        n0 = gdn.gdn_launch_count()
+        gdn.gdn_chunk_prefill(d["q"], d["k"], d["v"], d["log_alpha"], d["beta"], d["initial_state"], d["out"], d["final_state"])
+        assert gdn.gdn_launch_count() - n0 == launches
+        assert gdn.gdn_query_status_stream() == 0
+    finally:
+        gdn.gdn_set_workspace(None)
+    o, fin = run_oracle(x)
+    assert_close(f64(d["out"]), o, BF16_REL_L2, BF16_MAX_ABS, "out")
+    assert_close(f64(d["final_state"]), fin, BF16_REL_L2, BF16_MAX_ABS, "final_state")
