@@ -18,7 +18,7 @@
 // What bounds it: fp32 FMAs of one SM (about 460 k multiply-adds per chunk and CTA at d_k = d_v = 128, 3600
 // cycles at full rate) and the shared-memory loads that feed them (six 16-byte loads per 32 FMAs).  The form
 // v_new = Tm (V - K S) needs neither W nor U, so what a CTA fetches per chunk is 34 KiB instead of 66 KiB.
-// Measured on a B200 (2048 tokens, 16 heads, d = 128): 321 us against 2480 us; 256 tokens, 2 heads, d = 64: 35 us against 256 us.  Before, one
+// Measured on a B200 (2048 tokens, 16 heads, d = 128): 324 us against 2480 us; 256 tokens, 2 heads, d = 64: 32 us against 256 us.  Before, one
 // CTA per 32 value columns did every step of every chunk itself.
 //
 // Rows past the end of a sequence are identity tokens (beta = 0, log_alpha = 0,
@@ -528,7 +528,9 @@ __global__ void __launch_bounds__(NT, 1) gdn_simt_kernel(SimtParams p) {
 }
 
 constexpr int kMaxDevices = 64;
-constexpr long kWalk = 330, kPrep = 900;      // time per chunk of the walk and of steps a, b (10 ns units, d = 128)
+// Time per chunk of the walk and of steps a, b in units of 10 ns (one B200, d = 128: 8.9 us a chunk in clusters of eight, which
+// prepare eight chunks at a time, 9.75 us in clusters of four; the ratio is the same with d = 96 and 64)
+constexpr long kWalk = 800, kPrep = 680;
 
 template <typename TIO, int NC>
 int launch_typed(const SimtParams& p, cudaStream_t stream) {
@@ -565,8 +567,9 @@ int launch_typed(const SimtParams& p, cudaStream_t stream) {
         }
     }
     // Cluster size: eight CTAs prepare eight chunks at a time for 8 NC columns; four prepare four for 4 NC columns, so
-    // steps a and b cost four times as much per column, but more of the SMs can be covered (a B200 runs 15
-    // clusters of eight or 33 of four of the largest shape).  Whichever ends first: rounds x time per chunk.
+    // steps a and b cost twice as much per chunk of the walk, but more of the SMs can be covered (a B200 runs 15
+    // clusters of eight or 33 of four of the largest shape).  Whichever ends first: rounds x time per chunk (512 tokens, d = 128,
+    // eights / fours: 48 chains 291 / 240 us, 60 296 / 318, 64 365 / 320, 75 372 / 402, 80 441 / 405, 99 522 / 492, 120 601 / 648).
     const long groups = (long)p.B * p.H * (p.dv / NC);
     const long t8 = (groups / 8 + active8[dev] - 1) / active8[dev] * (kWalk + kPrep / 8);
     const long t4 = (groups / 4 + active4[dev] - 1) / active4[dev] * (kWalk + kPrep / 4);

@@ -5,7 +5,7 @@ import torch
 
 import paper_2607_14568_b200 as gdn
 from workloads import get_config, make_inputs
-from gdn_testlib import BF16_MAX_ABS, BF16_REL_L2, assert_close, f64, run_oracle, to_device
+from gdn_testlib import BF16_MAX_ABS, BF16_REL_L2, F32_REL_L2, assert_close, f64, run_lib, run_oracle, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -29,3 +29,14 @@ def test_sequence_split_by_the_rule(T, H, d_v, launches):
     o, fin = run_oracle(x)
     assert_close(f64(d["out"]), o, BF16_REL_L2, BF16_MAX_ABS, "out")
     assert_close(f64(d["final_state"]), fin, BF16_REL_L2, BF16_MAX_ABS, "final_state")
+
+
+# fp32: clusters of eight CTAs up to 60 chains of this size, of four from 61 to 66, of eight again from 67 (rounds on 148 SMs)
+@pytest.mark.parametrize("B,H", [(4, 15), (1, 61), (2, 33), (1, 67)])
+def test_fp32_clusters_on_both_sides_of_the_line(B, H):
+    x = make_inputs(get_config("tiny", B=B, T=64 * 9 + 5, H=H, init_std=0.1, seed=82))
+    d = to_device(x)
+    out, fin = run_lib(gdn.gdn_chunk_prefill_f32, d)
+    o, f = run_oracle(x)
+    assert_close(f64(out), o, F32_REL_L2, None, "out")
+    assert_close(f64(fin), f, F32_REL_L2, None, "final_state")
