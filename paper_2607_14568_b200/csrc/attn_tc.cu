@@ -20,8 +20,6 @@
 
 #include <cuda.h>
 
-#include <atomic>
-
 #include "gdn_internal.h"
 #include "sm100_ptx.cuh"
 
@@ -502,14 +500,8 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, const in
     // 2^(c s - m) is 1 with it)
     const float c = scale * 1.4426950408889634f;
     AttnParams p{static_cast<__nv_bfloat16*>(out), cu_seqlens, B, T, Hq, Hkv, 2, c > 1.17549435e-38f ? c : 1.17549435e-38f};
-    static std::atomic<int> sms_of_device[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GDN_ERR_CUDA;
-    int sms = dev < 64 ? sms_of_device[dev].load(std::memory_order_relaxed) : 0;
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return GDN_ERR_CUDA;
-        if (dev < 64) sms_of_device[dev].store(sms, std::memory_order_relaxed);
-    }
+    const int sms = sm_count();
+    if (sms <= 0) return GDN_ERR_CUDA;
     // Single tiles while they are fewer than two per SM: a round of one tile takes 1.5 us, of a pair 1.76 us, so halving the
     // longest item pays as long as no SM gets more than about its length (16 heads: 1024 tokens 19.2 -> 16.4 us, 2304 tokens 38.4 -> 34.4;
     // 3000 tokens, 384 single tiles: 48 -> 66 us with a CTA each).  Packed: sum over sequences of ceil(len / span) <= T / span + B.

@@ -12,6 +12,18 @@ namespace gdn {
 static std::atomic<unsigned long long> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
 
+int sm_count() {
+    static std::atomic<int> sms_of_device[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    int sms = dev < 64 ? sms_of_device[dev].load(std::memory_order_relaxed) : 0;
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        if (dev < 64) sms_of_device[dev].store(sms, std::memory_order_relaxed);
+    }
+    return sms;
+}
+
 namespace {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

@@ -133,9 +133,11 @@ int launch_decode(const void* q, const void* k, const void* v, const float* log_
     if (H > 65535 || B > 65535) return GDN_ERR_UNSUPPORTED;
     DecodeParams p{static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
                    static_cast<const __nv_bfloat16*>(v), log_alpha, beta, state, static_cast<__nv_bfloat16*>(out), H, d_k, d_v};
-    // 32 columns per CTA while the CTAs of 128 would not give every (148) SM one: 64 of them 5.0 -> 3.4 us, 80 6.0 -> 4.7 us,
+    // 32 columns per CTA while the CTAs of 128 would not give every SM one (148 on a B200): 64 of them 5.0 -> 3.4 us, 80 6.0 -> 4.7 us,
     // 128 6.0 -> 5.3 us, but 256 6.4 -> 9 us (one B200, back to back)
-    const bool narrow = (long)B * H * (d_v / DVB) <= 148;
+    const int sms = sm_count();
+    if (sms <= 0) return GDN_ERR_CUDA;
+    const bool narrow = (long)B * H * (d_v / DVB) <= sms;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(d_v / (narrow ? 32 : DVB), H, B);
     cfg.blockDim = dim3(NW * 32);

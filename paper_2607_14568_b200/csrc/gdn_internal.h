@@ -85,5 +85,6 @@ int launch_attn(const void* q, const void* k, const void* v, void* out, const in
 int attn_query_status();
 
 void count_launch(int n = 1);
+int sm_count();                       // SMs of the current device, looked up once per device; 0 if that fails
 
 }  // namespace gdn

@@ -3,8 +3,9 @@ oracle's result on both sides of a line."""
 import pytest
 import torch
 
+import oracle
 import paper_2607_14568_b200 as gdn
-from workloads import get_config, make_inputs
+from workloads import get_config, make_inputs, widen
 from gdn_testlib import BF16_MAX_ABS, BF16_REL_L2, F32_REL_L2, assert_close, f64, run_lib, run_oracle, to_device
 
 pytestmark = pytest.mark.gpu
@@ -40,3 +41,18 @@ def test_fp32_clusters_on_both_sides_of_the_line(B, H):
     o, f = run_oracle(x)
     assert_close(f64(out), o, F32_REL_L2, None, "out")
     assert_close(f64(fin), f, F32_REL_L2, None, "final_state")
+
+
+# decode: slices of 32 value columns while the slices of 128 are no more than the SMs
+@pytest.mark.parametrize("blocks,d_v", [(0, 128), (1, 128), (0, 256), (2, 256)])
+def test_decode_on_both_sides_of_the_line(blocks, d_v):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    H = sms * 128 // d_v + blocks * 128 // d_v
+    x = make_inputs(get_config("long", B=1, T=1, H=H, d_v=d_v, init_std=0.5, seed=83))
+    d = to_device(x)
+    state, out = d["initial_state"].clone(), d["out"][:, 0].contiguous()
+    gdn.gdn_decode_step(*(d[n][:, 0].contiguous() for n in ("q", "k", "v", "log_alpha", "beta")), state, out)
+    torch.cuda.synchronize()
+    o, s = oracle.sequential(widen(x.q), widen(x.k), widen(x.v), x.log_alpha, x.beta, x.initial_state)
+    assert_close(f64(out), o[:, 0], BF16_REL_L2, BF16_MAX_ABS, "out")      # one rounding of the output to bf16
+    assert_close(f64(state), s, F32_REL_L2, None, "state")
