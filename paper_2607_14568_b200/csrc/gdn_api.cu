@@ -391,7 +391,8 @@ int gdn_query_status_stream(gdn_stream_t stream_) {
 void gdn_debug_force_path(int path) { g_force_path = path; }
 
 // Not part of the public header: failure-path test hooks.  gdn_debug_drop_chunk(c) makes the chain
-// kernel's TMA thread of one CTA skip chunk c, so the bounded waits on that data expire;
+// kernel's TMA thread of one CTA skip chunk c, so the bounded waits on that data expire; -2 makes one CTA not raise a counter that
+// others wait for, -3 makes the prepare kernel wait for more bytes than its tiles have;
 // gdn_debug_reset_status() clears the status word afterwards.
 void gdn_debug_drop_chunk(int chunk) { lean_set_drop_chunk(chunk); }
 int gdn_debug_reset_status(void) { return lean_reset_status(); }

@@ -45,7 +45,8 @@ static bool g_lean_timing = false;
 static cudaEvent_t g_lean_events[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
 static bool g_lean_split_last = false;
 static float* g_lean_dbg = nullptr;        // debug: time stamps of the chain kernel
-static int g_lean_drop_chunk = -1;         // tests: chunk the chain kernel's TMA thread skips (-1 = none)
+static int g_lean_drop_chunk = -1;         // tests: chunk the chain kernel's TMA thread skips (-1 = none, -2 = a hand-over between CTAs
+                                           // that is not made, -3 = the prepare kernel waits for more bytes than its tiles have)
 static int g_lean_l2_hints = 3;            // tests: bit 0 = L2 eviction-priority hints on the K, Q, V tile loads, bit 1 = on the
                                            // scratch images W and T2 (measured on the 10240-token workload, chain kernel:
                                            // 51.3 us without, 49.0 / 49.4 us with either, 47.2 us with both)
@@ -83,18 +84,23 @@ constexpr uint32_t LDA = 68;
 // passes give the bound of about a second.  (An out-of-line function is not an option next to setmaxnreg.)
 constexpr uint32_t WAIT_PASS_NS = 1000000u;
 constexpr int WAIT_PASSES = 1024;
-struct Waiter {
+// CUT: a wait is given up at once when another role of the CTA has given one up.  The prepare kernel's are not: each runs to its end or
+// its own bound, so that no copy or product is in flight when the CTA ends.
+template <bool CUT>
+struct BoundedWaiter {
     uint32_t bars;              // shared address of barrier 0
     volatile int* abort_flag;
     __device__ __forceinline__ uint32_t bar(uint32_t i) const { return bars + i * 8; }
-    __device__ __forceinline__ void wait_slow(uint32_t b, uint32_t parity) const {
+    template <int PASSES = WAIT_PASSES>
+    __device__ __forceinline__ bool wait_slow(uint32_t b, uint32_t parity) const {
 #pragma unroll 1
-        for (int i = 0; i < WAIT_PASSES; ++i) {
-            if (mbar_try_wait_suspend(b, parity, WAIT_PASS_NS)) return;
-            if (*abort_flag) return;
+        for (int i = 0; i < PASSES; ++i) {
+            if (mbar_try_wait_suspend(b, parity, WAIT_PASS_NS)) return true;
+            if (CUT && *abort_flag) return false;
         }
         *abort_flag = 1;
         atomicCAS(&g_lean_status, 0, (int)GDN_ERR_TIMEOUT);
+        return false;
     }
     // For waits on the sequential chain: poll without suspending for a short while (a suspended
     // thread wakes up late), then fall back to the bounded suspending wait.
@@ -110,7 +116,13 @@ struct Waiter {
         if (mbar_try_wait(b, parity)) return;
         wait_slow(b, parity);
     }
+    // For what follows, without fail, on another role's bounded wait: its bound outlasts that one's.  False when it ran out.
+    __device__ __forceinline__ bool wait_on_waiter(uint32_t idx, uint32_t parity) const {
+        const uint32_t b = bar(idx);
+        return mbar_try_wait(b, parity) || wait_slow<4 * WAIT_PASSES>(b, parity);
+    }
 };
+using Waiter = BoundedWaiter<true>;
 
 __device__ __forceinline__ uint32_t swz(uint32_t row, uint32_t chunk) {
     return row * 128u + ((chunk ^ (row & 7u)) << 4);
@@ -209,6 +221,7 @@ struct PrepParams {
     int* ticket;               // next item beyond the first one of every CTA: zero before the launch; the chain kernel zeroes it again
     int l2;                    // bit 0: the K tiles are read again by later kernels of this call and fit in L2: keep them there;
                                // bit 1: the same for the W and T2 images this kernel writes
+    uint32_t tile_bytes;       // of an item's K and Q tiles, 32768 (tests: 16 more, so that the waits on them run out)
 };
 
 constexpr uint32_t ID_G = make_idesc(128, 64, kFmtBF16, kFmtBF16, kMajorK, kMajorK);
@@ -255,7 +268,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     float* gates = reinterpret_cast<float*>(sm + PS_GATES);
     float* sRN = reinterpret_cast<float*>(sm + PS_RN);
     volatile uint32_t* sMisc = reinterpret_cast<volatile uint32_t*>(sm + PS_MISC);
-    Waiter w{base + PS_BARS, reinterpret_cast<volatile int*>(sm + PS_MISC + 4)};
+    BoundedWaiter<false> w{base + PS_BARS, reinterpret_cast<volatile int*>(sm + PS_MISC + 4)};
 
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int H = p.H;
@@ -308,12 +321,15 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (warp == 4) publish(0, draw((int)blockIdx.x));
     int it = 0;     // items this CTA has processed (barrier phases)
     while (true) {
-        w.wait(PB_ITEM, it & 1);
+        // Nobody leaves on the abort flag: it may rise between two warps' reads of it, and the ones that went on would wait in the
+        // named barriers below for the others.  The end is what the issuing warp publishes, which on an abort it does after the
+        // item at hand.
+        const bool drawn = w.wait_on_waiter(PB_ITEM, it & 1);
         volatile uint32_t* m_item = sMisc + 4 + 4 * (it & 1);
-        const long item = (int)m_item[0];
+        const long item = drawn ? (int)m_item[0] : -1;
         const int h = (int)m_item[1], R = (int)m_item[3];
         const long tok = (int)m_item[2];
-        if (item < 0 || *w.abort_flag) break;
+        if (item < 0) break;
         uint8_t* out_item = p.items + (size_t)item * ITEM_BYTES;
         const uint32_t par = it & 1;
 
@@ -348,7 +364,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             // the -W^T image of the previous item has left the space of A by now; everybody is about to write there
             if (tp == 0) bulk_wait_read_all();
             named_bar_sync(1, 128);
-            w.wait(PB_G, par);
+            w.wait_on_waiter(PB_G, par);
             tc_fence_after_sync();
             // ---- step b1: decay masks on G = [K;Q] K^T ----
             {
@@ -632,7 +648,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 const uint64_t pol_k = (p.l2 & 1) ? l2_policy_evict_last() : l2_policy_evict_normal();
                 auto load_tiles = [&](int hh, long tk) {
                     if (!lead) return;
-                    mbar_arrive_expect_tx(full, 32768);
+                    mbar_arrive_expect_tx(full, p.tile_bytes);
                     tma_load_3d_hint(kq, &map_k, 0, hh, (int)tk, full, pol_k);
                     tma_load_3d_hint(kq + 16384, &map_k, 64, hh, (int)tk, full, pol_k);
                     tma_load_3d(kq + 8192, &map_q, 0, hh, (int)tk, full);
@@ -648,7 +664,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     if (lead) mma_ss(tmem, make_smem_desc(kq + off, 16, 1024), make_smem_desc(kq + off, 16, 1024), ID_G, ks > 0);
                 }
                 if (lead) mma_commit(w.bar(PB_G));
-                const int nxt = draw(-1);                           // the atomic's latency hides behind the solve
+                int nxt = draw(-1);                                 // the atomic's latency hides behind the solve
                 if (!COMPACT) {
                 w.wait(PB_TREADY, par);
                 tc_fence_after_sync();
@@ -662,6 +678,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 // (the end is published no earlier: everybody must have taken this item before the next phase of PB_ITEM
                 //  completes, or a wait for this one would see the parity of the one after)
                 w.wait(PB_KQFREE, par);
+                if (__any_sync(0xffffffffu, *w.abort_flag != 0)) nxt = -1;
                 if (nxt >= 0) load_tiles(nh, ntok);
                 publish((it + 1) & 1, nxt);
             }
@@ -2228,7 +2245,8 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // With a split, K (and V) are read by two or three kernels of the call; when they fit in L2 comfortably the
     // earlier readers ask L2 to keep them and the last reader releases them.
     const int l2 = (nseg > 1 && tokens * a.H * (uint64_t)(a.d_k + a.d_v) * 2 <= (96ull << 20)) ? (g_lean_l2_hints & 3) : 0;
-    PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, nslots, a.B, a.T, a.H, opt.gate_scale, opt.eps, ticket, l2};
+    PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, nslots, a.B, a.T, a.H, opt.gate_scale, opt.eps, ticket, l2,
+                  g_lean_drop_chunk == -3 ? 32784u : 32768u};
     // Items without -W^T (24 % less memory traffic over both kernels, one hop more per chain step) are for calls of one segment
     // per chain and equal lengths.  A plain or raw call takes them when its chains together are bound by memory: at least three
     // fifths of the SMs busy to the end, every chain reading its own K and Q (with d_v = 256 two chains share them through
@@ -2402,7 +2420,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
         return GDN_ERR_CUDA;
     const long nitems = (long)nslots * a.H;
     const long cap = 4L * sms_of_device[dev];
-    PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, (long)nslots, a.B, a.T, a.H, 1.f, 0.f, static_cast<int*>(ticket_of_device[dev])};
+    PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, (long)nslots, a.B, a.T, a.H, 1.f, 0.f, static_cast<int*>(ticket_of_device[dev]), 0, 32768u};
     gdn_prep_kernel<false, false><<<(int)(nitems < cap ? nitems : cap), PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;

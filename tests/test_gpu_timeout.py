@@ -76,3 +76,47 @@ def test_expired_counter_wait_in_the_merged_kernel_is_reported_and_the_context_s
     o_ref, f_ref = run_oracle(x)
     assert_close(f64(d["out"]), o_ref, BF16_REL_L2, BF16_MAX_ABS, "out after a timed-out merged call")
     assert_close(f64(d["final_state"]), f_ref, BF16_REL_L2, BF16_MAX_ABS, "state after a timed-out merged call")
+
+
+@pytest.mark.parametrize("raw,compact", [(False, 0), (False, 1), (True, 0)])
+def test_expired_wait_in_the_prepare_kernel_is_reported_and_the_context_survives(raw, compact):
+    """Every CTA expects more bytes than its tiles have: the wait on its first item's runs out, the item is gone through all the
+    same, and the roles of the CTA leave their loop together."""
+    cfg = get_config("short", B=1, T=64 * 100, H=16, raw=raw, seed=97)     # more items than CTAs
+    x = make_inputs(cfg)
+    d = to_device(x)
+    L = gdn.lib()
+    ws = torch.zeros(gdn.gdn_workspace_bytes(cfg.B, cfg.T, cfg.H, cfg.d_k, cfg.d_v, False), dtype=torch.uint8, device="cuda")
+    args = (d["q"], d["k"], d["v"], d["log_alpha"], d["beta"])
+
+    def call():
+        if raw:
+            gdn.gdn_chunk_prefill_raw(*args, cfg.gate_scale, 1e-6, None, d["out"], d["final_state"])
+        else:
+            gdn.gdn_chunk_prefill(*args, None, d["out"], d["final_state"])
+
+    gdn.gdn_set_workspace(ws)
+    L.gdn_debug_force_path(2)
+    L.gdn_debug_force_segments(1)
+    L.gdn_debug_set_compact(compact)
+    try:
+        call()
+        assert gdn.gdn_query_status() == 0
+        want = d["out"].clone(), d["final_state"].clone()
+        L.gdn_debug_drop_chunk(-3)
+        call()
+        assert gdn.gdn_query_status() == 5           # GDN_ERR_TIMEOUT; the kernels returned on their own
+        L.gdn_debug_drop_chunk(-1)
+        assert L.gdn_debug_reset_status() == 0
+        torch.cuda.synchronize()                     # no sticky CUDA error
+        gdn.gdn_set_workspace(ws)                    # as the header asks for after a time-out
+        d["out"].zero_(); d["final_state"].zero_()
+        call()
+        assert gdn.gdn_query_status() == 0
+        assert torch.equal(d["out"], want[0]) and torch.equal(d["final_state"], want[1])
+    finally:
+        L.gdn_debug_drop_chunk(-1)
+        L.gdn_debug_set_compact(-1)
+        L.gdn_debug_force_segments(0)
+        L.gdn_debug_force_path(0)
+        gdn.gdn_set_workspace(None)
