@@ -1021,7 +1021,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         if (RELAY) {                                    // publish the piece; the last one leaves the counter at zero
             __threadfence();
             named_bar_sync(3, 256);
-            if (tid == 0) {
+            // (test hook: drop_chunk == -2 makes the first piece of the first chain keep its state to itself)
+            if (tid == 0 && !(p.drop_chunk == -2 && cta.z == 0 && h == 0 && dvb == 0)) {
                 __threadfence();
                 atomicExch(done(), seg == p.nseg - 1 ? 0 : seg + 1);
             }

@@ -120,3 +120,38 @@ def test_expired_wait_in_the_prepare_kernel_is_reported_and_the_context_survives
         L.gdn_debug_force_segments(0)
         L.gdn_debug_force_path(0)
         gdn.gdn_set_workspace(None)
+
+
+@pytest.mark.parametrize("compact", [0, 1])
+def test_expired_counter_wait_of_a_relayed_chain_is_reported_and_the_context_survives(compact):
+    """The first piece of one chain does not say that it is done: the piece behind it gives up after a second, reports the time-out
+    and runs to its end, so do the others, and the next call on the workspace, set again as the header asks, is correct."""
+    cfg = get_config("short", B=1, T=64 * 9 + 3, H=3, seed=98)
+    x = make_inputs(cfg)
+    d = to_device(x)
+    L = gdn.lib()
+    ws = torch.zeros(gdn.gdn_workspace_bytes(cfg.B, cfg.T, cfg.H, cfg.d_k, cfg.d_v, False), dtype=torch.uint8, device="cuda")
+    call = lambda: gdn.gdn_chunk_prefill(d["q"], d["k"], d["v"], d["log_alpha"], d["beta"], None, d["out"], d["final_state"])
+    gdn.gdn_set_workspace(ws)
+    L.gdn_debug_force_path(2)
+    L.gdn_debug_set_relay(3)
+    L.gdn_debug_set_compact(compact)
+    L.gdn_debug_drop_chunk(-2)
+    try:
+        call()
+        assert gdn.gdn_query_status() == 5
+        L.gdn_debug_drop_chunk(-1)
+        assert L.gdn_debug_reset_status() == 0
+        torch.cuda.synchronize()
+        gdn.gdn_set_workspace(ws)
+        call()
+        assert gdn.gdn_query_status() == 0
+    finally:
+        L.gdn_debug_drop_chunk(-1)
+        L.gdn_debug_set_compact(-1)
+        L.gdn_debug_set_relay(-1)
+        L.gdn_debug_force_path(0)
+        gdn.gdn_set_workspace(None)
+    o_ref, f_ref = run_oracle(x)
+    assert_close(f64(d["out"]), o_ref, BF16_REL_L2, BF16_MAX_ABS, "out after a timed-out relay")
+    assert_close(f64(d["final_state"]), f_ref, BF16_REL_L2, BF16_MAX_ABS, "state after a timed-out relay")
