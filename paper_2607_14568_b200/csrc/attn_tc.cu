@@ -213,8 +213,8 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t ts = tmem + lane_base + TM_S + X * 128, to = tmem + lane_base + TM_O + X * 128;
         const float c = p.scale_log2e;
-        uint32_t tiles = 0, outs = 0, kt0 = 0;             // of this warpgroup, over all items (barrier phases); the item's first key tile
-        for (int k = 0; fetch(k, it); ++k, kt0 += it.ntiles) {
+        uint32_t tiles = 0, outs = 0;                      // of this warpgroup, over all items (barrier phases)
+        for (int k = 0; fetch(k, it); ++k) {
             __syncwarp();
             if (lane == 0) mbar_arrive(w.bar(AB_QFREE));   // the slot has been read
             const int nX = X ? it.nB : it.nA, qt = p.per * it.t + (int)X;
@@ -259,18 +259,6 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     #pragma unroll
                         for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
                         tmem_st16(to + 16 * q4, o);
-                    }
-                }
-                // The last key tile is completed with the rows that follow the sequence in memory.  Their probabilities are zero, but
-                // zero times what is not finite is not zero: the value rows are cleared before P V of this tile, which waits for P.
-                if (j == qt && it.len - qt * BM < BM) {
-                    const uint32_t s = (kt0 + j) & 1;
-                    w.wait(AB_VFULL0 + s, ((kt0 + j) >> 1) & 1);
-                    if (r >= it.len - qt * BM) {
-#pragma unroll 1
-                        for (uint32_t x = 0; x < 16; ++x)
-                            *reinterpret_cast<uint4*>(sm + AS_V + s * TILE_BYTES + (x >> 3) * 16384 + r * 128 + (x & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
-                        fence_proxy_async_smem();
                     }
                 }
                 // P = 2^(c s - m) as bf16 over the first 64 columns of the scores it came from.  The first 64 keys are handed
@@ -372,7 +360,18 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     // the tiles are normally there long before the probabilities: these waits come first, so that
                     // nothing but the MMAs sits between "P ready" and "next scores ready"
                     w.wait(AB_VFULL0 + s, (kt >> 1) & 1);
-                    if (more) w.wait(AB_KFULL0 + s1, ((kt + 1) >> 1) & 1);
+                    if (more) {
+                        w.wait(AB_KFULL0 + s1, ((kt + 1) >> 1) & 1);
+                    } else if (it.ntiles * BN > it.len) {
+                        // The last key tile is completed with the rows that follow the sequence in memory.  Their probabilities are
+                        // zero, but zero times what is not finite is not zero: the value rows are cleared before P V of the tile
+                        // (by this warp, which has the time of a softmax for it; in the softmax it cost 0.7 % on every call)
+#pragma unroll 1
+                        for (int x = (it.len & (BN - 1)) * 16 + lane; x < BN * 16; x += 32)
+                            *reinterpret_cast<uint4*>(sm + AS_V + s * TILE_BYTES + ((x >> 3) & 1) * 16384 + (x >> 4) * 128 + (x & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                    }
                     if (j < it.nA) {
                         issue_pv(0, kt, pa++, j == 0);
                         if (j + 1 < it.nA) {
