@@ -54,7 +54,7 @@ constexpr uint32_t ATTN_SMEM = AS_TOTAL + 1024;
 
 enum ABar : uint32_t { AB_Q = 0, AB_KFULL0 = 1, AB_KFREE0 = 3, AB_VFULL0 = 5, AB_VFREE0 = 7, AB_SFULL0 = 9 /* A, B */,
                        AB_PFULL0 = 11 /* A, B: first 64 keys */, AB_PVDONE0 = 13 /* A, B */, AB_PFULL1 = 15 /* A, B: other 64 */,
-                       AB_QFREE = 17 /* Q tiles and item slot read */, AB_TAKEN = 18 };
+                       AB_QFREE = 17 /* Q tiles and item slot read */, AB_TAKEN = 18, AB_DRAIN = 19 };
 
 struct AWaiter {
     uint32_t bars;
@@ -129,7 +129,8 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         w.wait(AB_Q, k & 1);
         volatile uint32_t* m = sMisc + 4 + 4 * (k & 1);
         it.tok0 = (int)m[0]; it.len = (int)m[1]; it.t = (int)m[2]; it.h = (int)m[3];
-        if (it.t < 0 || *w.abort_flag) return false;
+        // (a whole warp leaves or none of its lanes: the flag may rise between two lanes' reads of it)
+        if (__any_sync(0xffffffffu, it.t < 0 || *w.abort_flag)) return false;
         shape(it);
         return true;
     };
@@ -185,7 +186,7 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if (warp == 9 && !p.cu) find(blockIdx.x, it);                   // the first one under the setup
 
     if (tid == 0) {
-        mbar_init(w.bar(AB_Q), 1); mbar_init(w.bar(AB_TAKEN), 1);
+        mbar_init(w.bar(AB_Q), 1); mbar_init(w.bar(AB_TAKEN), 1); mbar_init(w.bar(AB_DRAIN), 1);
         mbar_init(w.bar(AB_QFREE), 9);                     // 8 softmax warps and the tensor core
         for (uint32_t s = 0; s < 2; ++s) {
             mbar_init(w.bar(AB_KFULL0 + s), 1); mbar_init(w.bar(AB_KFREE0 + s), 1);
@@ -392,6 +393,11 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (more && lead) mma_commit(w.bar(AB_KFREE0 + s1));
                     if (j + 2 == it.ntiles && lead) mma_commit(w.bar(AB_QFREE));      // the last Q K^T of the item is issued
                 }
+            }
+            if (__any_sync(0xffffffffu, *w.abort_flag != 0)) {     // nobody may be waiting for the products in flight: they end first (bounded)
+                if (lead) mma_commit(w.bar(AB_DRAIN));
+#pragma unroll 1
+                for (int i = 0; i < 1024 && !mbar_try_wait_suspend(w.bar(AB_DRAIN), 0, 1000000u); ++i) {}
             }
         }
     } else {
