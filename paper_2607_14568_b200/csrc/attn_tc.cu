@@ -505,7 +505,7 @@ int attn_query_status() {
 int launch_attn(const void* q, const void* k, const void* v, void* out, const int32_t* cu_seqlens, int B, int T,
                 int Hq, int Hkv, int d, float scale, cudaStream_t stream) {
     if (!attn_supported(Hq, Hkv, d)) return GDN_ERR_UNSUPPORTED;
-    if (B > 65535 || T / (2 * BM) + B + 1 > 65535) return GDN_ERR_UNSUPPORTED;
+    if (B > 65535 || T / (2 * BM) + B + 1 > 65535) return GDN_ERR_UNSUPPORTED;      // (the range accepted; the grid below would take more)
     if (B == 0 || T == 0) return GDN_OK;
     const uint64_t tokens = cu_seqlens ? (uint64_t)T : (uint64_t)B * T;
     if (tokens > 0x7fffffffull) return GDN_ERR_TOO_LARGE;

@@ -55,7 +55,7 @@ static bool g_lean_use_scan = false;       // true = summary, combination and ch
                                            // the 10240-token workload, 0.074 vs 0.060 ms at 2048 tokens, so it is off by default)
 static bool g_lean_scan_last = false;
 static int g_lean_relay = -1;              // tests: pieces per chain (0 = never, -1 = by the rule)
-static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size (-1 = by the rule)
+static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size, without a split (-1 = by the rule)
 
 namespace {
 
@@ -169,7 +169,6 @@ __device__ __forceinline__ void bulk_store_hint(void* gdst, uint32_t smem_src, u
                  ::"l"(reinterpret_cast<uint64_t>(gdst)), "r"(smem_src), "r"(bytes), "l"(pol) : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
@@ -1445,8 +1444,7 @@ __device__ __forceinline__ uint32_t sum_ds(int inst) { return inst ? 288u : 64u;
 __device__ __forceinline__ uint32_t sum_vt(int inst) { return inst ? 416u : 192u; }   // bf16 decayed v_new^T
 constexpr uint32_t SUM_COLS = 512;
 
-enum SBar : uint32_t { SB_FULL0 = 0, SB_FREE0 = 3, SB_V0 = 6, SB_S0 = 8, SB_SREADY0 = 10, SB_VREADY0 = 12,
-                       SB_X0 = 14, SB_YREADY0 = 16 };
+enum SBar : uint32_t { SB_FULL0 = 0, SB_FREE0 = 3, SB_V0 = 6, SB_S0 = 8, SB_SREADY0 = 10, SB_VREADY0 = 12 };
 
 struct SummaryParams {
     const int32_t* cu;
@@ -1466,12 +1464,11 @@ __device__ __forceinline__ void summary_init_bars(const Waiter& w, int ninst) {
     for (uint32_t i = 0; i < 2; ++i) {
         mbar_init(w.bar(SB_V0 + i), 1); mbar_init(w.bar(SB_S0 + i), 1);
         mbar_init(w.bar(SB_SREADY0 + i), 128); mbar_init(w.bar(SB_VREADY0 + i), 128);
-        mbar_init(w.bar(SB_X0 + i), 1); mbar_init(w.bar(SB_YREADY0 + i), 128);
     }
 }
 
-// Segment summary (M_seg, N_seg) of one CTA; cta.z = sequence * (nseg - 1) + segment.  COMPACT: as in chain_body.
-template <bool SCAN, bool COMPACT>
+// Segment summary (M_seg, N_seg) of one CTA; cta.z = sequence * (nseg - 1) + segment.
+template <bool SCAN>
 __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUtensorMap* map_v, const SummaryParams& p,
                                              const Cta& cta, const Waiter& w) {
     constexpr int CW = SCAN ? 12 : 8;                 // first warp of the control warpgroup
@@ -1516,29 +1513,6 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
             for (int c = 0; c < nchunks; ++c) {
                 const uint32_t s = c % SUM_STAGES;
                 const float* gates = reinterpret_cast<const float*>(sm + s * SUM_STAGE + SS_GATES);
-                if (COMPACT) {
-                    // Y^T = -e^g (S^T K^T): accumulator in the upper columns of dS^T, bf16 in the place of the decayed v_new
-                    w.wait_hot(SB_X0 + inst, c & 1);
-                    tc_fence_after_sync();
-                    uint32_t x[2][32];
-                    tmem_ld32(tmem + lane_base + sum_ds(inst) + 64, x[0]);
-                    tmem_wait_ld();
-                    tmem_ld32(tmem + lane_base + sum_ds(inst) + 96, x[1]);
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const float2 eg = *reinterpret_cast<const float2*>(gates + 32 * hh + 2 * i);
-                            pk[i] = pack_bf16(-eg.x * __uint_as_float(x[hh][2 * i]), -eg.y * __uint_as_float(x[hh][2 * i + 1]));
-                        }
-                        tmem_st16(tmem + lane_base + sum_vt(inst) + 16 * hh, pk);
-                        if (hh == 0) tmem_wait_ld();
-                    }
-                    tmem_wait_st();
-                    tc_fence_before_sync();
-                    mbar_arrive(w.bar(SB_YREADY0 + inst));
-                }
                 w.wait_hot(SB_V0 + inst, c & 1);
                 tc_fence_after_sync();
 #pragma unroll
@@ -1627,24 +1601,10 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                     }
                     w.wait_hot(SB_SREADY0 + inst, c & 1);
                     tc_fence_after_sync();
-                    if (COMPACT) {
-                        const uint64_t dKk = make_smem_desc(sb + SS_K, 16, 1024), dT = make_smem_desc(sb + SS_T2, 1024, 1024);
 #pragma unroll
-                        for (uint32_t ks = 0; ks < 8; ++ks)        // X^T = S^T K^T
-                            if (lead) mma_ts(tmem + sum_ds(inst) + 64, tmem + sum_ds(inst) + ks * 8,
-                                   dKk + (uint64_t)(((ks >> 2) * 8192 + (ks & 3) * 32) >> 4), ID_O, ks > 0);
-                        if (lead) mma_commit(w.bar(SB_X0 + inst));
-                        w.wait_hot(SB_YREADY0 + inst, c & 1);
-                        tc_fence_after_sync();
-#pragma unroll
-                        for (uint32_t ks = 0; ks < 4; ++ks)        // v^T = U^T + Y^T (T diag(b))^T
-                            if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_vt(inst) + ks * 8, dT + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
-                    } else {
-#pragma unroll
-                        for (uint32_t ks = 0; ks < 8; ++ks)        // v^T = U^T - S^T W^T   (U = 0 for the identity chain)
-                            if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_ds(inst) + ks * 8,
-                                   dW + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
-                    }
+                    for (uint32_t ks = 0; ks < 8; ++ks)            // v^T = U^T - S^T W^T   (U = 0 for the identity chain)
+                        if (lead) mma_ts(tmem + sum_dv(inst), tmem + sum_ds(inst) + ks * 8,
+                               dW + ks * 128, ID_1, (inst == 0 || ks > 0) ? 1u : 0u);
                     if (lead) mma_commit(w.bar(SB_V0 + inst));
                     w.wait_hot(SB_VREADY0 + inst, c & 1);
                     tc_fence_after_sync();
@@ -1667,12 +1627,12 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                 const uint32_t full = w.bar(SB_FULL0 + s);
                 const int tok = (int)(tok0 + (long)c * C);
                 const uint8_t* item = p.items + (size_t)((slot0 + c) * H + h) * ITEM_BYTES;
-                mbar_arrive_expect_tx(full, COMPACT ? SUM_STAGE_TX - 16384 : SUM_STAGE_TX);
+                mbar_arrive_expect_tx(full, SUM_STAGE_TX);
                 tma_load_3d_hint(sb + SS_K, map_k, 0, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_K + 8192, map_k, 64, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_V, map_v, dvb * DVB, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_V + 8192, map_v, dvb * DVB + 64, h, tok, full, pol_keep);
-                if (!COMPACT) bulk_load_hint(sb + SS_W, item + IT_W, 16384, full, pol_item);
+                bulk_load_hint(sb + SS_W, item + IT_W, 16384, full, pol_item);
                 bulk_load_hint(sb + SS_T2, item + IT_T2, 8192, full, pol_item);
                 bulk_load(sb + SS_GATES, item + IT_GATES, 1280, full);
             }
@@ -1687,7 +1647,6 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     }
 }
 
-template <bool COMPACT>
 __global__ void __launch_bounds__(SUM_THREADS, 1)
 gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    SummaryParams p) {
@@ -1713,7 +1672,7 @@ gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     pdl_trigger();
     pdl_wait();                         // the scratch items come from the prepare kernel
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
-    summary_body<false, COMPACT>(&map_k, &map_v, p, cta, w);
+    summary_body<false>(&map_k, &map_v, p, cta, w);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1991,7 +1950,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // ---------------- phase 1: summary of this segment (the last segment needs none) ----------------
         if (seg < nseg - 1) {
             const Cta c1{base, sm, tmem, 0, h, n * (nseg - 1) + seg};
-            summary_body<true, false>(&map_k, &map_v, p.sp, c1, w1);
+            summary_body<true>(&map_k, &map_v, p.sp, c1, w1);
             __threadfence();
             tc_fence_before_sync();
             cta_sync();
@@ -2181,7 +2140,7 @@ static int device_setup(int* sms_out) {
             !smem_limit(GDN_K(gdn_chain_kernel<kPlain, true, true>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kRelay, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, false, true>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kRelay, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, true, true>), CHAIN_SMEM_GATED) ||
-            !smem_limit(GDN_K(gdn_summary_kernel<false>), SUM_SMEM) || !smem_limit(GDN_K(gdn_summary_kernel<true>), SUM_SMEM) ||
+            !smem_limit(GDN_K(gdn_summary_kernel), SUM_SMEM) ||
             !smem_limit(GDN_K(gdn_combine_kernel), CMB_SMEM) ||
             !smem_limit(GDN_K(gdn_scan_kernel<false>), SCAN_SMEM) || !smem_limit(GDN_K(gdn_scan_kernel<true>), SCAN_SMEM))
             return GDN_ERR_CUDA;
@@ -2258,9 +2217,9 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // the chain sets the step, which hides the hop, so there is no line: 64 tokens 1 to 24 chains 4 to 5 % less, 1500
     // tokens 1 chain 54.7 / 54.4 us, 16 58.9 / 59.4, 32 65.7 / 67.6, 56 72.0 / 73.7, 64 73.5 / 77.1, 96 87 / 94, 144 113 / 126; 4096 tokens
     // 32 155 / 158 us, 64 178 / 184, 128 271 / 288; 8192 tokens 48 319 / 329 us, 96 445 / 462.
-    const bool compact = !g_lean_dbg && !g_lean_use_scan &&
+    const bool compact = !g_lean_dbg && !g_lean_use_scan && nseg == 1 &&
                          (g_lean_compact >= 0 ? g_lean_compact == 1
-                                              : !packed && nseg == 1 && a.d_v == DVB && (opt.gate_z || (long)a.B * a.H * 5 >= 3L * num_sms));
+                                              : !packed && a.d_v == DVB && (opt.gate_z || (long)a.B * a.H * 5 >= 3L * num_sms));
     const int pgrid = (int)(nitems < 4L * num_sms ? nitems : 4L * num_sms);
     auto mark = [&](int i) { if (g_lean_timing && g_lean_events[i]) cudaEventRecord(g_lean_events[i], stream); };
     mark(0);
@@ -2297,7 +2256,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
             return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
         }
         dim3 sgrid(a.d_v / DVB, a.H, a.B * (nseg - 1));
-        launch_after(compact ? gdn_summary_kernel<true> : gdn_summary_kernel<false>, sgrid, SUM_THREADS, SUM_SMEM, stream, mk, mv, sp);
+        launch_after(gdn_summary_kernel, sgrid, SUM_THREADS, SUM_SMEM, stream, mk, mv, sp);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
         mark(2);

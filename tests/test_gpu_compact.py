@@ -1,6 +1,7 @@
 """The form of the chain that reads no W (scratch items of (T diag beta)^T, P and the gate vectors only; used for grids that
 are bound by memory) against the fp64 oracle, forced on small inputs: one chunk and less, ragged tails, more chunks than
-any ring has slots, packed neighbours, wide values, the sequence split, raw projections and the fused output stage."""
+any ring has slots, packed neighbours, wide values, raw projections and the fused output stage; a split (four or three segments)
+keeps its W whatever is asked for."""
 import numpy as np
 import pytest
 import torch
