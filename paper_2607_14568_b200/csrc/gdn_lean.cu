@@ -51,8 +51,8 @@ static int g_lean_l2_hints = 3;            // tests: bit 0 = L2 eviction-priorit
                                            // scratch images W and T2 (measured on the 10240-token workload, chain kernel:
                                            // 51.3 us without, 49.0 / 49.4 us with either, 47.2 us with both)
 static bool g_lean_use_scan = false;       // true = summary, combination and chain of a split run as one resident launch (measured
-                                           // slower than the three kernels under programmatic dependent launch: 0.162 vs 0.152 ms on
-                                           // the 10240-token workload, 0.074 vs 0.060 ms at 2048 tokens, so it is off by default)
+                                           // slower than the three kernels under programmatic dependent launch: 129 against 126 us on
+                                           // the 10240-token workload, 56 against 45 us at 2048 tokens, so it is off by default)
 static bool g_lean_scan_last = false;
 static int g_lean_relay = -1;              // tests: pieces per chain (0 = never, -1 = by the rule)
 static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size, without a split (-1 = by the rule)
@@ -852,6 +852,8 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 
 // Steps c and d for one CTA.  SCAN: called from the merged scan kernel (register budgets are set there, the
 // incoming state is awaited through `hv` and read past the L1 cache, since another SM wrote it in this launch).
+// There the warp index stays a plain shift of the thread index, so that each warpgroup's copy of the phases reduces to its role:
+// behind the shuffle of warp_uniform every copy held all roles and spilled 5.4 KB.
 //
 // COMPACT: v_new = T diag(b) (V - diag(e^g) K S) instead of U - W S: S^T K^T, a conversion that applies -e^g, and a product
 // with (T diag(b))^T onto U^T.  One hop more per step (about 0.25 us), but 16 KB less to write and to read
@@ -868,7 +870,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     constexpr int CW = 8 + 4 * NOUT;                         // first warp of the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
-    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
+    const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
     if (tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
     const int n = cta.z / p.nseg, seg = cta.z % p.nseg;
@@ -1474,7 +1476,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     constexpr int CW = SCAN ? 12 : 8;                 // first warp of the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
-    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
+    const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
     const int nsum = p.nseg - 1;                      // the last segment needs no summary
     const int n = cta.z / nsum, seg = cta.z % nsum;
@@ -1723,7 +1725,7 @@ __device__ __forceinline__ void combine_init_bars(const Waiter& w) {
 template <bool SCAN>
 __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& cta, const Waiter& w, int issue_warp) {
     const uint32_t base = cta.base, tmem = cta.tmem;
-    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
+    const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int j0 = cta.dvb * CMB_COLS, h = cta.h, n = cta.z;
     const int H = p.H, dv = p.dv, nhops = p.nseg - 1;
     auto seg_off = [&](int seg) { return ((size_t)(n * p.nseg + seg) * H + h) * DK * dv; };
@@ -1945,7 +1947,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     // behind that role's register budget, so the phase bodies (which branch on the warp index themselves)
     // reduce to the one role; CTA-wide synchronisation therefore uses a named barrier, not __syncthreads.
     auto cta_sync = [&]() { named_bar_sync(4, SCAN_THREADS); };
-    auto phases = [&]() {
+    auto split_phases = [&]() {
         stamp(0);
         // ---------------- phase 1: summary of this segment (the last segment needs none) ----------------
         if (seg < nseg - 1) {
@@ -1985,6 +1987,8 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (tid == 0) { __threadfence(); atomicAdd(fl + 1, 1); }
         }
         stamp(3);
+    };
+    auto chain_phase = [&]() {
         // ---------------- phase 3: chain over this segment's chunks ----------------
         const Cta c3{base, sm, tmem, 0, h, (int)blockIdx.z};
         chain_body<DBG ? kStamps : kPlain, true, false, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
@@ -1992,12 +1996,13 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         tc_fence_before_sync();
         cta_sync();
     };
-    // register budgets: warpgroups 0 and 1 hold the fp32 states (a 128-value row per thread in the summary phase), warpgroup
-    // 2 writes the outputs, warpgroup 3 issues and copies
-    if (warp < 4) { setmaxnreg_inc<184>(); phases(); }
-    else if (warp < 8) { setmaxnreg_inc<184>(); phases(); }
-    else if (warp < 12) { setmaxnreg_dec<88>(); phases(); }
-    else { setmaxnreg_dec<56>(); phases(); }
+    // Register budgets (the shares add up to the 4 x 128 of the launch in both halves).  Summary and hops: warpgroups 0 and 1 hold a
+    // 128-value row of the state per thread, warpgroup 2 has nothing to do, warpgroup 3 issues and copies.  Chain: warpgroups 0 and 1
+    // hold half a row each, warpgroup 2 writes the outputs.  (Whoever gives registers up waits for nobody in between, so
+    // the increases cannot block for good.)
+    if (warp < 8) { setmaxnreg_inc<216>(); split_phases(); setmaxnreg_dec<160>(); chain_phase(); }
+    else if (warp < 12) { setmaxnreg_dec<40>(); split_phases(); setmaxnreg_inc<136>(); chain_phase(); }
+    else { setmaxnreg_dec<40>(); split_phases(); setmaxnreg_inc<56>(); chain_phase(); }
     if (tid == 0) {                     // the last CTA of this head to get here clears the counters
         __threadfence();
         if (atomicAdd(fl + 2, 1) == nseg - 1) {
