@@ -1987,6 +1987,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (tid == 0) { __threadfence(); atomicAdd(fl + 1, 1); }
         }
         stamp(3);
+        cta_sync();         // every warp has its budget of these phases before any asks for its next one, see below
     };
     auto chain_phase = [&]() {
         // ---------------- phase 3: chain over this segment's chunks ----------------
@@ -1998,8 +1999,10 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     };
     // Register budgets (the shares add up to the 4 x 128 of the launch in both halves).  Summary and hops: warpgroups 0 and 1 hold a
     // 128-value row of the state per thread, warpgroup 2 has nothing to do, warpgroup 3 issues and copies.  Chain: warpgroups 0 and 1
-    // hold half a row each, warpgroup 2 writes the outputs.  (Whoever gives registers up waits for nobody in between, so
-    // the increases cannot block for good.)
+    // hold half a row each, warpgroup 2 writes the outputs.  The barrier at the end of the first half stands between the two
+    // requests of every warp: without it (a CTA with neither a summary nor a slice passes no other one) warpgroup 2 could take
+    // its second share before warpgroups 0 and 1 had their first, which then would never come.  Behind it warpgroups 0 and 1 give up
+    // theirs without waiting for anybody, so the increases of the others are served.
     if (warp < 8) { setmaxnreg_inc<216>(); split_phases(); setmaxnreg_dec<160>(); chain_phase(); }
     else if (warp < 12) { setmaxnreg_dec<40>(); split_phases(); setmaxnreg_inc<136>(); chain_phase(); }
     else { setmaxnreg_dec<40>(); split_phases(); setmaxnreg_inc<56>(); chain_phase(); }
