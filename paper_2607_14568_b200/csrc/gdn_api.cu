@@ -123,13 +123,20 @@ struct HostPipe {
         return true;
     }
 };
-HostPipe g_host_pipe;
+// One per device (streams and events belong to one), and one call enqueues at a time: the calls share the events, and a wait
+// takes the record made last before it.
+HostPipe g_host_pipe_of_device[kMaxDevices];
+std::mutex g_host_pipe_mutex;
 
 int host_pipelined(const void* q_host, const void* k_host, const void* v_host, const float* a_host, const float* b_host,
                    const float* s0_host, void* out_host, float* sT_host, int T, int H, int d_k, int d_v, char* base,
                    const Staging& L, cudaStream_t stream) {
     const int npieces = (T + kHostPiece - 1) / kHostPiece;
-    HostPipe& hp = g_host_pipe;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return GDN_ERR_CUDA;
+    if (dev < 0 || dev >= kMaxDevices) return GDN_ERR_UNSUPPORTED;
+    std::lock_guard<std::mutex> lock(g_host_pipe_mutex);
+    HostPipe& hp = g_host_pipe_of_device[dev];
     if (!hp.ensure(2 * (size_t)npieces + 2)) return GDN_ERR_CUDA;
     auto ok = [](cudaError_t e) { return e == cudaSuccess; };
     cudaEvent_t ev_start = hp.ev[0], ev_done = hp.ev[1];
