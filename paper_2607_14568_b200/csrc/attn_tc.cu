@@ -367,9 +367,11 @@ attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         // The last key tile is completed with the rows that follow the sequence in memory.  Their probabilities are
                         // zero, but zero times what is not finite is not zero: the value rows are cleared before P V of the tile
                         // (by this warp, which has the time of a softmax for it; in the softmax it cost 0.7 % on every call)
-#pragma unroll 1
-                        for (int x = (it.len & (BN - 1)) * 16 + lane; x < BN * 16; x += 32)
-                            *reinterpret_cast<uint4*>(sm + AS_V + s * TILE_BYTES + ((x >> 3) & 1) * 16384 + (x >> 4) * 128 + (x & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        uint32_t row = (uint32_t)(it.len & (BN - 1)) + (lane >> 4);       // two rows of 256 bytes at a time
+                        uint32_t dst = base + AS_V + s * TILE_BYTES + ((lane >> 3) & 1) * 16384 + row * 128 + (lane & 7) * 16;
+#pragma unroll 4
+                        for (; row < BN; row += 2, dst += 256)
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0u) : "memory");
                         fence_proxy_async_smem();
                         __syncwarp();
                     }
