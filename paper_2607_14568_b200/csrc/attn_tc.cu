@@ -98,8 +98,9 @@ constexpr uint32_t ID_PV = make_idesc(128, 128, kFmtBF16, kFmtBF16, kMajorK, kMa
 // CTA that has not started (which then never does), so every SM goes on to the longest item that is left, and the copies,
 // first Q K^T and softmax of the next item run under the last softmax and the output of the current one; started as a
 // CTA, each item left 5 us open.  16 heads: 6000 tokens 136 -> 124 us, 10240 tokens 400 -> 383 us at the power limit,
-// packed 1711 + 402 + 2048 + 65 + 977 tokens 54 -> 43 us, eight packed prompts of 33 to 3000 tokens 84 -> 66 us.  (One CTA per SM and
-// the items dealt out back and forth in advance: 126, 383, 47, 75 us.)
+// packed 1711 + 402 + 2048 + 65 + 977 tokens 54 -> 43 us, eight packed prompts of 33 to 3000 tokens 84 -> 66 us (short runs; in a long
+// alternation of builds the first packed case takes 50 us, 10240 tokens 390).  (One CTA per SM and the items dealt out back and forth in
+// advance: 126, 383, 47, 75 us.)
 // The copy warp looks the items up and publishes them in shared memory (item k in slot k & 1, barrier AB_Q; t < 0 is the
 // end); a slot and the Q tiles are free again when the softmax warps have read the one and the tensor core the others
 // (AB_QFREE).
