@@ -413,6 +413,7 @@ int gdn_debug_get_timing(float* ms5) { return ms5 ? lean_get_timing(ms5) : GDN_E
 void gdn_debug_force_segments(int nseg) { lean_force_segments(nseg); }
 void gdn_debug_set_relay(int pieces) { lean_set_relay(pieces); }
 void gdn_debug_set_compact(int mode) { lean_set_compact(mode); }
+void gdn_debug_set_pair(int mode) { lean_set_pair(mode); }
 void gdn_debug_set_scan(int enable) { lean_set_scan(enable); }
 void gdn_debug_set_l2_hints(int enable) { lean_set_l2_hints(enable); }
 

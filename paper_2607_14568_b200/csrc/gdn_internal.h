@@ -42,7 +42,7 @@ int attn_status_async(int* host_dst, cudaStream_t stream);
 void tc_set_debug_dump(float* p);    // tests only: stage dump of chunk 0 of CTA (0,0,0)
 
 // [tokens, H, d] bf16 tensor map, box = 64 tokens x 1 head x 64 features, 128-byte swizzle
-bool tc_make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d);
+bool tc_make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d, uint32_t rows = 64);
 
 // Two-kernel pipeline (prepare on all SMs, then the chain) using caller-provided scratch.
 size_t lean_workspace_bytes(int B, int T, int H, int d_k, int d_v, bool packed);
@@ -70,6 +70,7 @@ int lean_set_timing(int enable);      // benchmark only: record events around ea
 int lean_get_timing(float* ms5);      // {prepare, summary, combine, chain, scan} of the last call
 void lean_set_l2_hints(int enable);   // tests only: 0 = no L2 eviction-priority hints
 void lean_set_relay(int pieces);      // tests only: pieces per chain (0 = never, -1 = by the rule)
+void lean_set_pair(int mode);         // tests only: 0 / 1 = fused output stage of a chain on one CTA / on two, -1 = by the rule
 void lean_set_compact(int mode);      // tests only: 0 / 1 = scratch items with / without W, -1 = by the rule
 void lean_set_scan(int enable);       // tests only: 0 = never merge summary, combine and chain into one launch
 

@@ -55,6 +55,7 @@ static bool g_lean_use_scan = false;       // true = summary, combination and ch
                                            // the 10240-token workload, 56 against 45 us at 2048 tokens, so it is off by default)
 static bool g_lean_scan_last = false;
 static int g_lean_relay = -1;              // tests: pieces per chain (0 = never, -1 = by the rule)
+static int g_lean_pair = -1;               // tests: 0 / 1 = the fused output stage of a chain on one CTA / on two (-1 = by the rule)
 static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size, without a split (-1 = by the rule)
 
 namespace {
@@ -172,11 +173,14 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// z / (1 + e^-z) with the hardware reciprocal (one unit in the last place; 0 for e^-z = inf)
-__device__ __forceinline__ float silu(float z) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + ex2(z * -LOG2E)));
-    return z * r;
+// weight * z / (1 + e^-z) of two bf16 values (low, high half), with the hardware reciprocal (one unit in the last place; 0 for e^-z = inf)
+__device__ __forceinline__ float2 weighted_silu2(uint32_t zz, float w) {
+    const float2 z = as_float2(zz << 16, zz & 0xffff0000u), t = mul2(z, make_float2(-LOG2E, -LOG2E));
+    const float2 d = add2(make_float2(ex2(t.x), ex2(t.y)), make_float2(1.f, 1.f));
+    float2 r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(d.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(d.y));
+    return mul2(make_float2(w, w), mul2(z, r));
 }
 
 // slot of chunk 0 of sequence n: disjoint ranges for any lengths, total <= tokens/64 + B
@@ -227,6 +231,7 @@ constexpr uint32_t ID_G = make_idesc(128, 64, kFmtBF16, kFmtBF16, kMajorK, kMajo
 constexpr uint32_t ID_WU = make_idesc(128, 64, kFmtBF16, kFmtBF16, kMajorMN, kMajorMN);
 constexpr uint32_t ID_1 = make_idesc(128, 64, kFmtBF16, kFmtBF16, kMajorK, kMajorMN);
 constexpr uint32_t ID_O = make_idesc(128, 64, kFmtBF16, kFmtBF16, kMajorK, kMajorK);
+constexpr uint32_t ID_OH = make_idesc(128, 32, kFmtBF16, kFmtBF16, kMajorK, kMajorK);
 constexpr uint32_t ID_2 = make_idesc(128, 128, kFmtBF16, kFmtBF16, kMajorK, kMajorMN);
 
 // item -> (head, first token, valid rows); false for a slot no sequence uses
@@ -723,7 +728,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // chain kernel (steps c and d)
 // =====================================================================================
 constexpr int CHAIN_THREADS = 512;          // two chain warpgroups, output warpgroup, control warpgroup
-constexpr int CHAIN_THREADS_GATED = 640;    // two output warpgroups, 32 tokens each
+constexpr int CHAIN_THREADS_GATED = 768;    // two output warpgroups and one that forms the gates
 // tensor memory columns
 constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384,
                    TM_OG = 448;   // fused output stage: norm_w * silu(gate_z) of the chunk, fp32
@@ -748,17 +753,21 @@ constexpr uint32_t GATE_SLOTS = 6;
 constexpr uint32_t CS_OST = CS_B + 2 * STAGE_B;        // two output tiles [2 halves of the columns][64 tokens][64], 128-byte swizzle
 constexpr uint32_t CS_GATES = CS_OST + 2 * 16384;
 constexpr uint32_t CS_BARS = (CS_GATES + GATE_SLOTS * 1280 + 1023) / 1024 * 1024;
-constexpr uint32_t CS_MISC = CS_BARS + 32 * 8;
+constexpr uint32_t CS_MISC = CS_BARS + 42 * 8;
 constexpr uint32_t CS_TOTAL = CS_MISC + 64;
 constexpr uint32_t CHAIN_SMEM = CS_TOTAL + 1024;
-// fused output stage only: the gate_z tile of a chunk, the partial row sums of two chunks, the inverse norms of each warp
-constexpr uint32_t CS_Z = (CS_TOTAL + 1023) / 1024 * 1024, CS_RED = CS_Z + 16384, CS_INV = CS_RED + 2 * 4 * 64 * 4;
-constexpr uint32_t CHAIN_SMEM_GATED = CS_INV + 4 * 64 * 4 + 1024;
+// fused output stage only, tiles of 32 tokens [2 halves of the columns][32][64]: an output tile per output warpgroup in the place of the
+// first output tile above; gate_z of two chunks, one in the place of the second output tile; the partial row sums of two chunks and the
+// inverse norms per output warpgroup
+constexpr uint32_t CS_Z = (CS_TOTAL + 1023) / 1024 * 1024, CS_Z1 = CS_OST + 16384, CS_RED = CS_Z + 16384, CS_INV = CS_RED + 2 * 2 * 4 * 32 * 4;
+constexpr uint32_t CHAIN_SMEM_GATED = CS_INV + 2 * 4 * 32 * 4 + 1024;
 static_assert(CS_OST % 1024 == 0 && CHAIN_SMEM_GATED <= 232448, "shared memory per CTA");
 
 enum CBar : uint32_t { CB_FULLW0 = 0, CB_FREEW0 = 2, CB_FULLQ0 = 4, CB_FREEQ0 = 6, CB_FULLK0 = 8, CB_FREEK0 = 10, CB_FULLP0 = 12, CB_FREEP0 = 14,
-                       CB_FULLB0 = 16, CB_FREEB0 = 18, CB_ZFULL = 20, CB_ZFREE, CB_V, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE, CB_U, CB_O1, CB_CLEAN, CB_VPLAIN };
-static_assert(CB_VPLAIN < 32, "barrier area");
+                       CB_FULLB0 = 16, CB_FREEB0 = 18, CB_V = 20, CB_S, CB_O, CB_SREADY, CB_VREADY, CB_OFREE0, CB_OFREE1, CB_U, CB_O1, CB_CLEAN, CB_VPLAIN,
+                       CB_ZFULL0, CB_ZFULL1, CB_ZFREE0, CB_ZFREE1, CB_GFULL0, CB_GFULL1, CB_GFREE0, CB_GFREE1,      // fused output stage
+                       CB_OH0, CB_OH1 };                                                                            // ... of a pair
+static_assert(CB_OH1 < 42, "barrier area");
 // COMPACT chains read no -W^T: K has a third slot in its place (it is used from the first to the last MMA of a step), and
 // the barriers of the -W^T ring serve that slot and the extra hand-over.
 enum CBarCompact : uint32_t { CB_FULLK2 = CB_FULLW0, CB_X = CB_FULLW0 + 1, CB_FREEK2 = CB_FREEW0, CB_YREADY = CB_FREEW0 + 1 };
@@ -806,6 +815,7 @@ struct Cta {
     uint8_t* sm;
     uint32_t tmem;
     int dvb, h, z;
+    int half;                 // of a pair: which 32 tokens of every chunk this CTA writes
 };
 // Grid-level hand-over inside the merged scan kernel: `flag` is a counter in global memory that the CTAs of one
 // (sequence, head) raise when their part of a phase is written; a consumer waits (bounded) until it reads
@@ -837,13 +847,29 @@ __device__ __forceinline__ bool handover_wait(const Handover& hv, volatile int* 
     return true;
 }
 
-__device__ __forceinline__ void chain_init_bars(const Waiter& w, int out_threads, bool compact) {
+// What the fused output stage adds to the chain kernel.  kGate: two output warpgroups, each with 32 of the 64 tokens of every chunk, and a
+// warpgroup that forms the gates.  The stage is then bound by the SM: 7300 warp instructions a chunk against 3350 without it, 54 % of
+// all issue slots and, with the special-function unit, 1.6 us a chunk (2.05 us when the output warpgroups formed the gates as well).
+// kGatePair: a cluster of two CTAs runs the same chain twice, with no word between them but the barrier that keeps the final state from
+// overwriting an initial state in the same array, and each writes 32 tokens of every chunk.  The output warpgroups take turns there, a
+// chunk each, with accumulators and gates of their own, so that the chain sets the step again: 1.2 us.
+enum GateMode : int { kNoGate = 0, kGate = 1, kGatePair = 2 };
+
+__device__ __forceinline__ void chain_init_bars(const Waiter& w, int gate, bool compact) {
     for (uint32_t i = CB_FULLW0; i < CB_V; ++i)
-        mbar_init(w.bar(i), i == CB_ZFREE ? out_threads : (compact && i == CB_YREADY) ? 256 : 1);
+        mbar_init(w.bar(i), (compact && i == CB_YREADY) ? 256 : 1);
     mbar_init(w.bar(CB_U), 1); mbar_init(w.bar(CB_O1), 1);
     mbar_init(w.bar(CB_V), 1); mbar_init(w.bar(CB_S), 1); mbar_init(w.bar(CB_O), 1);
-    mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256); mbar_init(w.bar(CB_OFREE), out_threads);
+    mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256);
     mbar_init(w.bar(CB_CLEAN), 128);
+    const uint32_t readers = gate == kGate ? 256 : 128;          // of one accumulator
+    for (uint32_t i = 0; i < 2; ++i) mbar_init(w.bar(CB_OFREE0 + i), readers);
+    if (gate != kNoGate)
+        for (uint32_t i = 0; i < 2; ++i) {
+            mbar_init(w.bar(CB_ZFULL0 + i), 1); mbar_init(w.bar(CB_ZFREE0 + i), 128);
+            mbar_init(w.bar(CB_GFULL0 + i), 128); mbar_init(w.bar(CB_GFREE0 + i), readers);
+            mbar_init(w.bar(CB_OH0 + i), 1);
+        }
 }
 
 // fragment loads and stores by the number of registers
@@ -862,12 +888,13 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 // MODE: what only a debug build (time stamps) or a relay needs stays out of the plain kernel: as run-time branches the relay cost
 // the other calls 1 to 2 %.
 enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2 };
-template <int MODE, bool SCAN, bool GATED, bool COMPACT>
+template <int MODE, bool SCAN, int GATE, bool COMPACT>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
     constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay;
-    constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments of each
-    constexpr int CW = 8 + 4 * NOUT;                         // first warp of the control warpgroup
+    constexpr bool GATED = GATE != kNoGate, PAIR = GATE == kGatePair;
+    constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments that each handles at a time
+    constexpr int OW = 8 + 4 * NOUT, CW = GATED ? OW + 4 : OW;  // warps behind the output warpgroups: the gate warpgroup, the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
@@ -934,6 +961,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             tc_fence_before_sync();
             mbar_arrive(w.bar(CB_SREADY));
         }
+        if (PAIR) cluster_arrive();                     // the incoming state has been read: it may be the array the final state goes to
         for (int c = 0; c < nchunks; ++c) {
             const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
             if (COMPACT) {
@@ -984,7 +1012,23 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             tc_fence_after_sync();
             if (tid == 0) stamp(0, c, 2);
             const float gamma = gates[256];
-            {
+            if (GATED) {
+                // (fewer registers: 16 columns at a time, the second load in flight over half of the first)
+                uint32_t d[2][32];
+                tmem_ld32(t_ds, d[0]);
+                tmem_wait_ld();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t pk[8];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) S[16 * q + i] = fmaf(gamma, S[16 * q + i], __uint_as_float(d[q >> 1][16 * (q & 1) + i]));
+                    if (q == 0) tmem_ld32(t_ds + 32, d[1]);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) pk[i] = pack_bf16(S[16 * q + 2 * i], S[16 * q + 2 * i + 1]);
+                    tmem_st8(t_sbf + 8 * q, pk);
+                    if (q == 1) tmem_wait_ld();
+                }
+            } else {
                 // S^T <- e^{gC} S^T + dS^T, 32 columns at a time, both loads in flight
                 uint32_t d[2][32];
                 tmem_ld32(t_ds, d[0]);
@@ -1015,7 +1059,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 }
             }
         }
-        if (p.sT && (RELAY || seg == p.nseg - 1)) {
+        if (PAIR) cluster_wait();
+        if (p.sT && (RELAY || seg == p.nseg - 1) && (!PAIR || cta.half == 0)) {
 #pragma unroll
             for (int m = 0; m < 64; ++m) p.sT[state_off + soff + (size_t)m * dv] = S[m];
         }
@@ -1028,31 +1073,32 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 atomicExch(done(), seg == p.nseg - 1 ? 0 : seg + 1);
             }
         }
-    } else if (warp < CW) {
+    } else if (warp < OW) {
         // =============================== output warpgroup(s) ===============================
-        if (!SCAN) { if (GATED) setmaxnreg_dec<80>(); else setmaxnreg_inc<136>(); }
-        const int og = (warp - 8) >> 2, q0 = og * QN;            // this warpgroup's tokens: 8 q0 .. 8 (q0 + QN) - 1
+        if (!SCAN) { if (GATED) setmaxnreg_dec<64>(); else setmaxnreg_inc<136>(); }
+        if (PAIR) cluster_arrive();
+        const int og = (warp - 8) >> 2;
         const int j = (tid - 256) & 127, we = j >> 5;
         const uint32_t lane_base = (uint32_t)(we * 32) << 16;
         // The accumulators are read as matrix fragments (thread: 4 value columns x 16 tokens, tokens in pairs), so that a
         // pair of tokens packs into one register and stmatrix transposes 8x8 blocks into rows of the output tile,
         // which leaves as two TMA stores (a last, partial chunk by plain stores: the rows behind it belong to others).
         // This role must stay shorter than a chain step: with one 2-byte store per value and row copies by
-        // the threads it took 1.6 us a chunk and set the pace of the whole kernel.  (With the fused output stage a single
-        // warpgroup is limited by how fast one warp per scheduler can issue, so two of them take 32 tokens each.)
-        const int l4 = lane & 3, l8 = lane >> 2;                 // fragment: columns 8q + 2 l4 (+1) are tokens, rows l8 (+8) values
-        // lane's part in stmatrix / ldmatrix: value columns 8 piece .. +7 of token 8q + (lane & 7)
+        // the threads it took 1.6 us a chunk and set the pace of the whole kernel.
+        const int l4 = lane & 3;                                 // fragment: columns 8q + 2 l4 (+1) are tokens, rows lane / 4 (+8) values
+        // lane's part in stmatrix: value columns 8 piece .. +7 of token 8q + (lane & 7)
+        constexpr uint32_t TILE_TOK = 8 * QN, TILE_HALF = TILE_TOK * 128;         // tokens of an output tile, bytes of half its columns
         const uint32_t piece = 4u * (uint32_t)we + (uint32_t)(lane >> 3);
-        const uint32_t frag_off = (piece >> 3) * 8192 + (uint32_t)(lane & 7) * 128 + (((piece & 7) ^ (uint32_t)(lane & 7)) << 4);
-        float wv[4] = {0.f, 0.f, 0.f, 0.f};
-        if (GATED) {
-#pragma unroll
-            for (int m = 0; m < 4; ++m) wv[m] = __ldg(p.norm_w + 32 * we + 8 * m + l8);
-        }
-        for (int c = 0; c < nchunks; ++c) {
-            const int R = min(C, len - c * C);
+        const uint32_t frag_off = (piece >> 3) * TILE_HALF + (uint32_t)(lane & 7) * 128 + (((piece & 7) ^ (uint32_t)(lane & 7)) << 4);
+        const int tk0 = GATED ? 32 * (PAIR ? cta.half : og) : 0;                  // first token of this warpgroup in a chunk
+        const uint32_t t_o1 = tmem + lane_base + TM_O1 + 32 * og, t_o2 = tmem + lane_base + TM_O2 + 32 * og;
+        for (int c = PAIR ? og : 0; c < nchunks; c += PAIR ? 2 : 1) {
+            const uint32_t par = PAIR ? (uint32_t)(c >> 1) & 1u : (uint32_t)c & 1u;      // of what this warpgroup waits for once per chunk of its own
+            const uint32_t own = PAIR ? (uint32_t)og : 0u;
+            const int R = min((int)TILE_TOK, len - c * C - tk0);
             const float* gates = reinterpret_cast<const float*>(sm + CS_GATES + (c % (int)GATE_SLOTS) * 1280);
-            if (og == 0 && tail_c >= 0 && c == max(tail_c - 1, 0)) {
+            // (of a pair: by the warpgroup that has seen the outputs of chunk tail_c - 2, so that the phases waited for below are those of tail_c)
+            if (PAIR ? c == tail_c : og == 0 && tail_c >= 0 && c == max(tail_c - 1, 0)) {
                 const int Rt = len - tail_c * C;
                 const uint32_t ks = KRing<COMPACT>::slot(tail_c), sk = base + KRing<COMPACT>::offset(ks);
                 const uint32_t sv = base + CS_B + (uint32_t)(tail_c & 1) * STAGE_B + ST_V;
@@ -1067,64 +1113,52 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 fence_proxy_async_smem();
                 mbar_arrive(w.bar(CB_CLEAN));
             }
-            if (GATED) {
-                // The gates do not depend on the chain: they are formed while this chunk's outputs are still on their way, and
-                // wait in tensor memory, which takes a running address where registers do not (unrolled, the
-                // gates made 14 KB of straight-line code that the instruction cache had lost by the next chunk).
-                w.wait(CB_ZFULL, c & 1);
-#pragma unroll 2
-                for (uint32_t q = q0; q < (uint32_t)(q0 + QN); ++q) {
-                    uint32_t z[4], y[2][4];
-                    ldmatrix_x4_trans(base + CS_Z + frag_off + q * 1024, z[0], z[1], z[2], z[3]);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {                // matrix m: value rows 8m + l8 of the warp's 32
-                        y[m >> 1][2 * (m & 1)] = __float_as_uint(wv[m] * silu(__uint_as_float(z[m] << 16)));
-                        y[m >> 1][2 * (m & 1) + 1] = __float_as_uint(wv[m] * silu(__uint_as_float(z[m] & 0xffff0000u)));
-                    }
-                    tmem_st_frag8(tmem + lane_base + TM_OG + 8 * q, y[0]);
-                    tmem_st_frag8(tmem + lane_base + (16u << 16) + TM_OG + 8 * q, y[1]);
-                }
-                tmem_wait_st();
-                mbar_arrive(w.bar(CB_ZFREE));
-            }
-            w.wait_hot(CB_O, c & 1);
+            w.wait_hot(PAIR ? CB_OH0 + own : (uint32_t)CB_O, par);
             tc_fence_after_sync();
-            // take both accumulators out of tensor memory first and hand them back at once: the next
+            // take both accumulators out of tensor memory first and hand them back at once: a later
             // chunk's output MMAs wait for this
-            const uint32_t ost = base + CS_OST + (uint32_t)(c & 1) * 16384;
+            const uint32_t ostoff = CS_OST + (GATED ? (uint32_t)og * 8192 : (uint32_t)(c & 1) * 16384), ost = base + ostoff;
             float o[2][4 * QN];
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
                 uint32_t o1[4 * QN], o2[4 * QN];
-                tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O1 + 8 * q0, o1);
-                tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_O2 + 8 * q0, o2);
+                tmem_ld_frags(t_o1 + ((uint32_t)(16 * hh) << 16), o1);
+                tmem_ld_frags(t_o2 + ((uint32_t)(16 * hh) << 16), o2);
                 tmem_wait_ld();
-                if (hh == 1) {
+                if (!PAIR && hh == 1) {
                     tc_fence_before_sync();
-                    mbar_arrive(w.bar(CB_OFREE));
+                    mbar_arrive(w.bar(CB_OFREE0 + own));
                 }
 #pragma unroll
                 for (int q = 0; q < QN; ++q) {
-                    const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + 8 * (q0 + q) + 2 * l4);
+                    const float2 eg = *reinterpret_cast<const float2*>(gates + 128 + tk0 + 8 * q + 2 * l4);
 #pragma unroll
-                    for (int x = 0; x < 4; ++x)
-                        o[hh][4 * q + x] = fmaf((x & 1) ? eg.y : eg.x, __uint_as_float(o1[4 * q + x]), __uint_as_float(o2[4 * q + x]));
+                    for (int x = 0; x < 4; x += 2) {
+                        const float2 y = fma2(eg, as_float2(o1[4 * q + x], o1[4 * q + x + 1]), as_float2(o2[4 * q + x], o2[4 * q + x + 1]));
+                        o[hh][4 * q + x] = y.x;
+                        o[hh][4 * q + x + 1] = y.y;
+                    }
                 }
+            }
+            if (PAIR) {                                          // (behind the use of the gate vectors: their slot may be refilled two chunks on)
+                tc_fence_before_sync();
+                mbar_arrive(w.bar(CB_OFREE0 + own));
             }
             if (GATED) {
                 // Fused output stage (the per-position kernels behind the scan, Section "Prefill projections:
                 // dequantize, then call the vendor"): root-mean-square norm of each output row over the value
                 // axis, weight vector, SiLU gate.  A token's squares lie in the eight lanes of equal l4 of every warp:
                 // a butterfly that halves the tokens at each step leaves two tokens' sums per lane, the four warps' sums meet
-                // in shared memory.  gate_z comes by TMA a chunk ahead and is read in the same fragments.
+                // in shared memory.  The gates come from a warpgroup of their own, in the same fragments.
                 float ss[2 * QN];
 #pragma unroll
-                for (int q = 0; q < QN; ++q)
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        const float a0 = o[0][4 * q + x], a1 = o[0][4 * q + 2 + x], a2 = o[1][4 * q + x], a3 = o[1][4 * q + 2 + x];
-                        ss[2 * q + x] = fmaf(a0, a0, a1 * a1) + fmaf(a2, a2, a3 * a3);
-                    }
+                for (int q = 0; q < QN; ++q) {
+                    const float2 a0 = make_float2(o[0][4 * q], o[0][4 * q + 1]), a1 = make_float2(o[0][4 * q + 2], o[0][4 * q + 3]);
+                    const float2 a2 = make_float2(o[1][4 * q], o[1][4 * q + 1]), a3 = make_float2(o[1][4 * q + 2], o[1][4 * q + 3]);
+                    const float2 y = add2(fma2(a0, a0, mul2(a1, a1)), fma2(a2, a2, mul2(a3, a3)));
+                    ss[2 * q] = y.x;
+                    ss[2 * q + 1] = y.y;
+                }
                 // eight values over eight lanes: after the three steps a lane holds one token's sum over its warp
 #pragma unroll
                 for (int st = 0; st < 3; ++st) {
@@ -1136,59 +1170,114 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                         ss[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16 >> st);
                     }
                 }
-                // value index = lane bits 4, 3, 2 = 2 q + x: token 8 (q0 + q) + 2 l4 + x
-                float* red = reinterpret_cast<float*>(sm + CS_RED) + (c & 1) * 256;
-                red[we * 64 + 8 * (q0 + (lane >> 4) * 2 + ((lane >> 3) & 1)) + 2 * l4 + ((lane >> 2) & 1)] = ss[0];
+                // value index = lane bits 4, 3, 2 = 2 q + x: token 8 q + 2 l4 + x of this warpgroup's
+                float* red = reinterpret_cast<float*>(sm + CS_RED) + og * 256 + par * 128;
+                red[we * 32 + 8 * ((lane >> 4) * 2 + ((lane >> 3) & 1)) + 2 * l4 + ((lane >> 2) & 1)] = ss[0];
+                if (j == 0) bulk_wait_read_all();                // this warpgroup's output tile has left: it is written again below
                 named_bar_sync(5 + og, 128);
-                float* inv = reinterpret_cast<float*>(sm + CS_INV) + we * 64;
-                {
-                    const int tk = 8 * q0 + lane;                // 32 tokens, one per lane
-                    const float sum = (red[tk] + red[64 + tk]) + (red[128 + tk] + red[192 + tk]);
-                    inv[tk] = rsqrtf(sum * (1.0f / DVB) + p.norm_eps);
-                }
+                float* inv = reinterpret_cast<float*>(sm + CS_INV) + (4 * og + we) * 32;
+                inv[lane] = rsqrtf(((red[lane] + red[32 + lane]) + (red[64 + lane] + red[96 + lane])) * (1.0f / DVB) + p.norm_eps);   // a token per lane
                 __syncwarp();
+                w.wait(CB_GFULL0 + own, par);
+                tc_fence_after_sync();
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     uint32_t g[4 * QN];
-                    tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_OG + 8 * q0, g);
+                    tmem_ld_frags(tmem + lane_base + ((uint32_t)(16 * hh) << 16) + TM_OG + 32 * og, g);
                     tmem_wait_ld();
+                    if (hh == 1) {
+                        tc_fence_before_sync();
+                        mbar_arrive(w.bar(CB_GFREE0 + own));
+                    }
 #pragma unroll
                     for (int q = 0; q < QN; ++q) {
-                        const float2 iv = *reinterpret_cast<const float2*>(inv + 8 * (q0 + q) + 2 * l4);
+                        const float2 iv = *reinterpret_cast<const float2*>(inv + 8 * q + 2 * l4);
 #pragma unroll
-                        for (int x = 0; x < 4; ++x) o[hh][4 * q + x] *= ((x & 1) ? iv.y : iv.x) * __uint_as_float(g[4 * q + x]);
+                        for (int x = 0; x < 4; x += 2) {
+                            const float2 y = mul2(make_float2(o[hh][4 * q + x], o[hh][4 * q + x + 1]), mul2(iv, as_float2(g[4 * q + x], g[4 * q + x + 1])));
+                            o[hh][4 * q + x] = y.x;
+                            o[hh][4 * q + x + 1] = y.y;
+                        }
                     }
                 }
             }
 #pragma unroll
             for (int q = 0; q < QN; ++q)
-                stmatrix_x4_trans(ost + frag_off + (uint32_t)(q0 + q) * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
+                stmatrix_x4_trans(ost + frag_off + (uint32_t)q * 1024, pack_bf16(o[0][4 * q], o[0][4 * q + 1]), pack_bf16(o[0][4 * q + 2], o[0][4 * q + 3]),
                                   pack_bf16(o[1][4 * q], o[1][4 * q + 1]), pack_bf16(o[1][4 * q + 2], o[1][4 * q + 3]));
-            if (R == C) {
+            if (R == (int)TILE_TOK) {
                 fence_proxy_async_smem();
-                if (j == 0 && og == 0) bulk_wait_read_all();              // the tile the next chunk writes has left (stored a chunk ago)
-                named_bar_sync(2, 128 * NOUT);
-                if (j == 0 && og == 0) {
-                    const int tok = (int)(tok0 + (long)c * C);
+                if (!GATED && j == 0) bulk_wait_read_all();      // the tile the next chunk writes has left (stored a chunk ago)
+                named_bar_sync(GATED ? 5 + og : 2, 128);
+                if (j == 0) {
+                    const int tok = (int)(tok0 + (long)c * C) + tk0;
                     tma_store_3d(map_o, dvb * DVB, h, tok, ost);
-                    tma_store_3d(map_o, dvb * DVB + 64, h, tok, ost + 8192);
+                    tma_store_3d(map_o, dvb * DVB + 64, h, tok, ost + TILE_HALF);
                     bulk_commit();
                 }
             } else {
-                named_bar_sync(2, 128 * NOUT);
-                __nv_bfloat16* obase = p.out + ((size_t)(tok0 + c * C) * H + h) * dv + (size_t)dvb * DVB;
+                named_bar_sync(GATED ? 5 + og : 2, 128);
+                __nv_bfloat16* obase = p.out + ((size_t)(tok0 + c * C + tk0) * H + h) * dv + (size_t)dvb * DVB;
 #pragma unroll 1
-                for (int qd = j + 128 * og; qd < R * 16; qd += 128 * NOUT) {
+                for (int qd = j; qd < R * 16; qd += 128) {
                     const uint32_t r = (uint32_t)qd >> 4, pc = (uint32_t)qd & 15u;
-                    const uint4 val = *reinterpret_cast<const uint4*>(sm + CS_OST + (c & 1) * 16384 + (pc >> 3) * 8192 + swz(r, pc & 7));
+                    const uint4 val = *reinterpret_cast<const uint4*>(sm + ostoff + (pc >> 3) * TILE_HALF + swz(r, pc & 7));
                     *reinterpret_cast<uint4*>(obase + (size_t)r * H * dv + pc * 8) = val;
                 }
             }
         }
-        if (j == 0 && og == 0) bulk_wait_all();
+        if (j == 0) bulk_wait_all();
+    } else if (GATED && warp < CW) {
+        // =============================== gate warpgroup ===============================
+        // norm_w * silu(gate_z) of a chunk, in the fragments the output warpgroups read and ahead of them: gate_z comes by TMA,
+        // the gates wait in tensor memory.  The output warpgroups used to form them as well, 0.9 of the 2.18 us that
+        // they took for a chunk and that set the step of the whole kernel.
+        setmaxnreg_dec<40>();
+        if (PAIR) cluster_arrive();
+        const int wq = warp - OW;
+        const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
+        const uint32_t piece = 4u * (uint32_t)wq + (uint32_t)(lane >> 3);
+        const uint32_t frag_off = (piece >> 3) * 4096 + (uint32_t)(lane & 7) * 128 + (((piece & 7) ^ (uint32_t)(lane & 7)) << 4);
+        float wv[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) wv[m] = __ldg(p.norm_w + 32 * wq + 8 * m + (lane >> 2));
+        for (int c = 0; c < nchunks; ++c) {
+            const uint32_t zt = base + ((c & 1) ? CS_Z1 : CS_Z) + frag_off, own = PAIR ? (uint32_t)c & 1u : 0u;
+            const uint32_t t_og = tmem + lane_base + TM_OG + 32 * own;
+            w.wait(CB_ZFULL0 + (c & 1), (c >> 1) & 1);
+            if (c >= (PAIR ? 2 : 1)) w.wait(CB_GFREE0 + own, PAIR ? ((c >> 1) - 1) & 1 : (c - 1) & 1);
+            tc_fence_after_sync();
+            // (a rolled loop, with a running address into tensor memory: unrolled it was 14 KB of straight-line code that the instruction
+            //  cache had lost by the next chunk)
+#pragma unroll 1
+            for (uint32_t q = 0; q < (PAIR ? 4 : 8); q += 2) {   // two fragments at once, to cover the latency of the special functions
+                uint32_t z[2][4], y[2][2][4];
+#pragma unroll
+                for (uint32_t f = 0; f < 2; ++f)
+                    ldmatrix_x4_trans(zt + (q >> 2) * 8192 + ((q & 3) + f) * 1024, z[f][0], z[f][1], z[f][2], z[f][3]);
+#pragma unroll
+                for (int f = 0; f < 2; ++f)
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {                // matrix m: value rows 8m + lane / 4 of the warp's 32
+                        const float2 g = weighted_silu2(z[f][m], wv[m]);
+                        y[f][m >> 1][2 * (m & 1)] = __float_as_uint(g.x);
+                        y[f][m >> 1][2 * (m & 1) + 1] = __float_as_uint(g.y);
+                    }
+#pragma unroll
+                for (uint32_t f = 0; f < 2; ++f) {
+                    tmem_st_frag8(t_og + 8 * (q + f), y[f][0]);
+                    tmem_st_frag8(t_og + (16u << 16) + 8 * (q + f), y[f][1]);
+                }
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+            mbar_arrive(w.bar(CB_GFULL0 + own));
+            mbar_arrive(w.bar(CB_ZFREE0 + (c & 1)));
+        }
     } else {
         // =============================== control warpgroup ===============================
-        if (!SCAN) setmaxnreg_dec<GATED ? 48 : 56>();
+        if (!SCAN) setmaxnreg_dec<GATED ? 40 : 56>();
+        if (PAIR) cluster_arrive();
         if (warp == CW) {
             const bool lead = elect_one();
             // ---- MMA issuer of the sequential chain: v_new and the state update, nothing else ----
@@ -1248,19 +1337,21 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             // (descriptors are built once; a stage or a k-step is an add on the 16-byte address field.  Every warp
             //  role runs its loop at the same time, so the size of these loops shows in the instruction cache.)
             const uint64_t dV0 = make_smem_desc(base + CS_B + ST_V, 8192, 1024), dT0 = make_smem_desc(base + CS_B + ST_T2, 1024, 1024);
+            constexpr uint32_t ID_OUT = PAIR ? ID_OH : ID_O, Q_HALF = PAIR ? 4096 : 8192;       // (a pair: 32 rows of Q and P)
             const uint64_t dQ0 = make_smem_desc(base + CS_Q, 16, 1024), dP0 = make_smem_desc(base + CS_P, 16, 1024);
             for (int c = -1; c < nchunks; ++c) {
                 const uint32_t s = c & 1, par = (c >> 1) & 1;
                 if (c >= 0) {
                     w.wait(CB_SREADY, c & 1);
                     w.wait(CB_FULLQ0 + s, par);
-                    if (c > 0) w.wait(CB_OFREE, (c - 1) & 1);  // the epilogue has read the previous O1, O2
+                    if (PAIR && c > 1) w.wait(CB_OFREE0 + s, ((c >> 1) - 1) & 1);   // the accumulators' previous contents have been read
+                    if (!PAIR && c > 0) w.wait(CB_OFREE0, (c - 1) & 1);
                     w.wait_hot(COMPACT ? (uint32_t)CB_X : (uint32_t)CB_V, c & 1);   // stay out of the tensor pipe until v_new (COMPACT: X) is done
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 8; ++ks)        // O1^T = S^T Q^T
-                        if (lead) mma_ts(tmem + TM_O1, tmem + TM_SBF + ks * 8, dQ0 + (uint64_t)((s * 16384 + (ks >> 2) * 8192 + (ks & 3) * 32) >> 4),
-                               ID_O, ks > 0);
+                        if (lead) mma_ts(tmem + TM_O1 + (PAIR ? 32 * s : 0u), tmem + TM_SBF + ks * 8, dQ0 + (uint64_t)((s * 16384 + (ks >> 2) * Q_HALF + (ks & 3) * 32) >> 4),
+                               ID_OUT, ks > 0);
                     if (lead) mma_commit(w.bar(CB_O1));
                     if (lead) mma_commit(w.bar(CB_FREEQ0 + s));
                     w.wait(CB_VREADY, c & 1);
@@ -1283,8 +1374,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks)        // O2^T = v^T P^T
-                        if (lead) mma_ts(tmem + TM_O2, tmem + TM_V + ks * 8, dP0 + (uint64_t)((s * 8192) >> 4) + ks * 2, ID_O, ks > 0);
+                        if (lead) mma_ts(tmem + TM_O2 + (PAIR ? 32 * s : 0u), tmem + TM_V + ks * 8, dP0 + (uint64_t)((s * 8192) >> 4) + ks * 2, ID_OUT, ks > 0);
                     if (lead) mma_commit(w.bar(CB_O));
+                    if (PAIR && lead) mma_commit(w.bar(CB_OH0 + s));
                     if (lead) mma_commit(w.bar(CB_FREEP0 + s));
                 }
             }
@@ -1320,9 +1412,10 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 {
                     const uint32_t full = w.bar(CB_FULLQ0 + s), dst = base + CS_Q + s * 16384;
                     if (c >= 2) w.wait(CB_FREEQ0 + s, par);
-                    mbar_arrive_expect_tx(full, 16384);
-                    tma_load_3d_hint(dst, map_q, 0, h, tok, full, pol_done);
-                    tma_load_3d_hint(dst + 8192, map_q, 64, h, tok, full, pol_done);
+                    const int tq = tok + (PAIR ? 32 * cta.half : 0);
+                    mbar_arrive_expect_tx(full, PAIR ? 8192 : 16384);
+                    tma_load_3d_hint(dst, map_q, 0, h, tq, full, pol_done);
+                    tma_load_3d_hint(dst + (PAIR ? 4096 : 8192), map_q, 64, h, tq, full, pol_done);
                 }
                 {
                     const uint32_t sk = KRing<COMPACT>::slot(c), full = w.bar(KRing<COMPACT>::full(sk)), dst = base + KRing<COMPACT>::offset(sk);
@@ -1336,8 +1429,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 {
                     const uint32_t full = w.bar(CB_FULLP0 + s);
                     if (c >= 2) w.wait(CB_FREEP0 + s, par);
-                    mbar_arrive_expect_tx(full, 8192);
-                    bulk_load(base + CS_P + s * 8192, item + IT_P, 8192, full);
+                    constexpr uint32_t bytes = PAIR ? 4096 : 8192;
+                    mbar_arrive_expect_tx(full, bytes);
+                    bulk_load(base + CS_P + s * 8192, item + IT_P + (PAIR ? (uint32_t)cta.half * 4096 : 0u), bytes, full);
                 }
             }
             if (*w.abort_flag) {
@@ -1352,26 +1446,30 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                                globaltimer_ns() - t0 < TIMEOUT_NS) {}
             }
         } else if (GATED && warp == CW + 3 && lane == 0) {
-            // ---- TMA producer of the gate tile ----
+            // ---- TMA producer of the gate tiles ----
             prefetch_tensormap(map_z);
-            const uint32_t full = w.bar(CB_ZFULL);
             for (int c = 0; c < nchunks; ++c) {
-                if (c > 0) w.wait(CB_ZFREE, (c - 1) & 1);
-                const int tok = (int)(tok0 + (long)c * C);
-                mbar_arrive_expect_tx(full, 16384);
-                tma_load_3d(base + CS_Z, map_z, 0, h, tok, full);
-                tma_load_3d(base + CS_Z + 8192, map_z, 64, h, tok, full);
+                const uint32_t full = w.bar(CB_ZFULL0 + (c & 1)), dst = base + ((c & 1) ? CS_Z1 : CS_Z);
+                if (c >= 2) w.wait(CB_ZFREE0 + (c & 1), ((c >> 1) - 1) & 1);
+                const int tok = (int)(tok0 + (long)c * C) + (PAIR ? 32 * cta.half : 0);
+                mbar_arrive_expect_tx(full, PAIR ? 8192 : 16384);
+                for (uint32_t t = 0; t < (PAIR ? 1 : 2); ++t) {
+                    tma_load_3d(dst + t * 8192, map_z, 0, h, tok + 32 * (int)t, full);
+                    tma_load_3d(dst + t * 8192 + 4096, map_z, 64, h, tok + 32 * (int)t, full);
+                }
             }
             if (*w.abort_flag) {
                 const unsigned long long t0 = globaltimer_ns();
-                while (!mbar_try_wait(full, (nchunks - 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+                for (int c = max(0, nchunks - 2); c < nchunks; ++c)
+                    while (!mbar_try_wait(w.bar(CB_ZFULL0 + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
             }
         }
     }
+    if (PAIR && warp >= 8) cluster_wait();
 }
 
-template <int MODE, bool GATED, bool COMPACT>
-__global__ void __launch_bounds__(GATED ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
+template <int MODE, int GATE, bool COMPACT>
+__global__ void __launch_bounds__(GATE != kNoGate ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
 gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                  const __grid_constant__ CUtensorMap map_z, ChainParams p) {
@@ -1382,7 +1480,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     Waiter w{base + CS_BARS, reinterpret_cast<volatile int*>(sm + CS_MISC + 4)};
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        chain_init_bars(w, GATED ? 256 : 128, COMPACT);
+        chain_init_bars(w, GATE, COMPACT);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -1396,7 +1494,8 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();                      // the next call's prepare kernel may set itself up as SMs come free
     pdl_wait();                         // scratch items and incoming states come from the kernels before this one
-    int dvb = (int)blockIdx.x, h = (int)blockIdx.y, z = (int)blockIdx.z;
+    int dvb = GATE == kGatePair ? 0 : (int)blockIdx.x, h = (int)blockIdx.y, z = (int)blockIdx.z;
+    const int half = GATE == kGatePair ? (int)blockIdx.x : 0;
     if (MODE == kRelay) {
         if (threadIdx.x == 0) sMisc[2] = (uint32_t)atomicAdd(p.ticket + 1, 1);
         __syncthreads();
@@ -1406,8 +1505,8 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         h = (c / D) % p.H;
         z = (c / (D * p.H)) * p.nseg + seg;
     }
-    const Cta cta{base, sm, tmem, dvb, h, z};
-    chain_body<MODE, false, GATED, COMPACT>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
+    const Cta cta{base, sm, tmem, dvb, h, z, half};
+    chain_body<MODE, false, GATE, COMPACT>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1673,7 +1772,7 @@ gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
     pdl_wait();                         // the scratch items come from the prepare kernel
-    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
+    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0};
     summary_body<false>(&map_k, &map_v, p, cta, w);
     tc_fence_before_sync();
     __syncthreads();
@@ -1856,7 +1955,7 @@ __global__ void __launch_bounds__(CMB_THREADS, 1) gdn_combine_kernel(CombinePara
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
-    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
+    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0};
     combine_body<false>(p, cta, w, 4);
     tc_fence_before_sync();
     __syncthreads();
@@ -1888,7 +1987,7 @@ constexpr int SCAN_THREADS = 512;
 constexpr uint32_t SC_BARS1 = CS_BARS;                 // behind the largest data layout (the chain phase's)
 constexpr uint32_t SC_BARS2 = SC_BARS1 + 24 * 8;
 constexpr uint32_t SC_BARS3 = SC_BARS2 + 16 * 8;
-constexpr uint32_t SC_MISC = SC_BARS3 + 32 * 8;
+constexpr uint32_t SC_MISC = SC_BARS3 + 42 * 8;
 constexpr uint32_t SCAN_SMEM = SC_MISC + 64 + 1024;
 static_assert(SUS_BARS <= CS_BARS && CM_BARS <= CS_BARS, "phase layouts must end before the barrier area");
 static_assert(SCAN_SMEM <= 232448, "shared memory per CTA");
@@ -1926,7 +2025,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (tid == 0) {
         summary_init_bars(w1, 2);
         combine_init_bars(w2);
-        chain_init_bars(w3, 128, false);
+        chain_init_bars(w3, kNoGate, false);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -1992,7 +2091,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     auto chain_phase = [&]() {
         // ---------------- phase 3: chain over this segment's chunks ----------------
         const Cta c3{base, sm, tmem, 0, h, (int)blockIdx.z};
-        chain_body<DBG ? kStamps : kPlain, true, false, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
+        chain_body<DBG ? kStamps : kPlain, true, kNoGate, false>(&map_q, &map_k, &map_v, &map_o, &map_o, p.cp, c3, w3, Handover{fl + 1, nowners});
         stamp(4);
         tc_fence_before_sync();
         cta_sync();
@@ -2086,20 +2185,27 @@ int lean_init_workspace(void* workspace) {
     return cudaMemset(workspace, 0, kWorkspaceHeader) == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
-// Launch a kernel that may begin (set-up only, up to its pdl_wait) before the previous kernel in the stream ends.
+// Launch a kernel that may begin (set-up only, up to its pdl_wait) before the previous kernel in the stream ends, in clusters of so many CTAs.
 template <typename... KArgs, typename... Args>
-static void launch_after(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+static void launch_cluster_after(int cluster, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = g_lean_timing ? 0 : 1;   // events between kernels: plain order
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+static void launch_after(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+    launch_cluster_after(1, kernel, grid, threads, smem, stream, args...);
 }
 
 // Split scratch per segment and sequence batch: incoming state, N_seg (fp32 [d_k, d_v] each) and the two
@@ -2143,11 +2249,12 @@ static int device_setup(int* sms_out) {
 #define GDN_K(...) reinterpret_cast<const void*>(__VA_ARGS__)
         if (!smem_limit(GDN_K(gdn_prep_kernel<false, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, false>), PREP_SMEM) ||
             !smem_limit(GDN_K(gdn_prep_kernel<false, true>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, true>), PREP_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kStamps, false, false>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, false, true>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, true, true>), CHAIN_SMEM_GATED) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kRelay, false, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, false, true>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kRelay, true, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, true, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kStamps, kNoGate, false>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGatePair, false>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kNoGate, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kGate, true>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_summary_kernel), SUM_SMEM) ||
             !smem_limit(GDN_K(gdn_combine_kernel), CMB_SMEM) ||
             !smem_limit(GDN_K(gdn_scan_kernel<false>), SCAN_SMEM) || !smem_limit(GDN_K(gdn_scan_kernel<true>), SCAN_SMEM))
@@ -2199,12 +2306,19 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                  : g_lean_relay < 0 && chain_ctas > num_sms ? plan_relay(chain_ctas, nch_all, num_sms) : 1;
     const int piece_chunks = pieces > 1 ? (nch_all + pieces - 1) / pieces : seg_chunks;
     if (pieces > 1) pieces = (nch_all + piece_chunks - 1) / piece_chunks;
-    CUtensorMap mq, mk, mv, mo, mz;
+    // The fused output stage on two CTAs per chain where the SMs would be idle otherwise (see GateMode).  One B200, calls with one / two:
+    // 16 heads, 1500 tokens 53.5 / 45.4 us, 2 x 4000 139 / 110, 3 packed sequences of 1123 to 2992 tokens 104 / 89, 4 x 1500 67.7 / 65.4
+    // (128 CTAs: what the second one reads again shows).  The line at four chunks: 400 tokens 22.7 / 20.6 us, 200 17.3 / 17.1, 128 12.9 /
+    // 13.4, 64 11.3 / 12.4 (the cluster's start).  The lengths of packed sequences are not known here: their mean stands for them.
+    const bool pair = opt.gate_z && pieces == 1 &&
+                      (g_lean_pair >= 0 ? g_lean_pair == 1 : chain_ctas * nseg * 2 <= num_sms && (packed ? (uint64_t)a.T > 192ull * a.B : a.T > 192));
+    CUtensorMap mq, mk, mv, mo, mz, mqc;
     if (!tc_make_map(&mq, a.q, tokens, a.H, a.d_k) || !tc_make_map(&mk, a.k, tokens, a.H, a.d_k) ||
-        !tc_make_map(&mv, a.v, tokens, a.H, a.d_v) || !tc_make_map(&mo, a.out, tokens, a.H, a.d_v) ||
-        (opt.gate_z && !tc_make_map(&mz, opt.gate_z, tokens, a.H, a.d_v)))
+        !tc_make_map(&mv, a.v, tokens, a.H, a.d_v) || !tc_make_map(&mo, a.out, tokens, a.H, a.d_v, opt.gate_z ? 32 : 64) ||
+        (opt.gate_z && !tc_make_map(&mz, opt.gate_z, tokens, a.H, a.d_v, 32)) || (pair && !tc_make_map(&mqc, a.q, tokens, a.H, a.d_k, 32)))
         return GDN_ERR_CUDA;
     if (!opt.gate_z) mz = mo;
+    if (!pair) mqc = mq;
     int* ticket = static_cast<int*>(workspace);                      // header, zeroed by lean_init_workspace
     uint8_t* ws = static_cast<uint8_t*>(workspace) + kWorkspaceHeader;
     const long nslots = (long)(tokens >> 6) + a.B;
@@ -2224,8 +2338,9 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // 70 at 1500 tokens to 100 at 8192, with at most 3 % to gain on either side of it.)  With the fused output stage that stage and not
     // the chain sets the step, which hides the hop, so there is no line: 64 tokens 1 to 24 chains 4 to 5 % less, 1500
     // tokens 1 chain 54.7 / 54.4 us, 16 58.9 / 59.4, 32 65.7 / 67.6, 56 72.0 / 73.7, 64 73.5 / 77.1, 96 87 / 94, 144 113 / 126; 4096 tokens
-    // 32 155 / 158 us, 64 178 / 184, 128 271 / 288; 8192 tokens 48 319 / 329 us, 96 445 / 462.
-    const bool compact = !g_lean_dbg && !g_lean_use_scan && nseg == 1 &&
+    // 32 155 / 158 us, 64 178 / 184, 128 271 / 288; 8192 tokens 48 319 / 329 us, 96 445 / 462.  (A pair of CTAs per chain is different: there
+    // the chain does set the step, and W is worth it: 16 heads, 1000 tokens 39.1 / 34.4 us, 4 x 1500 74.5 / 65.4.)
+    const bool compact = !g_lean_dbg && !g_lean_use_scan && nseg == 1 && !pair &&
                          (g_lean_compact >= 0 ? g_lean_compact == 1
                                               : !packed && a.d_v == DVB && (opt.gate_z || (long)a.B * a.H * 5 >= 3L * num_sms));
     const int pgrid = (int)(nitems < 4L * num_sms ? nitems : 4L * num_sms);
@@ -2279,14 +2394,15 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                    ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, pieces > 1 ? pieces : nseg, piece_chunks,
                    snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket,
                    pieces > 1 ? static_cast<int*>(workspace) + kScanFlagOffset : nullptr};
-    dim3 grid(a.d_v / DVB, a.H, a.B * (pieces > 1 ? pieces : nseg));
-    auto chain = pieces > 1 ? (opt.gate_z ? (compact ? gdn_chain_kernel<kRelay, true, true> : gdn_chain_kernel<kRelay, true, false>)
-                                          : (compact ? gdn_chain_kernel<kRelay, false, true> : gdn_chain_kernel<kRelay, false, false>))
-                 : opt.gate_z ? (compact ? gdn_chain_kernel<kPlain, true, true> : gdn_chain_kernel<kPlain, true, false>)
-                 : g_lean_dbg ? gdn_chain_kernel<kStamps, false, false>
-                              : (compact ? gdn_chain_kernel<kPlain, false, true> : gdn_chain_kernel<kPlain, false, false>);
-    launch_after(chain, grid, opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
-                 mq, mk, mv, mo, mz, cp);
+    dim3 grid(pair ? 2 : a.d_v / DVB, a.H, a.B * (pieces > 1 ? pieces : nseg));
+    auto chain = pieces > 1 ? (opt.gate_z ? (compact ? gdn_chain_kernel<kRelay, kGate, true> : gdn_chain_kernel<kRelay, kGate, false>)
+                                          : (compact ? gdn_chain_kernel<kRelay, kNoGate, true> : gdn_chain_kernel<kRelay, kNoGate, false>))
+                 : pair ? gdn_chain_kernel<kPlain, kGatePair, false>
+                 : opt.gate_z ? (compact ? gdn_chain_kernel<kPlain, kGate, true> : gdn_chain_kernel<kPlain, kGate, false>)
+                 : g_lean_dbg ? gdn_chain_kernel<kStamps, kNoGate, false>
+                              : (compact ? gdn_chain_kernel<kPlain, kNoGate, true> : gdn_chain_kernel<kPlain, kNoGate, false>);
+    launch_cluster_after(pair ? 2 : 1, chain, grid, opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
+                 mqc, mk, mv, mo, mz, cp);
     count_launch();
     mark(4);
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
@@ -2294,6 +2410,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
 
 void lean_set_relay(int pieces) { g_lean_relay = pieces; }
 void lean_set_compact(int mode) { g_lean_compact = mode; }
+void lean_set_pair(int mode) { g_lean_pair = mode; }
 void lean_set_scan(int enable) { g_lean_use_scan = enable != 0; }
 void lean_set_l2_hints(int enable) { g_lean_l2_hints = enable; }
 void lean_force_segments(int nseg) { g_lean_force_nseg = nseg; }
@@ -2376,7 +2493,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
             return GDN_ERR_CUDA;
         if (cudaFuncSetAttribute(gdn_prep_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(gdn_prep_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(gdn_chain_kernel<kPlain, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
+            cudaFuncSetAttribute(gdn_chain_kernel<kPlain, kNoGate, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
             return GDN_ERR_CUDA;
         sms_of_device[dev] = sms;
         scratch_of_device[dev] = ptr;
@@ -2397,7 +2514,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
                    ws, nullptr, nullptr, -1, a.B, a.T, a.H, a.d_v, 1, packed ? (1 << 24) : (nch > 0 ? nch : 1),
                    nullptr, 1, 0, 0, nullptr, nullptr, 0.f, static_cast<int*>(ticket_of_device[dev])};
     dim3 grid(a.d_v / DVB, a.H, a.B);
-    gdn_chain_kernel<kPlain, false, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
+    gdn_chain_kernel<kPlain, kNoGate, false><<<grid, CHAIN_THREADS, CHAIN_SMEM, stream>>>(mq, mk, mv, mo, mo, cp);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }

@@ -764,13 +764,13 @@ EncodeTiledFn encode_fn() {
 // [tokens, H, d] bf16, box = 64 tokens x 1 head x 64 features, 128-byte swizzle.
 // A map is a pure function of (address, tokens, H, d): a serving loop calls with the same few buffers again and
 // again, so the last few encodings are kept per host thread and the driver call is skipped on a repeat.
-bool make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d) {
-    struct Entry { const void* ptr; uint64_t tokens, H, d; CUtensorMap map; bool used; };
+bool make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d, uint32_t rows = 64) {
+    struct Entry { const void* ptr; uint64_t tokens, H, d; uint32_t rows; CUtensorMap map; bool used; };
     constexpr int kEntries = 32;          // four to five tensors a call, a handful of buffer sets in rotation
     static thread_local Entry cache[kEntries] = {};
     static thread_local int next = 0;
     for (int i = 0; i < kEntries; ++i)
-        if (cache[i].used && cache[i].ptr == ptr && cache[i].tokens == tokens && cache[i].H == H && cache[i].d == d) {
+        if (cache[i].used && cache[i].ptr == ptr && cache[i].tokens == tokens && cache[i].H == H && cache[i].d == d && cache[i].rows == rows) {
             *map = cache[i].map;
             return true;
         }
@@ -778,13 +778,13 @@ bool make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, ui
     if (!fn) return false;
     const cuuint64_t dims[3] = {d, H, tokens};
     const cuuint64_t strides[2] = {d * 2, H * d * 2};
-    const cuuint32_t box[3] = {64, 1, 64};
+    const cuuint32_t box[3] = {64, 1, rows};
     const cuuint32_t estr[3] = {1, 1, 1};
     if (fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
-    cache[next] = Entry{ptr, tokens, H, d, *map, true};
+    cache[next] = Entry{ptr, tokens, H, d, rows, *map, true};
     next = (next + 1) % kEntries;
     return true;
 }
@@ -793,8 +793,8 @@ bool make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, ui
 
 bool tc_supported(int d_k, int d_v) { return d_k == DK && d_v > 0 && d_v % DVB == 0; }
 
-bool tc_make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d) {
-    return make_map(map, ptr, tokens, H, d);
+bool tc_make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H, uint64_t d, uint32_t rows) {
+    return make_map(map, ptr, tokens, H, d, rows);
 }
 
 int launch_tc(const PrefillArgs& a, cudaStream_t stream) {

@@ -1,0 +1,98 @@
+"""The fused output stage on one CTA per chain and on two (each writes 32 tokens of every chunk): both against the oracle, at the
+edges of the 32-token halves, and a chain of every length in chunks up to where the rings have wrapped."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2607_14568_b200 as gdn
+from workloads import epilogue_inputs, get_config, make_inputs, widen
+from gdn_testlib import BF16_MAX_ABS, BF16_REL_L2, assert_close, f64, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _bf16(bits):
+    return torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16).cuda()
+
+
+def _run(x, d, e, pair, nseg=0, state=None):
+    cfg, packed, L = x.cfg, d["cu_seqlens"] is not None, gdn.lib()
+    gdn.gdn_set_workspace(torch.empty(gdn.gdn_workspace_bytes(len(x.lengths), x.T_arg, cfg.H, cfg.d_k, cfg.d_v, packed),
+                                      dtype=torch.uint8, device="cuda"))
+    L.gdn_debug_set_pair(pair)
+    L.gdn_debug_force_segments(nseg)
+    try:
+        gdn.gdn_chunk_prefill_gated(d["q"], d["k"], d["v"], d["log_alpha"], d["beta"], d["initial_state"] if state is None else state,
+                                    _bf16(e["z"]), torch.from_numpy(e["weight"]).cuda(), 1e-6, d["out"],
+                                    d["final_state"] if state is None else state, d["cu_seqlens"])
+        return gdn.gdn_query_status()
+    finally:
+        L.gdn_debug_set_pair(-1)
+        L.gdn_debug_force_segments(0)
+        gdn.gdn_set_workspace(None)
+
+
+def _check(x, d, e, fin, what):
+    o, want_fin = oracle.sequential(widen(x.q), widen(x.k), widen(x.v), x.log_alpha, x.beta, x.initial_state, x.cu_seqlens)
+    want = oracle.epilogue(o, widen(e["z"]), e["weight"], 1e-6)
+    # the norm and the gate rescale every row: the absolute bar scales with the values they produce
+    scale = max(1.0, float(np.abs(want).max() / np.abs(o).max()))
+    assert_close(f64(d["out"]), want, BF16_REL_L2, BF16_MAX_ABS * scale, what + ", out")
+    assert_close(f64(fin), want_fin, BF16_REL_L2, BF16_MAX_ABS, what + ", state")
+
+
+@pytest.mark.parametrize("pair", [0, 1])
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 63, 64, 65, 128 + 5, 192 + 32, 256 + 40, 64 * 9 + 63])
+def test_lengths(T, pair):
+    cfg = get_config("short", B=2, T=T, H=2, init_std=0.2, seed=T)
+    x = make_inputs(cfg)
+    d, e = to_device(x), epilogue_inputs(cfg, x.q.shape[:-2])
+    assert _run(x, d, e, pair) == 0
+    _check(x, d, e, d["final_state"], f"T {T}, pair {pair}")
+
+
+@pytest.mark.parametrize("pair", [0, 1])
+@pytest.mark.parametrize("nseg", [0, 4])
+def test_packed_or_split_and_the_state_in_place(nseg, pair):
+    """Packed sequences of every kind, the first followed by rows that are not finite; a split whose last segment ends in five tokens.
+    The state is updated in place: one CTA of a pair must not write it before the other has read it."""
+    kw = dict(T=64 * 20 + 5, B=1) if nseg else dict(B=4, T=0, lengths=(130, 0, 7, 64 * 5 + 33))
+    cfg = get_config("short", H=2, init_std=0.2, seed=5, **kw)
+    x = make_inputs(cfg)
+    d, e = to_device(x), epilogue_inputs(cfg, x.q.shape[:-2])
+    state = d["initial_state"].clone()
+    assert _run(x, d, e, pair, nseg, state) == 0
+    _check(x, d, e, state, f"nseg {nseg}, pair {pair}")
+    if not nseg:
+        for name in ("k", "v"):
+            d[name][130:170] = float("nan")
+        good = d["out"][:130].clone()
+        assert _run(x, d, e, pair) == 0
+        assert torch.equal(d["out"][:130], good)
+
+
+def test_rule_launches_two_kernels_either_way():
+    """Around the line (four chunks, two CTAs per chain within the SMs): same results bit for bit as the form that the rule takes."""
+    for B, T, H, pair in ((1, 192, 2, 0), (1, 193, 2, 1), (2, 256, 60, 0)):
+        cfg = get_config("short", B=B, T=T, H=H, init_std=0.2, seed=T)
+        x = make_inputs(cfg)
+        d, e = to_device(x), epilogue_inputs(cfg, x.q.shape[:-2])
+        assert _run(x, d, e, -1) == 0
+        by_rule = d["out"].clone()
+        assert _run(x, d, e, pair) == 0
+        assert torch.equal(by_rule, d["out"])
+
+
+def test_expired_wait_in_a_pair_is_reported_and_the_context_survives():
+    cfg = get_config("short", B=1, T=320, H=2, init_std=0.2, seed=9)
+    x = make_inputs(cfg)
+    d, e = to_device(x), epilogue_inputs(cfg, x.q.shape[:-2])
+    gdn.lib().gdn_debug_drop_chunk(2)                    # chunk 2 of the first chain is never loaded, by neither CTA
+    try:
+        assert _run(x, d, e, 1) == 5                     # GDN_ERR_TIMEOUT; the kernel returned on its own
+    finally:
+        gdn.lib().gdn_debug_drop_chunk(-1)
+    assert gdn.lib().gdn_debug_reset_status() == 0
+    assert _run(x, d, e, 1) == 0
+    _check(x, d, e, d["final_state"], "after a timed-out call")
