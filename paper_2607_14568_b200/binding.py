@@ -76,6 +76,8 @@ def lib():
         L.gdn_debug_set_scan.restype = None
         L.gdn_debug_set_relay.argtypes = [i]
         L.gdn_debug_set_relay.restype = None
+        L.gdn_debug_set_ahead.argtypes = [i]
+        L.gdn_debug_set_ahead.restype = None
         L.gdn_debug_set_pair.argtypes = [i]
         L.gdn_debug_set_pair.restype = None
         L.gdn_debug_set_compact.argtypes = [i]

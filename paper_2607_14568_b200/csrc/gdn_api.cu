@@ -350,7 +350,7 @@ int gdn_chunk_prefill_gated(const void* q, const void* k, const void* v, const f
 
 size_t gdn_workspace_bytes(int B, int T, int H, int d_k, int d_v, int chunk, int packed) {
     if (chunk != kChunk) return 0;
-    return lean_workspace_bytes(B, T, H, d_k, d_v, packed != 0);
+    return lean_workspace_bytes_full(B, T, H, d_k, d_v, packed != 0);
 }
 
 int gdn_set_workspace(void* device_ptr, size_t bytes) {
@@ -360,7 +360,7 @@ int gdn_set_workspace(void* device_ptr, size_t bytes) {
     if (dev < 0 || dev >= kMaxDevices) return GDN_ERR_UNSUPPORTED;
     Workspace ws;
     if (device_ptr && bytes >= 4096) {
-        if (int rc = lean_init_workspace(device_ptr)) return rc;
+        if (int rc = lean_init_workspace(device_ptr, bytes)) return rc;
         ws.ptr = device_ptr;
         ws.bytes = bytes;
     }
@@ -414,6 +414,7 @@ void gdn_debug_force_segments(int nseg) { lean_force_segments(nseg); }
 void gdn_debug_set_relay(int pieces) { lean_set_relay(pieces); }
 void gdn_debug_set_compact(int mode) { lean_set_compact(mode); }
 void gdn_debug_set_pair(int mode) { lean_set_pair(mode); }
+void gdn_debug_set_ahead(int mode) { lean_set_ahead(mode); }
 void gdn_debug_set_scan(int enable) { lean_set_scan(enable); }
 void gdn_debug_set_l2_hints(int enable) { lean_set_l2_hints(enable); }
 

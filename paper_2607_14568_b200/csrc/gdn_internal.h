@@ -46,7 +46,8 @@ bool tc_make_map(CUtensorMap* map, const void* ptr, uint64_t tokens, uint64_t H,
 
 // Two-kernel pipeline (prepare on all SMs, then the chain) using caller-provided scratch.
 size_t lean_workspace_bytes(int B, int T, int H, int d_k, int d_v, bool packed);
-int lean_init_workspace(void* workspace);   // zeroes the header of a newly provided workspace (synchronous)
+size_t lean_workspace_bytes_full(int B, int T, int H, int d_k, int d_v, bool packed);   // with what lets chains start early
+int lean_init_workspace(void* workspace, size_t bytes);   // zeroes the counters of a newly provided workspace (synchronous)
 struct LeanOptions {
     float* snaps = nullptr;    // optional (batched input only): [B, (T/64)/snap_every, H, d_k, d_v], the state
     int snap_every = 1;        //   after every snap_every chunks
@@ -70,6 +71,7 @@ int lean_set_timing(int enable);      // benchmark only: record events around ea
 int lean_get_timing(float* ms5);      // {prepare, summary, combine, chain, scan} of the last call
 void lean_set_l2_hints(int enable);   // tests only: 0 = no L2 eviction-priority hints
 void lean_set_relay(int pieces);      // tests only: pieces per chain (0 = never, -1 = by the rule)
+void lean_set_ahead(int mode);        // tests only: 0 = chains start behind the prepare kernel, 1 = by the rule
 void lean_set_pair(int mode);         // tests only: 0 / 1 = fused output stage of a chain on one CTA / on two, -1 = by the rule
 void lean_set_compact(int mode);      // tests only: 0 / 1 = scratch items with / without W, -1 = by the rule
 void lean_set_scan(int enable);       // tests only: 0 = never merge summary, combine and chain into one launch

@@ -46,7 +46,8 @@ static cudaEvent_t g_lean_events[5] = {nullptr, nullptr, nullptr, nullptr, nullp
 static bool g_lean_split_last = false;
 static float* g_lean_dbg = nullptr;        // debug: time stamps of the chain kernel
 static int g_lean_drop_chunk = -1;         // tests: chunk the chain kernel's TMA thread skips (-1 = none, -2 = a hand-over between CTAs
-                                           // that is not made, -3 = the prepare kernel waits for more bytes than its tiles have)
+                                           // that is not made, -3 = the prepare kernel waits for more bytes than its tiles have, -4 = no item is
+                                           // ever said to be ready)
 static int g_lean_l2_hints = 3;            // tests: bit 0 = L2 eviction-priority hints on the K, Q, V tile loads, bit 1 = on the
                                            // scratch images W and T2 (measured on the 10240-token workload, chain kernel:
                                            // 51.3 us without, 49.0 / 49.4 us with either, 47.2 us with both)
@@ -55,6 +56,7 @@ static bool g_lean_use_scan = false;       // true = summary, combination and ch
                                            // the 10240-token workload, 56 against 45 us at 2048 tokens, so it is off by default)
 static bool g_lean_scan_last = false;
 static int g_lean_relay = -1;              // tests: pieces per chain (0 = never, -1 = by the rule)
+static int g_lean_ahead = 1;               // tests: 0 / 2 = no / every chain starts before the prepare kernel has ended (1 = by the rule)
 static int g_lean_pair = -1;               // tests: 0 / 1 = the fused output stage of a chain on one CTA / on two (-1 = by the rule)
 static int g_lean_compact = -1;            // tests: 0 / 1 = items with / without -W^T whatever the size, without a split (-1 = by the rule)
 
@@ -112,10 +114,11 @@ struct BoundedWaiter {
             if (mbar_try_wait(b, parity)) return;
         wait_slow(b, parity);
     }
-    __device__ __forceinline__ void wait(uint32_t idx, uint32_t parity) const {
+    // False when given up.  Who issues copies must stop there: a further copy would arrive a second time on a barrier whose phase is open,
+    // and some tens of them overflow its byte count, which is a fault.
+    __device__ __forceinline__ bool wait(uint32_t idx, uint32_t parity) const {
         const uint32_t b = bar(idx);
-        if (mbar_try_wait(b, parity)) return;
-        wait_slow(b, parity);
+        return mbar_try_wait(b, parity) || wait_slow(b, parity);
     }
     // For what follows, without fail, on another role's bounded wait: its bound outlasts that one's.  False when it ran out.
     __device__ __forceinline__ bool wait_on_waiter(uint32_t idx, uint32_t parity) const {
@@ -171,6 +174,8 @@ __device__ __forceinline__ void bulk_store_hint(void* gdst, uint32_t smem_src, u
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// ... and what they wrote is visible to this thread, which may pass it on
+__device__ __forceinline__ void bulk_wait_all_global() { asm volatile("cp.async.bulk.wait_group 0;\n\tfence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // weight * z / (1 + e^-z) of two bf16 values (low, high half), with the hardware reciprocal (one unit in the last place; 0 for e^-z = inf)
@@ -206,13 +211,27 @@ constexpr uint32_t PS_GATES = PS_A + 64 * LDA * 4;
 constexpr uint32_t PS_RN = PS_GATES + GATE_FLOATS * 4;     // raw inputs: 1/|k_i| (64), 1/|q_r| (64)
 constexpr uint32_t PS_BARS = PS_RN + 128 * 4;
 constexpr uint32_t PS_MISC = PS_BARS + 16 * 8;
-constexpr uint32_t PS_TOTAL = PS_MISC + 64;          // tensor-memory address, abort flag, two item slots of four words
-constexpr uint32_t PREP_SMEM = PS_TOTAL + 1024;
+constexpr uint32_t PS_ORDER = PS_MISC + 64;          // (PS_MISC: tensor-memory address, abort flag, two item slots of four words)
+constexpr uint32_t PREP_SMEM = PS_ORDER + 1024;
+constexpr uint32_t PREP_SMEM_AHEAD = PREP_SMEM + 5 * 128 + 32;      // ItemOrder
 constexpr int PREP_THREADS = 192;
 constexpr uint32_t PT_COLS = 64;
 
-enum PBar : uint32_t { PB_FULL = 0, PB_G, PB_W, PB_TREADY, PB_GREADY, PB_DONE, PB_KQFREE, PB_ITEM };
+enum PBar : uint32_t { PB_FULL = 0, PB_G, PB_W, PB_TREADY, PB_GREADY, PB_DONE, PB_KQFREE, PB_ITEM, PB_STORED };
 
+// Whether chains start while items are still prepared.  Both kernels ask it of the same integers, so that they agree.
+struct AheadPlan {
+    int sms, chain_ctas;       // SMs; chain CTAs of a sequence
+    int step;                  // time of a chain step, in sixteenths of the time an SM spends on an item
+    int least;                 // least gain, in the same units: what the hand-over costs
+    // longest: chunks of the longest sequence; chunks: of all; items: chunks * heads.  All SMs together prepare, and then the chains run
+    // as long as the longest or as all of them take on all SMs; against the longer of the longest chain and everything on all SMs.
+    __host__ __device__ bool gains(long longest, long chunks, long items) const {
+        const long a = 16 * items, b = (long)step * longest * sms, c = (long)step * chain_ctas * chunks;
+        const long before = a + (b > c ? b : c), after = b > a + c ? b : a + c;
+        return 100 * (before - after) >= 100L * least * sms + 3 * (a + c);
+    }
+};
 struct PrepParams {
     const float* a;
     const float* beta;
@@ -225,6 +244,10 @@ struct PrepParams {
     int l2;                    // bit 0: the K tiles are read again by later kernels of this call and fit in L2: keep them there;
                                // bit 1: the same for the W and T2 images this kernel writes
     uint32_t tile_bytes;       // of an item's K and Q tiles, 32768 (tests: 16 more, so that the waits on them run out)
+    // Chains that start while this kernel still runs (see plan_ahead), or ready = nullptr:
+    int* ready;                // per item, zero before and after every call: set to `readers` once the item is in memory; every chain CTA that
+    int readers;               //   has taken the item counts it down by one
+    AheadPlan plan;
 };
 
 constexpr uint32_t ID_G = make_idesc(128, 64, kFmtBF16, kFmtBF16, kMajorK, kMajorK);
@@ -253,6 +276,109 @@ __device__ __forceinline__ bool decode_item(const PrepParams& p, long item, int*
     return true;
 }
 
+// Everything that this thread knows to be written, by itself or by the copies and threads it has waited for, is visible to who acquires the value.
+__device__ __forceinline__ void set_ready(int* flag, int value) {
+    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(flag), "r"(value) : "memory");
+}
+
+// The order of the items when chains start before all of them are done: what the chain with most left to do needs next comes
+// first.  With L chunks behind and including it, an item's level is L, and the levels go down from the longest sequence's length, at each
+// level the sequences that are as long, longest first, and their heads.  Equal lengths: chunk by chunk.  Packed input: every lane of a
+// warp holds the sequence of its rank by length (at most 32 of them), and between the lengths of two ranks the number of items per level does not
+// change, so that a ticket is found by its segment and two divisions.
+struct ItemOrder {                                  // in shared memory: as registers of one warp's role they would cost every role as many
+    int chunks[32], tok0[32], len[32], seq[32];     // (packed) of the sequence of rank i
+    int first[32];                                  // ticket of the first item of the levels that ranks 0 .. i share
+    int total;                                      // items of the call
+    int retire;                                     // a CTA that has drawn this ticket or a later one ends: its SM is for the chains
+    int last;                                       // ticket that the CTA has drawn last
+    int on;                                         // chains do start early (packed: decided here); otherwise nobody waits for single items, and
+                                                    // the first tickets are dealt out by CTA index
+    int stored;                                     // item that it has stored last
+    int pad[3];
+};
+static_assert(sizeof(ItemOrder) == PREP_SMEM_AHEAD - PREP_SMEM, "shared memory of the prepare kernel");
+__device__ __forceinline__ int warp_sum(int x) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
+    return x;
+}
+constexpr int kKeepSms = 12, kKeepCtas = 4;         // SMs, and CTAs wherever they are, that prepare items to the end
+__device__ __forceinline__ void make_order(const PrepParams& p, int lane, ItemOrder* o) {
+    const int H = p.H, cc = p.plan.chain_ctas, sms = p.plan.sms;
+    const float step = p.plan.step * (1.f / 16.f);
+    uint32_t smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    const int place = (int)smid;
+    // When does the chain CTA that this SM is meant for have to start?  All chains end together at the earliest time at which the longest
+    // one can have run and all SMs together can have done the work; each starts its own length earlier; until then its SM
+    // prepares items.  Times in units of an item on an SM.
+    float items_before;                             // what the SMs have prepared by that start
+    bool ok = place < sms - kKeepSms && blockIdx.x >= kKeepCtas;
+    int total;
+    bool on = true;                                 // (for equal lengths the host has asked)
+    if (p.cu) {
+        int t0 = 0, len = 0;
+        if (lane < p.B) { t0 = __ldcg(p.cu + lane); len = __ldcg(p.cu + lane + 1) - t0; }
+        const int k = (len + C - 1) / C;
+        int rank = 0;
+        for (int m = 0; m < 32; ++m) {
+            const int km = __shfl_sync(0xffffffffu, k, m);
+            rank += (km > k || (km == k && m < lane)) ? 1 : 0;
+        }
+        o->chunks[rank] = k; o->tok0[rank] = t0; o->len[rank] = len; o->seq[rank] = lane;
+        __syncwarp();
+        const int mine = o->chunks[lane], below = lane < 31 ? o->chunks[lane + 1] : 0;
+        const int size = (lane + 1) * (mine - below) * H;
+        int incl = size;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += up;
+        }
+        o->first[lane] = incl - size;
+        total = __shfl_sync(0xffffffffu, incl, 31);
+        const int q = min(place / cc, 31), kq = o->chunks[q];
+        const int all = warp_sum(mine);
+        const float chains = step * cc * all, longer = step * cc * warp_sum(lane < q ? mine - kq : 0);
+        const float end = fmaxf(step * o->chunks[0], (total + chains) / sms);
+        items_before = sms * (end - step * kq) - longer;
+        ok = ok && place / cc < 32 && kq > 0;
+        on = p.plan.gains(o->chunks[0], all, (long)all * H);
+    } else {
+        const int k = (p.T + C - 1) / C;
+        total = p.B * k * H;
+        const float one = step * k;
+        items_before = sms * (fmaxf(one, (total + one * p.B * cc) / sms) - one);
+        ok = ok && place < p.B * cc;
+    }
+    if (lane == 0) {
+        o->total = total;
+        o->retire = ok && on ? max(0, (int)items_before) : 0x7fffffff;
+        o->last = 0;
+        o->on = on;
+    }
+    __syncwarp();
+}
+// ticket -> item, head, first token, valid rows (all lanes of the warp)
+__device__ __forceinline__ int order_item(const PrepParams& p, const ItemOrder* o, int t, int lane, int* h, long* tok, int* R) {
+    const int H = p.H;
+    if (p.cu) {
+        const int r = 31 - __clz((int)__ballot_sync(0xffffffffu, o->first[lane] <= t));
+        const int x = t - o->first[r], per = (r + 1) * H, level = x / per, rem = x - level * per, i = rem / H;
+        *h = rem - i * H;
+        const int c = o->chunks[i] - o->chunks[r] + level;
+        *tok = o->tok0[i] + c * C;
+        *R = min(C, o->len[i] - c * C);
+        return (int)(slot_base(o->tok0[i], o->seq[i]) + c) * H + *h;
+    }
+    const int per = p.B * H, c = t / per, rem = t - c * per, n = rem / H;
+    *h = rem - n * H;
+    *tok = (long)n * p.T + c * C;
+    *R = min(C, p.T - c * C);
+    return (int)(slot_base((long)n * p.T, n) + c) * H + *h;
+}
+
 // RAW: q and k are raw projections and a, beta pre-activations.  The norms and the gating
 // (Section "Prefill projections: dequantize, then call the vendor": per-position kernels around the projections) are folded in here: the
 // inverse row norms scale A, P and the columns of T diag(b e^g), and they ride to the chain kernels
@@ -261,7 +387,8 @@ __device__ __forceinline__ bool decode_item(const PrepParams& p, long item, int*
 // COMPACT: the item is (T diag(b))^T, P and the gate vectors only, 17 KB instead of 33: the chain kernels then form
 // S^T K^T where they used S^T W^T and multiply by T diag(b) afterwards (see chain_body).  The first row of the gate vectors is
 // e^g / |k| there instead of g.
-template <bool RAW, bool COMPACT>
+// AHEAD: chains start while this kernel runs, so items come in the order of ItemOrder, and each is made known when it is in memory.
+template <bool RAW, bool COMPACT, bool AHEAD>
 __global__ void __launch_bounds__(PREP_THREADS, 4)
 gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, PrepParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -276,12 +403,13 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int H = p.H;
-    pdl_trigger();                      // the next kernel of the call may set itself up while this one runs
+    if (!AHEAD) pdl_trigger();          // the next kernel of the call may set itself up while this one runs
     if (warp == 4) { prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); }
     if (tid == 0) {
         mbar_init(w.bar(PB_FULL), 1); mbar_init(w.bar(PB_G), 1); mbar_init(w.bar(PB_W), 1);
         mbar_init(w.bar(PB_TREADY), 128); mbar_init(w.bar(PB_GREADY), 32); mbar_init(w.bar(PB_DONE), 128);
         mbar_init(w.bar(PB_KQFREE), 1); mbar_init(w.bar(PB_ITEM), 1);
+        if (AHEAD) mbar_init(w.bar(PB_STORED), 128);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -295,6 +423,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t tmem = warp_uniform(sMisc[0]);
 
     pdl_wait();                         // the scratch may still be read, and the inputs written, by what ran before
+    if (AHEAD) pdl_trigger();           // (chains that start ahead read inputs: what ran before has to have ended first)
     if (blockIdx.x == 0 && tid == 0) p.ticket[1] = 0;                 // (the chain kernel's, see ChainParams::relay)
 
     // Every CTA starts with the item of its own index; further ones are handed out through a global ticket: the time per
@@ -315,6 +444,19 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             t = -1;
         }
     };
+    ItemOrder* const order = reinterpret_cast<ItemOrder*>(sm + PS_ORDER);
+    if (AHEAD && warp == 4) make_order(p, lane, order);
+    auto draw_ordered = [&](bool first) -> int {
+        int t = order->last;
+        if (t >= order->retire) return -1;
+        __syncwarp();
+        if (first && !order->on) t = (int)blockIdx.x;
+        else {
+            if (lane == 0) t = order->last = (order->on ? 0 : (int)gridDim.x) + atomicAdd(p.ticket, 1);
+            t = (int)warp_uniform((uint32_t)t);
+        }
+        return t < order->total ? order_item(p, order, t, lane, &nh, &ntok, &nR) : -1;
+    };
     auto publish = [&](int slot, int item) {
         if (lane == 0) {
             volatile uint32_t* m = sMisc + 4 + 4 * slot;
@@ -322,7 +464,12 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             mbar_arrive(w.bar(PB_ITEM));
         }
     };
-    if (warp == 4) publish(0, draw((int)blockIdx.x));
+    if (warp == 4) publish(0, AHEAD ? draw_ordered(true) : draw((int)blockIdx.x));
+    auto store_first = [&](int it) {                 // (warps 0-3) the end of the CTA's first item
+        if (!AHEAD || it > 0 || !order->on) return;
+        if (tid == 0) bulk_wait_all_global();
+        mbar_arrive(w.bar(PB_STORED));
+    };
     int it = 0;     // items this CTA has processed (barrier phases)
     while (true) {
         // Nobody leaves on the abort flag: it may rise between two warps' reads of it, and the ones that went on would wait in the
@@ -367,6 +514,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
             // the -W^T image of the previous item has left the space of A by now; everybody is about to write there
             if (tp == 0) bulk_wait_read_all();
+            else if (AHEAD && it > 1 && order->on) mbar_arrive(w.bar(PB_STORED));
             named_bar_sync(1, 128);
             w.wait_on_waiter(PB_G, par);
             tc_fence_after_sync();
@@ -449,7 +597,16 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             // The images leave the SM as bulk copies from shared memory (a thread-per-row store would
             // touch 32 different lines per instruction); thread 0 issues them and later waits for their
             // shared-memory reads before the staging space is reused.
-            if (tp == 0) { bulk_store(out_item + IT_P, base + PS_KQ + 8192, 8192); bulk_commit(); }
+            if (tp == 0) {
+                // AHEAD: by now the previous item has long been in memory; warp 5 makes that known.  (Waited for at the top of the item, it
+                // held the whole CTA up.  The CTA's first item, which a chain may be waiting for to start, is: see store_first.)
+                if (AHEAD && it > 1 && order->on) {
+                    bulk_wait_all_global();
+                    mbar_arrive(w.bar(PB_STORED));
+                }
+                bulk_store(out_item + IT_P, base + PS_KQ + 8192, 8192);
+                bulk_commit();
+            }
             // ---- step b2: T = (I + A)^{-1}, blocked forward substitution (fp32) ----
             if (tp < 64) {   // level 0: four 16x16 diagonal blocks, one column per thread
                 const int I = tp >> 4, cc = tp & 15;
@@ -609,6 +766,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
             if (COMPACT) {
                 mbar_arrive(w.bar(PB_DONE));           // the gate vectors have been read
+                store_first(it);
                 ++it;
                 continue;
             }
@@ -644,6 +802,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 bulk_store_hint(out_item + IT_W, base + PS_A, 16384, (p.l2 & 2) ? l2_policy_evict_last() : l2_policy_evict_normal());
                 bulk_commit();
             }
+            store_first(it);
         } else if (warp == 4) {
             // ================= TMA + MMA issue (one elected thread) =================
             {
@@ -668,7 +827,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     if (lead) mma_ss(tmem, make_smem_desc(kq + off, 16, 1024), make_smem_desc(kq + off, 16, 1024), ID_G, ks > 0);
                 }
                 if (lead) mma_commit(w.bar(PB_G));
-                int nxt = draw(-1);                                 // the atomic's latency hides behind the solve
+                int nxt = AHEAD ? draw_ordered(false) : draw(-1);        // the atomic's latency hides behind the solve
                 if (!COMPACT) {
                 w.wait(PB_TREADY, par);
                 tc_fence_after_sync();
@@ -712,10 +871,24 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             gates[256 + lane] = (lane == 0) ? ex2(gC * LOG2E) : 0.f;
             gates[288 + lane] = 0.f;
             mbar_arrive(w.bar(PB_GREADY));
+            if (AHEAD && order->on) {
+                if (it > 0) w.wait_on_waiter(PB_STORED, (it - 1) & 1);
+                if (lane == 0) {
+                    if (it > 0) set_ready(p.ready + order->stored, p.readers);
+                    order->stored = (int)item;
+                }
+            }
         }
         ++it;
     }
-    if (tid == 0) bulk_wait_all();
+    if (tid == 0) { if (AHEAD) bulk_wait_all_global(); else bulk_wait_all(); }
+    if (AHEAD && it > 0 && order->on) {
+        if (warp < 4 && it > 1) mbar_arrive(w.bar(PB_STORED));
+        if (warp == 5) {
+            w.wait_on_waiter(PB_STORED, (it - 1) & 1);
+            if (lane == 0) set_ready(p.ready + order->stored, p.readers);
+        }
+    }
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -806,6 +979,8 @@ struct ChainParams {
     // possibly on another SM.  Pieces are taken in order through ticket[1], all first pieces before all second ones, so
     // whoever waits for a piece knows that it is running or done; the state travels through sT.
     int* relay;                    // [chains] pieces of the chain that are done (zero before and after every call), or nullptr
+    int* ready;                    // kAhead, see PrepParams
+    AheadPlan plan;
 };
 
 // One CTA's identity inside a kernel: aligned shared-memory base (address and pointer), tensor-memory base,
@@ -816,6 +991,8 @@ struct Cta {
     uint32_t tmem;
     int dvb, h, z;
     int half;                 // of a pair: which 32 tokens of every chunk this CTA writes
+    SeqInfo sq;               // kAhead: the sequence,
+    bool on;                  // and whether items are waited for one by one
 };
 // Grid-level hand-over inside the merged scan kernel: `flag` is a counter in global memory that the CTAs of one
 // (sequence, head) raise when their part of a phase is written; a consumer waits (bounded) until it reads
@@ -887,11 +1064,11 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 // here, W there.
 // MODE: what only a debug build (time stamps) or a relay needs stays out of the plain kernel: as run-time branches the relay cost
 // the other calls 1 to 2 %.
-enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2 };
+enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2, kAhead = 3 };
 template <int MODE, bool SCAN, int GATE, bool COMPACT>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
-    constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay;
+    constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay, AHEAD = MODE == kAhead;
     constexpr bool GATED = GATE != kNoGate, PAIR = GATE == kGatePair;
     constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments that each handles at a time
     constexpr int OW = 8 + 4 * NOUT, CW = GATED ? OW + 4 : OW;  // warps behind the output warpgroups: the gate warpgroup, the control warpgroup
@@ -899,10 +1076,10 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
-    if (tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
+    if (!AHEAD && tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
     const int n = cta.z / p.nseg, seg = cta.z % p.nseg;
     const int H = p.H, dv = p.dv;
-    const SeqInfo sq = seq_info(p.cu, n, p.T);
+    const SeqInfo sq = AHEAD ? cta.sq : seq_info(p.cu, n, p.T);
     // this CTA walks chunks [seg * seg_chunks, ...) of the sequence
     const int cbeg = seg * p.seg_chunks;
     const long tok0 = sq.tok0 + (long)cbeg * C;
@@ -942,9 +1119,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             if (tid == 0) handover_wait(SCAN ? hv : Handover{done(), seg}, w.abort_flag);
             named_bar_sync(3, 256);
         }
-        if (s_in) {                                     // (SCAN, RELAY: past the L1 cache, another SM may have written it during this launch)
+        if (s_in) {                                     // (SCAN, RELAY, AHEAD: past the L1 cache, another SM may have written it since this launch began)
 #pragma unroll
-            for (int m = 0; m < 64; ++m) S[m] = (SCAN || RELAY) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
+            for (int m = 0; m < 64; ++m) S[m] = (SCAN || RELAY || AHEAD) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
         } else {
 #pragma unroll
             for (int m = 0; m < 64; ++m) S[m] = 0.f;
@@ -1075,7 +1252,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
     } else if (warp < OW) {
         // =============================== output warpgroup(s) ===============================
-        if (!SCAN) { if (GATED) setmaxnreg_dec<64>(); else setmaxnreg_inc<136>(); }
+        if (!SCAN) { if (GATED) setmaxnreg_dec<64>(); else if (!AHEAD || COMPACT) setmaxnreg_inc<136>(); }      // (AHEAD with W: 128, as launched)
         if (PAIR) cluster_arrive();
         const int og = (warp - 8) >> 2;
         const int j = (tid - 256) & 127, we = j >> 5;
@@ -1240,7 +1417,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         const uint32_t frag_off = (piece >> 3) * 4096 + (uint32_t)(lane & 7) * 128 + (((piece & 7) ^ (uint32_t)(lane & 7)) << 4);
         float wv[4];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) wv[m] = __ldg(p.norm_w + 32 * wq + 8 * m + (lane >> 2));
+        for (int m = 0; m < 4; ++m) wv[m] = AHEAD ? __ldcg(p.norm_w + 32 * wq + 8 * m + (lane >> 2)) : __ldg(p.norm_w + 32 * wq + 8 * m + (lane >> 2));
         for (int c = 0; c < nchunks; ++c) {
             const uint32_t zt = base + ((c & 1) ? CS_Z1 : CS_Z) + frag_off, own = PAIR ? (uint32_t)c & 1u : 0u;
             const uint32_t t_og = tmem + lane_base + TM_OG + 32 * own;
@@ -1276,8 +1453,23 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
     } else {
         // =============================== control warpgroup ===============================
-        if (!SCAN) setmaxnreg_dec<GATED ? 40 : 56>();
+        if (!SCAN) setmaxnreg_dec<GATED ? 40 : AHEAD && !COMPACT ? 64 : 56>();
         if (PAIR) cluster_arrive();
+        volatile int* const upto = w.abort_flag + 4;            // (AHEAD) chunks whose items are known to be ready
+        auto load_z = [&](int c) {
+            const uint32_t full = w.bar(CB_ZFULL0 + (c & 1)), dst = base + ((c & 1) ? CS_Z1 : CS_Z);
+            const int tok = (int)(tok0 + (long)c * C) + (PAIR ? 32 * cta.half : 0);
+            mbar_arrive_expect_tx(full, PAIR ? 8192 : 16384);
+            for (uint32_t t = 0; t < (PAIR ? 1 : 2); ++t) {
+                tma_load_3d(dst + t * 8192, map_z, 0, h, tok + 32 * (int)t, full);
+                tma_load_3d(dst + t * 8192 + 4096, map_z, 64, h, tok + 32 * (int)t, full);
+            }
+        };
+        auto drain_z = [&](int n) {                             // n tiles were requested: let them land before shared memory is released (bounded)
+            const unsigned long long t0 = globaltimer_ns();
+            for (int c = max(0, n - 2); c < n; ++c)
+                while (!mbar_try_wait(w.bar(CB_ZFULL0 + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+        };
         if (warp == CW) {
             const bool lead = elect_one();
             // ---- MMA issuer of the sequential chain: v_new and the state update, nothing else ----
@@ -1388,81 +1580,139 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             prefetch_tensormap(map_o);
             const uint64_t pol_done = (p.l2 & 1) ? l2_policy_evict_first() : l2_policy_evict_normal();
             const uint64_t pol_item = (p.l2 & 2) ? l2_policy_evict_first() : l2_policy_evict_normal();
+            int issued = 0;                                    // five loads a chunk, in the order in which the slots come free
+            int known = AHEAD ? 0 : nchunks;                   // chunks whose items are known to be ready
             for (int c = 0; c < nchunks; ++c) {
-                if (c == p.drop_chunk && dvb == 0 && h == 0 && cta.z == 0) continue;
+                if (c == p.drop_chunk && dvb == 0 && h == 0 && cta.z == 0) { issued += 5; continue; }
+                if (AHEAD && c >= known) {
+                    while ((known = *upto) <= c && !*w.abort_flag) {}     // (bounded by the warp that looks)
+                    if (known <= c) break;
+                    // the items were written by other SMs during this launch, and bulk copies are about to read them
+                    __threadfence_block();
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                }
                 const int tok = (int)(tok0 + (long)c * C);
                 const uint8_t* item = p.items + (size_t)((slot0 + c) * H + h) * ITEM_BYTES;
-                // in the order in which the slots come free
                 const uint32_t s = c & 1, par = ((c >> 1) - 1) & 1;
                 {   // V tile and (T diag b)^T
                     const uint32_t bb = base + CS_B + s * STAGE_B, full = w.bar(CB_FULLB0 + s);
-                    if (c >= 2) w.wait(CB_FREEB0 + s, par);
+                    if (c >= 2 && !w.wait(CB_FREEB0 + s, par)) break;
                     mbar_arrive_expect_tx(full, STAGE_B_TX);
                     tma_load_3d_hint(bb + ST_V, map_v, dvb * DVB, h, tok, full, pol_done);
                     tma_load_3d_hint(bb + ST_V + 8192, map_v, dvb * DVB + 64, h, tok, full, pol_done);
                     bulk_load_hint(bb + ST_T2, item + IT_T2, 8192, full, pol_item);
                 }
+                ++issued;
                 if (!COMPACT) {
                     const uint32_t full = w.bar(CB_FULLW0 + s);
-                    if (c >= 2) w.wait(CB_FREEW0 + s, par);
+                    if (c >= 2 && !w.wait(CB_FREEW0 + s, par)) break;
                     mbar_arrive_expect_tx(full, 16384 + 1280);
                     bulk_load_hint(base + CS_W + s * 16384, item + IT_W, 16384, full, pol_item);
                     bulk_load(base + CS_GATES + (c % (int)GATE_SLOTS) * 1280, item + IT_GATES, 1280, full);
                 }
+                ++issued;
                 {
                     const uint32_t full = w.bar(CB_FULLQ0 + s), dst = base + CS_Q + s * 16384;
-                    if (c >= 2) w.wait(CB_FREEQ0 + s, par);
+                    if (c >= 2 && !w.wait(CB_FREEQ0 + s, par)) break;
                     const int tq = tok + (PAIR ? 32 * cta.half : 0);
                     mbar_arrive_expect_tx(full, PAIR ? 8192 : 16384);
                     tma_load_3d_hint(dst, map_q, 0, h, tq, full, pol_done);
                     tma_load_3d_hint(dst + (PAIR ? 4096 : 8192), map_q, 64, h, tq, full, pol_done);
                 }
+                ++issued;
                 {
                     const uint32_t sk = KRing<COMPACT>::slot(c), full = w.bar(KRing<COMPACT>::full(sk)), dst = base + KRing<COMPACT>::offset(sk);
                     constexpr int KD = COMPACT ? 3 : 2;
-                    if (c >= KD) w.wait(KRing<COMPACT>::free(sk), KRing<COMPACT>::parity(c - KD));
+                    if (c >= KD && !w.wait(KRing<COMPACT>::free(sk), KRing<COMPACT>::parity(c - KD))) break;
                     mbar_arrive_expect_tx(full, 16384 + (COMPACT ? 1280 : 0));
                     tma_load_3d_hint(dst, map_k, 0, h, tok, full, pol_done);
                     tma_load_3d_hint(dst + 8192, map_k, 64, h, tok, full, pol_done);
                     if (COMPACT) bulk_load(base + CS_GATES + (c % (int)GATE_SLOTS) * 1280, item + IT_GATES, 1280, full);
                 }
+                ++issued;
                 {
-                    const uint32_t full = w.bar(CB_FULLP0 + s);
-                    if (c >= 2) w.wait(CB_FREEP0 + s, par);
                     constexpr uint32_t bytes = PAIR ? 4096 : 8192;
+                    const uint32_t full = w.bar(CB_FULLP0 + s);
+                    if (c >= 2 && !w.wait(CB_FREEP0 + s, par)) break;
                     mbar_arrive_expect_tx(full, bytes);
                     bulk_load(base + CS_P + s * 8192, item + IT_P + (PAIR ? (uint32_t)cta.half * 4096 : 0u), bytes, full);
                 }
+                ++issued;
             }
             if (*w.abort_flag) {
                 // let copies in flight land before shared memory is released (bounded)
                 const unsigned long long t0 = globaltimer_ns();
-                for (int c = max(0, nchunks - 2); c < nchunks; ++c)
-                    for (uint32_t b = COMPACT ? CB_FULLQ0 : CB_FULLW0; b <= CB_FULLB0; b += 4)
-                        while (!(COMPACT && b == CB_FULLK0) && !mbar_try_wait(w.bar(b + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
-                if (COMPACT)
-                    for (int c = max(0, nchunks - 3); c < nchunks; ++c)
-                        while (!mbar_try_wait(w.bar(KRing<COMPACT>::full(KRing<COMPACT>::slot(c))), KRing<COMPACT>::parity(c)) &&
-                               globaltimer_ns() - t0 < TIMEOUT_NS) {}
-            }
-        } else if (GATED && warp == CW + 3 && lane == 0) {
-            // ---- TMA producer of the gate tiles ----
-            prefetch_tensormap(map_z);
-            for (int c = 0; c < nchunks; ++c) {
-                const uint32_t full = w.bar(CB_ZFULL0 + (c & 1)), dst = base + ((c & 1) ? CS_Z1 : CS_Z);
-                if (c >= 2) w.wait(CB_ZFREE0 + (c & 1), ((c >> 1) - 1) & 1);
-                const int tok = (int)(tok0 + (long)c * C) + (PAIR ? 32 * cta.half : 0);
-                mbar_arrive_expect_tx(full, PAIR ? 8192 : 16384);
-                for (uint32_t t = 0; t < (PAIR ? 1 : 2); ++t) {
-                    tma_load_3d(dst + t * 8192, map_z, 0, h, tok + 32 * (int)t, full);
-                    tma_load_3d(dst + t * 8192 + 4096, map_z, 64, h, tok + 32 * (int)t, full);
+#pragma unroll 1
+                for (int r = 0; r < 5; ++r) {
+                    const int n = (issued + 4 - r) / 5;         // loads of this ring
+                    const bool is_k = r == 3;
+                    if (COMPACT && r == 1) continue;
+#pragma unroll 1
+                    for (int c = max(0, n - (is_k && COMPACT ? 3 : 2)); c < n; ++c) {
+                        const uint32_t b = is_k ? KRing<COMPACT>::full(KRing<COMPACT>::slot(c))
+                                                : (r == 0 ? CB_FULLB0 : r == 1 ? CB_FULLW0 : r == 2 ? CB_FULLQ0 : CB_FULLP0) + (uint32_t)(c & 1);
+                        while (!mbar_try_wait(w.bar(b), is_k ? KRing<COMPACT>::parity(c) : (uint32_t)(c >> 1) & 1u) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+                    }
                 }
             }
-            if (*w.abort_flag) {
-                const unsigned long long t0 = globaltimer_ns();
-                for (int c = max(0, nchunks - 2); c < nchunks; ++c)
-                    while (!mbar_try_wait(w.bar(CB_ZFULL0 + (c & 1)), (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+        } else if (AHEAD && warp == CW + 3) {
+            // ---- which items are ready (the whole warp, a lane each), and the TMA producer of the gate tiles ----
+            // A warp of its own: an answer from memory takes 0.7 us, which the producer's loads would start late.
+            if (GATED) prefetch_tensormap(map_z);
+            int* const flags = p.ready + (slot0 * H + h);
+            int zc = GATED ? 0 : nchunks, n = 0;
+            unsigned long long t0 = globaltimer_ns();
+            if (!cta.on) {                             // all of them, when the prepare kernel has ended
+                pdl_wait();
+                n = nchunks;
+                if (lane == 0) *upto = n;
             }
+            while (zc < nchunks || n < nchunks) {
+                bool moved = false;
+                if (GATED && zc < nchunks) {
+                    const bool slot = zc < 2 || mbar_test_wait(w.bar(CB_ZFREE0 + (zc & 1)), ((zc >> 1) - 1) & 1);
+                    if (__shfl_sync(0xffffffffu, slot, 0)) {
+                        if (lane == 0) load_z(zc);
+                        ++zc;
+                        moved = true;
+                    }
+                }
+                if (n < nchunks) {
+                    int* const mine = flags + (long)(n + lane) * H;
+                    const uint32_t there = __ballot_sync(0xffffffffu, n + lane < nchunks && ld_acquire_gpu(mine) > 0);
+                    const int m = there == 0xffffffffu ? 32 : __ffs((int)~there) - 1;
+                    if (m > 0) {
+                        if (lane < m) asm volatile("red.relaxed.gpu.global.add.s32 [%0], -1;" ::"l"(mine) : "memory");
+                        n += m;
+                        __threadfence_block();
+                        __syncwarp();
+                        if (lane == 0) *upto = n;
+                        moved = true;
+                    }
+                }
+                const bool late = globaltimer_ns() - t0 > TIMEOUT_NS;
+                if (moved) t0 = globaltimer_ns();
+                else if (late && lane == 0) {
+                    *w.abort_flag = 1;
+                    atomicCAS(&g_lean_status, 0, (int)GDN_ERR_TIMEOUT);
+                }
+                if (__any_sync(0xffffffffu, (late && !moved) || *w.abort_flag)) break;
+                if (!moved) __nanosleep(100);
+            }
+            if (lane == 0) {
+                pdl_wait();                    // who waits for this kernel waits for the prepare kernel as well
+                if (blockIdx.x + blockIdx.y + blockIdx.z == 0) *p.ticket = 0;
+                if (GATED && *w.abort_flag) drain_z(zc);
+            }
+        } else if (!AHEAD && GATED && warp == CW + 3 && lane == 0) {
+            // ---- TMA producer of the gate tiles ----
+            prefetch_tensormap(map_z);
+            int c = 0;
+            for (; c < nchunks; ++c) {
+                if (c >= 2 && !w.wait(CB_ZFREE0 + (c & 1), ((c >> 1) - 1) & 1)) break;
+                load_z(c);
+            }
+            if (*w.abort_flag) drain_z(c);
         }
     }
     if (PAIR && warp >= 8) cluster_wait();
@@ -1482,19 +1732,49 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (threadIdx.x == 0) {
         chain_init_bars(w, GATE, COMPACT);
         sMisc[1] = 0;
+        sMisc[5] = 0;
         fence_mbar_init();
     }
     if (warp == 0) {
         tmem_alloc(base + CS_MISC, CT_COLS);
         tmem_relinquish();
     }
+    // AHEAD: the prepare kernel still runs; what ran before it has ended, or its CTAs would not have let this one start.  What that wrote is
+    // read past the L1 cache.  Packed sequences start longest first: blockIdx.z is the rank, the sequence is found by a warp, a sequence per lane.
+    if (MODE == kAhead && warp == 1 && p.cu) {
+        const int lane = threadIdx.x & 31;
+        int t0 = 0, len = 0, rank = 0;
+        if (lane < p.B) { t0 = __ldcg(p.cu + lane); len = __ldcg(p.cu + lane + 1) - t0; }
+        const int k = (len + C - 1) / C;
+        for (int m = 0; m < 32; ++m) {
+            const int km = __shfl_sync(0xffffffffu, k, m);
+            rank += (km > k || (km == k && m < lane)) ? 1 : 0;
+        }
+        const int all = warp_sum(k);
+        const int longest = __reduce_max_sync(0xffffffffu, k);
+        const bool on = p.plan.gains(longest, all, (long)all * p.H);
+        if ((on || longest * p.B >= 2 * all ? rank : lane) == (int)blockIdx.z) { sMisc[2] = (uint32_t)lane; sMisc[3] = (uint32_t)t0; sMisc[4] = (uint32_t)len; sMisc[6] = on; }
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();                      // the next call's prepare kernel may set itself up as SMs come free
-    pdl_wait();                         // scratch items and incoming states come from the kernels before this one
     int dvb = GATE == kGatePair ? 0 : (int)blockIdx.x, h = (int)blockIdx.y, z = (int)blockIdx.z;
+    SeqInfo sq{0, 0};
+    bool on = true;
+    if (MODE == kAhead) {
+        if (p.cu) {
+            z = (int)warp_uniform(sMisc[2]);
+            sq.tok0 = (long)warp_uniform(sMisc[3]);
+            sq.len = (int)warp_uniform(sMisc[4]);
+            on = sMisc[6] != 0;
+        } else {
+            sq = seq_info(nullptr, z, p.T);
+        }
+    } else {
+        pdl_wait();                     // scratch items and incoming states come from the kernels before this one
+    }
     const int half = GATE == kGatePair ? (int)blockIdx.x : 0;
     if (MODE == kRelay) {
         if (threadIdx.x == 0) sMisc[2] = (uint32_t)atomicAdd(p.ticket + 1, 1);
@@ -1505,7 +1785,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         h = (c / D) % p.H;
         z = (c / (D * p.H)) * p.nseg + seg;
     }
-    const Cta cta{base, sm, tmem, dvb, h, z, half};
+    const Cta cta{base, sm, tmem, dvb, h, z, half, sq, on};
     chain_body<MODE, false, GATE, COMPACT>(&map_q, &map_k, &map_v, &map_o, &map_z, p, cta, w, Handover{nullptr, 0});
     tc_fence_before_sync();
     __syncthreads();
@@ -1722,9 +2002,10 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
             prefetch_tensormap(map_v);
             const uint64_t pol_keep = (p.l2 & 1) ? l2_policy_evict_last() : l2_policy_evict_normal();
             const uint64_t pol_item = (p.l2 & 2) ? l2_policy_evict_last() : l2_policy_evict_normal();
-            for (int c = 0; c < nchunks; ++c) {
+            int c = 0;
+            for (; c < nchunks; ++c) {
                 const uint32_t s = c % SUM_STAGES, sb = base + s * SUM_STAGE;
-                if (c >= (int)SUM_STAGES) w.wait(SB_FREE0 + s, ((c / SUM_STAGES) - 1) & 1);
+                if (c >= (int)SUM_STAGES && !w.wait(SB_FREE0 + s, ((c / SUM_STAGES) - 1) & 1)) break;
                 const uint32_t full = w.bar(SB_FULL0 + s);
                 const int tok = (int)(tok0 + (long)c * C);
                 const uint8_t* item = p.items + (size_t)((slot0 + c) * H + h) * ITEM_BYTES;
@@ -1738,10 +2019,10 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                 bulk_load(sb + SS_GATES, item + IT_GATES, 1280, full);
             }
             if (*w.abort_flag) {
-                for (int c = max(0, nchunks - (int)SUM_STAGES); c < nchunks; ++c) {
-                    const uint32_t bar = w.bar(SB_FULL0 + (c % SUM_STAGES));
+                for (int i = max(0, c - (int)SUM_STAGES); i < c; ++i) {
+                    const uint32_t bar = w.bar(SB_FULL0 + (i % SUM_STAGES));
                     const unsigned long long t0 = globaltimer_ns();
-                    while (!mbar_try_wait(bar, (c / SUM_STAGES) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+                    while (!mbar_try_wait(bar, (i / SUM_STAGES) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
                 }
             }
         }
@@ -1772,7 +2053,7 @@ gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
     pdl_wait();                         // the scratch items come from the prepare kernel
-    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0};
+    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0, SeqInfo{0, 0}, false};
     summary_body<false>(&map_k, &map_v, p, cta, w);
     tc_fence_before_sync();
     __syncthreads();
@@ -1906,8 +2187,9 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
 #pragma unroll
             for (uint32_t q = 0; q < 4; ++q) bulk_load(base + st * CMB_IMG + q * 16384, src + q * 16384, 16384, full);
         };
+        int loaded = 0;
         if (prod == 0)
-            for (int sg = 0; sg < (int)CMB_STAGES && sg < nhops; ++sg) load_m(sg);
+            for (; loaded < (int)CMB_STAGES && loaded < nhops; ++loaded) load_m(loaded);
         const uint64_t dB0 = make_smem_desc(base + CM_B + boff, 16, 1024);
         for (int seg = 0; seg < nhops; ++seg) {
             const uint32_t st = seg % CMB_STAGES, ma = base + st * CMB_IMG + aoff;
@@ -1921,13 +2203,13 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
             if (lead) mma_commit(w.bar(MB_D));
             if (lead) mma_commit(w.bar(MB_FREE0 + st));
             if (prod == 0 && seg + (int)CMB_STAGES < nhops) {
-                w.wait(MB_FREE0 + st, (seg / CMB_STAGES) & 1);   // the tensor core has read this stage for all three products
-                load_m(seg + CMB_STAGES);
+                const bool read = w.wait(MB_FREE0 + st, (seg / CMB_STAGES) & 1);   // by the tensor core, for all three products
+                if (__all_sync(0xffffffffu, read) && loaded == seg + (int)CMB_STAGES) { load_m(loaded); ++loaded; }
             }
         }
         if (prod == 0 && *w.abort_flag) {   // let copies in flight land before shared memory is released (bounded)
             const unsigned long long t0 = globaltimer_ns();
-            for (int seg = max(0, nhops - (int)CMB_STAGES); seg < nhops; ++seg)
+            for (int seg = max(0, loaded - (int)CMB_STAGES); seg < loaded; ++seg)
                 while (!mbar_try_wait(w.bar(MB_FULL0 + seg % CMB_STAGES), (seg / CMB_STAGES) & 1) &&
                        globaltimer_ns() - t0 < TIMEOUT_NS) {}
         }
@@ -1955,7 +2237,7 @@ __global__ void __launch_bounds__(CMB_THREADS, 1) gdn_combine_kernel(CombinePara
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
-    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0};
+    const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0, SeqInfo{0, 0}, false};
     combine_body<false>(p, cta, w, 4);
     tc_fence_before_sync();
     __syncthreads();
@@ -2180,9 +2462,15 @@ constexpr int kScanFlagOffset = 16;
 constexpr long kMaxRelayChains = (long)(kWorkspaceHeader / sizeof(int) - kScanFlagOffset);
 constexpr long kMaxScanChains = (long)(kWorkspaceHeader / sizeof(int) - kScanFlagOffset) / SCAN_FLAG_INTS;
 
-// The ticket must read zero before the first launch; every launch leaves it zero again.
-int lean_init_workspace(void* workspace) {
-    return cudaMemset(workspace, 0, kWorkspaceHeader) == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
+// At the end of the workspace: a counter per item that the workspace can hold (PrepParams::ready; 0.012 % of its bytes).  Its place depends on the
+// workspace's size alone, so that it is zero before every call whatever the sizes of the calls before.
+static size_t ready_bytes(size_t workspace_bytes) { return (workspace_bytes / ITEM_BYTES + 1) * sizeof(int); }
+static size_t ready_offset(size_t workspace_bytes) { return workspace_bytes / sizeof(int) * sizeof(int) - ready_bytes(workspace_bytes); }
+
+// The ticket and the counters must read zero before the first launch; every call leaves them zero again.
+int lean_init_workspace(void* workspace, size_t bytes) {
+    return cudaMemset(workspace, 0, kWorkspaceHeader) == cudaSuccess &&
+           cudaMemset(static_cast<uint8_t*>(workspace) + ready_offset(bytes), 0, ready_bytes(bytes)) == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
 // Launch a kernel that may begin (set-up only, up to its pdl_wait) before the previous kernel in the stream ends, in clusters of so many CTAs.
@@ -2231,6 +2519,12 @@ size_t lean_workspace_bytes(int B, int T, int H, int d_k, int d_v, bool packed) 
     return bytes;
 }
 
+// What a caller should provide: the counters of items ready on top of what a call has to have.
+size_t lean_workspace_bytes_full(int B, int T, int H, int d_k, int d_v, bool packed) {
+    const size_t need = lean_workspace_bytes(B, T, H, d_k, d_v, packed);
+    return need ? (need + ready_bytes(need + need / 4096) + 4 + 255) / 256 * 256 : 0;
+}
+
 // Set-up done once per device: the SM count and the kernels' dynamic shared-memory limits.
 constexpr int kMaxDevices = 64;
 static int device_setup(int* sms_out) {
@@ -2247,14 +2541,19 @@ static int device_setup(int* sms_out) {
             return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
         };
 #define GDN_K(...) reinterpret_cast<const void*>(__VA_ARGS__)
-        if (!smem_limit(GDN_K(gdn_prep_kernel<false, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, false>), PREP_SMEM) ||
-            !smem_limit(GDN_K(gdn_prep_kernel<false, true>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, true>), PREP_SMEM) ||
+        if (!smem_limit(GDN_K(gdn_prep_kernel<false, false, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, false, false>), PREP_SMEM) ||
+            !smem_limit(GDN_K(gdn_prep_kernel<false, true, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, true, false>), PREP_SMEM) ||
+            !smem_limit(GDN_K(gdn_prep_kernel<false, false, true>), PREP_SMEM_AHEAD) || !smem_limit(GDN_K(gdn_prep_kernel<true, false, true>), PREP_SMEM_AHEAD) ||
+            !smem_limit(GDN_K(gdn_prep_kernel<false, true, true>), PREP_SMEM_AHEAD) || !smem_limit(GDN_K(gdn_prep_kernel<true, true, true>), PREP_SMEM_AHEAD) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kStamps, kNoGate, false>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, true>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, true>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGatePair, false>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kNoGate, true>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kGate, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kNoGate, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kGate, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kGatePair, false>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_summary_kernel), SUM_SMEM) ||
             !smem_limit(GDN_K(gdn_combine_kernel), CMB_SMEM) ||
             !smem_limit(GDN_K(gdn_scan_kernel<false>), SCAN_SMEM) || !smem_limit(GDN_K(gdn_scan_kernel<true>), SCAN_SMEM))
@@ -2343,12 +2642,46 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     const bool compact = !g_lean_dbg && !g_lean_use_scan && nseg == 1 && !pair &&
                          (g_lean_compact >= 0 ? g_lean_compact == 1
                                               : !packed && a.d_v == DVB && (opt.gate_z || (long)a.B * a.H * 5 >= 3L * num_sms));
-    const int pgrid = (int)(nitems < 4L * num_sms ? nitems : 4L * num_sms);
+    const size_t used = kWorkspaceHeader + items_bytes + (nseg > 1 ? split_scratch_bytes(a.B, a.H, a.d_k, a.d_v, nseg) : 0);
+    const bool tail_free = used <= ready_offset(workspace_bytes);
+    // (a workspace without room for the counters: what the call has written over them is cleared behind it)
+    auto finish = [&]() {
+        if (cudaGetLastError() != cudaSuccess) return (int)GDN_ERR_CUDA;
+        if (!tail_free && cudaMemsetAsync(static_cast<uint8_t*>(workspace) + ready_offset(workspace_bytes), 0, ready_bytes(workspace_bytes), stream) != cudaSuccess)
+            return (int)GDN_ERR_CUDA;
+        return (int)GDN_OK;
+    };
+    const int per_seq = a.H * (a.d_v / DVB) * (pair ? 2 : 1);         // chain CTAs of a sequence
+    // Chains that start while the prepare kernel still runs, as the items of their first chunks are ready (AheadPlan; a step and the least gain
+    // in sixteenths of an item on an SM, 2.6 us with W and 2.0 without).  The hand-over costs about 6 us a call, so equal lengths take it where
+    // the plan says that it gains more; with d_v = 256, where calls of the same size came out 6 % faster or slower, twice that.  Packed
+    // lengths are known on the device only, which decides again; here the line is the number of items: with few of them all are in
+    // flight at once.  Measured without / with, one B200: 2 x 24 heads x 4096 tokens 121 / 110 us, 4 x 12 x 8192 221 / 191, 4 x 16 x 2048 73.0 / 67.1,
+    // 3 x 12 x 3508 93.8 / 83.9; the line for equal lengths: 3 x 16 x 1024 38.1 / 36.0, 4 x 32 x 4096 190 / 193 (not taken), 3 x 32 x 768
+    // 38.9 / 40.5 (not taken).  Packed, 16 heads: 590 to 7880 tokens 240 / 203 us, 37 to 2320 78.1 / 70.6; 8 heads 62.3 / 57.7; uniform lengths
+    // lose 2 to 4 % (6 x 800 tokens, 32 heads 88.3 / 90.1), few items 3 to 5 % (not taken).
+    const int D = a.d_v / DVB;
+    const AheadPlan plan{num_sms, per_seq, compact ? 18 : pair ? 8 : 12, compact ? 128 : D > 1 ? 160 : 72};
+    const bool gains = packed ? a.B <= 32 && 2 * nitems > (D > 1 ? 24L : chain_ctas * 20 <= 13L * num_sms ? 12L : 21L) * num_sms
+                              : plan.gains(nch_all, (long)a.B * nch_all, (long)a.B * nch_all * a.H);
+    const bool ahead = tail_free && g_lean_ahead && nseg == 1 && pieces == 1 && !g_lean_dbg && tokens > 0 && (gains || (g_lean_ahead == 2 && (!packed || a.B <= 32)));
+    int* const ready = ahead ? reinterpret_cast<int*>(static_cast<uint8_t*>(workspace) + ready_offset(workspace_bytes)) : nullptr;
+    if (ahead) {
+        pp.ready = ready;
+        pp.readers = g_lean_drop_chunk == -4 ? 0 : (a.d_v / DVB) * (pair ? 2 : 1);
+        pp.plan = plan;
+    }
     auto mark = [&](int i) { if (g_lean_timing && g_lean_events[i]) cudaEventRecord(g_lean_events[i], stream); };
     mark(0);
-    auto prep = compact ? (opt.raw ? gdn_prep_kernel<true, true> : gdn_prep_kernel<false, true>)
-                        : (opt.raw ? gdn_prep_kernel<true, false> : gdn_prep_kernel<false, false>);
-    launch_after(prep, dim3(pgrid), PREP_THREADS, PREP_SMEM, stream, mq, mk, pp);
+    auto pick = [&](auto plain, auto in_order) { return ahead ? in_order : plain; };
+    auto prep = compact ? (opt.raw ? pick(gdn_prep_kernel<true, true, false>, gdn_prep_kernel<true, true, true>)
+                                   : pick(gdn_prep_kernel<false, true, false>, gdn_prep_kernel<false, true, true>))
+                        : (opt.raw ? pick(gdn_prep_kernel<true, false, false>, gdn_prep_kernel<true, false, true>)
+                                   : pick(gdn_prep_kernel<false, false, false>, gdn_prep_kernel<false, false, true>));
+    // (ahead: the CTAs on the SMs that the first chains are for may end at once)
+    const long want = nitems + (ahead ? 4L * (per_seq * (long)a.B < num_sms ? per_seq * (long)a.B : num_sms) : 0L);
+    const int pgrid = (int)(want < 4L * num_sms ? want : 4L * num_sms);
+    launch_after(prep, dim3(pgrid), PREP_THREADS, ahead ? PREP_SMEM_AHEAD : PREP_SMEM, stream, mq, mk, pp);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
     mark(1);
@@ -2376,7 +2709,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
             count_launch();
             g_lean_scan_last = true;
             mark(4);
-            return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
+            return finish();
         }
         dim3 sgrid(a.d_v / DVB, a.H, a.B * (nseg - 1));
         launch_after(gdn_summary_kernel, sgrid, SUM_THREADS, SUM_SMEM, stream, mk, mv, sp);
@@ -2393,10 +2726,13 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     ChainParams cp{a.initial_state, static_cast<__nv_bfloat16*>(a.out), a.final_state, a.cu_seqlens,
                    ws, seg_sin, g_lean_dbg, g_lean_drop_chunk, a.B, a.T, a.H, a.d_v, pieces > 1 ? pieces : nseg, piece_chunks,
                    snaps, snap_every, nsnap, l2, opt.gate_z, opt.norm_w, opt.norm_eps, ticket,
-                   pieces > 1 ? static_cast<int*>(workspace) + kScanFlagOffset : nullptr};
+                   pieces > 1 ? static_cast<int*>(workspace) + kScanFlagOffset : nullptr, ready, plan};
     dim3 grid(pair ? 2 : a.d_v / DVB, a.H, a.B * (pieces > 1 ? pieces : nseg));
     auto chain = pieces > 1 ? (opt.gate_z ? (compact ? gdn_chain_kernel<kRelay, kGate, true> : gdn_chain_kernel<kRelay, kGate, false>)
                                           : (compact ? gdn_chain_kernel<kRelay, kNoGate, true> : gdn_chain_kernel<kRelay, kNoGate, false>))
+                 : ahead && pair ? gdn_chain_kernel<kAhead, kGatePair, false>
+                 : ahead ? (opt.gate_z ? (compact ? gdn_chain_kernel<kAhead, kGate, true> : gdn_chain_kernel<kAhead, kGate, false>)
+                                       : (compact ? gdn_chain_kernel<kAhead, kNoGate, true> : gdn_chain_kernel<kAhead, kNoGate, false>))
                  : pair ? gdn_chain_kernel<kPlain, kGatePair, false>
                  : opt.gate_z ? (compact ? gdn_chain_kernel<kPlain, kGate, true> : gdn_chain_kernel<kPlain, kGate, false>)
                  : g_lean_dbg ? gdn_chain_kernel<kStamps, kNoGate, false>
@@ -2405,12 +2741,13 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                  mqc, mk, mv, mo, mz, cp);
     count_launch();
     mark(4);
-    return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
+    return finish();
 }
 
 void lean_set_relay(int pieces) { g_lean_relay = pieces; }
 void lean_set_compact(int mode) { g_lean_compact = mode; }
 void lean_set_pair(int mode) { g_lean_pair = mode; }
+void lean_set_ahead(int mode) { g_lean_ahead = mode; }
 void lean_set_scan(int enable) { g_lean_use_scan = enable != 0; }
 void lean_set_l2_hints(int enable) { g_lean_l2_hints = enable; }
 void lean_force_segments(int nseg) { g_lean_force_nseg = nseg; }
@@ -2491,8 +2828,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             return GDN_ERR_CUDA;
-        if (cudaFuncSetAttribute(gdn_prep_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
-        cudaFuncSetAttribute(gdn_prep_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
+        if (cudaFuncSetAttribute(gdn_prep_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PREP_SMEM) != cudaSuccess ||
             cudaFuncSetAttribute(gdn_chain_kernel<kPlain, kNoGate, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM) != cudaSuccess)
             return GDN_ERR_CUDA;
         sms_of_device[dev] = sms;
@@ -2506,7 +2842,7 @@ int launch_lean_static(const PrefillArgs& a, cudaStream_t stream) {
     const long nitems = (long)nslots * a.H;
     const long cap = 4L * sms_of_device[dev];
     PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, (long)nslots, a.B, a.T, a.H, 1.f, 0.f, static_cast<int*>(ticket_of_device[dev]), 0, 32768u};
-    gdn_prep_kernel<false, false><<<(int)(nitems < cap ? nitems : cap), PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
+    gdn_prep_kernel<false, false, false><<<(int)(nitems < cap ? nitems : cap), PREP_THREADS, PREP_SMEM, stream>>>(mq, mk, pp);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return GDN_ERR_CUDA;
     const int nch = packed ? 1 : (a.T + C - 1) / C;            // one segment: the whole sequence

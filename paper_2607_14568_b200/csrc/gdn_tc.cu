@@ -710,9 +710,11 @@ gdn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             prefetch_tensormap(&map_q);
             prefetch_tensormap(&map_k);
             prefetch_tensormap(&map_v);
-            for (int c = 0; c < nchunks; ++c) {
+            int c = 0;
+            for (; c < nchunks; ++c) {
                 const uint32_t stage = c & 1;
                 if (c >= 2) wait(cta, B_FREE0 + stage, ((c - 2) >> 1) & 1);
+                if (*cta.abort_flag) break;        // (a further copy could arrive twice in one phase of its barrier)
                 const uint32_t kq = cta.base + SM_KQ + stage * 32768, vb = cta.base + SM_V + stage * 16384;
                 const uint32_t full = cta.bar(B_FULL0 + stage);
                 const int tok = (int)(tok0 + (long)c * C);
@@ -726,10 +728,10 @@ gdn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             }
             if (*cta.abort_flag) {
                 // let copies in flight land before shared memory is released (bounded)
-                for (int c = max(0, nchunks - 2); c < nchunks; ++c) {
-                    const uint32_t bar = cta.bar(B_FULL0 + (c & 1));
+                for (int i = max(0, c - 2); i < c; ++i) {
+                    const uint32_t bar = cta.bar(B_FULL0 + (i & 1));
                     const unsigned long long t0 = globaltimer_ns();
-                    while (!mbar_try_wait(bar, (c >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
+                    while (!mbar_try_wait(bar, (i >> 1) & 1) && globaltimer_ns() - t0 < TIMEOUT_NS) {}
                 }
             }
         }

@@ -1,0 +1,185 @@
+"""Chains that start while the prepare kernel still runs: the same calls with and without, bit for bit, over the forms that the call has
+(items with and without W, raw projections, output stage on one and on two CTAs, wide values, snapshots, packed input of every kind),
+and the state that such a call leaves behind."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_14568_b200 as gdn
+from workloads import epilogue_inputs, get_config, make_inputs
+from gdn_testlib import BF16_MAX_ABS, BF16_REL_L2, assert_close, f64, run_oracle, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _bytes(x):
+    cfg = x.cfg
+    return gdn.gdn_workspace_bytes(len(x.lengths), x.T_arg, cfg.H, cfg.d_k, cfg.d_v, x.cu_seqlens is not None)
+
+
+def _call(x, d, entry, ahead, hooks=(), snaps=None):
+    L = gdn.lib()
+    L.gdn_debug_set_ahead(ahead)
+    L.gdn_debug_force_segments(1)
+    for name, value in hooks:
+        getattr(L, name)(value)
+    try:
+        a = (d["q"], d["k"], d["v"], d["log_alpha"], d["beta"])
+        if entry == "raw":
+            gdn.gdn_chunk_prefill_raw(*a, 0.05, 1e-6, d["initial_state"], d["out"], d["final_state"], d["cu_seqlens"])
+        elif entry == "gated":
+            e = epilogue_inputs(x.cfg, x.q.shape[:-2])
+            z = torch.from_numpy(e["z"].view(np.int16)).view(torch.bfloat16).cuda()
+            gdn.gdn_chunk_prefill_gated(*a, d["initial_state"], z, torch.from_numpy(e["weight"]).cuda(), 1e-6, d["out"], d["final_state"], d["cu_seqlens"])
+        elif entry == "snapshots":
+            gdn.gdn_chunk_prefill_snapshots(*a, d["initial_state"], d["out"], d["final_state"], 2, snaps)
+        else:
+            gdn.gdn_chunk_prefill(*a, d["initial_state"], d["out"], d["final_state"], d["cu_seqlens"])
+        return gdn.gdn_query_status()
+    finally:
+        L.gdn_debug_set_ahead(1)
+        L.gdn_debug_force_segments(0)
+        for name, _ in hooks:
+            getattr(L, name)(-1)
+
+
+def _both(x, entry="plain", hooks=(), ws=None):
+    """out, final state without and with; the counters at the end of the workspace are back at zero."""
+    d = to_device(x)
+    snaps = torch.zeros(len(x.lengths), max(x.cfg.T // 128, 1), x.cfg.H, 128, x.cfg.d_v, device="cuda") if entry == "snapshots" else None
+    if ws is None:
+        ws = torch.full((_bytes(x),), 0x55, dtype=torch.uint8, device="cuda")
+    got = []
+    try:
+        for ahead in (0, 2, 2):
+            gdn.gdn_set_workspace(ws)
+            d["out"].zero_(); d["final_state"].zero_()
+            assert _call(x, d, entry, ahead, hooks, snaps) == 0
+            got.append([t.clone() for t in (d["out"], d["final_state"]) + ((snaps,) if snaps is not None else ())])
+            n = ws.numel()
+            tail = ws[n // 4 * 4 - (n // 34048 + 1) * 4: n // 4 * 4].view(torch.int32)
+            assert int(tail.abs().sum()) == 0
+    finally:
+        gdn.gdn_set_workspace(None)
+    for g in got[1:]:
+        for a, b in zip(g, got[0]):
+            assert torch.equal(a, b)
+    return got[1]
+
+
+W, C = ("gdn_debug_set_compact", 0), ("gdn_debug_set_compact", 1)
+ONE, TWO = ("gdn_debug_set_pair", 0), ("gdn_debug_set_pair", 1)
+
+
+@pytest.mark.parametrize("entry,hooks,kw", [
+    ("plain", (W,), dict(B=3, T=64 * 9 + 1, H=5)), ("plain", (C,), dict(B=3, T=64 * 9 + 63, H=5)), ("plain", (W,), dict(B=1, T=1, H=1)),
+    ("plain", (W,), dict(B=2, T=64 * 40, H=40)), ("plain", (C,), dict(B=2, T=64 * 40, H=90)), ("plain", (W,), dict(B=2, T=64 * 20, H=7, d_v=256)),
+    ("raw", (W,), dict(B=2, T=64 * 5 + 9, H=3, raw=True)), ("raw", (C,), dict(B=2, T=64 * 5 + 9, H=3, raw=True)),
+    ("gated", (W, ONE), dict(B=2, T=64 * 7 + 33, H=3)), ("gated", (C, ONE), dict(B=2, T=64 * 7 + 33, H=3)), ("gated", (TWO,), dict(B=2, T=64 * 7 + 33, H=3)),
+    ("gated", (TWO,), dict(B=2, T=64 * 30, H=36)), ("snapshots", (W,), dict(B=2, T=64 * 8 + 5, H=3))])
+def test_equal_lengths(entry, hooks, kw):
+    _both(make_inputs(get_config("short", init_std=0.2, seed=31, **kw)), entry, hooks)
+
+
+@pytest.mark.parametrize("entry,hooks", [("plain", (W,)), ("plain", (C,)), ("raw", (W,)), ("gated", (ONE,)), ("gated", (TWO,))])
+@pytest.mark.parametrize("lengths,H", [((130,), 2), ((0, 64 * 30, 1, 0, 65, 700), 3), ((64,) * 32, 2), ((5, 64 * 33, 200) + (7,) * 20, 8),
+                                       ((64 * 60, 64 * 50 + 1, 64 * 9), 50)])
+def test_packed(entry, hooks, lengths, H):
+    x = make_inputs(get_config("short", init_std=0.2, seed=32, B=len(lengths), T=0, H=H, lengths=lengths, raw=entry == "raw"))
+    _both(x, entry, hooks)
+
+
+@pytest.mark.parametrize("kw", [dict(B=4, T=2048, H=12), dict(B=3, T=0, H=16, lengths=(5000, 1300, 64))])
+def test_taken_by_the_rule_and_right(kw):
+    x = make_inputs(get_config("short", init_std=0.2, seed=33, **kw))
+    out, fin = _both(x)
+    d = to_device(x)
+    gdn.gdn_set_workspace(torch.empty(_bytes(x), dtype=torch.uint8, device="cuda"))
+    try:
+        assert _call(x, d, "plain", 1) == 0
+    finally:
+        gdn.gdn_set_workspace(None)
+    assert torch.equal(d["out"], out) and torch.equal(d["final_state"], fin)
+    o_ref, f_ref = run_oracle(x)
+    assert_close(f64(out), o_ref, BF16_REL_L2, BF16_MAX_ABS, "out")
+    assert_close(f64(fin), f_ref, BF16_REL_L2, BF16_MAX_ABS, "state")
+
+
+def test_workspace_without_room_for_the_counters():
+    """As many bytes as a call cannot do without: the call runs, without early starts, and leaves the counters' place at zero for smaller
+    calls, which have room.  Calls of other sizes before do not matter either."""
+    kw = dict(B=2, T=0, H=3, init_std=0.2)
+    big, small = make_inputs(get_config("short", lengths=(64 * 12 + 5, 64 * 8), seed=34, **kw)), make_inputs(get_config("short", lengths=(64 * 2, 64 * 4 + 1), seed=35, **kw))
+    need = 4096 + (22 * 3 * 34048 + 255) // 256 * 256
+    ws = torch.full((need,), 0x55, dtype=torch.uint8, device="cuda")
+    gdn.gdn_set_workspace(ws)
+    try:
+        d, e = to_device(big), to_device(small)
+        assert _call(big, d, "plain", 2) == 0
+        n = need // 34048 + 1
+        assert int(ws[need - 4 * n:].view(torch.int32).abs().sum()) == 0
+        for x, y in ((small, e), (big, d), (small, e)):
+            assert _call(x, y, "plain", 2) == 0
+    finally:
+        gdn.gdn_set_workspace(None)
+    assert torch.equal(e["out"], _both(small)[0]) and torch.equal(d["out"], _both(big)[0])
+
+
+@pytest.mark.parametrize("packed", [False, True])
+def test_inputs_written_just_before_and_captured(packed):
+    """Every input, the sequence boundaries included, copied in front of the call on the same stream, eagerly and in a graph."""
+    L = gdn.lib()
+    kw = dict(B=3, T=0, lengths=(64 * 25 + 7, 64 * 3, 64 * 12 + 1)) if packed else dict(B=2, T=64 * 20 + 7)
+    kv = dict(B=3, T=0, lengths=(64 * 3, 64 * 12 + 1, 64 * 25 + 7)) if packed else dict(B=2, T=64 * 20 + 7)
+    xs = [make_inputs(get_config("short", H=6, init_std=0.3, seed=s, **k)) for s, k in ((36, kw), (37, kv))]
+    want = [_both(x) for x in xs]
+    src = [to_device(x) for x in xs]
+    d = {n: t.clone() if t is not None else None for n, t in src[0].items()}
+    names = [n for n in ("q", "k", "v", "log_alpha", "beta", "initial_state", "cu_seqlens") if d[n] is not None]
+    gdn.gdn_set_workspace(torch.empty(_bytes(xs[0]), dtype=torch.uint8, device="cuda"))
+    L.gdn_debug_set_ahead(2)
+    L.gdn_debug_force_segments(1)
+
+    def call():
+        gdn.gdn_chunk_prefill(d["q"], d["k"], d["v"], d["log_alpha"], d["beta"], d["initial_state"], d["out"], d["final_state"], d["cu_seqlens"])
+    try:
+        for i in range(8):
+            for n in names:
+                d[n].copy_(src[i & 1][n])
+            call()
+            got = d["out"].clone(), d["final_state"].clone()
+            assert torch.equal(got[0], want[i & 1][0]) and torch.equal(got[1], want[i & 1][1])
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=side):
+            call()
+        for i in range(4):
+            for n in names:
+                d[n].copy_(src[i & 1][n])
+            torch.cuda.synchronize()
+            graph.replay()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert gdn.gdn_query_status() == 0
+            assert torch.equal(d["out"], want[i & 1][0]) and torch.equal(d["final_state"], want[i & 1][1])
+    finally:
+        L.gdn_debug_set_ahead(1)
+        L.gdn_debug_force_segments(0)
+        gdn.gdn_set_workspace(None)
+
+
+@pytest.mark.parametrize("entry", ["plain", "gated"])
+def test_items_that_are_never_ready(entry):
+    """Every chain gives up after about a second, has nothing in flight, and the call returns with GDN_ERR_TIMEOUT; the next one is right."""
+    x = make_inputs(get_config("short", B=2, T=64 * 30, H=3, init_std=0.2, seed=38))
+    d = to_device(x)
+    ws = torch.empty(_bytes(x), dtype=torch.uint8, device="cuda")
+    gdn.gdn_set_workspace(ws)
+    gdn.lib().gdn_debug_drop_chunk(-4)
+    try:
+        assert _call(x, d, entry, 2) == 5
+    finally:
+        gdn.lib().gdn_debug_drop_chunk(-1)
+        gdn.gdn_set_workspace(None)
+    assert gdn.lib().gdn_debug_reset_status() == 0
+    _both(x, entry)
