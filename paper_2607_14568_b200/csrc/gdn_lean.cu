@@ -2609,8 +2609,13 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // 16 heads, 1500 tokens 53.5 / 45.4 us, 2 x 4000 139 / 110, 3 packed sequences of 1123 to 2992 tokens 104 / 89, 4 x 1500 67.7 / 65.4
     // (128 CTAs: what the second one reads again shows).  The line at four chunks: 400 tokens 22.7 / 20.6 us, 200 17.3 / 17.1, 128 12.9 /
     // 13.4, 64 11.3 / 12.4 (the cluster's start).  The lengths of packed sequences are not known here: their mean stands for them.
+    // Chains on more than half of that many SMs do not take two where they can start while items are still prepared (below), which then has
+    // the other SMs: 4 x 16 heads x 1500 tokens, two CTAs / early start 67.8 / 61.2 us, x 3000 116 / 102, x 6000 220 / 184, 3 x 2000 78.0 / 74.3.
+    const bool many = !packed && nseg == 1 && chain_ctas * 40 > 11L * num_sms &&
+                      AheadPlan{num_sms, a.H, 18, 128}.gains(nch_all, (long)a.B * nch_all, (long)a.B * nch_all * a.H);
     const bool pair = opt.gate_z && pieces == 1 &&
-                      (g_lean_pair >= 0 ? g_lean_pair == 1 : chain_ctas * nseg * 2 <= num_sms && (packed ? (uint64_t)a.T > 192ull * a.B : a.T > 192));
+                      (g_lean_pair >= 0 ? g_lean_pair == 1
+                                        : !many && chain_ctas * nseg * 2 <= num_sms && (packed ? (uint64_t)a.T > 192ull * a.B : a.T > 192));
     CUtensorMap mq, mk, mv, mo, mz, mqc;
     if (!tc_make_map(&mq, a.q, tokens, a.H, a.d_k) || !tc_make_map(&mk, a.k, tokens, a.H, a.d_k) ||
         !tc_make_map(&mv, a.v, tokens, a.H, a.d_v) || !tc_make_map(&mo, a.out, tokens, a.H, a.d_v, opt.gate_z ? 32 : 64) ||
@@ -2659,10 +2664,10 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // flight at once.  Measured without / with, one B200: 2 x 24 heads x 4096 tokens 121 / 110 us, 4 x 12 x 8192 221 / 191, 4 x 16 x 2048 73.0 / 67.1,
     // 3 x 12 x 3508 93.8 / 83.9; the line for equal lengths: 3 x 16 x 1024 38.1 / 36.0, 4 x 32 x 4096 190 / 193 (not taken), 3 x 32 x 768
     // 38.9 / 40.5 (not taken).  Packed, 16 heads: 590 to 7880 tokens 240 / 203 us, 37 to 2320 78.1 / 70.6; 8 heads 62.3 / 57.7; uniform lengths
-    // lose 2 to 4 % (6 x 800 tokens, 32 heads 88.3 / 90.1), few items 3 to 5 % (not taken).
+    // lose 2 to 4 % (6 x 800 tokens, 32 heads 88.3 / 90.1), few items 3 to 5 %, and two CTAs on each of many chains 6 % (not taken).
     const int D = a.d_v / DVB;
     const AheadPlan plan{num_sms, per_seq, compact ? 18 : pair ? 8 : 12, compact ? 128 : D > 1 ? 160 : 72};
-    const bool gains = packed ? a.B <= 32 && 2 * nitems > (D > 1 ? 24L : chain_ctas * 20 <= 13L * num_sms ? 12L : 21L) * num_sms
+    const bool gains = packed ? a.B <= 32 && !(pair && chain_ctas * 40 > 13L * num_sms) && 2 * nitems > (D > 1 ? 24L : chain_ctas * 20 <= 13L * num_sms ? 12L : 21L) * num_sms
                               : plan.gains(nch_all, (long)a.B * nch_all, (long)a.B * nch_all * a.H);
     const bool ahead = tail_free && g_lean_ahead && nseg == 1 && pieces == 1 && !g_lean_dbg && tokens > 0 && (gains || (g_lean_ahead == 2 && (!packed || a.B <= 32)));
     int* const ready = ahead ? reinterpret_cast<int*>(static_cast<uint8_t*>(workspace) + ready_offset(workspace_bytes)) : nullptr;
