@@ -902,6 +902,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // =====================================================================================
 constexpr int CHAIN_THREADS = 512;          // two chain warpgroups, output warpgroup, control warpgroup
 constexpr int CHAIN_THREADS_GATED = 768;    // two output warpgroups and one that forms the gates
+constexpr int CHAIN_THREADS_PAIR = 1024;    // and four chain warpgroups
 // tensor memory columns
 constexpr uint32_t TM_DV = 0, TM_DS = 64, TM_SBF = 192, TM_V = 256, TM_VT = 288, TM_O1 = 320, TM_O2 = 384,
                    TM_OG = 448;   // fused output stage: norm_w * silu(gate_z) of the chunk, fp32
@@ -1032,12 +1033,12 @@ __device__ __forceinline__ bool handover_wait(const Handover& hv, volatile int* 
 // chunk each, with accumulators and gates of their own, so that the chain sets the step again: 1.2 us.
 enum GateMode : int { kNoGate = 0, kGate = 1, kGatePair = 2 };
 
-__device__ __forceinline__ void chain_init_bars(const Waiter& w, int gate, bool compact) {
+__device__ __forceinline__ void chain_init_bars(const Waiter& w, int gate, bool compact, uint32_t chain_threads) {
     for (uint32_t i = CB_FULLW0; i < CB_V; ++i)
-        mbar_init(w.bar(i), (compact && i == CB_YREADY) ? 256 : 1);
+        mbar_init(w.bar(i), (compact && i == CB_YREADY) ? chain_threads : 1);
     mbar_init(w.bar(CB_U), 1); mbar_init(w.bar(CB_O1), 1);
     mbar_init(w.bar(CB_V), 1); mbar_init(w.bar(CB_S), 1); mbar_init(w.bar(CB_O), 1);
-    mbar_init(w.bar(CB_SREADY), 256); mbar_init(w.bar(CB_VREADY), 256); mbar_init(w.bar(CB_VPLAIN), 256);
+    mbar_init(w.bar(CB_SREADY), chain_threads); mbar_init(w.bar(CB_VREADY), chain_threads); mbar_init(w.bar(CB_VPLAIN), chain_threads);
     mbar_init(w.bar(CB_CLEAN), 128);
     const uint32_t readers = gate == kGate ? 256 : 128;          // of one accumulator
     for (uint32_t i = 0; i < 2; ++i) mbar_init(w.bar(CB_OFREE0 + i), readers);
@@ -1071,7 +1072,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay, AHEAD = MODE == kAhead;
     constexpr bool GATED = GATE != kNoGate, PAIR = GATE == kGatePair;
     constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments that each handles at a time
-    constexpr int OW = 8 + 4 * NOUT, CW = GATED ? OW + 4 : OW;  // warps behind the output warpgroups: the gate warpgroup, the control warpgroup
+    constexpr int NCH = PAIR ? 4 : 2, TW = C / NCH, SW = DK / NCH;      // chain warpgroups; tokens and state columns of each
+    constexpr int OW = 4 * NCH + 4 * NOUT, CW = GATED ? OW + 4 : OW;  // warps behind the output warpgroups: the gate warpgroup, the control warpgroup
     const uint32_t base = cta.base, tmem = cta.tmem;
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
@@ -1105,30 +1107,32 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                       : p.seg_sin ? p.seg_sin + ((size_t)(n * p.nseg + seg) * H + h) * DK * dv + (size_t)dvb * DVB
                                   : (p.s0 ? p.s0 + state_off : nullptr);
 
-    if (warp < 8) {
+    if (warp < 4 * NCH) {
         // =============================== chain warpgroups ===============================
         // Two of them share the conversions that sit between two dependent MMA batches: each takes half of the tokens
-        // of v_new and half of the state's d_k columns (64 fp32 values per thread).  Short prompts: 27 -> 25 us for the kernel.
-        if (!SCAN) setmaxnreg_inc<GATED ? 136 : 160>();
+        // of v_new and half of the state's d_k columns (64 fp32 values per thread).  Short prompts: 27 -> 25 us for the kernel.  In a pair, where
+        // everything else leaves the chain alone but has taken the registers for this, four (3 packed sequences of 1123 to 2992 tokens, 16
+        // heads: 88.7 -> 80.7 us); without the output stage four are 2 % slower than two.
+        if (!SCAN) setmaxnreg_inc<PAIR ? 72 : GATED ? 136 : 160>();
         const int wg = warp >> 2, j = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t t_sbf = tmem + lane_base + TM_SBF + 32 * wg, t_ds = tmem + lane_base + TM_DS + 64 * wg;
-        const size_t soff = (size_t)(64 * wg) * dv + j;          // this thread's first state element: row 64 wg, column j
-        float S[64];
+        const uint32_t t_sbf = tmem + lane_base + TM_SBF + SW / 2 * wg, t_ds = tmem + lane_base + TM_DS + SW * wg;
+        const size_t soff = (size_t)(SW * wg) * dv + j;          // this thread's first state element: row SW wg, column j
+        float S[SW];
         if (SCAN || (RELAY && seg > 0)) {               // the combine phase of every slice of this head, or the previous piece, has been written
             if (tid == 0) handover_wait(SCAN ? hv : Handover{done(), seg}, w.abort_flag);
-            named_bar_sync(3, 256);
+            named_bar_sync(3, 128 * NCH);
         }
         if (s_in) {                                     // (SCAN, RELAY, AHEAD: past the L1 cache, another SM may have written it since this launch began)
 #pragma unroll
-            for (int m = 0; m < 64; ++m) S[m] = (SCAN || RELAY || AHEAD) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
+            for (int m = 0; m < SW; ++m) S[m] = (SCAN || RELAY || AHEAD) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
         } else {
 #pragma unroll
-            for (int m = 0; m < 64; ++m) S[m] = 0.f;
+            for (int m = 0; m < SW; ++m) S[m] = 0.f;
         }
         if (nchunks > 0) {
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
+            for (int q = 0; q < SW / 32; ++q) {
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(S[32 * q + 2 * i], S[32 * q + 2 * i + 1]);
@@ -1145,15 +1149,15 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 // Y^T = -e^g (S^T K^T) as bf16; the accumulator borrows columns of dS^T, which is idle now
                 w.wait_hot(CB_X, c & 1);
                 tc_fence_after_sync();
-                uint32_t x[32], pk[16];
-                tmem_ld32(tmem + lane_base + TM_DS + 32 * wg, x);
+                uint32_t x[TW], pk[TW / 2];
+                tmem_ld_cols(tmem + lane_base + TM_DS + TW * wg, x);
                 tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float2 eg = *reinterpret_cast<const float2*>(gates + 32 * wg + 2 * i);
+                for (int i = 0; i < TW / 2; ++i) {
+                    const float2 eg = *reinterpret_cast<const float2*>(gates + TW * wg + 2 * i);
                     pk[i] = pack_bf16(-eg.x * __uint_as_float(x[2 * i]), -eg.y * __uint_as_float(x[2 * i + 1]));
                 }
-                tmem_st16(tmem + lane_base + TM_DS + 64 + 16 * wg, pk);
+                tmem_st_cols(tmem + lane_base + TM_DS + 64 + TW / 2 * wg, pk);
                 tmem_wait_st();
                 tc_fence_before_sync();
                 mbar_arrive(w.bar(CB_YREADY));
@@ -1164,22 +1168,22 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             if (tid == 0) stamp(0, c, 0);
             {
                 // v_new^T: first the decayed copy the state update waits for, then the plain one of the output product
-                uint32_t x[32], pk[16];
-                tmem_ld32(tmem + lane_base + TM_DV + 32 * wg, x);
+                uint32_t x[TW], pk[TW / 2];
+                tmem_ld_cols(tmem + lane_base + TM_DV + TW * wg, x);
                 tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float2 dec = *reinterpret_cast<const float2*>(gates + 192 + 32 * wg + 2 * i);
+                for (int i = 0; i < TW / 2; ++i) {
+                    const float2 dec = *reinterpret_cast<const float2*>(gates + 192 + TW * wg + 2 * i);
                     pk[i] = pack_bf16(__uint_as_float(x[2 * i]) * dec.x, __uint_as_float(x[2 * i + 1]) * dec.y);
                 }
-                tmem_st16(tmem + lane_base + TM_VT + 16 * wg, pk);
+                tmem_st_cols(tmem + lane_base + TM_VT + TW / 2 * wg, pk);
                 tmem_wait_st();
                 tc_fence_before_sync();
                 mbar_arrive(w.bar(CB_VREADY));
                 if (tid == 0) stamp(0, c, 1);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
-                tmem_st16(tmem + lane_base + TM_V + 16 * wg, pk);
+                for (int i = 0; i < TW / 2; ++i) pk[i] = pack_bf16(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+                tmem_st_cols(tmem + lane_base + TM_V + TW / 2 * wg, pk);
                 tmem_wait_st();
                 tc_fence_before_sync();
                 mbar_arrive(w.bar(CB_VPLAIN));
@@ -1189,13 +1193,13 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             tc_fence_after_sync();
             if (tid == 0) stamp(0, c, 2);
             const float gamma = gates[256];
-            if (GATED) {
+            if (GATED && !PAIR) {
                 // (fewer registers: 16 columns at a time, the second load in flight over half of the first)
                 uint32_t d[2][32];
                 tmem_ld32(t_ds, d[0]);
                 tmem_wait_ld();
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < SW / 16; ++q) {
                     uint32_t pk[8];
 #pragma unroll
                     for (int i = 0; i < 16; ++i) S[16 * q + i] = fmaf(gamma, S[16 * q + i], __uint_as_float(d[q >> 1][16 * (q & 1) + i]));
@@ -1207,19 +1211,19 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                 }
             } else {
                 // S^T <- e^{gC} S^T + dS^T, 32 columns at a time, both loads in flight
-                uint32_t d[2][32];
+                uint32_t d[SW / 32][32];
                 tmem_ld32(t_ds, d[0]);
                 tmem_wait_ld();
-                tmem_ld32(t_ds + 32, d[1]);
+                if (SW > 32) tmem_ld32(t_ds + 32, d[SW / 32 - 1]);
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
+                for (int q = 0; q < SW / 32; ++q) {
                     uint32_t pk[16];
 #pragma unroll
                     for (int i = 0; i < 32; ++i) S[32 * q + i] = fmaf(gamma, S[32 * q + i], __uint_as_float(d[q][i]));
 #pragma unroll
                     for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(S[32 * q + 2 * i], S[32 * q + 2 * i + 1]);
                     tmem_st16(t_sbf + 16 * q, pk);
-                    if (q == 0) tmem_wait_ld();
+                    if (SW > 32 && q == 0) tmem_wait_ld();
                 }
             }
             tmem_wait_st();
@@ -1232,18 +1236,18 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
                     float* dst = p.snaps + (((size_t)n * p.nsnap + (gc / p.snap_every - 1)) * H + h) * DK * dv +
                                  (size_t)dvb * DVB + soff;
 #pragma unroll
-                    for (int m = 0; m < 64; ++m) dst[(size_t)m * dv] = S[m];
+                    for (int m = 0; m < SW; ++m) dst[(size_t)m * dv] = S[m];
                 }
             }
         }
         if (PAIR) cluster_wait();
         if (p.sT && (RELAY || seg == p.nseg - 1) && (!PAIR || cta.half == 0)) {
 #pragma unroll
-            for (int m = 0; m < 64; ++m) p.sT[state_off + soff + (size_t)m * dv] = S[m];
+            for (int m = 0; m < SW; ++m) p.sT[state_off + soff + (size_t)m * dv] = S[m];
         }
         if (RELAY) {                                    // publish the piece; the last one leaves the counter at zero
             __threadfence();
-            named_bar_sync(3, 256);
+            named_bar_sync(3, 128 * NCH);
             // (test hook: drop_chunk == -2 makes the first piece of the first chain keep its state to itself)
             if (tid == 0 && !(p.drop_chunk == -2 && cta.z == 0 && h == 0 && dvb == 0)) {
                 __threadfence();
@@ -1252,10 +1256,10 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
     } else if (warp < OW) {
         // =============================== output warpgroup(s) ===============================
-        if (!SCAN) { if (GATED) setmaxnreg_dec<64>(); else if (!AHEAD || COMPACT) setmaxnreg_inc<136>(); }      // (AHEAD with W: 128, as launched)
+        if (!SCAN && !PAIR) { if (GATED) setmaxnreg_dec<64>(); else if (!AHEAD || COMPACT) setmaxnreg_inc<136>(); }      // (a pair: 64, AHEAD with W: 128, as launched)
         if (PAIR) cluster_arrive();
-        const int og = (warp - 8) >> 2;
-        const int j = (tid - 256) & 127, we = j >> 5;
+        const int og = (warp - 4 * NCH) >> 2;
+        const int j = tid & 127, we = j >> 5;
         const uint32_t lane_base = (uint32_t)(we * 32) << 16;
         // The accumulators are read as matrix fragments (thread: 4 value columns x 16 tokens, tokens in pairs), so that a
         // pair of tokens packs into one register and stmatrix transposes 8x8 blocks into rows of the output tile,
@@ -1409,7 +1413,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         // norm_w * silu(gate_z) of a chunk, in the fragments the output warpgroups read and ahead of them: gate_z comes by TMA,
         // the gates wait in tensor memory.  The output warpgroups used to form them as well, 0.9 of the 2.18 us that
         // they took for a chunk and that set the step of the whole kernel.
-        setmaxnreg_dec<40>();
+        setmaxnreg_dec<PAIR ? 48 : 40>();
         if (PAIR) cluster_arrive();
         const int wq = warp - OW;
         const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
@@ -1453,7 +1457,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
     } else {
         // =============================== control warpgroup ===============================
-        if (!SCAN) setmaxnreg_dec<GATED ? 40 : AHEAD && !COMPACT ? 64 : 56>();
+        if (!SCAN) setmaxnreg_dec<PAIR ? 48 : GATED ? 40 : AHEAD && !COMPACT ? 64 : 56>();
         if (PAIR) cluster_arrive();
         volatile int* const upto = w.abort_flag + 4;            // (AHEAD) chunks whose items are known to be ready
         auto load_z = [&](int c) {
@@ -1715,11 +1719,11 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             if (*w.abort_flag) drain_z(c);
         }
     }
-    if (PAIR && warp >= 8) cluster_wait();
+    if (PAIR && warp >= 4 * NCH) cluster_wait();
 }
 
 template <int MODE, int GATE, bool COMPACT>
-__global__ void __launch_bounds__(GATE != kNoGate ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
+__global__ void __launch_bounds__(GATE == kGatePair ? CHAIN_THREADS_PAIR : GATE == kGate ? CHAIN_THREADS_GATED : CHAIN_THREADS, 1)
 gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                  const __grid_constant__ CUtensorMap map_z, ChainParams p) {
@@ -1730,7 +1734,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     Waiter w{base + CS_BARS, reinterpret_cast<volatile int*>(sm + CS_MISC + 4)};
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        chain_init_bars(w, GATE, COMPACT);
+        chain_init_bars(w, GATE, COMPACT, GATE == kGatePair ? 512 : 256);
         sMisc[1] = 0;
         sMisc[5] = 0;
         fence_mbar_init();
@@ -2307,7 +2311,7 @@ gdn_scan_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (tid == 0) {
         summary_init_bars(w1, 2);
         combine_init_bars(w2);
-        chain_init_bars(w3, kNoGate, false);
+        chain_init_bars(w3, kNoGate, false, 256);
         sMisc[1] = 0;
         fence_mbar_init();
     }
@@ -2742,7 +2746,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                  : opt.gate_z ? (compact ? gdn_chain_kernel<kPlain, kGate, true> : gdn_chain_kernel<kPlain, kGate, false>)
                  : g_lean_dbg ? gdn_chain_kernel<kStamps, kNoGate, false>
                               : (compact ? gdn_chain_kernel<kPlain, kNoGate, true> : gdn_chain_kernel<kPlain, kNoGate, false>);
-    launch_cluster_after(pair ? 2 : 1, chain, grid, opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
+    launch_cluster_after(pair ? 2 : 1, chain, grid, pair ? CHAIN_THREADS_PAIR : opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
                  mqc, mk, mv, mo, mz, cp);
     count_launch();
     mark(4);
