@@ -244,6 +244,7 @@ struct PrepParams {
     int l2;                    // bit 0: the K tiles are read again by later kernels of this call and fit in L2: keep them there;
                                // bit 1: the same for the W and T2 images this kernel writes
     uint32_t tile_bytes;       // of an item's K and Q tiles, 32768 (tests: 16 more, so that the waits on them run out)
+    int split;                 // the next kernel is not the chain kernel: it waits for this one before it reads anything
     // Chains that start while this kernel still runs (see plan_ahead), or ready = nullptr:
     int* ready;                // per item, zero before and after every call: set to `readers` once the item is in memory; every chain CTA that
     int readers;               //   has taken the item counts it down by one
@@ -403,7 +404,7 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int H = p.H;
-    if (!AHEAD) pdl_trigger();          // the next kernel of the call may set itself up while this one runs
+    if (!AHEAD && p.split) pdl_trigger();        // the next kernel of the call may set itself up while this one runs
     if (warp == 4) { prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); }
     if (tid == 0) {
         mbar_init(w.bar(PB_FULL), 1); mbar_init(w.bar(PB_G), 1); mbar_init(w.bar(PB_W), 1);
@@ -423,7 +424,9 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t tmem = warp_uniform(sMisc[0]);
 
     pdl_wait();                         // the scratch may still be read, and the inputs written, by what ran before
-    if (AHEAD) pdl_trigger();           // (chains that start ahead read inputs: what ran before has to have ended first)
+    // Chains may start.  Not before this point: they read inputs before this kernel has ended, and find those of the call written, as every
+    // CTA has to come by here before one of theirs starts.
+    if (AHEAD || !p.split) pdl_trigger();
     if (blockIdx.x == 0 && tid == 0) p.ticket[1] = 0;                 // (the chain kernel's, see ChainParams::relay)
 
     // Every CTA starts with the item of its own index; further ones are handed out through a global ticket: the time per
@@ -1065,11 +1068,17 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 // here, W there.
 // MODE: what only a debug build (time stamps) or a relay needs stays out of the plain kernel: as run-time branches the relay cost
 // the other calls 1 to 2 %.
-enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2, kAhead = 3 };
+enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2, kAhead = 3, kEarly = 4 };
 template <int MODE, bool SCAN, int GATE, bool COMPACT>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
     constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay, AHEAD = MODE == kAhead;
+    // Directly behind the prepare kernel the inputs of the call are there when this one starts: only the thread that loads the items waits for
+    // that kernel to end; the state is read and converted and the first gates are formed meanwhile.  (Behind the split's kernels, which let
+    // the next one start before their own wait, all of the kernel waits.)  A call takes 0.7 to 2.8 us less: one B200, 16 heads, 64 tokens
+    // 11.1 -> 10.1 us, with the output stage 11.2 -> 9.9, 6 x 16 heads x 300 24.4 -> 22.6, 1500 tokens with the output stage 46.4 -> 43.5,
+    // 8 x 32 x 2048 222 -> 218.
+    constexpr bool EARLY = MODE == kEarly;
     constexpr bool GATED = GATE != kNoGate, PAIR = GATE == kGatePair;
     constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments that each handles at a time
     constexpr int NCH = PAIR ? 4 : 2, TW = C / NCH, SW = DK / NCH;      // chain warpgroups; tokens and state columns of each
@@ -1078,10 +1087,11 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     uint8_t* sm = cta.sm;
     const int tid = threadIdx.x, warp = SCAN ? tid >> 5 : (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int dvb = cta.dvb, h = cta.h;
-    if (!AHEAD && tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
+    if (!AHEAD && !EARLY && tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
     const int n = cta.z / p.nseg, seg = cta.z % p.nseg;
     const int H = p.H, dv = p.dv;
-    const SeqInfo sq = AHEAD ? cta.sq : seq_info(p.cu, n, p.T);
+    SeqInfo sq = AHEAD ? cta.sq : seq_info(EARLY ? nullptr : p.cu, n, p.T);
+    if (EARLY && p.cu) { const int t0 = __ldcg(p.cu + n); sq.tok0 = t0; sq.len = __ldcg(p.cu + n + 1) - t0; }     // (not from L1, like all that is read early)
     // this CTA walks chunks [seg * seg_chunks, ...) of the sequence
     const int cbeg = seg * p.seg_chunks;
     const long tok0 = sq.tok0 + (long)cbeg * C;
@@ -1123,9 +1133,9 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             if (tid == 0) handover_wait(SCAN ? hv : Handover{done(), seg}, w.abort_flag);
             named_bar_sync(3, 128 * NCH);
         }
-        if (s_in) {                                     // (SCAN, RELAY, AHEAD: past the L1 cache, another SM may have written it since this launch began)
+        if (s_in) {     // (past the L1 cache where another SM may have written it since an earlier kernel of the call began)
 #pragma unroll
-            for (int m = 0; m < SW; ++m) S[m] = (SCAN || RELAY || AHEAD) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
+            for (int m = 0; m < SW; ++m) S[m] = (SCAN || RELAY || AHEAD || EARLY) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
         } else {
 #pragma unroll
             for (int m = 0; m < SW; ++m) S[m] = 0.f;
@@ -1256,7 +1266,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
     } else if (warp < OW) {
         // =============================== output warpgroup(s) ===============================
-        if (!SCAN && !PAIR) { if (GATED) setmaxnreg_dec<64>(); else if (!AHEAD || COMPACT) setmaxnreg_inc<136>(); }      // (a pair: 64, AHEAD with W: 128, as launched)
+        if (!SCAN && !PAIR) { if (GATED) setmaxnreg_dec<64>(); else if (!(AHEAD || EARLY) || COMPACT) setmaxnreg_inc<136>(); }      // (a pair: 64, AHEAD and EARLY with W: 128, as launched)
         if (PAIR) cluster_arrive();
         const int og = (warp - 4 * NCH) >> 2;
         const int j = tid & 127, we = j >> 5;
@@ -1421,7 +1431,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         const uint32_t frag_off = (piece >> 3) * 4096 + (uint32_t)(lane & 7) * 128 + (((piece & 7) ^ (uint32_t)(lane & 7)) << 4);
         float wv[4];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) wv[m] = AHEAD ? __ldcg(p.norm_w + 32 * wq + 8 * m + (lane >> 2)) : __ldg(p.norm_w + 32 * wq + 8 * m + (lane >> 2));
+        for (int m = 0; m < 4; ++m) wv[m] = __ldcg(p.norm_w + 32 * wq + 8 * m + (lane >> 2));
         for (int c = 0; c < nchunks; ++c) {
             const uint32_t zt = base + ((c & 1) ? CS_Z1 : CS_Z) + frag_off, own = PAIR ? (uint32_t)c & 1u : 0u;
             const uint32_t t_og = tmem + lane_base + TM_OG + 32 * own;
@@ -1457,7 +1467,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
         }
     } else {
         // =============================== control warpgroup ===============================
-        if (!SCAN) setmaxnreg_dec<PAIR ? 48 : GATED ? 40 : AHEAD && !COMPACT ? 64 : 56>();
+        if (!SCAN) setmaxnreg_dec<PAIR ? 48 : GATED ? 40 : (AHEAD || EARLY) && !COMPACT ? 64 : 56>();
         if (PAIR) cluster_arrive();
         volatile int* const upto = w.abort_flag + 4;            // (AHEAD) chunks whose items are known to be ready
         auto load_z = [&](int c) {
@@ -1584,6 +1594,10 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             prefetch_tensormap(map_o);
             const uint64_t pol_done = (p.l2 & 1) ? l2_policy_evict_first() : l2_policy_evict_normal();
             const uint64_t pol_item = (p.l2 & 2) ? l2_policy_evict_first() : l2_policy_evict_normal();
+            if (EARLY) {
+                pdl_wait();
+                if (dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
+            }
             int issued = 0;                                    // five loads a chunk, in the order in which the slots come free
             int known = AHEAD ? 0 : nchunks;                   // chunks whose items are known to be ready
             for (int c = 0; c < nchunks; ++c) {
@@ -1776,7 +1790,7 @@ gdn_chain_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         } else {
             sq = seq_info(nullptr, z, p.T);
         }
-    } else {
+    } else if (MODE != kEarly) {
         pdl_wait();                     // scratch items and incoming states come from the kernels before this one
     }
     const int half = GATE == kGatePair ? (int)blockIdx.x : 0;
@@ -2550,9 +2564,10 @@ static int device_setup(int* sms_out) {
             !smem_limit(GDN_K(gdn_prep_kernel<false, false, true>), PREP_SMEM_AHEAD) || !smem_limit(GDN_K(gdn_prep_kernel<true, false, true>), PREP_SMEM_AHEAD) ||
             !smem_limit(GDN_K(gdn_prep_kernel<false, true, true>), PREP_SMEM_AHEAD) || !smem_limit(GDN_K(gdn_prep_kernel<true, true, true>), PREP_SMEM_AHEAD) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kStamps, kNoGate, false>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, true>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, true>), CHAIN_SMEM_GATED) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGatePair, false>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGatePair, false>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kNoGate, true>), CHAIN_SMEM) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kGate, true>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kGatePair, false>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kNoGate, true>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kRelay, kGate, true>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kAhead, kNoGate, true>), CHAIN_SMEM) ||
@@ -2611,8 +2626,8 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     if (pieces > 1) pieces = (nch_all + piece_chunks - 1) / piece_chunks;
     // The fused output stage on two CTAs per chain where the SMs would be idle otherwise (see GateMode).  One B200, calls with one / two:
     // 16 heads, 1500 tokens 53.5 / 45.4 us, 2 x 4000 139 / 110, 3 packed sequences of 1123 to 2992 tokens 104 / 89, 4 x 1500 67.7 / 65.4
-    // (128 CTAs: what the second one reads again shows).  The line at four chunks: 400 tokens 22.7 / 20.6 us, 200 17.3 / 17.1, 128 12.9 /
-    // 13.4, 64 11.3 / 12.4 (the cluster's start).  The lengths of packed sequences are not known here: their mean stands for them.
+    // (128 CTAs: what the second one reads again shows).  The line at four chunks: 448 tokens 21.0 / 18.3 us, 226 16.2 / 15.3, 192 13.2 /
+    // 13.0, and for 64 chains 26.9 / 25.5, 20.1 / 20.6, 17.1 / 17.9 (the cluster's start).  The lengths of packed sequences are not known here: their mean stands for them.
     // Chains on more than half of that many SMs do not take two where they can start while items are still prepared (below), which then has
     // the other SMs: 4 x 16 heads x 1500 tokens, two CTAs / early start 67.8 / 61.2 us, x 3000 116 / 102, x 6000 220 / 184, 3 x 2000 78.0 / 74.3.
     const bool many = !packed && nseg == 1 && chain_ctas * 40 > 11L * num_sms &&
@@ -2636,7 +2651,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // earlier readers ask L2 to keep them and the last reader releases them.
     const int l2 = (nseg > 1 && tokens * a.H * (uint64_t)(a.d_k + a.d_v) * 2 <= (96ull << 20)) ? (g_lean_l2_hints & 3) : 0;
     PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, nslots, a.B, a.T, a.H, opt.gate_scale, opt.eps, ticket, l2,
-                  g_lean_drop_chunk == -3 ? 32784u : 32768u};
+                  g_lean_drop_chunk == -3 ? 32784u : 32768u, nseg > 1};
     // Items without -W^T (24 % less memory traffic over both kernels, one hop more per chain step) are for calls of one segment
     // per chain and equal lengths.  A plain or raw call takes them when its chains together are bound by memory: at least three
     // fifths of the SMs busy to the end, every chain reading its own K and Q (with d_v = 256 two chains share them through
@@ -2742,10 +2757,11 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                  : ahead && pair ? gdn_chain_kernel<kAhead, kGatePair, false>
                  : ahead ? (opt.gate_z ? (compact ? gdn_chain_kernel<kAhead, kGate, true> : gdn_chain_kernel<kAhead, kGate, false>)
                                        : (compact ? gdn_chain_kernel<kAhead, kNoGate, true> : gdn_chain_kernel<kAhead, kNoGate, false>))
-                 : pair ? gdn_chain_kernel<kPlain, kGatePair, false>
-                 : opt.gate_z ? (compact ? gdn_chain_kernel<kPlain, kGate, true> : gdn_chain_kernel<kPlain, kGate, false>)
-                 : g_lean_dbg ? gdn_chain_kernel<kStamps, kNoGate, false>
-                              : (compact ? gdn_chain_kernel<kPlain, kNoGate, true> : gdn_chain_kernel<kPlain, kNoGate, false>);
+                 : g_lean_dbg && !opt.gate_z ? gdn_chain_kernel<kStamps, kNoGate, false>
+                 : nseg > 1 ? (pair ? gdn_chain_kernel<kPlain, kGatePair, false> : opt.gate_z ? gdn_chain_kernel<kPlain, kGate, false> : gdn_chain_kernel<kPlain, kNoGate, false>)
+                 : pair ? gdn_chain_kernel<kEarly, kGatePair, false>
+                 : opt.gate_z ? (compact ? gdn_chain_kernel<kEarly, kGate, true> : gdn_chain_kernel<kEarly, kGate, false>)
+                              : (compact ? gdn_chain_kernel<kEarly, kNoGate, true> : gdn_chain_kernel<kEarly, kNoGate, false>);
     launch_cluster_after(pair ? 2 : 1, chain, grid, pair ? CHAIN_THREADS_PAIR : opt.gate_z ? CHAIN_THREADS_GATED : CHAIN_THREADS, opt.gate_z ? CHAIN_SMEM_GATED : CHAIN_SMEM, stream,
                  mqc, mk, mv, mo, mz, cp);
     count_launch();

@@ -1,0 +1,68 @@
+"""The chain kernel reads the inputs of a call (initial state, gate_z, norm weight, offsets) while the prepare kernel still runs.  Here all of
+them are written by what comes just before on the stream: the result has to be bit for bit that of the same call after a
+synchronisation."""
+import pytest
+import torch
+
+import paper_2607_14568_b200 as gdn
+from workloads import get_config, make_inputs
+from gdn_testlib import to_device
+
+pytestmark = pytest.mark.gpu
+
+
+# one chunk, a tail, the line of the second CTA per chain; lengths, one of them empty; one and two CTAs per chain, items with and without W
+@pytest.mark.parametrize("H,lens,packed,pair,compact", [(2, [64], False, 0, 1), (2, [64], False, 0, 0), (2, [64], False, 1, 0), (3, [129], False, 0, 0),
+                                                        (3, [451], False, -1, -1), (2, [451] * 3, False, 0, 1), (2, [70, 0, 333], True, 0, 0),
+                                                        (2, [333, 70, 1], True, 1, 0)])
+@pytest.mark.parametrize("gated", [False, True])
+def test_inputs_written_just_before(H, lens, packed, pair, compact, gated):
+    if pair == 1 and not gated:
+        pytest.skip("two CTAs per chain belong to the output stage")
+    L, n, T = gdn.lib(), len(lens), sum(lens)
+    B = 1 if packed else n
+    x = to_device(make_inputs(get_config("short", B=B, T=T // B, H=H, init_std=0.3, seed=5)))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    z0 = torch.randn(x["v"].shape, device="cuda", generator=g).to(torch.bfloat16)
+    w0 = torch.rand(128, device="cuda", generator=g) + 0.5
+    s00 = torch.randn(n, H, 128, 128, device="cuda", generator=g) * 0.3
+    cu0 = torch.tensor([0, *torch.tensor(lens).cumsum(0).tolist()], dtype=torch.int32, device="cuda")
+    shape = (lambda t: t[0]) if packed else (lambda t: t)
+    v, z, w, s0, cu = (torch.empty_like(t) for t in (x["v"], z0, w0, s00, cu0))
+    fin, out = torch.empty_like(s00), torch.empty_like(x["v"])
+    big = torch.ones(64 << 20, device="cuda")
+
+    def write():
+        big.mul_(1.0001)                                   # the writes below are queued, not done, when the call is made
+        for dst, src in ((v, x["v"]), (z, z0), (w, w0), (s0, s00), (cu, cu0)):
+            dst.copy_(src)
+
+    def call():
+        a = [shape(x["q"]), shape(x["k"]), shape(v), shape(x["log_alpha"]), shape(x["beta"]), s0]
+        tail = [shape(out), fin] + ([cu] if packed else [])
+        if gated:
+            gdn.gdn_chunk_prefill_gated(*a, shape(z), w, 1e-6, *tail)
+        else:
+            gdn.gdn_chunk_prefill(*a, *tail)
+
+    ws = torch.empty(gdn.gdn_workspace_bytes(n, T if packed else T // B, H, 128, 128, packed), dtype=torch.uint8, device="cuda")
+    gdn.gdn_set_workspace(ws)
+    L.gdn_debug_force_segments(1); L.gdn_debug_set_pair(pair); L.gdn_debug_set_compact(compact); L.gdn_debug_set_ahead(0)
+    try:
+        write()
+        torch.cuda.synchronize()
+        call()
+        torch.cuda.synchronize()
+        want = out.clone(), fin.clone()
+        for _ in range(5):
+            for t in (v, z, w, s0, cu, out, fin):
+                t.zero_()
+            torch.cuda.synchronize()
+            write()
+            call()
+            torch.cuda.synchronize()
+            assert gdn.gdn_query_status() == 0
+            assert torch.equal(out, want[0]) and torch.equal(fin, want[1])
+    finally:
+        L.gdn_debug_force_segments(0); L.gdn_debug_set_pair(-1); L.gdn_debug_set_compact(-1); L.gdn_debug_set_ahead(1)
+        gdn.gdn_set_workspace(None)
