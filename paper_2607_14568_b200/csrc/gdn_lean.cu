@@ -1068,16 +1068,16 @@ __device__ __forceinline__ void tmem_ld_frags(uint32_t a, uint32_t (&r)[16]) { t
 // here, W there.
 // MODE: what only a debug build (time stamps) or a relay needs stays out of the plain kernel: as run-time branches the relay cost
 // the other calls 1 to 2 %.
-enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2, kAhead = 3, kEarly = 4 };
+enum ChainMode : int { kPlain = 0, kStamps = 1, kRelay = 2, kAhead = 3, kEarly = 4 };     // (kPlain: calls without a workspace, merged scan)
 template <int MODE, bool SCAN, int GATE, bool COMPACT>
 __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUtensorMap* map_k, const CUtensorMap* map_v,
                                            const CUtensorMap* map_o, const CUtensorMap* map_z, const ChainParams& p, const Cta& cta, const Waiter& w, const Handover& hv) {
     constexpr bool DBG = MODE == kStamps, RELAY = MODE == kRelay, AHEAD = MODE == kAhead;
-    // Directly behind the prepare kernel the inputs of the call are there when this one starts: only the thread that loads the items waits for
-    // that kernel to end; the state is read and converted and the first gates are formed meanwhile.  (Behind the split's kernels, which let
-    // the next one start before their own wait, all of the kernel waits.)  A call takes 0.7 to 2.8 us less: one B200, 16 heads, 64 tokens
-    // 11.1 -> 10.1 us, with the output stage 11.2 -> 9.9, 6 x 16 heads x 300 24.4 -> 22.6, 1500 tokens with the output stage 46.4 -> 43.5,
-    // 8 x 32 x 2048 222 -> 218.
+    // The inputs of the call are there when this kernel starts: only the thread that loads the items waits for the prepare kernel to end;
+    // the state is read and converted and the first gates are formed meanwhile.  Behind a combine kernel, which lets this one start after
+    // its own wait, the items are there too, and only the incoming state is waited for.  A call takes 0.7 to 2.8 us less: one B200, 16 heads,
+    // 64 tokens 11.1 -> 10.1 us, with the output stage 11.2 -> 9.9, 6 x 16 heads x 300 24.4 -> 22.6, 1500 tokens with the output stage 46.4 ->
+    // 43.5, 8 x 32 x 2048 222 -> 218; split, 2048 tokens 48.3 -> 46.1, 8192 104.6 -> 101.6, 8 heads x 8192 with the output stage 89.8 -> 83.7.
     constexpr bool EARLY = MODE == kEarly;
     constexpr bool GATED = GATE != kNoGate, PAIR = GATE == kGatePair;
     constexpr int NOUT = GATED ? 2 : 1, QN = 8 / NOUT;       // output warpgroups, eight-token fragments that each handles at a time
@@ -1133,6 +1133,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             if (tid == 0) handover_wait(SCAN ? hv : Handover{done(), seg}, w.abort_flag);
             named_bar_sync(3, 128 * NCH);
         }
+        if (EARLY && p.nseg > 1) pdl_wait();            // (the combine kernel writes it)
         if (s_in) {     // (past the L1 cache where another SM may have written it since an earlier kernel of the call began)
 #pragma unroll
             for (int m = 0; m < SW; ++m) S[m] = (SCAN || RELAY || AHEAD || EARLY) ? __ldcg(s_in + soff + (size_t)m * dv) : __ldg(s_in + soff + (size_t)m * dv);
@@ -1595,7 +1596,8 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
             const uint64_t pol_done = (p.l2 & 1) ? l2_policy_evict_first() : l2_policy_evict_normal();
             const uint64_t pol_item = (p.l2 & 2) ? l2_policy_evict_first() : l2_policy_evict_normal();
             if (EARLY) {
-                pdl_wait();
+                if (p.nseg == 1) pdl_wait();
+                else asm volatile("fence.proxy.async;" ::: "memory");       // the items are complete: the combine kernel has waited
                 if (dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
             }
             int issued = 0;                                    // five loads a chunk, in the order in which the slots come free
@@ -2196,7 +2198,10 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
         //      three products are independent); the first of them also copies the M images ----
         const uint32_t prod = (uint32_t)(warp - issue_warp);            // hi*hi, lo*hi, hi*lo
         const uint32_t aoff = (prod == 1) ? CMB_IMG / 2 : 0u, boff = (prod == 2) ? CMB_BIMG : 0u;
-        if (!SCAN) pdl_wait();
+        if (!SCAN) {
+            pdl_wait();
+            pdl_trigger();              // (not earlier: the chain kernel reads items without waiting for this kernel to end)
+        }
         auto load_m = [&](int seg) {
             const uint32_t st = seg % CMB_STAGES, full = w.bar(MB_FULL0 + st);
             const uint8_t* src = reinterpret_cast<const uint8_t*>(p.seg_mt) + ((size_t)(n * p.nseg + seg) * H + h) * CMB_IMG;
@@ -2254,7 +2259,6 @@ __global__ void __launch_bounds__(CMB_THREADS, 1) gdn_combine_kernel(CombinePara
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
-    pdl_trigger();
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0, SeqInfo{0, 0}, false};
     combine_body<false>(p, cta, w, 4);
     tc_fence_before_sync();
@@ -2563,8 +2567,7 @@ static int device_setup(int* sms_out) {
             !smem_limit(GDN_K(gdn_prep_kernel<false, true, false>), PREP_SMEM) || !smem_limit(GDN_K(gdn_prep_kernel<true, true, false>), PREP_SMEM) ||
             !smem_limit(GDN_K(gdn_prep_kernel<false, false, true>), PREP_SMEM_AHEAD) || !smem_limit(GDN_K(gdn_prep_kernel<true, false, true>), PREP_SMEM_AHEAD) ||
             !smem_limit(GDN_K(gdn_prep_kernel<false, true, true>), PREP_SMEM_AHEAD) || !smem_limit(GDN_K(gdn_prep_kernel<true, true, true>), PREP_SMEM_AHEAD) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kStamps, kNoGate, false>), CHAIN_SMEM) ||
-            !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kPlain, kGatePair, false>), CHAIN_SMEM_GATED) ||
+            !smem_limit(GDN_K(gdn_chain_kernel<kStamps, kNoGate, false>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kNoGate, false>), CHAIN_SMEM) || !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kNoGate, true>), CHAIN_SMEM) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kGate, false>), CHAIN_SMEM_GATED) || !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kGate, true>), CHAIN_SMEM_GATED) ||
             !smem_limit(GDN_K(gdn_chain_kernel<kEarly, kGatePair, false>), CHAIN_SMEM_GATED) ||
@@ -2758,7 +2761,6 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
                  : ahead ? (opt.gate_z ? (compact ? gdn_chain_kernel<kAhead, kGate, true> : gdn_chain_kernel<kAhead, kGate, false>)
                                        : (compact ? gdn_chain_kernel<kAhead, kNoGate, true> : gdn_chain_kernel<kAhead, kNoGate, false>))
                  : g_lean_dbg && !opt.gate_z ? gdn_chain_kernel<kStamps, kNoGate, false>
-                 : nseg > 1 ? (pair ? gdn_chain_kernel<kPlain, kGatePair, false> : opt.gate_z ? gdn_chain_kernel<kPlain, kGate, false> : gdn_chain_kernel<kPlain, kNoGate, false>)
                  : pair ? gdn_chain_kernel<kEarly, kGatePair, false>
                  : opt.gate_z ? (compact ? gdn_chain_kernel<kEarly, kGate, true> : gdn_chain_kernel<kEarly, kGate, false>)
                               : (compact ? gdn_chain_kernel<kEarly, kNoGate, true> : gdn_chain_kernel<kEarly, kNoGate, false>);

@@ -1,4 +1,4 @@
-"""The chain kernel reads the inputs of a call (initial state, gate_z, norm weight, offsets) while the prepare kernel still runs.  Here all of
+"""The kernels of a call read its inputs (initial state, values, gate_z, norm weight, offsets) while the one before still runs.  Here all of
 them are written by what comes just before on the stream: the result has to be bit for bit that of the same call after a
 synchronisation."""
 import pytest
@@ -11,12 +11,14 @@ from gdn_testlib import to_device
 pytestmark = pytest.mark.gpu
 
 
-# one chunk, a tail, the line of the second CTA per chain; lengths, one of them empty; one and two CTAs per chain, items with and without W
-@pytest.mark.parametrize("H,lens,packed,pair,compact", [(2, [64], False, 0, 1), (2, [64], False, 0, 0), (2, [64], False, 1, 0), (3, [129], False, 0, 0),
-                                                        (3, [451], False, -1, -1), (2, [451] * 3, False, 0, 1), (2, [70, 0, 333], True, 0, 0),
-                                                        (2, [333, 70, 1], True, 1, 0)])
+# one chunk, a tail, the line of the second CTA per chain; lengths, one of them empty; one and two CTAs per chain, items with and without W;
+# two and four segments
+@pytest.mark.parametrize("H,lens,packed,pair,compact,nseg", [
+    (2, [64], False, 0, 1, 1), (2, [64], False, 0, 0, 1), (2, [64], False, 1, 0, 1), (3, [129], False, 0, 0, 1), (3, [451], False, -1, -1, 1),
+    (2, [451] * 3, False, 0, 1, 1), (2, [70, 0, 333], True, 0, 0, 1), (2, [333, 70, 1], True, 1, 0, 1), (3, [451], False, 0, 0, 2),
+    (3, [1300], False, 1, 0, 4)])
 @pytest.mark.parametrize("gated", [False, True])
-def test_inputs_written_just_before(H, lens, packed, pair, compact, gated):
+def test_inputs_written_just_before(H, lens, packed, pair, compact, nseg, gated):
     if pair == 1 and not gated:
         pytest.skip("two CTAs per chain belong to the output stage")
     L, n, T = gdn.lib(), len(lens), sum(lens)
@@ -47,7 +49,7 @@ def test_inputs_written_just_before(H, lens, packed, pair, compact, gated):
 
     ws = torch.empty(gdn.gdn_workspace_bytes(n, T if packed else T // B, H, 128, 128, packed), dtype=torch.uint8, device="cuda")
     gdn.gdn_set_workspace(ws)
-    L.gdn_debug_force_segments(1); L.gdn_debug_set_pair(pair); L.gdn_debug_set_compact(compact); L.gdn_debug_set_ahead(0)
+    L.gdn_debug_force_segments(nseg); L.gdn_debug_set_pair(pair); L.gdn_debug_set_compact(compact); L.gdn_debug_set_ahead(0)
     try:
         write()
         torch.cuda.synchronize()
