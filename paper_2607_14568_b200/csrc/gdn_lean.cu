@@ -198,6 +198,12 @@ __device__ __forceinline__ SeqInfo seq_info(const int32_t* cu, int n, int T) {
     else    { s.tok0 = (long)n * T; s.len = T; }
     return s;
 }
+// the same past the L1 cache, for a kernel that has not waited for the one before it
+__device__ __forceinline__ SeqInfo seq_info_early(const int32_t* cu, int n, int T) {
+    SeqInfo s{(long)n * T, T};
+    if (cu) { const int t0 = __ldcg(cu + n); s.tok0 = t0; s.len = __ldcg(cu + n + 1) - t0; }
+    return s;
+}
 
 // =====================================================================================
 // prepare kernel
@@ -244,7 +250,6 @@ struct PrepParams {
     int l2;                    // bit 0: the K tiles are read again by later kernels of this call and fit in L2: keep them there;
                                // bit 1: the same for the W and T2 images this kernel writes
     uint32_t tile_bytes;       // of an item's K and Q tiles, 32768 (tests: 16 more, so that the waits on them run out)
-    int split;                 // the next kernel is not the chain kernel: it waits for this one before it reads anything
     // Chains that start while this kernel still runs (see plan_ahead), or ready = nullptr:
     int* ready;                // per item, zero before and after every call: set to `readers` once the item is in memory; every chain CTA that
     int readers;               //   has taken the item counts it down by one
@@ -404,7 +409,6 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
     const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     const int H = p.H;
-    if (!AHEAD && p.split) pdl_trigger();        // the next kernel of the call may set itself up while this one runs
     if (warp == 4) { prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); }
     if (tid == 0) {
         mbar_init(w.bar(PB_FULL), 1); mbar_init(w.bar(PB_G), 1); mbar_init(w.bar(PB_W), 1);
@@ -424,9 +428,9 @@ gdn_prep_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t tmem = warp_uniform(sMisc[0]);
 
     pdl_wait();                         // the scratch may still be read, and the inputs written, by what ran before
-    // Chains may start.  Not before this point: they read inputs before this kernel has ended, and find those of the call written, as every
-    // CTA has to come by here before one of theirs starts.
-    if (AHEAD || !p.split) pdl_trigger();
+    // The next kernel may start.  Not before this point: it and those behind it read inputs before this kernel has ended, and find those of the
+    // call written, as every CTA has to come by here before one of theirs starts.
+    pdl_trigger();
     if (blockIdx.x == 0 && tid == 0) p.ticket[1] = 0;                 // (the chain kernel's, see ChainParams::relay)
 
     // Every CTA starts with the item of its own index; further ones are handed out through a global ticket: the time per
@@ -1090,8 +1094,7 @@ __device__ __forceinline__ void chain_body(const CUtensorMap* map_q, const CUten
     if (!AHEAD && !EARLY && tid == 0 && dvb == 0 && h == 0 && cta.z == 0) *p.ticket = 0;
     const int n = cta.z / p.nseg, seg = cta.z % p.nseg;
     const int H = p.H, dv = p.dv;
-    SeqInfo sq = AHEAD ? cta.sq : seq_info(EARLY ? nullptr : p.cu, n, p.T);
-    if (EARLY && p.cu) { const int t0 = __ldcg(p.cu + n); sq.tok0 = t0; sq.len = __ldcg(p.cu + n + 1) - t0; }     // (not from L1, like all that is read early)
+    const SeqInfo sq = AHEAD ? cta.sq : EARLY ? seq_info_early(p.cu, n, p.T) : seq_info(p.cu, n, p.T);
     // this CTA walks chunks [seg * seg_chunks, ...) of the sequence
     const int cbeg = seg * p.seg_chunks;
     const long tok0 = sq.tok0 + (long)cbeg * C;
@@ -1880,7 +1883,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     const int nsum = p.nseg - 1;                      // the last segment needs no summary
     const int n = cta.z / nsum, seg = cta.z % nsum;
     const int H = p.H, dv = p.dv;
-    const SeqInfo sq = seq_info(p.cu, n, p.T);
+    const SeqInfo sq = SCAN ? seq_info(p.cu, n, p.T) : seq_info_early(p.cu, n, p.T);
     const int cbeg = seg * p.seg_chunks;
     const long tok0 = sq.tok0 + (long)cbeg * C;
     const int len = max(0, min(sq.len - cbeg * C, p.seg_chunks * C));
@@ -2022,6 +2025,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
             prefetch_tensormap(map_v);
             const uint64_t pol_keep = (p.l2 & 1) ? l2_policy_evict_last() : l2_policy_evict_normal();
             const uint64_t pol_item = (p.l2 & 2) ? l2_policy_evict_last() : l2_policy_evict_normal();
+            if (!SCAN && nchunks == 0) pdl_wait();    // (every CTA waits, so that the prepare kernel has ended when this one has)
             int c = 0;
             for (; c < nchunks; ++c) {
                 const uint32_t s = c % SUM_STAGES, sb = base + s * SUM_STAGE;
@@ -2034,6 +2038,7 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
                 tma_load_3d_hint(sb + SS_K + 8192, map_k, 64, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_V, map_v, dvb * DVB, h, tok, full, pol_keep);
                 tma_load_3d_hint(sb + SS_V + 8192, map_v, dvb * DVB + 64, h, tok, full, pol_keep);
+                if (!SCAN && c == 0) pdl_wait();     // the items come from the prepare kernel
                 bulk_load_hint(sb + SS_W, item + IT_W, 16384, full, pol_item);
                 bulk_load_hint(sb + SS_T2, item + IT_T2, 8192, full, pol_item);
                 bulk_load(sb + SS_GATES, item + IT_GATES, 1280, full);
@@ -2049,6 +2054,8 @@ __device__ __forceinline__ void summary_body(const CUtensorMap* map_k, const CUt
     }
 }
 
+// (The first K and V tiles, the identity state, and in the combine kernel the images of the initial state come before the wait for the kernel in
+// front: 2048 tokens, 16 heads 46.2 -> 45.4 us a call, 8192 102.3 -> 100.1.)
 __global__ void __launch_bounds__(SUM_THREADS, 1)
 gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    SummaryParams p) {
@@ -2072,7 +2079,6 @@ gdn_summary_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     tc_fence_after_sync();
     const uint32_t tmem = warp_uniform(sMisc[0]);
     pdl_trigger();
-    pdl_wait();                         // the scratch items come from the prepare kernel
     const Cta cta{base, sm, tmem, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, 0, SeqInfo{0, 0}, false};
     summary_body<false>(&map_k, &map_v, p, cta, w);
     tc_fence_before_sync();
@@ -2135,13 +2141,10 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
         const int m = tid;
         const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
         float s[CMB_COLS];
-        // M_seg, N_seg come from the summary kernel.  The initial state waits as well: with every kernel launched ahead of
-        // its predecessor's end, only this wait says that what ran before the call, which may have produced it, is done.
-        if (!SCAN) pdl_wait();
-        if (p.s0) {
+        if (p.s0) {                      // (there since before the prepare kernel's CTAs let the next kernel start)
             const float4* src = reinterpret_cast<const float4*>(p.s0 + (((size_t)n * H + h) * DK + m) * dv + j0);
 #pragma unroll
-            for (int q = 0; q < CMB_COLS / 4; ++q) { const float4 x = __ldg(src + q); s[4 * q] = x.x; s[4 * q + 1] = x.y; s[4 * q + 2] = x.z; s[4 * q + 3] = x.w; }
+            for (int q = 0; q < CMB_COLS / 4; ++q) { const float4 x = __ldcg(src + q); s[4 * q] = x.x; s[4 * q + 1] = x.y; s[4 * q + 2] = x.z; s[4 * q + 3] = x.w; }
         } else {
 #pragma unroll
             for (int j = 0; j < CMB_COLS; ++j) s[j] = 0.f;
@@ -2158,7 +2161,7 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
             float4 nv[CMB_COLS / 4];
             const float4* nsrc = reinterpret_cast<const float4*>(p.seg_n + seg_off(seg) + (size_t)m * dv + j0);
 #pragma unroll
-            for (int q = 0; q < CMB_COLS / 4; ++q) nv[q] = SCAN ? __ldcg(nsrc + q) : __ldg(nsrc + q);
+            for (int q = 0; q < CMB_COLS / 4; ++q) if (SCAN || seg > 0) nv[q] = __ldcg(nsrc + q);
 #pragma unroll
             for (int j = 0; j < CMB_COLS; ++j) {
                 const __nv_bfloat16 hi = __float2bfloat16_rn(s[j]);
@@ -2171,6 +2174,11 @@ __device__ __forceinline__ void combine_body(const CombineParams& p, const Cta& 
             tc_fence_before_sync();
             mbar_arrive(w.bar(MB_BREADY));
             store_sin(seg);              // S_in of this segment drains while the product runs
+            if (!SCAN && seg == 0) {     // M_seg, N_seg come from the summary kernel
+                pdl_wait();
+#pragma unroll
+                for (int q = 0; q < CMB_COLS / 4; ++q) nv[q] = __ldcg(nsrc + q);
+            }
             w.wait_hot(MB_D, seg & 1);
             tc_fence_after_sync();
 #pragma unroll
@@ -2654,7 +2662,7 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     // earlier readers ask L2 to keep them and the last reader releases them.
     const int l2 = (nseg > 1 && tokens * a.H * (uint64_t)(a.d_k + a.d_v) * 2 <= (96ull << 20)) ? (g_lean_l2_hints & 3) : 0;
     PrepParams pp{a.log_alpha, a.beta, a.cu_seqlens, ws, nslots, a.B, a.T, a.H, opt.gate_scale, opt.eps, ticket, l2,
-                  g_lean_drop_chunk == -3 ? 32784u : 32768u, nseg > 1};
+                  g_lean_drop_chunk == -3 ? 32784u : 32768u};
     // Items without -W^T (24 % less memory traffic over both kernels, one hop more per chain step) are for calls of one segment
     // per chain and equal lengths.  A plain or raw call takes them when its chains together are bound by memory: at least three
     // fifths of the SMs busy to the end, every chain reading its own K and Q (with d_v = 256 two chains share them through
