@@ -2688,17 +2688,19 @@ int launch_lean(const PrefillArgs& a, void* workspace, size_t workspace_bytes, c
     };
     const int per_seq = a.H * (a.d_v / DVB) * (pair ? 2 : 1);         // chain CTAs of a sequence
     // Chains that start while the prepare kernel still runs, as the items of their first chunks are ready (AheadPlan; a step and the least gain
-    // in sixteenths of an item on an SM, 2.6 us with W and 2.0 without).  The hand-over costs about 6 us a call, so equal lengths take it where
-    // the plan says that it gains more; with d_v = 256, where calls of the same size came out 6 % faster or slower, twice that.  Packed
-    // lengths are known on the device only, which decides again; here the line is the number of items: with few of them all are in
-    // flight at once.  Measured without / with, one B200: 2 x 24 heads x 4096 tokens 121 / 110 us, 4 x 12 x 8192 221 / 191, 4 x 16 x 2048 73.0 / 67.1,
-    // 3 x 12 x 3508 93.8 / 83.9; the line for equal lengths: 3 x 16 x 1024 38.1 / 36.0, 4 x 32 x 4096 190 / 193 (not taken), 3 x 32 x 768
-    // 38.9 / 40.5 (not taken).  Packed, 16 heads: 590 to 7880 tokens 240 / 203 us, 37 to 2320 78.1 / 70.6; 8 heads 62.3 / 57.7; uniform lengths
-    // lose 2 to 4 % (6 x 800 tokens, 32 heads 88.3 / 90.1), few items 3 to 5 %, and two CTAs on each of many chains 6 % (not taken).
+    // in sixteenths of an item on an SM, 2.6 us with W and 2.0 without).  The hand-over costs about 8 us a call more than kEarly, so equal lengths
+    // take it where the plan says that it gains more; with W and chains on more than a third of the SMs, which contend for
+    // memory with the prepare kernel, only for twice that, on more than four ninths not at all (3 x 24 heads x 1500 tokens, without / with 60.9 / 63.9 us, 4 x 20 x 4096 150 / 153), and with d_v = 256, where calls of
+    // the same size came out 6 % faster or slower, for three times that.  Packed lengths are known on the device only, which decides
+    // again; here the line is the number of items: with few of them all are in flight at once.  Measured without / with, one B200: 4 x 12 heads
+    // x 8192 221 / 191 us, 4 x 24 x 4096 (no W) 181 / 166, 4 x 16 x 4096 131 / 126, 3 x 16 x 1500 50.5 / 48.7, with the output stage 4 x 16 x 1500
+    // 69.0 / 59.3; the line for equal lengths: 2 x 24 x 1500 50.2 / 51.7, 4 x 16 x 1500 57.9 / 58.1, 4 x 16 x 1024 40.6 / 41.9 (not taken).
+    // Packed, 16 heads: 590 to 7880 tokens 205 / 179 us, 786 to 3322 88.0 / 81.1, 222 to 1654 59.5 / 57.5; at 14 items a pair of SMs 48.0 / 51.1, 47.9 / 48.8
+    // (not taken); two CTAs on each of many chains lose 6 % (not taken).
     const int D = a.d_v / DVB;
-    const AheadPlan plan{num_sms, per_seq, compact ? 18 : pair ? 8 : 12, compact ? 128 : D > 1 ? 160 : 72};
-    const bool gains = packed ? a.B <= 32 && !(pair && chain_ctas * 40 > 13L * num_sms) && 2 * nitems > (D > 1 ? 24L : chain_ctas * 20 <= 13L * num_sms ? 12L : 21L) * num_sms
-                              : plan.gains(nch_all, (long)a.B * nch_all, (long)a.B * nch_all * a.H);
+    const AheadPlan plan{num_sms, per_seq, compact ? 18 : pair ? 8 : 12, compact ? 128 : D > 1 ? (packed ? 160 : 240) : packed || chain_ctas * 3 <= num_sms ? 72 : 140};
+    const bool gains = packed ? a.B <= 32 && !(pair && chain_ctas * 40 > 13L * num_sms) && 2 * nitems > (D > 1 ? 24L : chain_ctas * 20 <= 13L * num_sms ? 18L : 21L) * num_sms
+                              : (compact || D > 1 || pair || chain_ctas * 9 <= 4L * num_sms) && plan.gains(nch_all, (long)a.B * nch_all, (long)a.B * nch_all * a.H);
     const bool ahead = tail_free && g_lean_ahead && nseg == 1 && pieces == 1 && !g_lean_dbg && tokens > 0 && (gains || (g_lean_ahead == 2 && (!packed || a.B <= 32)));
     int* const ready = ahead ? reinterpret_cast<int*>(static_cast<uint8_t*>(workspace) + ready_offset(workspace_bytes)) : nullptr;
     if (ahead) {
