@@ -250,7 +250,7 @@ struct PrepParams {
     int l2;                    // bit 0: the K tiles are read again by later kernels of this call and fit in L2: keep them there;
                                // bit 1: the same for the W and T2 images this kernel writes
     uint32_t tile_bytes;       // of an item's K and Q tiles, 32768 (tests: 16 more, so that the waits on them run out)
-    // Chains that start while this kernel still runs (see plan_ahead), or ready = nullptr:
+    // Chains that start while this kernel still runs (see AheadPlan), or ready = nullptr:
     int* ready;                // per item, zero before and after every call: set to `readers` once the item is in memory; every chain CTA that
     int readers;               //   has taken the item counts it down by one
     AheadPlan plan;
@@ -2503,7 +2503,7 @@ int lean_init_workspace(void* workspace, size_t bytes) {
            cudaMemset(static_cast<uint8_t*>(workspace) + ready_offset(bytes), 0, ready_bytes(bytes)) == cudaSuccess ? GDN_OK : GDN_ERR_CUDA;
 }
 
-// Launch a kernel that may begin (set-up only, up to its pdl_wait) before the previous kernel in the stream ends, in clusters of so many CTAs.
+// Launch a kernel that may begin (set-up and reads of inputs, up to its pdl_wait) before the previous kernel in the stream ends, in clusters of so many CTAs.
 template <typename... KArgs, typename... Args>
 static void launch_cluster_after(int cluster, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
